@@ -59,6 +59,32 @@ static void qlaunch(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, 
 // --------------------------------------------------------------------------
 // block reduction helpers (fixed order: deterministic for a fixed launch shape)
 // --------------------------------------------------------------------------
+// sums over a warp of five values each lane holds; lane 0 receives them.  Two
+// exchanges first split the values over the lanes (4 + 2 additions), so the
+// warp issues 10 FP64 additions instead of 25.
+__device__ __forceinline__ void warp_sum5(double& a, double& b, double& c, double& d, double& e) {
+  const unsigned FULL = 0xffffffffu;
+  const int lane = (threadIdx.y * BX + threadIdx.x) & 31;
+  const bool b4 = lane & 16, b3 = lane & 8;
+  // lanes 0..15 keep a, b, e, lanes 16..31 keep c, d (and a zero)
+  double x = (b4 ? c : a) + __shfl_xor_sync(FULL, b4 ? a : c, 16);
+  double y = (b4 ? d : b) + __shfl_xor_sync(FULL, b4 ? b : d, 16);
+  double z = e + __shfl_xor_sync(FULL, e, 16);  // the same on both halves
+  // lanes with bit 3 clear keep x, the others y
+  double w = (b3 ? y : x) + __shfl_xor_sync(FULL, b3 ? x : y, 8);
+  // e on the lanes with bit 2 set in a register of its own: two values, three exchanges
+  z += __shfl_xor_sync(FULL, z, 8);
+  const bool b2 = lane & 4;
+  double wz = (b2 ? z : w) + __shfl_xor_sync(FULL, b2 ? w : z, 4);
+  wz += __shfl_xor_sync(FULL, wz, 2);
+  wz += __shfl_xor_sync(FULL, wz, 1);
+  a = __shfl_sync(FULL, wz, 0);
+  b = __shfl_sync(FULL, wz, 8);
+  c = __shfl_sync(FULL, wz, 16);
+  d = __shfl_sync(FULL, wz, 24);
+  e = __shfl_sync(FULL, wz, 4);
+}
+
 template <int NV>
 __device__ __forceinline__ void block_sum_store(double (&val)[NV], double* part, int nmax_first) {
   // first `nmax_first` values are reduced with max, the rest with sum.  The
@@ -67,6 +93,7 @@ __device__ __forceinline__ void block_sum_store(double (&val)[NV], double* part,
   // 64-bit integers, off the FP64 pipe.
   __shared__ double sh[NT / 32][NV];
   int lane = (threadIdx.y * BX + threadIdx.x) & 31, warp = (threadIdx.y * BX + threadIdx.x) >> 5;
+  if constexpr (NV == 10) warp_sum5(val[5], val[6], val[7], val[8], val[9]);
 #pragma unroll
   for (int q = 0; q < NV; ++q) {
     double x = val[q];
@@ -77,7 +104,7 @@ __device__ __forceinline__ void block_sum_store(double (&val)[NV], double* part,
         b = c > b ? c : b;
       }
       x = __longlong_as_double(b);
-    } else {
+    } else if (NV != 10) {
       for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
     }
     if (lane == 0) sh[warp][q] = x;
@@ -86,10 +113,16 @@ __device__ __forceinline__ void block_sum_store(double (&val)[NV], double* part,
   if (warp == 0) {
 #pragma unroll
     for (int q = 0; q < NV; ++q) {
-      double x = lane < NT / 32 ? sh[lane][q] : (q < nmax_first ? 0.0 : 0.0);
-      for (int o = 16; o > 0; o >>= 1) {
-        double y = __shfl_down_sync(0xffffffffu, x, o);
-        x = (q < nmax_first) ? fmax(x, y) : x + y;
+      double x = sh[lane & (NT / 32 - 1)][q];  // lane 0 reduces the values of lanes 0 .. NT/32 - 1
+      if (q < nmax_first) {
+        long long b = __double_as_longlong(x);
+        for (int o = NT / 64; o > 0; o >>= 1) {
+          long long c = __shfl_down_sync(0xffffffffu, b, o);
+          b = c > b ? c : b;
+        }
+        x = __longlong_as_double(b);
+      } else {
+        for (int o = NT / 64; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
       }
       if (lane == 0) part[(blockIdx.y * gridDim.x + blockIdx.x) * NV + q] = x;
     }
@@ -124,6 +157,68 @@ __global__ void k_finalize(const double* part, int nparts, int nv, int nmax_firs
 // residual r = f - N(x) (mode 0, optional norms) or f += N(x) (mode 1)
 // thread (i,j): cell families at (i,j), u-edge (i,j) and v-edge (i,j)
 // --------------------------------------------------------------------------
+// The FP64 primitive operator in the fewest FP64 instructions (the pipe that
+// bounds the kernels that evaluate it): sums over the four faces of unscaled
+// differences, scaled once by the level's constants.
+// sum over the faces of (m(c^n) of both cells) (d mu + alpha d p): 2 h^2 Pe
+// times the diffusion of N_c
+template <typename T>
+__device__ __forceinline__ T flux_sum(const Prm<T>& P, const Lv<T>& L, int k) {
+  const int W = L.pitch;
+  const T *mob = L.mobn, *mu = L.mu, *p = L.p;
+  const int off[4] = {1, -1, W, -W};
+  T mk = mob[k], s = T(0);
+  if constexpr (sizeof(T) == 8) {
+    T fk = mu[k] + P.alpha * p[k];
+#pragma unroll
+    for (int f = 0; f < 4; ++f) {
+      int q = k + off[f];
+      s += (mk + mob[q]) * (mu[q] + P.alpha * p[q] - fk);
+    }
+  } else {  // differences first: the sums would round at the fields' own size
+#pragma unroll
+    for (int f = 0; f < 4; ++f) {
+      int q = k + off[f];
+      s += (mk + mob[q]) * ((mu[q] - mu[k]) + P.alpha * (p[q] - p[k]));
+    }
+  }
+  return s;
+}
+// the advection (e1e2) of N_c
+template <typename T>
+__device__ __forceinline__ T adv_sum(const Lv<T>& L, int k) {
+  const int W = L.pitch;
+  const T* rn = L.rhon;
+  return rn[k + 1] * L.Tx[k] * L.u[k] + rn[k - 1] * L.Tx[k - 1] * L.u[k - 1] +
+         rn[k + W] * L.Ty[k] * L.v[k] + rn[k - W] * L.Ty[k - W] * L.v[k - W];
+}
+// (pm-num-chem) (op_mu with its constants folded): with S = rho + rho^n, A(c) =
+// c (c - 1), 8 rho^{n+1/2} g = S (A + A^n)(c + c^n - 1) and 8 (F + F^n)/2 =
+// A^2 + (A^n)^2
+template <typename T>
+__device__ __forceinline__ T chem_full(const Prm<T>& P, const Lv<T>& L, int k, T rk,
+                                       const T (&rq)[4]) {
+  const int W = L.pitch;
+  const T *c = L.c, *cn = L.cn, *rn = L.rhon;
+  const int off[4] = {1, -1, W, -W};
+  T ck = c[k], cnk = cn[k], rnk = rn[k];
+  T S = rk + rnk, ch = ck + cnk;
+  T A = ck * ck - ck, An = cnk * cnk - cnk;
+  T G2 = T(0), div = T(0), SD = T(0);
+#pragma unroll
+  for (int f = 0; f < 4; ++f) {
+    int q = k + off[f];
+    T d = c[q] - ck, D = (c[q] + cn[q]) - ch;
+    G2 += d * d;
+    div += (rq[f] + rn[q]) * D;
+    SD += D;
+  }
+  div += S * SD;
+  T E = L.k.K8 * (A * A + An * An) + L.k.L4 * (L.k.hih2 * G2 + L.Gn[k]);
+  return rk * L.mu[k] + L.k.L8 * div - L.k.K8 * (S * ((A + An) * (ch - T(1)))) +
+         P.alpha * rk * rnk * E;
+}
+
 // r = f - N(x) (MODE 0; val receives |r| and r^2 per family) or f += N(x) (MODE 1)
 // at thread (i,j): cell families at (i,j), u-edge (i,j) and v-edge (i,j)
 template <typename T, int MODE, class Form>
@@ -133,16 +228,18 @@ __device__ __forceinline__ void residual_cell(const Prm<T>& P, const Lv<T>& L, i
   bool hu = i <= L.uhi(), hv = j < L.m2;
   T nc, nm, np, nu, nv;
   if constexpr (std::is_same<Form, FullForm>::value) {
-    // rho(c) of the cell and its neighbours, shared by the five rows
+    // rho(c) of the cell and its neighbours, shared by the five rows, and the
+    // flux sum shared by N_c and N_p
     const int W = L.pitch;
     const T* rc = L.rhoc;
     T rk = rc[k];
     const T rq[4] = {rc[k + 1], rc[k - 1], rc[k + W], rc[k - W]};
-    nc = op_c(P, L, k, rk);
-    nm = op_mu(P, L, k, rk, rq);
-    np = op_p(P, L, k);
-    nu = op_u(P, L, k, T(0.5) * (rk + rq[0]));  // also on boundary edges (padded arrays); masked below
-    nv = op_v(P, L, k, T(0.5) * (rk + rq[2]));  // also on boundary edges (padded arrays); masked below
+    T flux = flux_sum(P, L, k);
+    nc = rk * (L.c[k] - L.cn[k]) * P.idt + adv_sum(L, k) - L.k.dif * flux;
+    nm = chem_full(P, L, k, rk, rq);
+    np = (L.u[k] - L.u[k - 1] + L.v[k] - L.v[k - W]) * L.ih - L.k.adif * flux;
+    nu = op_u(P, L, k, rk + rq[0]);  // also on boundary edges (padded arrays); masked below
+    nv = op_v(P, L, k, rk + rq[2]);  // also on boundary edges (padded arrays); masked below
   } else if constexpr (std::is_same<Form, ProjForm>::value) {
     const int W = L.pitch;
     const T* rc = L.rhoc;
@@ -153,8 +250,8 @@ __device__ __forceinline__ void residual_cell(const Prm<T>& P, const Lv<T>& L, i
     nc = opp_c_w(P, L, k, rq, w);
     nm = op_mu_r(P, L, k, rk, rq, L.rhon[k]);
     np = opp_p_w(P, L, k, w);
-    nu = op_u<T, false>(P, L, k, T(0.5) * (rk + rq[0]));  // also on boundary edges (padded arrays); masked below
-    nv = op_v<T, false>(P, L, k, T(0.5) * (rk + rq[2]));  // also on boundary edges (padded arrays); masked below
+    nu = op_u<T, false>(P, L, k, rk + rq[0]);  // also on boundary edges (padded arrays); masked below
+    nv = op_v<T, false>(P, L, k, rk + rq[2]);  // also on boundary edges (padded arrays); masked below
   } else {
     nc = Form::Nc(P, L, k);
     nm = Form::Nmu(P, L, k);
@@ -221,6 +318,55 @@ static int residual_rows(const Lv<T>& L) {
 // of each cell with (i + j) % 2 == colour; neighbours frozen.  Faces on
 // Neumann walls do not contribute (their ghost follows the cell).
 // --------------------------------------------------------------------------
+// ch_system for the FP64 primitive form, with the constants and the terms
+// common to the residuals and the Jacobian folded (chem_full's notation; E =
+// K ((F + F^n)/2) + (Lam/4) Gbar): about 115 FP64 instructions where the
+// unfolded sums take about 190.  On a wall face the ghost's c and c^n are the
+// cell's own, so its differences vanish and only the coefficients of c (2 rho
+// sums) and the mobilities need the face left out.
+template <typename T>
+__device__ __forceinline__ void ch_system_full(const Prm<T>& P, const Lv<T>& L, int i, int j,
+                                               T (&J)[2][2], T (&R)[2]) {
+  const int W = L.pitch;
+  const int k = L.at(i, j);
+  const int off[4] = {1, -1, W, -W};
+  const bool wall[4] = {!L.px && i == L.m1, !L.px && i == 1, j == L.m2, j == 1};
+  const T *c = L.c, *cn = L.cn, *rn = L.rhon, *rc = L.rhoc, *mob = L.mobn, *mu = L.mu, *p = L.p;
+  T ck = c[k], cnk = cn[k], rk = rc[k], rnk = rn[k], muk = mu[k];
+  T mk = mob[k], fk = muk + P.alpha * p[k];
+  T S = rk + rnk, ch = ck + cnk;
+  T flux = T(0), sm = T(0), G2 = T(0), sd = T(0), div = T(0), SD = T(0), SW = T(0);
+#pragma unroll
+  for (int f = 0; f < 4; ++f) {
+    const int q = k + off[f];
+    T m = mk + mob[q], cq = c[q];
+    flux += m * (mu[q] + P.alpha * p[q] - fk);
+    T d = cq - ck, D = (cq + cn[q]) - ch, H = rc[q] + rn[q];
+    G2 += d * d;
+    sd += d;
+    div += H * D;
+    SD += D;
+    sm += wall[f] ? T(0) : m;
+    SW += wall[f] ? T(0) : H;
+  }
+  const int open = 4 - (wall[0] + wall[1] + wall[2] + wall[3]);
+  SW += (open == 4 ? T(4) : open == 3 ? T(3) : open == 2 ? T(2) : open == 1 ? T(1) : T(0)) * S;
+  div += S * SD;
+  T dck = ck - cnk, ar = -P.alpha * rk, drho = ar * rk, r = ar * rnk;
+  T dr = -P.alpha * rnk * drho;
+  T A = ck * ck - ck, An = cnk * cnk - cnk, sA = A + An, t = ch - T(1), g4 = sA * t;
+  T Gs = L.k.hih2 * G2 + L.Gn[k];
+  T E = L.k.K8 * (A * A + An * An) + L.k.L4 * Gs;
+  R[0] = rk * dck * P.idt - L.fc[k] + adv_sum(L, k) - L.k.dif * flux;
+  R[1] = rk * muk - L.fmu[k] + L.k.L8 * div - L.k.K8 * (S * g4) - r * E;
+  T tc = T(2) * ck - T(1);
+  J[0][0] = (rk + drho * dck) * P.idt;
+  J[0][1] = L.k.dif * sm;
+  J[1][0] = drho * (muk + L.k.L8 * SD - L.k.K8 * g4) - L.k.K8 * (S * (tc * t + sA)) -
+            r * (L.k.K4 * (A * tc) - L.k.L4h * sd) - dr * E - L.k.L8 * SW;
+  J[1][1] = rk;
+}
+
 // The 2x2 CH system of cell (i,j): residuals R = N - f of (N_c, N_mu) and their
 // Jacobian J in (c, mu), neighbours frozen, at the full values c, mu
 template <typename T, class Form>
@@ -229,6 +375,10 @@ __device__ __forceinline__ void ch_system(const Prm<T>& P, const Lv<T>& L, int i
   const int W = L.pitch;
   int k = L.at(i, j);
   const int off[4] = {1, -1, W, -W};
+  if constexpr (std::is_same<Form, FullForm>::value) {
+    ch_system_full(P, L, i, j, J, R);
+    return;
+  }
   // rho(c) of the cell and its four neighbours, shared by N_c, N_mu and J
   T rho, rq4[4];
   rho = Form::rho(P, L, k);
@@ -236,10 +386,7 @@ __device__ __forceinline__ void ch_system(const Prm<T>& P, const Lv<T>& L, int i
   for (int f = 0; f < 4; ++f) rq4[f] = Form::rho(P, L, k + off[f]);
   T Rc, Rm;
   T wf[4];  // projection method: the face velocities u^{n+1} (E, W, N, S)
-  if constexpr (std::is_same<Form, FullForm>::value) {
-    Rc = op_c(P, L, k, rho) - L.fc[k];
-    Rm = op_mu(P, L, k, rho, rq4) - L.fmu[k];
-  } else if constexpr (std::is_same<Form, ProjForm>::value) {
+  if constexpr (std::is_same<Form, ProjForm>::value) {
     proj_faces(P, L, i, j, rho, rq4, wf);
     Rc = opp_c_w(P, L, k, rq4, wf) - L.fc[k];
     Rm = op_mu_r(P, L, k, rho, rq4, L.rhon[k]) - L.fmu[k];
@@ -347,6 +494,30 @@ __device__ __forceinline__ T proj_face_team(const Prm<T>& P, const Lv<T>& L, int
   return open ? vel[a] + (st - dp) * P.iM / (Ar * P.idt) - grav : T(0);
 }
 
+// sums over the four lanes of a team of eight values each lane holds, every
+// lane receiving all eight: the first exchange halves what a lane adds up
+// (4 + 2 additions a lane where eight butterflies take 16; each addition is
+// that of team_sum, so the sums are the same)
+__device__ __forceinline__ void team_sum8(double (&v)[8]) {
+  const unsigned FULL = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  const bool b0 = lane & 1, b1 = lane & 2;
+  double r[4], t[2];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    double send = b0 ? v[i] : v[i + 4], keep = b0 ? v[i + 4] : v[i];
+    r[i] = keep + __shfl_xor_sync(FULL, send, 1);
+  }
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    double send = b1 ? r[i] : r[i + 2], keep = b1 ? r[i + 2] : r[i];
+    t[i] = keep + __shfl_xor_sync(FULL, send, 2);
+  }
+#pragma unroll
+  for (int m = 0; m < 8; ++m)
+    v[m] = __shfl_sync(FULL, t[m & 1], (lane & 28) | (m >> 2) | (m & 2));
+}
+
 // The CH rows of cell (i,j) for a team of four lanes (lane & 3 = q: face W,
 // E, S, N; open = face q is not a wall): residuals Rc = N_c - f_c,
 // Rm = N_mu - f_mu and the 2x2 Jacobian of ch_system, and for the coupled
@@ -360,9 +531,59 @@ struct ChRows {
   T sm, sflux, drho, gq;
 };
 
+// ch_team_rows for the FP64 primitive form: ch_system_full's sums, a face a lane
+__device__ __forceinline__ ChRows<double> ch_team_rows_full(const Prm<double>& P,
+                                                            const Lv<double>& L, int i, int j,
+                                                            int q, bool open) {
+  typedef double T;
+  const int W = L.pitch;
+  const int d = q >> 1;
+  const int k = L.at(i, j);
+  const int nq = k + (q == 0 ? -1 : q == 1 ? 1 : q == 2 ? -W : W);
+  const int kf = q == 0 ? k - 1 : (q == 2 ? k - W : k);  // edge of face q
+  const T *c = L.c, *cn = L.cn, *rn = L.rhon, *rc = L.rhoc, *mob = L.mobn;
+  T ck = c[k], cnk = cn[k], rk = rc[k], rnk = rn[k], muk = L.mu[k];
+  T cq = c[nq], rnq = rn[nq];
+  T gq = rnq * (d ? L.Ty[kf] : L.Tx[kf]);  // rho^n D c^n / 2 at face q
+  T m = mob[k] + mob[nq];
+  T S = rk + rnk, ch = ck + cnk, dq = cq - ck, D = (cq + cn[nq]) - ch, H = rc[nq] + rnq;
+  T v[8] = {m * (L.mu[nq] + P.alpha * L.p[nq] - (muk + P.alpha * L.p[k])),
+            open ? m : T(0),
+            gq * (d ? L.v[kf] : L.u[kf]),
+            dq * dq,
+            dq,
+            (H + S) * D,
+            D,
+            open ? H + S : T(0)};
+  team_sum8(v);
+  const T flux = v[0], sm = v[1], adv = v[2], G2 = v[3], sd = v[4], div = v[5], SD = v[6],
+          SW = v[7];
+  T dck = ck - cnk, ar = -P.alpha * rk, drho = ar * rk, r = ar * rnk;
+  T dr = -P.alpha * rnk * drho;
+  T A = ck * ck - ck, An = cnk * cnk - cnk, sA = A + An, t = ch - T(1), g4 = sA * t;
+  T Gs = L.k.hih2 * G2 + L.Gn[k];
+  T E = L.k.K8 * (A * A + An * An) + L.k.L4 * Gs;
+  T tc = T(2) * ck - T(1);
+  ChRows<T> R;
+  R.Rc = rk * dck * P.idt - L.fc[k] + adv - L.k.dif * flux;
+  R.Rm = rk * muk - L.fmu[k] + L.k.L8 * div - L.k.K8 * (S * g4) - r * E;
+  R.J11 = (rk + drho * dck) * P.idt;
+  R.J12 = L.k.dif * sm;
+  R.J21 = drho * (muk + L.k.L8 * SD - L.k.K8 * g4) - L.k.K8 * (S * (tc * t + sA)) -
+          r * (L.k.K4 * (A * tc) - L.k.L4h * sd) - dr * E - L.k.L8 * SW;
+  R.J22 = rk;
+  R.sm = sm;
+  R.sflux = flux;
+  R.drho = drho;
+  R.gq = gq;
+  return R;
+}
+
 template <typename T, class Form>
 __device__ __forceinline__ ChRows<T> ch_team_rows(const Prm<T>& P, const Lv<T>& L, int i, int j, int q,
                                                   bool open) {
+  if constexpr (std::is_same<Form, FullForm>::value)
+    return ch_team_rows_full(P, L, i, j, q, open);
   const int W = L.pitch;
   const int d = q >> 1;
   const T ih2 = L.ih2;
@@ -382,7 +603,7 @@ __device__ __forceinline__ ChRows<T> ch_team_rows(const Prm<T>& P, const Lv<T>& 
   T dlt = cq - ck;
   // face sums: diffusion flux (N_c and the mass row), sum A m over open faces,
   // advection of N_c, and the Jacobian's G, dG/dc and d(div)/dc terms
-  T sflux = team_sum<T>(T(0.5) * am * ((L.mu[nq] - L.mu[k]) + P.alpha * (L.p[nq] - L.p[k])));
+  T sflux = team_sum<T>(am * ((L.mu[nq] - L.mu[k]) + P.alpha * (L.p[nq] - L.p[k])));
   T sm = team_sum<T>(open ? am : T(0));
   T sadv = team_sum<T>(gq * (d ? L.v[kf] : L.u[kf]));
   T G2 = team_sum<T>(dlt * dlt);
@@ -394,7 +615,7 @@ __device__ __forceinline__ ChRows<T> ch_team_rows(const Prm<T>& P, const Lv<T>& 
     wq = proj_face_team(P, L, k, q, open, rho, rq);
     // advection a(rho(c) D c u^{n+1}) of (pj-num-phase) by faces
     T sadvp = team_sum<T>(T(0.5) * rq * ((q & 1) ? (cq - ck) : (ck - cq)) * L.ih * wq);
-    Nc = rnk * (ck - cnk) * P.idt + sadvp - P.iPe * ih2 * sflux;
+    Nc = rnk * (ck - cnk) * P.idt + sadvp - L.k.dif * sflux;
     T sdv = team_sum<T>((rh + T(0.5) * (rq + rn[nq])) * ((cq + cn[nq]) - chk));
     T r = -P.alpha * rho * rnk;
     T bulk = rh * gsec(ck, cnk) + T(0.5) * (Fdw(ck) + Fdw(cnk)) * r;
@@ -405,7 +626,7 @@ __device__ __forceinline__ ChRows<T> ch_team_rows(const Prm<T>& P, const Lv<T>& 
     const T *e = L.c, *B = L.Bc;
     T ek = e[k], Ck = B[k];
     T rC = rho_of(P, Ck);
-    Nc = ek * (rho + rsec_(P, rho, rC) * L.Bdc[k]) * P.idt + sadv - P.iPe * ih2 * sflux;
+    Nc = ek * (rho + rsec_(P, rho, rC) * L.Bdc[k]) * P.idt + sadv - L.k.dif * sflux;
     T dC = B[nq] - Ck, de = e[nq] - ek;
     T rCq = rho_of(P, B[nq]);
     T dr = rsec_(P, rho, rC) * ek;
@@ -422,7 +643,7 @@ __device__ __forceinline__ ChRows<T> ch_team_rows(const Prm<T>& P, const Lv<T>& 
     T dgrad = T(0.25) * P.Lam * (T(0.5) * sdGe * ih2 * r_new + (T(0.5) * sGC * ih2 + L.Gn[k]) * d_r);
     Nm = rho * L.mu[k] + dr * L.Bmu[k] - P.K * dbulk - dgrad + P.Lam * T(0.25) * ih2 * sddiv;
   } else {
-    Nc = rho * (ck - cnk) * P.idt + sadv - P.iPe * ih2 * sflux;
+    Nc = rho * (ck - cnk) * P.idt + sadv - L.k.dif * sflux;
     T sdv = team_sum<T>((rh + T(0.5) * (rq + rn[nq])) * ((cq + cn[nq]) - chk));
     T r = -P.alpha * rho * rnk;
     T bulk = rh * gsec(ck, cnk) + T(0.5) * (Fdw(ck) + Fdw(cnk)) * r;
@@ -434,7 +655,7 @@ __device__ __forceinline__ ChRows<T> ch_team_rows(const Prm<T>& P, const Lv<T>& 
   R.Rm = Nm - L.fmu[k];
   T r = -P.alpha * rho * rnk, drr = -P.alpha * drho * rnk;
   R.J11 = (rho + drho * (ck - cnk)) * P.idt;
-  R.J12 = T(0.5) * sm * P.iPe * ih2;
+  R.J12 = L.k.dif * sm;
   T Gs = T(0.5) * G2 * ih2 + L.Gn[k];
   T dbulkJ = T(0.5) * drho * gsec(ck, cnk) + rh * gsec_da(ck, cnk) + T(0.5) * fdw(ck) * r +
              T(0.5) * (Fdw(ck) + Fdw(cnk)) * drr;
@@ -522,25 +743,25 @@ __device__ __forceinline__ void vanka_system(const Prm<T>& P, const Lv<T>& L, in
 #pragma unroll
     for (int c = 0; c < 5; ++c) A[r][c] = T(0);
   const T third = T(1.0 / 3.0);
-  // density averages on the four edges from rho(c) of the cell and its four
+  // density sums on the four edges from rho(c) of the cell and its four
   // neighbours (c at kW + 1 is c at k, exactly: ghosts are copies)
   T Arq[4];
   {
     T rk = Form::rho(P, L, k);
-    Arq[0] = T(0.5) * (Form::rho(P, L, kW) + rk);
-    Arq[1] = T(0.5) * (rk + Form::rho(P, L, k + 1));
-    Arq[2] = T(0.5) * (Form::rho(P, L, k - W) + rk);
-    Arq[3] = T(0.5) * (rk + Form::rho(P, L, k + W));
+    Arq[0] = Form::rho(P, L, kW) + rk;
+    Arq[1] = rk + Form::rho(P, L, k + 1);
+    Arq[2] = Form::rho(P, L, k - W) + rk;
+    Arq[3] = rk + Form::rho(P, L, k + W);
   }
   // x-edge rows: q = 0 (west edge, index kW), q = 1 (east edge, index k)
 #pragma unroll
   for (int q = 0; q < 2; ++q) {
     int ke = q == 0 ? kW : k;
     T Arn = L.Aru[ke];
-    T Ar = Arq[q];
+    T Ar = T(0.5) * Arq[q];
     T gt = (j == L.m2) ? T(2) : T(1), gb = (j == 1) ? T(2) : T(1);
     if constexpr (!std::is_same<Form, ErrForm>::value) {  // per-step coefficients
-      A[q][q] = L.Dgu[ke] + T(0.5) * P.idt * Ar;
+      A[q][q] = L.Dgu[ke] + L.k.qidt * Arq[q];
       continue;
     }
     A[q][q] = Arn * P.idt + T(0.5) * (Ar - Arn) * P.idt +
@@ -550,26 +771,25 @@ __device__ __forceinline__ void vanka_system(const Prm<T>& P, const Lv<T>& L, in
                              gb * L.Av[ke - W]);
   }
   {
-    T vc = vis[k];
-    T v3 = vc * P.iRe * ih2 * third;
-    A[0][1] = T(0.5) * L.Sx[k] * ih - vc * P.iRe * ih2 - v3;
-    A[1][0] = -T(0.5) * L.Sx[k] * ih - vc * P.iRe * ih2 - v3;
+    T v3 = vis[k] * L.k.v3, v1 = vis[k] * L.k.v1, sc = L.k.hih * L.Sx[k];
+    A[0][1] = sc - v1 - v3;
+    A[1][0] = -sc - v1 - v3;
     A[0][2] = v3;
     A[0][3] = -v3;
     A[1][2] = -v3;
     A[1][3] = v3;
-    A[0][4] = ih * P.iM;
-    A[1][4] = -ih * P.iM;
+    A[0][4] = L.k.ihM;
+    A[1][4] = -L.k.ihM;
   }
   // y-edge rows: q = 2 (south edge, index k - W), q = 3 (north edge, index k)
 #pragma unroll
   for (int q = 2; q < 4; ++q) {
     int ke = q == 2 ? k - W : k;
     T Arn = L.Arv[ke];
-    T Ar = Arq[q];
+    T Ar = T(0.5) * Arq[q];
     T ge = (!L.px && i == L.m1) ? T(2) : T(1), gw = (!L.px && i == 1) ? T(2) : T(1);
     if constexpr (!std::is_same<Form, ErrForm>::value) {  // per-step coefficients
-      A[q][q] = L.Dgv[ke] + T(0.5) * P.idt * Ar;
+      A[q][q] = L.Dgv[ke] + L.k.qidt * Arq[q];
       continue;
     }
     A[q][q] = Arn * P.idt + T(0.5) * (Ar - Arn) * P.idt +
@@ -579,16 +799,15 @@ __device__ __forceinline__ void vanka_system(const Prm<T>& P, const Lv<T>& L, in
                              (vis[ke + W] + vis[ke]) * (T(1) + third));
   }
   {
-    T vc = vis[k];
-    T v3 = vc * P.iRe * ih2 * third;
-    A[2][3] = T(0.5) * L.Sy[k] * ih - vc * P.iRe * ih2 - v3;
-    A[3][2] = -T(0.5) * L.Sy[k] * ih - vc * P.iRe * ih2 - v3;
+    T v3 = vis[k] * L.k.v3, v1 = vis[k] * L.k.v1, sc = L.k.hih * L.Sy[k];
+    A[2][3] = sc - v1 - v3;
+    A[3][2] = -sc - v1 - v3;
     A[2][0] = v3;
     A[2][1] = -v3;
     A[3][0] = -v3;
     A[3][1] = v3;
-    A[2][4] = ih * P.iM;
-    A[3][4] = -ih * P.iM;
+    A[2][4] = L.k.ihM;
+    A[3][4] = -L.k.ihM;
   }
   {
     const T* mob = L.mobn;
@@ -602,7 +821,7 @@ __device__ __forceinline__ void vanka_system(const Prm<T>& P, const Lv<T>& L, in
     A[4][1] = ih;
     A[4][2] = -ih;
     A[4][3] = ih;
-    A[4][4] = T(0.5) * P.alpha * P.alpha * P.iPe * sm * ih2;
+    A[4][4] = L.k.a2dif * sm;
   }
   if constexpr (std::is_same<Form, FullForm>::value) {
     {
@@ -657,7 +876,7 @@ __device__ __forceinline__ void vanka_system(const Prm<T>& P, const Lv<T>& L, in
     }
   }
   if constexpr (std::is_same<Form, ProjForm>::value) b[4] = T(0);  // the 4x4 block has no p row
-  else b[4] = Form::Np(P, L, k) - L.fp[k];
+  else b[4] = (L.u[k] - L.u[k - 1] + L.v[k] - L.v[k - W]) * ih - L.k.adif * flux_sum(P, L, k) - L.fp[k];
 #pragma unroll
   for (int q = 0; q < 4; ++q)
     if (!act[q]) {
@@ -679,7 +898,7 @@ __device__ __forceinline__ void vanka_system(const Prm<T>& P, const Lv<T>& L, in
 // NP = 5 solves the full system, NP = 4 the velocity block alone.
 template <typename T, int NP>
 __device__ __forceinline__ void solve_vanka(const T (&A)[5][5], T (&b)[5], const bool (&act)[5],
-                                            T v3, T a, T ih) {
+                                            T v3, T a, T ih, T iha) {
   // w_q is +1, -1 or 0, so the products with w are selections
   T y[4], z[4];
 #pragma unroll
@@ -705,8 +924,10 @@ __device__ __forceinline__ void solve_vanka(const T (&A)[5][5], T (&b)[5], const
   T tdot = (y[0] - y[1]) + (y[2] - y[3]);
   T g = qrcp(T(1) + v3 * sdot);
   T pr = T(0);
-  if constexpr (NP == 5) pr = (b[4] + ih * tdot * g) * qrcp(A[4][4] + ih * a * sdot * g);
-  T f = g * (v3 * tdot + a * pr);
+  const T tg = tdot * g;
+  if constexpr (NP == 5) pr = (b[4] + ih * tg) * qrcp(A[4][4] + iha * (sdot * g));
+  T f = v3 * tg;
+  if constexpr (NP == 5) f += (a * g) * pr;
 #pragma unroll
   for (int q = 0; q < 4; ++q) b[q] = y[q] - z[q] * f;
   if constexpr (NP == 5) b[4] = pr;
@@ -719,7 +940,7 @@ __device__ __forceinline__ void vanka_cell(const Prm<T>& P, const Lv<T>& L, int 
   vanka_system<T, Form>(P, L, i, j, A, b, act);
   const int W = L.pitch;
   int k = L.at(i, j);
-  solve_vanka<T, 5>(A, b, act, L.visn[k] * P.iRe * L.ih2 * T(1.0 / 3.0), L.ih * P.iM, L.ih);
+  solve_vanka<T, 5>(A, b, act, L.visn[k] * L.k.v3, L.k.ihM, L.ih, L.k.ihaM);
   int eW = (L.px && i == 1) ? L.m1 : i - 1;
   int kW = L.at(eW, j);
   if (act[0]) store_u(L, eW, j, L.u[kW] - omega * b[0]);
@@ -738,7 +959,7 @@ __device__ __forceinline__ void vanka_cell(const Prm<T>& P, const Lv<T>& L, int 
 // coupling entries are zero and its Schur row is that of J_CH.
 template <typename T>
 __device__ __forceinline__ void solve_coupled7(const T (&A)[7][7], T (&b)[7], const bool (&act)[5],
-                                               T v3, T a, T ih) {
+                                               T v3, T a, T ih, T iha) {
   T B00[2], B01[2], B10[2], B11[2], idet[2], z[4];
 #pragma unroll
   for (int blk = 0; blk < 2; ++blk) {
@@ -754,7 +975,7 @@ __device__ __forceinline__ void solve_coupled7(const T (&A)[7][7], T (&b)[7], co
   }
   const T sdot = (z[0] - z[1]) + (z[2] - z[3]);
   const T g = qrcp(T(1) + v3 * sdot);
-  const T iden = qrcp(A[6][6] + ih * a * sdot * g);
+  const T iden = qrcp(A[6][6] + iha * (sdot * g)), ga = g * a;
   // x = A_NS^-1 r for a right-hand side r over (u_W, u_E, v_S, v_N, p)
   auto apply = [&](const T (&r)[5], T (&x)[5]) {
     T y[4];
@@ -765,8 +986,9 @@ __device__ __forceinline__ void solve_coupled7(const T (&A)[7][7], T (&b)[7], co
       y[p1] = (B00[blk] * r[p1] - B10[blk] * r[p0]) * idet[blk];
     }
     T t = (y[0] - y[1]) + (y[2] - y[3]);
-    T pr = (r[4] + ih * t * g) * iden;
-    T f = g * (v3 * t + a * pr);
+    T tg = t * g;
+    T pr = (r[4] + ih * tg) * iden;
+    T f = v3 * tg + ga * pr;
 #pragma unroll
     for (int q = 0; q < 4; ++q) x[q] = y[q] - z[q] * f;
     x[4] = pr;
@@ -845,7 +1067,7 @@ __device__ __forceinline__ void coupled_cell(const Prm<T>& P, const Lv<T>& L, in
   T gE = rn[k + 1] * L.Tx[k];
   T gS = rn[k - W] * L.Ty[k - W];
   T gN = rn[k + W] * L.Ty[k];
-  T diffc = T(0.5) * P.alpha * P.iPe * sm * L.ih2;
+  T diffc = L.k.adif * sm;
   A[0][2] = gW;
   A[0][3] = gE;
   A[0][4] = gS;
@@ -871,7 +1093,7 @@ __device__ __forceinline__ void coupled_cell(const Prm<T>& P, const Lv<T>& L, in
       }
       A[2 + q][2 + q] = T(1);
     }
-  solve_coupled7(A, b, act, L.visn[k] * P.iRe * L.ih2 * T(1.0 / 3.0), L.ih * P.iM, L.ih);
+  solve_coupled7(A, b, act, L.visn[k] * L.k.v3, L.k.ihM, L.ih, L.k.ihaM);
   T cnew = L.c[k] - omega * b[0];
   store_cell(L, L.c, i, j, cnew);
   if constexpr (!std::is_same<Form, ErrForm>::value) store_cell(L, L.rhoc, i, j, rho_of(P, cnew));
@@ -979,7 +1201,7 @@ __device__ __forceinline__ void vanka4_cell(const Prm<T>& P, const Lv<T>& L, int
   vanka_system<T, Form>(P, L, i, j, A5, b5, act);
   const int W = L.pitch;
   int k = L.at(i, j);
-  solve_vanka<T, 4>(A5, b5, act, L.visn[k] * P.iRe * L.ih2 * T(1.0 / 3.0), L.ih * P.iM, L.ih);
+  solve_vanka<T, 4>(A5, b5, act, L.visn[k] * L.k.v3, L.k.ihM, L.ih, L.k.ihaM);
   const T(&b)[5] = b5;
   int eW = (L.px && i == 1) ? L.m1 : i - 1;
   int kW = L.at(eW, j);
@@ -1307,7 +1529,8 @@ __device__ __forceinline__ void assemble_row(const Prm<T>& P, const Lv<T>& L, in
 }
 
 // per-step row coefficients of the momentum rows (needs k_frozen_coef2): time =
-// x T1 + T0 + A rho(c) x/(2dt); Dg = the iterate-independent part of the
+// x T1 + T0 + A rho(c) x/(2dt) (T0 of the y rows holds gravity, which P carries
+// for the primitive method only); Dg = the iterate-independent part of the
 // diagonal entry (the whole entry is Dg + A rho(c)/(2dt)), with the reflected
 // no-slip ghosts doubling the tangential wall terms (g = 2)
 template <typename T>
@@ -1336,7 +1559,7 @@ __global__ void k_frozen_coef3(Prm<T> P, Lv<T> L) {
     T ge = (!L.px && i == L.m1) ? T(2) : T(1), gw = (!L.px && i == 1) ? T(2) : T(1);
     T t1 = T(0.5) * Arn * P.idt + L.Dvv[k];
     L.T1v[k] = t1;
-    L.T0v[k] = -Arn * L.vn[k] * P.idt;
+    L.T0v[k] = -Arn * L.vn[k] * P.idt + P.Fr_inv * Arn;
     L.Dgv[k] = t1 + T(0.5) * L.ih * (-L.Qy[k] * ge + L.Qy[k - 1] * gw - L.Sy[k + W] + L.Sy[k]) +
                P.iRe * L.ih2 * (ge * L.Av[k] + gw * L.Av[k - 1] + (vis[k + W] + vis[k]) * (T(1) + third));
     assemble_row(P, L, k, W, 1, t1, L.Sy, L.Qy, L.Ty, L.Cv, L.aPv, L.aMv, L.tPv, L.tMv, L.M0v,
@@ -1608,12 +1831,11 @@ template <typename T>
 struct MomRow {
   const T *a, *b, *S, *Q, *Tf, *Arn, *Dv, *T1, *T0, *Dg, *B, *f;
   int s, t, d;
-  T grav;
 };
 
 // FullForm uses the per-step row coefficients T1, T0, Dg; ErrForm (the error
-// equation of the defect correction) has none of them, adds the base-state term
-// of the time derivative and has no gravity (it cancels in N(X + e) - N(X))
+// equation of the defect correction) has none of them and adds the base-state
+// term of the time derivative
 template <typename T, class Form>
 __device__ __forceinline__ MomRow<T> mom_row(const Prm<T>& P, const Lv<T>& L, int d) {
   MomRow<T> R;
@@ -1632,9 +1854,6 @@ __device__ __forceinline__ MomRow<T> mom_row(const Prm<T>& P, const Lv<T>& L, in
   R.s = d ? L.pitch : 1;
   R.t = d ? 1 : L.pitch;
   R.d = d;
-  // gravity: the primitive momentum row only (the error equation cancels it,
-  // the projection method puts it in the projection equation)
-  R.grav = (d && std::is_same<Form, FullForm>::value) ? P.Fr_inv : T(0);
   return R;
 }
 
@@ -1643,10 +1862,10 @@ __device__ __forceinline__ MomRow<T> mom_row(const Prm<T>& P, const Lv<T>& L, in
 template <typename T, class Form>
 __device__ __forceinline__ T mom_residual(const Prm<T>& P, const Lv<T>& L, const MomRow<T>& R, int k,
                                           T rl, T rr) {
-  T Ar = T(0.5) * (rl + rr);
   // FP64 primitive rows: the per-step assembled stencil
   if constexpr (std::is_same<Form, FullForm>::value && sizeof(T) == 8)
-    return mom_asm(P, L, R.d, k, Ar) - R.f[k];
+    return mom_asm(L, R.d, k, rl + rr) - R.f[k];
+  T Ar = T(0.5) * (rl + rr);
   const int s = R.s, t = R.t;
   const T *a = R.a, *b = R.b, *vis = L.visn, *rn = L.rhon;
   T ae = a[k];
@@ -1664,7 +1883,7 @@ __device__ __forceinline__ T mom_residual(const Prm<T>& P, const Lv<T>& L, const
     time = Arn * ae * P.idt + T(0.5) * (Ar - Arn) * P.idt * ae + T(0.5) * dAr * P.idt * R.B[k] +
            R.Dv[k] * ae;
   } else {
-    time = ae * R.T1[k] + R.T0[k] + T(0.5) * P.idt * Ar * ae;
+    time = ae * (R.T1[k] + L.k.qidt * (rl + rr)) + R.T0[k];
   }
   T press = T(0), st = T(0);  // the projection method's intermediate-velocity row has neither
   if constexpr (!std::is_same<Form, ProjForm>::value) {
@@ -1674,7 +1893,7 @@ __device__ __forceinline__ T mom_residual(const Prm<T>& P, const Lv<T>& L, const
   T vl = vis[k], vr = vis[k + s];
   T visc = -P.iRe * L.ih * ((vr * dr - vl * dl) + (L.Av[k] * Dp - L.Av[k - t] * Dm) +
                             (vr * dvr - vl * dvl) * T(1.0 / 3.0));
-  return time + conv + press + st + visc + R.grav * R.Arn[k] - R.f[k];
+  return time + conv + press + st + visc - R.f[k];
 }
 
 // Diagonal entry dq and residual bq = N - f (0 on a wall edge) of momentum row
@@ -1698,7 +1917,7 @@ __device__ __forceinline__ void team_row(const Prm<T>& P, const Lv<T>& L, int i,
          T(0.5) * ih * (-R.S[ke + R.s] + R.S[ke] - R.Q[ke] * gp + R.Q[ke - R.t] * gm) + R.Dv[ke] +
          P.iRe * ih2 * ((vis[ke + R.s] + vis[ke]) * (T(1) + third) + gp * L.Av[ke] + gm * L.Av[ke - R.t]);
   } else {
-    dq = R.Dg[ke] + T(0.5) * P.idt * Ar;
+    dq = R.Dg[ke] + L.k.qidt * (rl + rr);
   }
   bq = mom_residual<T, Form>(P, L, R, ke, rl, rr);  // wall edges too (padded arrays), then discarded
   if (!mine) bq = T(0);
@@ -1714,7 +1933,7 @@ __device__ __forceinline__ void team_row(const Prm<T>& P, const Lv<T>& L, int i,
 // identity rows with rq = 0.
 template <typename T>
 struct TeamSolve {
-  T B00, B01, B10, B11, idet, z, g, iden, v3, a, ih;
+  T B00, B01, B10, B11, idet, z, g, ga, iden, v3, ih;
   bool odd;
   // with_p = false: the 4x4 velocity block alone (the projection method's
   // intermediate-velocity block), solved as solve_vanka<T, 4> does
@@ -1722,15 +1941,15 @@ struct TeamSolve {
                                        T S, T vc, T A44, bool with_p = true) {
     const unsigned FULL = 0xffffffffu;
     ih = L.ih;
-    v3 = vc * P.iRe * L.ih2 * T(1.0 / 3.0);
-    a = with_p ? L.ih * P.iM : T(0);
+    v3 = vc * L.k.v3;
     odd = q & 1;
     T dqo = __shfl_xor_sync(FULL, dq, 1);
     T D0 = odd ? dqo : dq, D1 = odd ? dq : dqo;
     B00 = ap0 ? D0 - v3 : T(1);
     B11 = ap1 ? D1 - v3 : T(1);
-    B01 = (ap0 && ap1) ? T(0.5) * S * ih - vc * P.iRe * L.ih2 : T(0);
-    B10 = (ap0 && ap1) ? -T(0.5) * S * ih - vc * P.iRe * L.ih2 : T(0);
+    const T v1 = vc * L.k.v1, sc = L.k.hih * S;
+    B01 = (ap0 && ap1) ? sc - v1 : T(0);
+    B10 = (ap0 && ap1) ? -sc - v1 : T(0);
     idet = qrcp(B00 * B11 - B01 * B10);
     T zn = odd ? ((ap1 ? B00 : T(0)) + (ap0 ? B10 : T(0))) : ((ap0 ? B11 : T(0)) + (ap1 ? B01 : T(0)));
     z = (odd ? -zn : zn) * idet;
@@ -1738,7 +1957,8 @@ struct TeamSolve {
     sdot += __shfl_xor_sync(FULL, sdot, 1);
     sdot += __shfl_xor_sync(FULL, sdot, 2);
     g = qrcp(T(1) + v3 * sdot);
-    iden = with_p ? qrcp(A44 + ih * a * sdot * g) : T(0);
+    iden = with_p ? qrcp(A44 + L.k.ihaM * (sdot * g)) : T(0);
+    ga = with_p ? g * L.k.ihM : T(0);
   }
   __device__ __forceinline__ T apply(T rq, T r4, T& pr) const {
     const unsigned FULL = 0xffffffffu;
@@ -1748,8 +1968,9 @@ struct TeamSolve {
     T tdot = odd ? -y : y;
     tdot += __shfl_xor_sync(FULL, tdot, 1);
     tdot += __shfl_xor_sync(FULL, tdot, 2);
-    pr = (r4 + ih * tdot * g) * iden;
-    return y - z * (g * (v3 * tdot + a * pr));
+    const T tg = tdot * g;
+    pr = (r4 + ih * tg) * iden;
+    return y - z * (v3 * tg + ga * pr);
   }
 };
 
@@ -1780,10 +2001,10 @@ __device__ __forceinline__ void vanka_team(const Prm<T>& P, const Lv<T>& L, int 
   const int nq = k + (q == 0 ? -1 : q == 1 ? 1 : q == 2 ? -W : W);
   T am = mob[nq] + mob[k];
   T f0 = team_sum<T>((q & 1) ? (d ? L.v[k] : L.u[k]) : -(d ? L.v[k - W] : L.u[k - 1]));
-  T f1 = team_sum<T>(T(0.5) * am * ((L.mu[nq] - L.mu[k]) + P.alpha * (L.p[nq] - L.p[k])));
+  T f1 = team_sum<T>(am * ((L.mu[nq] - L.mu[k]) + P.alpha * (L.p[nq] - L.p[k])));
   T f2 = team_sum<T>(mine ? am : T(0));
-  T A44 = T(0.5) * P.alpha * P.alpha * P.iPe * f2 * ih2;
-  T b4 = f0 * ih - P.alpha * P.iPe * ih2 * f1 - L.fp[k];
+  T A44 = L.k.a2dif * f2;
+  T b4 = f0 * ih - L.k.adif * f1 - L.fp[k];
   TeamSolve<T> ts(P, L, q, dq, d ? a2 : a0, d ? a3 : a1, d ? L.Sy[k] : L.Sx[k], L.visn[k], A44);
   T pr;
   T x = ts.apply(bq, b4, pr);
@@ -1798,7 +2019,7 @@ __device__ __forceinline__ void vanka_team(const Prm<T>& P, const Lv<T>& L, int 
 }
 
 // One half of mom_residual for a lane pair of an eight-lane team: half 0 the
-// time term, the convection, gravity and -f; half 1 the pressure gradient,
+// time term (with gravity), the convection and -f; half 1 the pressure gradient,
 // the surface tension and the viscous terms.  The two halves sum to the
 // momentum row's N - f (up to the order of the additions).  FullForm only.
 template <typename T>
@@ -1810,10 +2031,9 @@ __device__ __forceinline__ T mom_residual_half(const Prm<T>& P, const Lv<T>& L, 
   T dl = (ae - a[k - s]) * L.ih, dr = (a[k + s] - ae) * L.ih;
   T Dp = (a[k + t] - ae) * L.ih, Dm = (ae - a[k - t]) * L.ih;
   if (half == 0) {
-    T Ar = T(0.5) * (rl + rr);
     T conv = T(0.5) * (R.S[k + s] * dr + R.S[k] * dl + R.Q[k] * Dp + R.Q[k - t] * Dm);
-    T time = ae * R.T1[k] + R.T0[k] + T(0.5) * P.idt * Ar * ae;
-    return time + conv + R.grav * R.Arn[k] - R.f[k];
+    T time = ae * (R.T1[k] + L.k.qidt * (rl + rr)) + R.T0[k];
+    return time + conv - R.f[k];
   }
   const T *vis = L.visn, *rn = L.rhon;
   T dvl = dl + (b[k] - b[k - t]) * L.ih;
@@ -1846,7 +2066,7 @@ __device__ __forceinline__ void vanka_team8(const Prm<T>& P, const Lv<T>& L, int
   int ke = q == 0 ? kW : (q == 2 ? k - W : k);
   MomRow<T> R = mom_row<T, FullForm>(P, L, d);
   T rl = L.rhoc[ke], rr = L.rhoc[ke + R.s];
-  T dq = R.Dg[ke] + T(0.5) * P.idt * (T(0.5) * (rl + rr));
+  T dq = R.Dg[ke] + L.k.qidt * (rl + rr);
   T bq = mom_residual_half<T>(P, L, R, ke, rl, rr, half);
   bq += __shfl_xor_sync(0xffffffffu, bq, 4);
   if (!mine) bq = T(0);
@@ -1854,10 +2074,10 @@ __device__ __forceinline__ void vanka_team8(const Prm<T>& P, const Lv<T>& L, int
   const int nq = k + (q == 0 ? -1 : q == 1 ? 1 : q == 2 ? -W : W);
   T am = mob[nq] + mob[k];
   T f0 = team_sum<T>((q & 1) ? (d ? L.v[k] : L.u[k]) : -(d ? L.v[k - W] : L.u[k - 1]));
-  T f1 = team_sum<T>(T(0.5) * am * ((L.mu[nq] - L.mu[k]) + P.alpha * (L.p[nq] - L.p[k])));
+  T f1 = team_sum<T>(am * ((L.mu[nq] - L.mu[k]) + P.alpha * (L.p[nq] - L.p[k])));
   T f2 = team_sum<T>(mine ? am : T(0));
-  T A44 = T(0.5) * P.alpha * P.alpha * P.iPe * f2 * ih2;
-  T b4 = f0 * ih - P.alpha * P.iPe * ih2 * f1 - L.fp[k];
+  T A44 = L.k.a2dif * f2;
+  T b4 = f0 * ih - L.k.adif * f1 - L.fp[k];
   TeamSolve<T> ts(P, L, q, dq, d ? a2 : a0, d ? a3 : a1, d ? L.Sy[k] : L.Sx[k], L.visn[k], A44);
   T pr;
   T x = ts.apply(bq, b4, pr);
@@ -1925,9 +2145,9 @@ __device__ __forceinline__ void coupled_team(const Prm<T>& P, const Lv<T>& L, in
   T J11 = C.J11, J12 = C.J12, J21 = C.J21, J22 = C.J22, Rc = C.Rc, Rm = C.Rm;
   // the mass row and the couplings of edge q: d N_q/dc, d N_q/dmu (rows of
   // the two CH columns), d N_c/d x_q = g_q (the CH row), d N_p/dmu = d N_c/dp
-  T A44 = T(0.5) * P.alpha * P.alpha * P.iPe * sm * ih2;
-  T b4 = sdiv * ih - P.alpha * P.iPe * ih2 * sflux - L.fp[k];
-  T diffc = T(0.5) * P.alpha * P.iPe * sm * ih2;
+  T A44 = L.k.a2dif * sm;
+  T b4 = sdiv * ih - L.k.adif * sflux - L.fp[k];
+  T diffc = L.k.adif * sm;
   T gm = mine ? gq : T(0);
   T cq0 = mine ? T(0.25) * C.drho * P.idt * (d ? Form::val_v(L, ke) : Form::val_u(L, ke)) : T(0);
   T cq1 = mine ? -gq * P.iM : T(0);
@@ -2049,36 +2269,36 @@ __device__ __forceinline__ void vanka_pair(const Prm<T>& P, const Lv<T>& L, int 
   const int n0 = k - off, n1 = k + off;
   T am0 = mob[n0] + mob[k], am1 = mob[n1] + mob[k];
   T fs0 = -(d ? L.v[k - W] : L.u[k - 1]) + (d ? L.v[k] : L.u[k]);
-  T fs1 = T(0.5) * am0 * ((L.mu[n0] - L.mu[k]) + P.alpha * (L.p[n0] - L.p[k])) +
-          T(0.5) * am1 * ((L.mu[n1] - L.mu[k]) + P.alpha * (L.p[n1] - L.p[k]));
+  T fs1 = am0 * ((L.mu[n0] - L.mu[k]) + P.alpha * (L.p[n0] - L.p[k])) +
+          am1 * ((L.mu[n1] - L.mu[k]) + P.alpha * (L.p[n1] - L.p[k]));
   T fs2 = (ap0 ? am0 : T(0)) + (ap1 ? am1 : T(0));
   fs0 += __shfl_xor_sync(FULL, fs0, 1);
   fs1 += __shfl_xor_sync(FULL, fs1, 1);
   fs2 += __shfl_xor_sync(FULL, fs2, 1);
-  T A44 = T(0.5) * P.alpha * P.alpha * P.iPe * fs2 * ih2;
-  T b4 = fs0 * ih - P.alpha * P.iPe * ih2 * fs1 - L.fp[k];
+  T A44 = L.k.a2dif * fs2;
+  T b4 = fs0 * ih - L.k.adif * fs1 - L.fp[k];
   // this pair's block B = A_vv - v3 w w^T (TeamSolve, both rows on one lane)
   T vc = L.visn[k];
   T S = d ? L.Sy[k] : L.Sx[k];
-  T v3 = vc * P.iRe * L.ih2 * T(1.0 / 3.0);
-  T a = L.ih * P.iM;
+  T v3 = vc * L.k.v3, v1 = vc * L.k.v1, sc = L.k.hih * S;
   T B00 = ap0 ? dq0 - v3 : T(1);
   T B11 = ap1 ? dq1 - v3 : T(1);
-  T B01 = (ap0 && ap1) ? T(0.5) * S * ih - vc * P.iRe * L.ih2 : T(0);
-  T B10 = (ap0 && ap1) ? -T(0.5) * S * ih - vc * P.iRe * L.ih2 : T(0);
+  T B01 = (ap0 && ap1) ? sc - v1 : T(0);
+  T B10 = (ap0 && ap1) ? -sc - v1 : T(0);
   T idet = qrcp(B00 * B11 - B01 * B10);
   T z0 = ((ap0 ? B11 : T(0)) + (ap1 ? B01 : T(0))) * idet;
   T z1 = -((ap1 ? B00 : T(0)) + (ap0 ? B10 : T(0))) * idet;
   T sdot = z0 + -z1;
   sdot += __shfl_xor_sync(FULL, sdot, 1);
   T g = qrcp(T(1) + v3 * sdot);
-  T iden = qrcp(A44 + ih * a * sdot * g);
+  T iden = qrcp(A44 + L.k.ihaM * (sdot * g));
   T y0 = (B11 * bq0 - B01 * bq1) * idet;
   T y1 = (B00 * bq1 - B10 * bq0) * idet;
   T tdot = y0 + -y1;
   tdot += __shfl_xor_sync(FULL, tdot, 1);
-  T pr = (b4 + ih * tdot * g) * iden;
-  T f = g * (v3 * tdot + a * pr);
+  T tg = tdot * g;
+  T pr = (b4 + ih * tg) * iden;
+  T f = v3 * tg + (g * L.k.ihM) * pr;
   T x0 = y0 - z0 * f, x1 = y1 - z1 * f;
   if (!ok) return;
   if (d == 0) {
@@ -2352,8 +2572,9 @@ __global__ void __launch_bounds__(NT) k_coarse_vcycle(Prm<T> P, CoarseLevels<T> 
 // writes) into shared memory at the compact pitch m1 + 3, runs the V-cycle
 // body unchanged on level descriptors that point into the copy, and writes
 // back the arrays the V-cycle writes: the unknowns, sources, residuals and the
-// kept restricted iterate (the first 20 arrays) and rho(c).  Same device code
-// on the same values: the results are those of k_coarse_vcycle.
+// kept restricted iterate (the first 20 arrays) and rho(c).  copy = 0 leaves
+// the descriptors on the level's own arrays: one instance of the code serves
+// both, so the two give the same bits.
 // --------------------------------------------------------------------------
 constexpr int QN_LV_NARR = 59;     // arrays of QN_LV_ARRAYS
 constexpr int QN_LV_WRITTEN = 20;  // arrays 0..19 are written; and rho(c):
@@ -2396,14 +2617,15 @@ __device__ __forceinline__ void coarse_copy(double* __restrict__ g, int pg, long
 
 template <int NT>
 __global__ void __launch_bounds__(NT) k_coarse_vcycle_smem(Prm<double> P, CoarseLevels<double> C,
-                                                           CoarseSmem M, int nu1, int nu2, int nuc,
-                                                           double omega, int coupled, int team8) {
+                                                           CoarseSmem M, int copy, int nu1, int nu2,
+                                                           int nuc, double omega, int coupled,
+                                                           int team8) {
   extern __shared__ __align__(16) double qn_coarse_smem[];
   pdl_enter();
   CoarseLevels<double>* S = reinterpret_cast<CoarseLevels<double>*>(qn_coarse_smem);
   double* arr = qn_coarse_smem + M.head;
   const int n = C.n;
-  for (int l = 0; l < n; ++l) {
+  for (int l = 0; copy && l < n; ++l) {
     const Lv<double>& G = C.L[l];
     const int cc = G.m1 + 3, rr = G.m2 + 3;
     coarse_copy<NT, true>(G.c - (G.pitch + 1), G.pitch, M.ng[l], arr + M.off[l], cc, rr, 0,
@@ -2412,13 +2634,15 @@ __global__ void __launch_bounds__(NT) k_coarse_vcycle_smem(Prm<double> P, Coarse
   if (threadIdx.x < n) {  // the descriptor of level l, its arrays in the copy
     const int l = threadIdx.x;
     Lv<double> X = C.L[l];
-    const int cc = X.m1 + 3, ns = cc * (X.m2 + 3);
-    double* o = arr + M.off[l] + cc + 1;  // origin (0,0) of array 0
-    int q = 0;
+    if (copy) {
+      const int cc = X.m1 + 3, ns = cc * (X.m2 + 3);
+      double* o = arr + M.off[l] + cc + 1;  // origin (0,0) of array 0
+      int q = 0;
 #define QN_REBASE(m) X.m = o + (q++) * ns;
-    QN_LV_ARRAYS(QN_REBASE)
+      QN_LV_ARRAYS(QN_REBASE)
 #undef QN_REBASE
-    X.pitch = cc;
+      X.pitch = cc;
+    }
     S->L[l] = X;
   }
   if (threadIdx.x == 0) {
@@ -2429,7 +2653,7 @@ __global__ void __launch_bounds__(NT) k_coarse_vcycle_smem(Prm<double> P, Coarse
   __syncthreads();
   coarse_vcycle_body<double, FullForm>(P, *S, nu1, nu2, nuc, omega, coupled, team8);
   __syncthreads();
-  for (int l = 0; l < n; ++l) {
+  for (int l = 0; copy && l < n; ++l) {
     const Lv<double>& G = C.L[l];
     const int cc = G.m1 + 3, rr = G.m2 + 3;
     double* g = G.c - (G.pitch + 1);
@@ -3037,7 +3261,8 @@ int nparts_cells(const Lv<T>& L) {
 }
 
 template <typename T, class Form>
-void launch_residual(const Prm<T>& P, const Lv<T>& L, double* part, cudaStream_t s) {
+void launch_residual(const Prm<T>& P, const Lv<T>& L0, double* part, cudaStream_t s) {
+  const Lv<T> L = level_consts(P, L0);
   if (residual_rows(L) == 2)
     qlaunch(&k_residual<T, 0, Form, 2>, grid2(L.m1, (L.m2 + 1) / 2), dim3(BX, BY), 0, s, P, L, part);
   else
@@ -3045,7 +3270,8 @@ void launch_residual(const Prm<T>& P, const Lv<T>& L, double* part, cudaStream_t
   ++g_launches;
 }
 template <typename T, class Form>
-void launch_add_op(const Prm<T>& P, const Lv<T>& L, cudaStream_t s) {
+void launch_add_op(const Prm<T>& P, const Lv<T>& L0, cudaStream_t s) {
+  const Lv<T> L = level_consts(P, L0);
   if (residual_rows(L) == 2)
     qlaunch(&k_residual<T, 1, Form, 2>, grid2(L.m1, (L.m2 + 1) / 2), dim3(BX, BY), 0, s, P, L, nullptr);
   else
@@ -3053,7 +3279,8 @@ void launch_add_op(const Prm<T>& P, const Lv<T>& L, cudaStream_t s) {
   ++g_launches;
 }
 template <typename T, class Form>
-void launch_ch(const Prm<T>& P, const Lv<T>& L, int colour, cudaStream_t s, int team_max) {
+void launch_ch(const Prm<T>& P, const Lv<T>& L0, int colour, cudaStream_t s, int team_max) {
+  const Lv<T> L = level_consts(P, L0);
   int n = (L.m1 + 1) / 2 * L.m2;
   if (n <= 0) return;
   if constexpr (sizeof(T) == 8 || std::is_same<Form, ErrForm>::value) {
@@ -3108,8 +3335,9 @@ int vanka_split_single(int n, int split) {
 }
 
 template <typename T, class Form>
-void launch_vanka(const Prm<T>& P, const Lv<T>& L, int colour, T omega, cudaStream_t s,
+void launch_vanka(const Prm<T>& P, const Lv<T>& L0, int colour, T omega, cudaStream_t s,
                   int team_max, int team8_max, int pair_max, int split) {
+  const Lv<T> L = level_consts(P, L0);
   int n = vanka_slots(L, colour).n;
   if (n <= 0) return;
   if constexpr (std::is_same<Form, FullForm>::value && sizeof(T) == 8) {
@@ -3197,18 +3425,16 @@ int launch_coarse_vcycle(const Prm<T>& P, const Lv<T>* levels, int n, int nu1, i
   CoarseLevels<T> C;
   C.n = n;
   C.base = std::is_same<Form, ErrForm>::value;
-  for (int l = 0; l < n; ++l) C.L[l] = levels[l];
+  for (int l = 0; l < n; ++l) C.L[l] = level_consts(P, levels[l]);
   constexpr int NT = sizeof(T) == 8 ? 256 : 512;
   if constexpr (std::is_same<Form, FullForm>::value && sizeof(T) == 8) {
-    if (smem && ctas <= 1) {
+    if (ctas <= 1) {
       CoarseSmem M = {};
-      const size_t bytes = coarse_smem_plan(levels, n, M);
-      if (bytes) {
-        qlaunch(&k_coarse_vcycle_smem<NT>, 1, NT, bytes, s, P, C, M, nu1, nu2, nuc, omega, coupled,
-                team8);
-        ++g_launches;
-        return 1;
-      }
+      const size_t bytes = smem ? coarse_smem_plan(levels, n, M) : 0;
+      qlaunch(&k_coarse_vcycle_smem<NT>, 1, NT, bytes ? bytes : sizeof(CoarseLevels<double>), s, P,
+              C, M, bytes ? 1 : 0, nu1, nu2, nuc, omega, coupled, team8);
+      ++g_launches;
+      return bytes ? 1 : 0;
     }
   }
   if (ctas <= 1) {
@@ -3279,8 +3505,9 @@ int coarse_cluster_blocks(int ctas) {
 }
 
 template <typename T, class Form>
-void launch_vanka4(const Prm<T>& P, const Lv<T>& L, int colour, T omega, cudaStream_t s,
+void launch_vanka4(const Prm<T>& P, const Lv<T>& L0, int colour, T omega, cudaStream_t s,
                    int team_max) {
+  const Lv<T> L = level_consts(P, L0);
   int n = vanka_slots(L, colour).n;
   if (n <= 0) return;
   if constexpr (std::is_same<Form, ProjForm>::value && sizeof(T) == 8) {
@@ -3294,7 +3521,8 @@ void launch_vanka4(const Prm<T>& P, const Lv<T>& L, int colour, T omega, cudaStr
   ++g_launches;
 }
 template <typename T>
-void launch_pgs(const Prm<T>& P, const Lv<T>& L, int colour, cudaStream_t s, int team_max) {
+void launch_pgs(const Prm<T>& P, const Lv<T>& L0, int colour, cudaStream_t s, int team_max) {
+  const Lv<T> L = level_consts(P, L0);
   int n = (L.m1 + 1) / 2 * L.m2;
   if (n <= 0) return;
   if (n <= team_max) {  // four lanes per cell: shorter critical path per visit
@@ -3319,8 +3547,9 @@ void launch_proj_diss(const Prm<T>& P, const Lv<T>& L, const T* uo, const T* vo,
   ++g_launches;
 }
 template <typename T, class Form>
-void launch_coupled(const Prm<T>& P, const Lv<T>& L, int colour, T omega, cudaStream_t s,
+void launch_coupled(const Prm<T>& P, const Lv<T>& L0, int colour, T omega, cudaStream_t s,
                     int team_max) {
+  const Lv<T> L = level_consts(P, L0);
   int n = vanka_slots(L, colour).n;
   if (n <= 0) return;
   if (n <= team_max) {  // four lanes per block: shorter critical path per visit
@@ -3483,8 +3712,9 @@ void launch_pack_out(const Lv<T>& L, double* dst, const T* src, int kind, cudaSt
 }
 
 template <typename T, class Form>
-void launch_wave(const Prm<T>& P, const Lv<T>& L, const WavePlan& W, T omega, unsigned* ctr,
+void launch_wave(const Prm<T>& P, const Lv<T>& L0, const WavePlan& W, T omega, unsigned* ctr,
                  double* flag, cudaStream_t s) {
+  const Lv<T> L = level_consts(P, L0);
   static std::atomic<int> blocks_per_sm{0};
   static std::atomic<int> sms{0};
   if (!sms.load()) {
@@ -3506,8 +3736,9 @@ void launch_wave(const Prm<T>& P, const Lv<T>& L, const WavePlan& W, T omega, un
 }
 
 template <typename T, class Form>
-int launch_skew(const Prm<T>& P, const Lv<T>& L, int nsteps, int coupled, int rows, T omega,
+int launch_skew(const Prm<T>& P, const Lv<T>& L0, int nsteps, int coupled, int rows, T omega,
                 cudaStream_t s) {
+  const Lv<T> L = level_consts(P, L0);
   const int per = coupled ? L.kcol : L.kcol + 2;
   const int H = std::max(rows, 1);
   const int group = std::max(1, SKEW_MAX_TASKS / per);  // steps per schedule

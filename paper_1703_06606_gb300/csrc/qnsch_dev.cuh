@@ -27,8 +27,27 @@ struct Prm {
   T idt;           // 1/dt
 };
 
+// Products of the parameters and a level's spacing that the operators multiply
+// by (level_consts, on the host at each launch).  A warp's FP64 instruction
+// holds its sub-partition's pipe for 64 to 76 cycles whether its operands vary
+// by lane or not, so a product of two kernel parameters costs a visit as much
+// as one of its own terms; formed here it costs nothing.
+template <typename T>
+struct LvK {
+  T qidt;              // 1/(4 dt): A rho(c) / (2 dt) from the sum of the edge's two densities
+  T ihM;               // 1/(M h)
+  T v1, v3;            // 1/(Re h^2), a third of it
+  T hih;               // 1/(2 h)
+  T dif, adif, a2dif;  // 1/(2 Pe h^2), alpha and alpha^2 times it
+  T ihaM;              // 1/(M h^2)
+  T hih2;              // 1/(2 h^2)
+  T K8, K4;            // K/8, K/4
+  T L4, L8, L4h;       // Lam/4, Lam/(8 h^2), Lam/(4 h^2)
+};
+
 template <typename T>
 struct Lv {
+  LvK<T> k;
   int m1, m2, px, pitch;
   // Vanka colours of this level: kcol colours, (2i+j) mod 8 when c8 is set
   // (periodic x with m1 = 0 mod 4), else (i+2j) mod kcol
@@ -50,7 +69,8 @@ struct Lv {
   // FP64 full-iterate levels only, built per step (they depend on dt): for each
   // momentum row (x-edges *u, y-edges *v) the time-term coefficients, time =
   // x T1 + T0 + (dt^-1/2) A rho(c) x with T1 = A rho^n/(2dt) + Dv and T0 =
-  // -A rho^n x^n/dt, and Dg, the part of the row's diagonal entry that does not
+  // -A rho^n x^n/dt (plus, in the primitive method's y rows, gravity
+  // (1/Fr) A_y rho^n), and Dg, the part of the row's diagonal entry that does not
   // depend on the iterate (the whole diagonal is Dg + A rho(c)/(2dt))
   T *T1u = nullptr, *T1v = nullptr, *T0u = nullptr, *T0v = nullptr, *Dgu = nullptr, *Dgv = nullptr;
   // FP64 full-iterate levels only: rho(c) of the iterate, ghosts included.
@@ -78,6 +98,18 @@ struct Lv {
   __device__ __forceinline__ int uhi() const { return px ? m1 : m1 - 1; }
 };
 
+// L with its constants for the parameters P
+template <typename T>
+inline Lv<T> level_consts(const Prm<T>& P, const Lv<T>& L) {
+  const double ih = L.ih, ih2 = L.ih2, iM = P.iM, dif = 0.5 * P.iPe * ih2, al = P.alpha;
+  Lv<T> X = L;
+  X.k = {T(0.25 * P.idt), T(ih * iM),       T(P.iRe * ih2),         T(P.iRe * ih2 / 3.0),
+         T(0.5 * ih),     T(dif),           T(al * dif),            T(al * al * dif),
+         T(ih * ih * iM), T(0.5 * ih2),     T(0.125 * P.K),         T(0.25 * P.K),
+         T(0.25 * P.Lam), T(0.125 * P.Lam * ih2), T(0.25 * P.Lam * ih2)};
+  return X;
+}
+
 // The arrays of an FP64 full-iterate level in the order in which they sit in
 // the level's block (one allocation, NFIELD arrays of the same padded size):
 // X(member) for each.
@@ -99,20 +131,25 @@ template <typename T> __device__ __forceinline__ T rho_of(const Prm<T>& P, T c) 
 template <typename T> __device__ __forceinline__ T qdiv(T a, T b) { return a / b; }
 template <> __device__ __forceinline__ float qdiv(float a, float b) { return __fdividef(a, b); }
 // 1/x for the pivots of the local block solves.  FP32: the fast division, as
-// qdiv.  FP64: the Newton-Raphson iteration r <- r + r (1 - x r) for the zero
-// of 1/r - x, which squares the relative error of r at every step, started
-// from the hardware's approximate reciprocal (rcp.approx.ftz.f64); after two
-// steps the result is within a few units in the last place of 1/x (tested
-// against IEEE division).  Normal-range x only: the pivots are determinants
-// and diagonal sums of the local systems, far from the subnormal range.
+// qdiv.  FP64: one step of the third-order iteration r <- r + r (e + e^2),
+// e = 1 - x r, which is Newton's for the zero of 1/r - x with the next term of
+// the geometric series 1/(1 - e) kept, so the relative error e of r becomes
+// e^3; started from the hardware's approximate reciprocal
+// (rcp.approx.ftz.f64) the result is within a few units in the last place of
+// 1/x (tested against IEEE division) in three FP64 instructions, where two
+// Newton steps take four and an IEEE division about ten.  Normal-range x only:
+// the pivots are determinants and diagonal sums of the local systems and the
+// densities' denominators, far from the subnormal range.
 template <typename T> __device__ __forceinline__ T qrcp(T x) { return qdiv(T(1), x); }
 template <> __device__ __forceinline__ double qrcp(double x) {
   double r;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
   double e = fma(-x, r, 1.0);
-  r = fma(r, e, r);
-  e = fma(-x, r, 1.0);
+  e = fma(e, e, e);
   return fma(r, e, r);
+}
+template <> __device__ __forceinline__ double rho_of(const Prm<double>& P, double c) {
+  return qrcp(P.ia * c + P.ib);
 }
 template <> __device__ __forceinline__ float rho_of(const Prm<float>& P, float c) {
   return qdiv(1.0f, P.ia * c + P.ib);
@@ -230,34 +267,32 @@ __device__ __forceinline__ T op_p(const Prm<T>& P, const Lv<T>& L, int k) {
 // Momentum row d (0: x row at x-edge k, unknown u; 1: y row at y-edge k,
 // unknown v) of (pm-num-mx) from the per-step assembled stencil (the arrays
 // Cu.. / Cv.. of Lv): the same sum as op_u / op_v, term by term, regrouped by
-// unknown.  Ar = A rho(c) on the edge.  s is the stride along the edge normal,
-// t across it; a the row's own velocity, b the other one.
+// unknown.  rs = the sum of rho(c) over the edge's two cells.  s is the stride
+// along the edge normal, t across it; a the row's own velocity, b the other one.
 template <typename T>
-__device__ __forceinline__ T mom_asm(const Prm<T>& P, const Lv<T>& L, int d, int k, T Ar) {
+__device__ __forceinline__ T mom_asm(const Lv<T>& L, int d, int k, T rs) {
   const int s = d ? L.pitch : 1, t = d ? 1 : L.pitch;
   const T *a = d ? L.v : L.u, *b = d ? L.u : L.v;
   const T *C = d ? L.Cv : L.Cu, *aP = d ? L.aPv : L.aPu, *aM = d ? L.aMv : L.aMu;
   const T *tP = d ? L.tPv : L.tPu, *tM = d ? L.tMv : L.tMu;
   const T *M0 = d ? L.M0v : L.M0u, *M1 = d ? L.M1v : L.M1u;
-  T ae = a[k];
-  T r = (d ? L.T0v : L.T0u)[k] + (C[k] + T(0.5) * P.idt * Ar) * ae;
+  T r = (d ? L.T0v : L.T0u)[k] + (C[k] + L.k.qidt * rs) * a[k];
   r += aP[k] * a[k + s] + aM[k] * a[k - s] + tP[k] * a[k + t] + tM[k] * a[k - t];
   // the grad-div term's cross derivative of the other velocity
   T vl = L.visn[k], vr = L.visn[k + s];
-  r -= (P.iRe * L.ih2 * T(1.0 / 3.0)) * (vr * (b[k + s] - b[k + s - t]) - vl * (b[k] - b[k - t]));
-  r += (L.p[k + s] - L.p[k]) * (L.ih * P.iM) + M0[k] * L.mu[k] + M1[k] * L.mu[k + s];
-  if (d) r += P.Fr_inv * L.Arv[k];
+  r -= L.k.v3 * (vr * (b[k + s] - b[k + s - t]) - vl * (b[k] - b[k - t]));
+  r += (L.p[k + s] - L.p[k]) * L.k.ihM + M0[k] * L.mu[k] + M1[k] * L.mu[k + s];
   return r;
 }
 
 // x row of (pm-num-mx) at edge u_{i+1/2,j} (array index k = at(i,j)); cells k (left), k+1 (right),
 // vertices k (top, (i+1/2, j+1/2)) and k-W (bottom); (e1e1-1), (e1e1-2) and (e1e1)
-// (Ar = (rho(c_k) + rho(c_{k+1})) / 2, the density average on the edge).  PST =
+// (rs = rho(c_k) + rho(c_{k+1}), twice the density average on the edge).  PST =
 // false drops the pressure and surface-tension terms: the intermediate-velocity
 // row of the projection method (pj-num-mx).
 template <typename T, bool PST = true>
-__device__ __forceinline__ T op_u(const Prm<T>& P, const Lv<T>& L, int k, T Ar) {
-  if constexpr (PST && sizeof(T) == 8) return mom_asm(P, L, 0, k, Ar);  // FP64 primitive row
+__device__ __forceinline__ T op_u(const Prm<T>& P, const Lv<T>& L, int k, T rs) {
+  if constexpr (PST && sizeof(T) == 8) return mom_asm(L, 0, k, rs);  // FP64 primitive row
   const int W = L.pitch;
   const T *u = L.u, *vis = L.visn, *rn = L.rhon;
   T ue = u[k];
@@ -266,7 +301,7 @@ __device__ __forceinline__ T op_u(const Prm<T>& P, const Lv<T>& L, int k, T Ar) 
   T dvr = dxr + (L.v[k + 1] - L.v[k + 1 - W]) * L.ih;
   T Dt = (u[k + W] - ue) * L.ih, Db = (ue - u[k - W]) * L.ih;
   T conv = T(0.5) * (L.Sx[k + 1] * dxr + L.Sx[k] * dxl + L.Qx[k] * Dt + L.Qx[k - W] * Db);
-  T time = ue * L.T1u[k] + L.T0u[k] + T(0.5) * P.idt * Ar * ue;
+  T time = ue * (L.T1u[k] + L.k.qidt * rs) + L.T0u[k];
   T r = time + conv;
   if constexpr (PST) {
     T press = (L.p[k + 1] - L.p[k]) * L.ih * P.iM;
@@ -280,16 +315,16 @@ __device__ __forceinline__ T op_u(const Prm<T>& P, const Lv<T>& L, int k, T Ar) 
 }
 template <typename T>
 __device__ __forceinline__ T op_u(const Prm<T>& P, const Lv<T>& L, int k) {
-  return op_u(P, L, k, T(0.5) * (rho_of(P, L.c[k]) + rho_of(P, L.c[k + 1])));
+  return op_u(P, L, k, rho_of(P, L.c[k]) + rho_of(P, L.c[k + 1]));
 }
 
 // y row of (pm-num-mx) at edge v_{i,j+1/2} (index k = at(i,j)); cells k (bottom), k+W (top),
-// vertices k (east, (i+1/2, j+1/2)) and k-1 (west); plus gravity (1/Fr) A_y rho^n
+// vertices k (east, (i+1/2, j+1/2)) and k-1 (west); gravity (1/Fr) A_y rho^n is in T0v
 // PST = false: the projection method's intermediate-velocity row, without
 // pressure, surface tension and gravity (those act in (pj-num-pjx))
 template <typename T, bool PST = true>
-__device__ __forceinline__ T op_v(const Prm<T>& P, const Lv<T>& L, int k, T Ar) {
-  if constexpr (PST && sizeof(T) == 8) return mom_asm(P, L, 1, k, Ar);  // FP64 primitive row
+__device__ __forceinline__ T op_v(const Prm<T>& P, const Lv<T>& L, int k, T rs) {
+  if constexpr (PST && sizeof(T) == 8) return mom_asm(L, 1, k, rs);  // FP64 primitive row
   const int W = L.pitch;
   const T *v = L.v, *vis = L.visn, *rn = L.rhon;
   T ve = v[k];
@@ -298,7 +333,7 @@ __device__ __forceinline__ T op_v(const Prm<T>& P, const Lv<T>& L, int k, T Ar) 
   T dvt = dyt + (L.u[k + W] - L.u[k + W - 1]) * L.ih;
   T De = (v[k + 1] - ve) * L.ih, Dw = (ve - v[k - 1]) * L.ih;
   T conv = T(0.5) * (L.Qy[k] * De + L.Qy[k - 1] * Dw + L.Sy[k + W] * dyt + L.Sy[k] * dyb);
-  T time = ve * L.T1v[k] + L.T0v[k] + T(0.5) * P.idt * Ar * ve;
+  T time = ve * (L.T1v[k] + L.k.qidt * rs) + L.T0v[k];
   T r = time + conv;
   if constexpr (PST) {
     T press = (L.p[k + W] - L.p[k]) * L.ih * P.iM;
@@ -308,12 +343,11 @@ __device__ __forceinline__ T op_v(const Prm<T>& P, const Lv<T>& L, int k, T Ar) 
   T vb = vis[k], vt = vis[k + W];
   T visc = -P.iRe * L.ih * ((L.Av[k] * De - L.Av[k - 1] * Dw) + (vt * dyt - vb * dyb) +
                             (vt * dvt - vb * dvb) * T(1.0 / 3.0));
-  if constexpr (PST) return r + visc + P.Fr_inv * L.Arv[k];
   return r + visc;
 }
 template <typename T>
 __device__ __forceinline__ T op_v(const Prm<T>& P, const Lv<T>& L, int k) {
-  return op_v(P, L, k, T(0.5) * (rho_of(P, L.c[k]) + rho_of(P, L.c[k + L.pitch])));
+  return op_v(P, L, k, rho_of(P, L.c[k]) + rho_of(P, L.c[k + L.pitch]));
 }
 
 // ---------------------------------------------------------------------------
@@ -405,11 +439,11 @@ __device__ __forceinline__ T opp_mu(const Prm<T>& P, const Lv<T>& L, int k) {
 }
 template <typename T>
 __device__ __forceinline__ T opp_u(const Prm<T>& P, const Lv<T>& L, int k) {
-  return op_u<T, false>(P, L, k, T(0.5) * (rho_of(P, L.c[k]) + rho_of(P, L.c[k + 1])));
+  return op_u<T, false>(P, L, k, rho_of(P, L.c[k]) + rho_of(P, L.c[k + 1]));
 }
 template <typename T>
 __device__ __forceinline__ T opp_v(const Prm<T>& P, const Lv<T>& L, int k) {
-  return op_v<T, false>(P, L, k, T(0.5) * (rho_of(P, L.c[k]) + rho_of(P, L.c[k + L.pitch])));
+  return op_v<T, false>(P, L, k, rho_of(P, L.c[k]) + rho_of(P, L.c[k + L.pitch]));
 }
 
 // ---------------------------------------------------------------------------

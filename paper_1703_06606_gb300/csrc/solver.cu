@@ -947,10 +947,12 @@ void queue_begin(qnsch_s* s, double dt) {
   cudaMemcpyAsync(F.un - pitch - 1, s->su - pitch - 1, bytes, cudaMemcpyDeviceToDevice, s->stream);
   cudaMemcpyAsync(F.vn - pitch - 1, s->sv - pitch - 1, bytes, cudaMemcpyDeviceToDevice, s->stream);
   qn::launch_rho_fill(P, F, s->stream);
-  qn::launch_frozen(P, F, s->stream);
+  Prm<double> Pf = P;  // the frozen rows carry gravity in the primitive method only
+  if (s->scheme) Pf.Fr_inv = 0.0;
+  qn::launch_frozen(Pf, F, s->stream);
   for (int l = 1; l < s->nlev; ++l) {
     qn::launch_restrict_frozen(s->L[l - 1], s->L[l], s->stream);
-    qn::launch_frozen(P, s->L[l], s->stream);
+    qn::launch_frozen(Pf, s->L[l], s->stream);
   }
   if (s->precision == 1) {
     for (int l = 0; l < s->nlev; ++l) qn::launch_cast_frozen(s->L[l], s->Ef[l], s->stream);
