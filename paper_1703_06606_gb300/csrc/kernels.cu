@@ -162,10 +162,10 @@ __global__ void k_finalize(const double* part, int nparts, int nv, int nmax_firs
 // differences, scaled once by the level's constants.
 // sum over the faces of (m(c^n) of both cells) (d mu + alpha d p): 2 h^2 Pe
 // times the diffusion of N_c
-template <typename T>
-__device__ __forceinline__ T flux_sum(const Prm<T>& P, const Lv<T>& L, int k) {
+template <typename T, class LV>
+__device__ __forceinline__ T flux_sum(const Prm<T>& P, const LV& L, int k) {
   const int W = L.pitch;
-  const T *mob = L.mobn, *mu = L.mu, *p = L.p;
+  auto mob = L.mobn; auto mu = L.mu; auto p = L.p;
   const int off[4] = {1, -1, W, -W};
   T mk = mob[k], s = T(0);
   if constexpr (sizeof(T) == 8) {
@@ -185,21 +185,22 @@ __device__ __forceinline__ T flux_sum(const Prm<T>& P, const Lv<T>& L, int k) {
   return s;
 }
 // the advection (e1e2) of N_c
-template <typename T>
-__device__ __forceinline__ T adv_sum(const Lv<T>& L, int k) {
+template <class LV>
+__device__ __forceinline__ typename LV::real adv_sum(const LV& L, int k) {
+  typedef typename LV::real T;
   const int W = L.pitch;
-  const T* rn = L.rhon;
+  auto rn = L.rhon;
   return rn[k + 1] * L.Tx[k] * L.u[k] + rn[k - 1] * L.Tx[k - 1] * L.u[k - 1] +
          rn[k + W] * L.Ty[k] * L.v[k] + rn[k - W] * L.Ty[k - W] * L.v[k - W];
 }
 // (pm-num-chem) (op_mu with its constants folded): with S = rho + rho^n, A(c) =
 // c (c - 1), 8 rho^{n+1/2} g = S (A + A^n)(c + c^n - 1) and 8 (F + F^n)/2 =
 // A^2 + (A^n)^2
-template <typename T>
-__device__ __forceinline__ T chem_full(const Prm<T>& P, const Lv<T>& L, int k, T rk,
+template <typename T, class LV>
+__device__ __forceinline__ T chem_full(const Prm<T>& P, const LV& L, int k, T rk,
                                        const T (&rq)[4]) {
   const int W = L.pitch;
-  const T *c = L.c, *cn = L.cn, *rn = L.rhon;
+  auto c = L.c; auto cn = L.cn; auto rn = L.rhon;
   const int off[4] = {1, -1, W, -W};
   T ck = c[k], cnk = cn[k], rnk = rn[k];
   T S = rk + rnk, ch = ck + cnk;
@@ -221,8 +222,8 @@ __device__ __forceinline__ T chem_full(const Prm<T>& P, const Lv<T>& L, int k, T
 
 // r = f - N(x) (MODE 0; val receives |r| and r^2 per family) or f += N(x) (MODE 1)
 // at thread (i,j): cell families at (i,j), u-edge (i,j) and v-edge (i,j)
-template <typename T, int MODE, class Form>
-__device__ __forceinline__ void residual_cell(const Prm<T>& P, const Lv<T>& L, int i, int j,
+template <typename T, int MODE, class Form, class LV>
+__device__ __forceinline__ void residual_cell(const Prm<T>& P, const LV& L, int i, int j,
                                               double (&val)[10]) {
   int k = L.at(i, j);
   bool hu = i <= L.uhi(), hv = j < L.m2;
@@ -231,7 +232,7 @@ __device__ __forceinline__ void residual_cell(const Prm<T>& P, const Lv<T>& L, i
     // rho(c) of the cell and its neighbours, shared by the five rows, and the
     // flux sum shared by N_c and N_p
     const int W = L.pitch;
-    const T* rc = L.rhoc;
+    auto rc = L.rhoc;
     T rk = rc[k];
     const T rq[4] = {rc[k + 1], rc[k - 1], rc[k + W], rc[k - W]};
     T flux = flux_sum(P, L, k);
@@ -242,7 +243,7 @@ __device__ __forceinline__ void residual_cell(const Prm<T>& P, const Lv<T>& L, i
     nv = op_v(P, L, k, rk + rq[2]);  // also on boundary edges (padded arrays); masked below
   } else if constexpr (std::is_same<Form, ProjForm>::value) {
     const int W = L.pitch;
-    const T* rc = L.rhoc;
+    auto rc = L.rhoc;
     T rk = rc[k];
     const T rq[4] = {rc[k + 1], rc[k - 1], rc[k + W], rc[k - W]};
     T w[4];
@@ -324,14 +325,14 @@ static int residual_rows(const Lv<T>& L) {
 // unfolded sums take about 190.  On a wall face the ghost's c and c^n are the
 // cell's own, so its differences vanish and only the coefficients of c (2 rho
 // sums) and the mobilities need the face left out.
-template <typename T>
-__device__ __forceinline__ void ch_system_full(const Prm<T>& P, const Lv<T>& L, int i, int j,
+template <typename T, class LV>
+__device__ __forceinline__ void ch_system_full(const Prm<T>& P, const LV& L, int i, int j,
                                                T (&J)[2][2], T (&R)[2]) {
   const int W = L.pitch;
   const int k = L.at(i, j);
   const int off[4] = {1, -1, W, -W};
   const bool wall[4] = {!L.px && i == L.m1, !L.px && i == 1, j == L.m2, j == 1};
-  const T *c = L.c, *cn = L.cn, *rn = L.rhon, *rc = L.rhoc, *mob = L.mobn, *mu = L.mu, *p = L.p;
+  auto c = L.c; auto cn = L.cn; auto rn = L.rhon; auto rc = L.rhoc; auto mob = L.mobn; auto mu = L.mu; auto p = L.p;
   T ck = c[k], cnk = cn[k], rk = rc[k], rnk = rn[k], muk = mu[k];
   T mk = mob[k], fk = muk + P.alpha * p[k];
   T S = rk + rnk, ch = ck + cnk;
@@ -369,8 +370,8 @@ __device__ __forceinline__ void ch_system_full(const Prm<T>& P, const Lv<T>& L, 
 
 // The 2x2 CH system of cell (i,j): residuals R = N - f of (N_c, N_mu) and their
 // Jacobian J in (c, mu), neighbours frozen, at the full values c, mu
-template <typename T, class Form>
-__device__ __forceinline__ void ch_system(const Prm<T>& P, const Lv<T>& L, int i, int j,
+template <typename T, class Form, class LV>
+__device__ __forceinline__ void ch_system(const Prm<T>& P, const LV& L, int i, int j,
                                           T (&J)[2][2], T (&R)[2]) {
   const int W = L.pitch;
   int k = L.at(i, j);
@@ -394,7 +395,7 @@ __device__ __forceinline__ void ch_system(const Prm<T>& P, const Lv<T>& L, int i
     Rc = Form::Nc(P, L, k) - L.fc[k];
     Rm = Form::Nmu(P, L, k) - L.fmu[k];
   }
-  const T *cn = L.cn, *rn = L.rhon, *mob = L.mobn;
+  auto cn = L.cn; auto rn = L.rhon; auto mob = L.mobn;
   // full values c, mu at which the local Jacobian is evaluated
   T ck = Form::val_c(L, k), cnk = cn[k], mk = Form::val_mu(L, k);
   T drho = -P.alpha * rho * rho;
@@ -443,8 +444,8 @@ __device__ __forceinline__ void ch_system(const Prm<T>& P, const Lv<T>& L, int i
   R[1] = Rm;
 }
 
-template <typename T, class Form>
-__device__ __forceinline__ void ch_cell(const Prm<T>& P, const Lv<T>& L, int i, int j) {
+template <typename T, class Form, class LV>
+__device__ __forceinline__ void ch_cell(const Prm<T>& P, const LV& L, int i, int j) {
   T J[2][2], R[2];
   ch_system<T, Form>(P, L, i, j, J, R);
   T idet = qrcp(J[0][0] * J[1][1] - J[0][1] * J[1][0]);
@@ -479,19 +480,33 @@ __device__ __forceinline__ T team_sum(T v) {
 
 // u^{n+1} at face q (W, E, S, N) of cell k (0 on a wall face), as proj_faces
 // gives it: rho(c) of the cell rk and of the face's neighbour rn
-template <typename T>
-__device__ __forceinline__ T proj_face_team(const Prm<T>& P, const Lv<T>& L, int k, int q, bool open, T rk,
+template <typename T, class LV>
+__device__ __forceinline__ T proj_face_team(const Prm<T>& P, const LV& L, int k, int q, bool open, T rk,
                                             T rn) {
   const int d = q >> 1, off = d ? L.pitch : 1;
   const bool hi = q & 1;  // E or N: the face's velocity sits at k
   const int a = hi ? k : k - off;
-  const T *vel = d ? L.v : L.u, *c = L.c, *mu = L.mu, *p = L.p;
+  auto vel = d ? L.v : L.u; auto c = L.c; auto mu = L.mu; auto p = L.p;
   T ra = hi ? rk : rn, rb = hi ? rn : rk;
   T Ar = T(0.5) * (ra + rb);
   T dp = (p[a + off] - p[a]) * L.ih;
   T st = T(0.5) * (rb * mu[a] + ra * mu[a + off]) * (c[a + off] - c[a]) * L.ih;
   T grav = d ? P.Fr_inv / P.idt : T(0);
   return open ? vel[a] + (st - dp) * P.iM / (Ar * P.idt) - grav : T(0);
+}
+
+// rho(c) of the full value at cell k and, on error levels, of the base: what
+// the rows of a team's lane need of a cell
+template <typename T>
+struct RhoPair {
+  T r, b;
+};
+template <typename T, class Form, class LV>
+__device__ __forceinline__ RhoPair<T> rho_pair(const Prm<T>& P, const LV& L, int k) {
+  if constexpr (std::is_same<Form, ErrForm>::value)
+    return {Form::rho(P, L, k), rho_of(P, L.Bc[k])};
+  else
+    return {Form::rho(P, L, k), T(0)};
 }
 
 // sums over the four lanes of a team of eight values each lane holds, every
@@ -534,22 +549,22 @@ struct ChRows {
 // ch_team_rows for the FP64 primitive form: ch_system_full's sums, a face a lane
 __device__ __forceinline__ ChRows<double> ch_team_rows_full(const Prm<double>& P,
                                                             const Lv<double>& L, int i, int j,
-                                                            int q, bool open) {
+                                                            int q, bool open, double rk, double rq) {
   typedef double T;
   const int W = L.pitch;
   const int d = q >> 1;
   const int k = L.at(i, j);
   const int nq = k + (q == 0 ? -1 : q == 1 ? 1 : q == 2 ? -W : W);
   const int kf = q == 0 ? k - 1 : (q == 2 ? k - W : k);  // edge of face q
-  const T *c = L.c, *cn = L.cn, *rn = L.rhon, *rc = L.rhoc, *mob = L.mobn;
-  T ck = c[k], cnk = cn[k], rk = rc[k], rnk = rn[k], muk = L.mu[k];
+  auto c = L.c; auto cn = L.cn; auto rn = L.rhon; auto mob = L.mobn;
+  T ck = c[k], cnk = cn[k], rnk = rn[k], muk = L.mu[k];
   T cq = c[nq], rnq = rn[nq];
-  T gq = rnq * (d ? L.Ty[kf] : L.Tx[kf]);  // rho^n D c^n / 2 at face q
+  T gq = rnq * L.pair(d, L.Tx, L.Ty)[kf];  // rho^n D c^n / 2 at face q
   T m = mob[k] + mob[nq];
-  T S = rk + rnk, ch = ck + cnk, dq = cq - ck, D = (cq + cn[nq]) - ch, H = rc[nq] + rnq;
+  T S = rk + rnk, ch = ck + cnk, dq = cq - ck, D = (cq + cn[nq]) - ch, H = rq + rnq;
   T v[8] = {m * (L.mu[nq] + P.alpha * L.p[nq] - (muk + P.alpha * L.p[k])),
             open ? m : T(0),
-            gq * (d ? L.v[kf] : L.u[kf]),
+            gq * L.pair(d, L.u, L.v)[kf],
             dq * dq,
             dq,
             (H + S) * D,
@@ -579,33 +594,34 @@ __device__ __forceinline__ ChRows<double> ch_team_rows_full(const Prm<double>& P
   return R;
 }
 
-template <typename T, class Form>
-__device__ __forceinline__ ChRows<T> ch_team_rows(const Prm<T>& P, const Lv<T>& L, int i, int j, int q,
-                                                  bool open) {
-  if constexpr (std::is_same<Form, FullForm>::value)
-    return ch_team_rows_full(P, L, i, j, q, open);
+template <typename T, class Form, class LV>
+__device__ __forceinline__ ChRows<T> ch_team_rows(const Prm<T>& P, const LV& L, int i, int j, int q,
+                                                  bool open, RhoPair<T> ra, RhoPair<T> rb) {
+  if constexpr (std::is_same<Form, FullForm>::value) {
+    return ch_team_rows_full(P, L, i, j, q, open, ra.r, rb.r);
+  } else {
   const int W = L.pitch;
   const int d = q >> 1;
   const T ih2 = L.ih2;
   int k = L.at(i, j);
-  const T *mob = L.mobn, *cn = L.cn, *rn = L.rhon;
+  auto mob = L.mobn; auto cn = L.cn; auto rn = L.rhon;
   const int nq = k + (q == 0 ? -1 : q == 1 ? 1 : q == 2 ? -W : W);
   const int kf = q == 0 ? k - 1 : (q == 2 ? k - W : k);  // edge of face q
   // full values at the cell and at the face's neighbour
   T ck = Form::val_c(L, k), cnk = cn[k], mk = Form::val_mu(L, k), rnk = rn[k];
-  T rho = Form::rho(P, L, k);
-  T cq = Form::val_c(L, nq), rq = Form::rho(P, L, nq);
+  T rho = ra.r;
+  T cq = Form::val_c(L, nq), rq = rb.r;
   T drho = -P.alpha * rho * rho;
   T rh = T(0.5) * (rho + rnk);
   T chk = ck + cnk;
   T am = mob[nq] + mob[k];
-  T gq = rn[nq] * (d ? L.Ty[kf] : L.Tx[kf]);  // rho^n D c^n / 2 at face q
+  T gq = rn[nq] * L.pair(d, L.Tx, L.Ty)[kf];  // rho^n D c^n / 2 at face q
   T dlt = cq - ck;
   // face sums: diffusion flux (N_c and the mass row), sum A m over open faces,
   // advection of N_c, and the Jacobian's G, dG/dc and d(div)/dc terms
   T sflux = team_sum<T>(am * ((L.mu[nq] - L.mu[k]) + P.alpha * (L.p[nq] - L.p[k])));
   T sm = team_sum<T>(open ? am : T(0));
-  T sadv = team_sum<T>(gq * (d ? L.v[kf] : L.u[kf]));
+  T sadv = team_sum<T>(gq * L.pair(d, L.u, L.v)[kf]);
   T G2 = team_sum<T>(dlt * dlt);
   T dG = team_sum<T>(open ? -dlt : T(0));
   T dd = team_sum<T>(open ? T(0.5) * drho * ((cq + cn[nq]) - chk) - (rh + T(0.5) * (rq + rn[nq])) : T(0));
@@ -623,12 +639,12 @@ __device__ __forceinline__ ChRows<T> ch_team_rows(const Prm<T>& P, const Lv<T>& 
     Nm = rnk * mk - P.K * bulk - grad + P.Lam * T(0.25) * ih2 * sdv;
     sJ11 = team_sum<T>(T(0.5) * ((q & 1) ? -rq * wq : rq * wq) * L.ih);
   } else if constexpr (std::is_same<Form, ErrForm>::value) {
-    const T *e = L.c, *B = L.Bc;
+    auto e = L.c; auto B = L.Bc;
     T ek = e[k], Ck = B[k];
-    T rC = rho_of(P, Ck);
+    T rC = ra.b;
     Nc = ek * (rho + rsec_(P, rho, rC) * L.Bdc[k]) * P.idt + sadv - L.k.dif * sflux;
     T dC = B[nq] - Ck, de = e[nq] - ek;
-    T rCq = rho_of(P, B[nq]);
+    T rCq = rb.b;
     T dr = rsec_(P, rho, rC) * ek;
     T drq = rsec_(P, rq, rCq) * e[nq];
     T chP = Ck + cnk;
@@ -674,16 +690,20 @@ __device__ __forceinline__ ChRows<T> ch_team_rows(const Prm<T>& P, const Lv<T>& 
   R.drho = drho;
   R.gq = gq;
   return R;
+  }
 }
 
 // CH step of cell (i,j) by a team of four lanes (ch_team_rows), every lane
 // solving the 2x2 Newton step; lane 0 stores.  All 32 lanes of the warp call
 // this (ok = false: a spare team on cell (1,1), no store).
-template <typename T, class Form>
-__device__ __forceinline__ void ch_team(const Prm<T>& P, const Lv<T>& L, int i, int j, bool ok) {
+template <typename T, class Form, class LV>
+__device__ __forceinline__ void ch_team(const Prm<T>& P, const LV& L, int i, int j, bool ok) {
   const int q = threadIdx.x & 3;
   const bool open = q == 0 ? (L.px || i > 1) : q == 1 ? (L.px || i < L.m1) : q == 2 ? j > 1 : j < L.m2;
-  ChRows<T> R = ch_team_rows<T, Form>(P, L, i, j, q, open);
+  const int k0 = L.at(i, j);
+  const int nq = k0 + (q == 0 ? -1 : q == 1 ? 1 : q == 2 ? -L.pitch : L.pitch);
+  ChRows<T> R = ch_team_rows<T, Form>(P, L, i, j, q, open, rho_pair<T, Form>(P, L, k0),
+                                      rho_pair<T, Form>(P, L, nq));
   T idet = qrcp(R.J11 * R.J22 - R.J12 * R.J21);
   T dc = (R.J22 * R.Rc - R.J12 * R.Rm) * idet;
   T dm = (R.J11 * R.Rm - R.J21 * R.Rc) * idet;
@@ -724,12 +744,12 @@ __global__ void __launch_bounds__(64) k_ch_team(Prm<T> P, Lv<T> L, int colour) {
 // The 5x5 Vanka system of cell (i,j): A = Jacobian of (N_u W, N_u E, N_v S,
 // N_v N, N_p) in (u_W, u_E, v_S, v_N, p), b = residuals N - f; rows and
 // columns of wall edges (act = false) replaced by the identity
-template <typename T, class Form>
-__device__ __forceinline__ void vanka_system(const Prm<T>& P, const Lv<T>& L, int i, int j,
+template <typename T, class Form, class LV>
+__device__ __forceinline__ void vanka_system(const Prm<T>& P, const LV& L, int i, int j,
                                              T (&A)[5][5], T (&b)[5], bool (&act)[5]) {
   const int W = L.pitch;
   const T ih = L.ih, ih2 = L.ih2;
-  const T* vis = L.visn;
+  auto vis = L.visn;
   int k = L.at(i, j);
   int eW = (L.px && i == 1) ? L.m1 : i - 1;
   int kW = L.at(eW, j);
@@ -810,7 +830,7 @@ __device__ __forceinline__ void vanka_system(const Prm<T>& P, const Lv<T>& L, in
     A[3][4] = -L.k.ihM;
   }
   {
-    const T* mob = L.mobn;
+    auto mob = L.mobn;
     bool wall[4] = {!L.px && i == L.m1, !L.px && i == 1, j == L.m2, j == 1};
     const int off[4] = {1, -1, W, -W};
     T sm = 0;
@@ -933,8 +953,8 @@ __device__ __forceinline__ void solve_vanka(const T (&A)[5][5], T (&b)[5], const
   if constexpr (NP == 5) b[4] = pr;
 }
 
-template <typename T, class Form>
-__device__ __forceinline__ void vanka_cell(const Prm<T>& P, const Lv<T>& L, int i, int j, T omega) {
+template <typename T, class Form, class LV>
+__device__ __forceinline__ void vanka_cell(const Prm<T>& P, const LV& L, int i, int j, T omega) {
   T A[5][5], b[5];
   bool act[5];
   vanka_system<T, Form>(P, L, i, j, A, b, act);
@@ -1027,8 +1047,8 @@ __device__ __forceinline__ void solve_coupled7(const T (&A)[7][7], T (&b)[7], co
 // the CH advection (e1e2) and (alpha/Pe) grad.(A m grad p) in N_c, the
 // (alpha/Pe) grad.(A m grad mu) term of N_p, and the rho(c) and surface-tension
 // (e1e1) terms of the momentum rows.
-template <typename T, class Form>
-__device__ __forceinline__ void coupled_cell(const Prm<T>& P, const Lv<T>& L, int i, int j, T omega) {
+template <typename T, class Form, class LV>
+__device__ __forceinline__ void coupled_cell(const Prm<T>& P, const LV& L, int i, int j, T omega) {
   T A5[5][5], b5[5], J2[2][2], R2[2];
   bool act[5];
   vanka_system<T, Form>(P, L, i, j, A5, b5, act);
@@ -1054,7 +1074,7 @@ __device__ __forceinline__ void coupled_cell(const Prm<T>& P, const Lv<T>& L, in
   int k = L.at(i, j);
   int eW = (L.px && i == 1) ? L.m1 : i - 1;
   int kW = L.at(eW, j);
-  const T *rn = L.rhon, *mob = L.mobn;
+  auto rn = L.rhon; auto mob = L.mobn;
   bool wall[4] = {!L.px && i == L.m1, !L.px && i == 1, j == L.m2, j == 1};
   const int off[4] = {1, -1, W, -W};
   T sm = T(0);
@@ -1107,15 +1127,17 @@ __device__ __forceinline__ void coupled_cell(const Prm<T>& P, const Lv<T>& L, in
 
 // Vanka colour of cell (i,j): (2i + j) mod 8 (periodic x, m1 = 0 mod 4) or
 // (i + 2j) mod kcol (kcol = 5 with walls, the smallest divisor >= 5 of m1 otherwise)
-template <typename T>
-__device__ __forceinline__ int vanka_colour(const Lv<T>& L, int i, int j) {
+template <class LV>
+__device__ __forceinline__ int vanka_colour(const LV& L, int i, int j) {
+  typedef typename LV::real T;
   return L.c8 ? (2 * i + j) & 7 : (i + 2 * j) % L.kcol;
 }
 
 // first cell i0 >= 1 of colour `colour` in row j and the stride between cells
 // of that colour in the row; false if the row has none
-template <typename T>
-__device__ __forceinline__ bool colour_row(const Lv<T>& L, int colour, int j, int& i0, int& stride) {
+template <class LV>
+__device__ __forceinline__ bool colour_row(const LV& L, int colour, int j, int& i0, int& stride) {
+  typedef typename LV::real T;
   if (L.c8) {
     int d = (colour - j) & 7;
     if (d & 1) return false;
@@ -1137,8 +1159,9 @@ struct ColourSlots {
   int j0, rstep, mpr, n;
 };
 
-template <typename T>
-__host__ __device__ __forceinline__ ColourSlots vanka_slots(const Lv<T>& L, int col) {
+template <class LV>
+__host__ __device__ __forceinline__ ColourSlots vanka_slots(const LV& L, int col) {
+  typedef typename LV::real T;
   ColourSlots cs;
   if (L.c8) {
     cs.j0 = ((col - 1) & 1) ? 2 : 1;  // rows with (col - j) even
@@ -1153,9 +1176,10 @@ __host__ __device__ __forceinline__ ColourSlots vanka_slots(const Lv<T>& L, int 
   return cs;
 }
 
-template <typename T>
-__device__ __forceinline__ bool vanka_slot_cell(const Lv<T>& L, int col, const ColourSlots& cs, int t,
+template <class LV>
+__device__ __forceinline__ bool vanka_slot_cell(const LV& L, int col, const ColourSlots& cs, int t,
                                                 int& i, int& j) {
+  typedef typename LV::real T;
   j = cs.j0 + cs.rstep * (t / cs.mpr);
   int i0, stride;
   if (!colour_row(L, col, j, i0, stride)) return false;
@@ -1194,8 +1218,8 @@ __global__ void __launch_bounds__(SNT) k_coupled(Prm<T> P, Lv<T> L, int colour, 
 // --------------------------------------------------------------------------
 // step 2: exact solve of the 4x4 block of the intermediate velocities
 // (ut_W, ut_E, vt_S, vt_N) of cell (i,j) in the rows of (pj-num-mx)
-template <typename T, class Form>
-__device__ __forceinline__ void vanka4_cell(const Prm<T>& P, const Lv<T>& L, int i, int j, T omega) {
+template <typename T, class Form, class LV>
+__device__ __forceinline__ void vanka4_cell(const Prm<T>& P, const LV& L, int i, int j, T omega) {
   T A5[5][5], b5[5];
   bool act[5];
   vanka_system<T, Form>(P, L, i, j, A5, b5, act);
@@ -1224,11 +1248,11 @@ __global__ void __launch_bounds__(SNT) k_vanka4(Prm<T> P, Lv<T> L, int colour, T
 // step 3: Gauss-Seidel on (pj-num-mass) for p_ij.  The row is affine in p_ij:
 // u^{n+1} on an open face carries -dt/(M h A rho(c)) times the pressure of each
 // adjacent cell, plus the diffusion term (alpha^2/Pe) A m / h^2.
-template <typename T>
-__device__ __forceinline__ void pgs_cell(const Prm<T>& P, const Lv<T>& L, int i, int j) {
+template <typename T, class LV>
+__device__ __forceinline__ void pgs_cell(const Prm<T>& P, const LV& L, int i, int j) {
   const int W = L.pitch;
   int k = L.at(i, j);
-  const T* rc = L.rhoc;
+  auto rc = L.rhoc;
   T rk = rc[k];
   const T rq[4] = {rc[k + 1], rc[k - 1], rc[k + W], rc[k - W]};
   T w[4];
@@ -1250,8 +1274,8 @@ __device__ __forceinline__ void pgs_cell(const Prm<T>& P, const Lv<T>& L, int i,
 // pgs_cell by a team of four lanes (lane & 3 = q: face W, E, S, N): lane q
 // takes u^{n+1} at face q, its share of the mass row and of the row's
 // derivative in p_ij; butterflies add them; lane 0 stores.
-template <typename T>
-__device__ __forceinline__ void pgs_team(const Prm<T>& P, const Lv<T>& L, int i, int j, bool ok) {
+template <typename T, class LV>
+__device__ __forceinline__ void pgs_team(const Prm<T>& P, const LV& L, int i, int j, bool ok) {
   const int W = L.pitch;
   const int q = threadIdx.x & 3;
   const bool open = q == 0 ? (L.px || i > 1) : q == 1 ? (L.px || i < L.m1) : q == 2 ? j > 1 : j < L.m2;
@@ -1360,8 +1384,9 @@ __device__ __forceinline__ bool frame_pos(int t, int m1, int m2, int& I, int& J)
   return false;
 }
 
-template <typename T>
-__device__ __forceinline__ void fill_cell_ghost(const Lv<T>& L, T* a, int I, int J) {
+template <class LV, class A>
+__device__ __forceinline__ void fill_cell_ghost(const LV& L, A a, int I, int J) {
+  typedef typename LV::real T;
   if (I < 0 || J < 0) return;
   bool gx = (I == 0 || I == L.m1 + 1), gy = (J == 0 || J == L.m2 + 1);
   if (!gx && !gy) return;
@@ -1370,8 +1395,9 @@ __device__ __forceinline__ void fill_cell_ghost(const Lv<T>& L, T* a, int I, int
   a[L.at(I, J)] = a[L.at(si, sj)];
 }
 
-template <typename T>
-__device__ __forceinline__ T u_interior_or_zero(const Lv<T>& L, const T* a, int I, int J) {
+template <class LV, class A>
+__device__ __forceinline__ typename LV::real u_interior_or_zero(const LV& L, A a, int I, int J) {
+  typedef typename LV::real T;
   // value of u(I, J) for J in 1..m2 after applying the x rule
   if (L.px) {
     int s = I;
@@ -1384,8 +1410,9 @@ __device__ __forceinline__ T u_interior_or_zero(const Lv<T>& L, const T* a, int 
   return a[L.at(I, J)];
 }
 
-template <typename T>
-__device__ __forceinline__ void fill_u_ghost(const Lv<T>& L, T* a, int I, int J) {
+template <class LV, class A>
+__device__ __forceinline__ void fill_u_ghost(const LV& L, A a, int I, int J) {
+  typedef typename LV::real T;
   if (J < 0) return;
   bool xg = L.px ? (I == 0 || I == -1 || I == L.m1 + 1) : (I <= 0 || I >= L.m1);
   bool yg = (J == 0 || J == L.m2 + 1);
@@ -1398,15 +1425,17 @@ __device__ __forceinline__ void fill_u_ghost(const Lv<T>& L, T* a, int I, int J)
   }
 }
 
-template <typename T>
-__device__ __forceinline__ T v_interior_or_zero(const Lv<T>& L, const T* a, int I, int J) {
+template <class LV, class A>
+__device__ __forceinline__ typename LV::real v_interior_or_zero(const LV& L, A a, int I, int J) {
+  typedef typename LV::real T;
   // value of v(I, J) for I in 1..m1 after applying the y (wall) rule
   if (J <= 0 || J >= L.m2) return T(0);
   return a[L.at(I, J)];
 }
 
-template <typename T>
-__device__ __forceinline__ void fill_v_ghost(const Lv<T>& L, T* a, int I, int J) {
+template <class LV, class A>
+__device__ __forceinline__ void fill_v_ghost(const LV& L, A a, int I, int J) {
+  typedef typename LV::real T;
   if (I < 0) return;
   bool xg = (I == 0 || I == L.m1 + 1);
   bool yg = (J <= 0 || J >= L.m2);
@@ -1469,7 +1498,7 @@ __global__ void k_frozen_coef1(Lv<T> L) {
   if (i > L.m1 + 1 || j > L.m2 + 1) return;
   const int W = L.pitch;
   int k = L.at(i, j);
-  const T *rn = L.rhon, *vis = L.visn, *un = L.un, *vn = L.vn, *cn = L.cn;
+  auto rn = L.rhon; auto vis = L.visn; auto un = L.un; auto vn = L.vn; auto cn = L.cn;
   L.Sx[k] = rn[k] * T(0.5) * (un[k] + un[k - 1]);   // cell (i,j)
   L.Sy[k] = rn[k] * T(0.5) * (vn[k] + vn[k - W]);
   if (i <= L.m1 && j <= L.m2) {  // vertex (i+1/2, j+1/2), edges (i+1/2, j), (i, j+1/2)
@@ -1507,9 +1536,9 @@ __global__ void k_frozen_coef2(Lv<T> L) {
 // each neighbour's coefficient is the sum of its convective and viscous
 // parts, and the edge's own coefficient is minus their sum plus t1.  Wall
 // edges keep the undoubled coefficients: the row reads the reflected ghosts.
-template <typename T>
-__device__ __forceinline__ void assemble_row(const Prm<T>& P, const Lv<T>& L, int k, int s, int t,
-                                             T t1, const T* S, const T* Q, const T* Tf, T* C,
+template <typename T, class LV, class A>
+__device__ __forceinline__ void assemble_row(const Prm<T>& P, const LV& L, int k, int s, int t,
+                                             T t1, A S, const T* Q, const T* Tf, T* C,
                                              T* aP, T* aM, T* tP, T* tM, T* M0, T* M1) {
   const T* vis = L.visn;
   const T hc = T(0.5) * L.ih, hv = P.iRe * L.ih2, f43 = T(4.0 / 3.0);
@@ -1541,7 +1570,7 @@ __global__ void k_frozen_coef3(Prm<T> P, Lv<T> L) {
   if (i > L.m1 || j > L.m2) return;
   const int W = L.pitch;
   int k = L.at(i, j);
-  const T* vis = L.visn;
+  auto vis = L.visn;
   const T third = T(1.0 / 3.0);
   if (j >= 1) {  // x-edge (i+1/2, j)
     T Arn = L.Aru[k];
@@ -1572,8 +1601,8 @@ __global__ void k_frozen_coef3(Prm<T> P, Lv<T> L) {
 // --------------------------------------------------------------------------
 // coarse iterate = R x_h (cells: 4-mean; edges: mean of the 2 coincident fine edges),
 // and a copy kept for the correction
-template <typename T>
-__device__ __forceinline__ void restrict_state_cell(const Prm<T>& P, const Lv<T>& F, const Lv<T>& C,
+template <typename T, class LV>
+__device__ __forceinline__ void restrict_state_cell(const Prm<T>& P, const LV& F, const LV& C,
                                                     int I, int J) {
   int kc = C.at(I, J);
   if (I >= 1 && J >= 1) {
@@ -1582,7 +1611,8 @@ __device__ __forceinline__ void restrict_state_cell(const Prm<T>& P, const Lv<T>
     T b = T(0.25) * (F.mu[kf] + F.mu[kf + 1] + F.mu[kf + W] + F.mu[kf + W + 1]);
     T d = T(0.25) * (F.p[kf] + F.p[kf + 1] + F.p[kf + W] + F.p[kf + W + 1]);
     C.c[kc] = a; C.sc[kc] = a;
-    if (C.rhoc) C.rhoc[kc] = rho_of(P, a);
+    if constexpr (LV::has_rho)
+      if (C.rhoc) C.rhoc[kc] = rho_of(P, a);
     C.mu[kc] = b; C.smu[kc] = b;
     C.p[kc] = d; C.sp[kc] = d;
   }
@@ -1609,8 +1639,9 @@ __global__ void k_restrict_state(Prm<T> P, Lv<T> F, Lv<T> C) {
   restrict_state_cell(P, F, C, I, J);
 }
 
-template <typename T>
-__device__ __forceinline__ T ru_at(const Lv<T>& F, int i, int j) {
+template <class LV>
+__device__ __forceinline__ typename LV::real ru_at(const LV& F, int i, int j) {
+  typedef typename LV::real T;
   if (F.px) {
     if (i > F.m1) i -= F.m1;
     if (i < 1) i += F.m1;
@@ -1619,16 +1650,18 @@ __device__ __forceinline__ T ru_at(const Lv<T>& F, int i, int j) {
   }
   return F.ru[F.at(i, j)];
 }
-template <typename T>
-__device__ __forceinline__ T rv_at(const Lv<T>& F, int i, int j) {
+template <class LV>
+__device__ __forceinline__ typename LV::real rv_at(const LV& F, int i, int j) {
+  typedef typename LV::real T;
   if (j <= 0 || j >= F.m2) return T(0);
   return F.rv[F.at(i, j)];
 }
 
 // coarse right-hand side f_H = R r_h (cells: 4-mean; edges: full weighting),
 // to which k_residual<MODE 1> then adds N_H(R x_h)
-template <typename T>
-__device__ __forceinline__ void restrict_res_cell(const Lv<T>& F, const Lv<T>& C, int I, int J) {
+template <class LV>
+__device__ __forceinline__ void restrict_res_cell(const LV& F, const LV& C, int I, int J) {
+  typedef typename LV::real T;
   int kc = C.at(I, J);
   int kf = F.at(2 * I - 1, 2 * J - 1), W = F.pitch;
   C.fc[kc] = T(0.25) * (F.rc[kf] + F.rc[kf + 1] + F.rc[kf + W] + F.rc[kf + W + 1]);
@@ -1688,14 +1721,15 @@ __global__ void k_restrict_frozen(Lv<T> F, Lv<T> C) {
 
 // x_h += P(x_H - saved_H): cells piecewise constant; edges coincident or linear
 // in the normal direction, constant in the tangential direction
-template <typename T>
-__device__ __forceinline__ void prolong_cell(const Prm<T>& P, const Lv<T>& F, const Lv<T>& C, int i,
+template <typename T, class LV>
+__device__ __forceinline__ void prolong_cell(const Prm<T>& P, const LV& F, const LV& C, int i,
                                              int j) {
   int k = F.at(i, j);
   int I = (i + 1) >> 1, J = (j + 1) >> 1;
   int kc = C.at(I, J);
   F.c[k] += C.c[kc] - C.sc[kc];
-  if (F.rhoc) F.rhoc[k] = rho_of(P, F.c[k]);
+  if constexpr (LV::has_rho)
+    if (F.rhoc) F.rhoc[k] = rho_of(P, F.c[k]);
   F.mu[k] += C.mu[kc] - C.smu[kc];
   F.p[k] += C.p[kc] - C.sp[kc];
   if (i <= F.uhi()) {
@@ -1740,8 +1774,9 @@ __global__ void k_prolong(Prm<T> P, Lv<T> F, Lv<T> C) {
 // kernels above, in the same colour order, so the results are the same.
 // --------------------------------------------------------------------------
 // coarse base X_H = R X_h (cells: 4-mean; edges: 2 coincident fine edges), one entry
-template <typename T>
-__device__ __forceinline__ void restrict_base_cell(const Lv<T>& F, const Lv<T>& C, int I, int J) {
+template <class LV>
+__device__ __forceinline__ void restrict_base_cell(const LV& F, const LV& C, int I, int J) {
+  typedef typename LV::real T;
   int kc = C.at(I, J);
   if (I >= 1 && J >= 1) {
     int kf = F.at(2 * I - 1, 2 * J - 1), W = F.pitch;
@@ -1760,8 +1795,9 @@ __device__ __forceinline__ void restrict_base_cell(const Lv<T>& F, const Lv<T>& 
 }
 
 // ghosts of the base arrays
-template <typename T>
-__device__ __forceinline__ void bc_base_cell(const Lv<T>& L, int I, int J) {
+template <class LV>
+__device__ __forceinline__ void bc_base_cell(const LV& L, int I, int J) {
+  typedef typename LV::real T;
   fill_cell_ghost(L, L.Bc, I, J);
   fill_cell_ghost(L, L.Bmu, I, J);
   fill_cell_ghost(L, L.Bdc, I, J);
@@ -1799,14 +1835,16 @@ struct CoarseLevels {
   int base;  // error equation: restrict the base state to L[1..n-1] first
 };
 
-template <typename T>
-__device__ __forceinline__ void bc_unknowns_block(const Lv<T>& L) {
+template <class LV>
+__device__ __forceinline__ void bc_unknowns_block(const LV& L) {
+  typedef typename LV::real T;
   int n = 4 * (L.m1 + 3) + 4 * (L.m2 + 3);
   for (int t = grp_rank(); t < n; t += grp_size()) {
     int I, J;
     if (!frame_pos(t, L.m1, L.m2, I, J)) continue;
     fill_cell_ghost(L, L.c, I, J);
-    if (L.rhoc) fill_cell_ghost(L, L.rhoc, I, J);
+    if constexpr (LV::has_rho)
+      if (L.rhoc) fill_cell_ghost(L, L.rhoc, I, J);
     fill_cell_ghost(L, L.mu, I, J);
     fill_cell_ghost(L, L.p, I, J);
     fill_u_ghost(L, L.u, I, J);
@@ -1823,103 +1861,83 @@ __device__ __forceinline__ void bc_unknowns_block(const Lv<T>& L) {
 // the cells of the colour, and on the smallest levels four lanes share one
 // Vanka block (one edge row each).
 // --------------------------------------------------------------------------
-// Momentum row of the full-form operator in one direction: d = 0 is the x row
-// (op_u, unknown u), d = 1 the y row (op_v, unknown v).  Both directions run
-// the same instructions on different arrays and strides (s along the edge
-// normal, t across it).
-template <typename T>
-struct MomRow {
-  const T *a, *b, *S, *Q, *Tf, *Arn, *Dv, *T1, *T0, *Dg, *B, *f;
-  int s, t, d;
-};
-
-// FullForm uses the per-step row coefficients T1, T0, Dg; ErrForm (the error
-// equation of the defect correction) has none of them and adds the base-state
-// term of the time derivative
-template <typename T, class Form>
-__device__ __forceinline__ MomRow<T> mom_row(const Prm<T>& P, const Lv<T>& L, int d) {
-  MomRow<T> R;
-  R.Dv = d ? L.Dvv : L.Dvu;
-  R.B = d ? L.Bv : L.Bu;
-  R.a = d ? L.v : L.u;
-  R.b = d ? L.u : L.v;
-  R.S = d ? L.Sy : L.Sx;
-  R.Q = d ? L.Qy : L.Qx;
-  R.Tf = d ? L.Ty : L.Tx;
-  R.Arn = d ? L.Arv : L.Aru;
-  R.T1 = d ? L.T1v : L.T1u;
-  R.T0 = d ? L.T0v : L.T0u;
-  R.Dg = d ? L.Dgv : L.Dgu;
-  R.f = d ? L.fv : L.fu;
-  R.s = d ? L.pitch : 1;
-  R.t = d ? 1 : L.pitch;
-  R.d = d;
-  return R;
-}
-
-// N - f of the momentum row at edge index k (op_u / op_v, or opd_u / opd_v for
-// ErrForm), from rho(c) of the edge's two cells (full values) passed in
-template <typename T, class Form>
-__device__ __forceinline__ T mom_residual(const Prm<T>& P, const Lv<T>& L, const MomRow<T>& R, int k,
-                                          T rl, T rr) {
+// N - f of the momentum row in direction d (0: the x row, op_u, unknown u; 1:
+// the y row, op_v, unknown v; opd_u / opd_v for ErrForm) at edge index k, from
+// rho(c) of the edge's two cells.  Both directions run the same instructions
+// on different arrays and strides (s along the edge normal, t across it).
+// FullForm uses the per-step row coefficients; ErrForm (the error equation of
+// the defect correction) has none of them and adds the base-state term of the
+// time derivative.
+template <typename T, class Form, class LV>
+__device__ __forceinline__ T mom_residual(const Prm<T>& P, const LV& L, int d, int k,
+                                          RhoPair<T> l, RhoPair<T> r) {
+  const T f = L.pair(d, L.fu, L.fv)[k];
   // FP64 primitive rows: the per-step assembled stencil
-  if constexpr (std::is_same<Form, FullForm>::value && sizeof(T) == 8)
-    return mom_asm(L, R.d, k, rl + rr) - R.f[k];
-  T Ar = T(0.5) * (rl + rr);
-  const int s = R.s, t = R.t;
-  const T *a = R.a, *b = R.b, *vis = L.visn, *rn = L.rhon;
-  T ae = a[k];
-  T dl = (ae - a[k - s]) * L.ih, dr = (a[k + s] - ae) * L.ih;
-  T dvl = dl + (b[k] - b[k - t]) * L.ih;
-  T dvr = dr + (b[k + s] - b[k + s - t]) * L.ih;
-  T Dp = (a[k + t] - ae) * L.ih, Dm = (ae - a[k - t]) * L.ih;
-  T conv = T(0.5) * (R.S[k + s] * dr + R.S[k] * dl + R.Q[k] * Dp + R.Q[k - t] * Dm);
-  T time;
-  if constexpr (std::is_same<Form, ErrForm>::value) {
-    // rho(X + e) - rho(X) of the two cells by the secant of rho, times the base velocity
-    T dAr = T(0.5) * (rsec_(P, rl, rho_of(P, L.Bc[k])) * L.c[k] +
-                      rsec_(P, rr, rho_of(P, L.Bc[k + s])) * L.c[k + s]);
-    T Arn = R.Arn[k];
-    time = Arn * ae * P.idt + T(0.5) * (Ar - Arn) * P.idt * ae + T(0.5) * dAr * P.idt * R.B[k] +
-           R.Dv[k] * ae;
+  if constexpr (std::is_same<Form, FullForm>::value && sizeof(T) == 8) {
+    return mom_asm(L, d, k, l.r + r.r) - f;
   } else {
-    time = ae * (R.T1[k] + L.k.qidt * (rl + rr)) + R.T0[k];
+    T Ar = T(0.5) * (l.r + r.r);
+    const int s = d ? L.pitch : 1, t = d ? 1 : L.pitch;
+    auto a = L.pair(d, L.u, L.v);
+    auto b = L.pair(1 - d, L.u, L.v);
+    auto S = L.pair(d, L.Sx, L.Sy);
+    auto Q = L.pair(d, L.Qx, L.Qy);
+    auto vis = L.visn;
+    auto rn = L.rhon;
+    T ae = a[k];
+    T dl = (ae - a[k - s]) * L.ih, dr = (a[k + s] - ae) * L.ih;
+    T dvl = dl + (b[k] - b[k - t]) * L.ih;
+    T dvr = dr + (b[k + s] - b[k + s - t]) * L.ih;
+    T Dp = (a[k + t] - ae) * L.ih, Dm = (ae - a[k - t]) * L.ih;
+    T conv = T(0.5) * (S[k + s] * dr + S[k] * dl + Q[k] * Dp + Q[k - t] * Dm);
+    T time;
+    if constexpr (std::is_same<Form, ErrForm>::value) {
+      // rho(X + e) - rho(X) of the two cells by the secant of rho, times the base velocity
+      T dAr = T(0.5) * (rsec_(P, l.r, l.b) * L.c[k] + rsec_(P, r.r, r.b) * L.c[k + s]);
+      T Arn = L.pair(d, L.Aru, L.Arv)[k];
+      time = Arn * ae * P.idt + T(0.5) * (Ar - Arn) * P.idt * ae +
+             T(0.5) * dAr * P.idt * L.pair(d, L.Bu, L.Bv)[k] + L.pair(d, L.Dvu, L.Dvv)[k] * ae;
+    } else {
+      time = ae * (L.pair(d, L.T1u, L.T1v)[k] + L.k.qidt * (l.r + r.r)) +
+             L.pair(d, L.T0u, L.T0v)[k];
+    }
+    T press = T(0), st = T(0);  // the projection method's intermediate-velocity row has neither
+    if constexpr (!std::is_same<Form, ProjForm>::value) {
+      press = (L.p[k + s] - L.p[k]) * L.k.ihM;
+      st = -(rn[k + s] * L.mu[k] + rn[k] * L.mu[k + s]) * L.pair(d, L.Tx, L.Ty)[k] * P.iM;
+    }
+    T vl = vis[k], vr = vis[k + s];
+    T visc = -P.iRe * L.ih * ((vr * dr - vl * dl) + (L.Av[k] * Dp - L.Av[k - t] * Dm) +
+                              (vr * dvr - vl * dvl) * T(1.0 / 3.0));
+    return time + conv + press + st + visc - f;
   }
-  T press = T(0), st = T(0);  // the projection method's intermediate-velocity row has neither
-  if constexpr (!std::is_same<Form, ProjForm>::value) {
-    press = (L.p[k + s] - L.p[k]) * L.ih * P.iM;
-    st = -(rn[k + s] * L.mu[k] + rn[k] * L.mu[k + s]) * R.Tf[k] * P.iM;
-  }
-  T vl = vis[k], vr = vis[k + s];
-  T visc = -P.iRe * L.ih * ((vr * dr - vl * dl) + (L.Av[k] * Dp - L.Av[k - t] * Dm) +
-                            (vr * dvr - vl * dvl) * T(1.0 / 3.0));
-  return time + conv + press + st + visc - R.f[k];
 }
 
 // Diagonal entry dq and residual bq = N - f (0 on a wall edge) of momentum row
 // q of the Vanka block of cell (i,j), for lane q of a team: direction d (0:
-// x-edge, 1: y-edge), edge index ke.  The x and y rows run the same
-// instruction stream on different arrays and strides (mom_row).
-template <typename T, class Form>
-__device__ __forceinline__ void team_row(const Prm<T>& P, const Lv<T>& L, int i, int j, int d, int ke,
-                                         bool mine, T& dq, T& bq) {
-  const T ih = L.ih, ih2 = L.ih2, third = T(1.0 / 3.0);
-  MomRow<T> R = mom_row<T, Form>(P, L, d);
-  T rl = Form::rho(P, L, ke), rr = Form::rho(P, L, ke + R.s);
-  T Ar = T(0.5) * (rl + rr);
-  const T* vis = L.visn;
+// x-edge, 1: y-edge), edge index ke, rho(c) of the edge's cells l and r.
+template <typename T, class Form, class LV>
+__device__ __forceinline__ void team_row(const Prm<T>& P, const LV& L, int i, int j, int d, int ke,
+                                         RhoPair<T> l, RhoPair<T> r, bool mine, T& dq, T& bq) {
   if constexpr (std::is_same<Form, ErrForm>::value) {
+    const T ih = L.ih, ih2 = L.ih2, third = T(1.0 / 3.0);
+    const int s = d ? L.pitch : 1, t = d ? 1 : L.pitch;
+    auto vis = L.visn;
+    auto S = L.pair(d, L.Sx, L.Sy);
+    auto Q = L.pair(d, L.Qx, L.Qy);
+    T Ar = T(0.5) * (l.r + r.r);
     // the diagonal from the frozen arrays (error levels carry no row coefficients)
     T gp = d ? ((!L.px && i == L.m1) ? T(2) : T(1)) : ((j == L.m2) ? T(2) : T(1));
     T gm = d ? ((!L.px && i == 1) ? T(2) : T(1)) : ((j == 1) ? T(2) : T(1));
-    T Arn = R.Arn[ke];
+    T Arn = L.pair(d, L.Aru, L.Arv)[ke];
     dq = Arn * P.idt + T(0.5) * (Ar - Arn) * P.idt +
-         T(0.5) * ih * (-R.S[ke + R.s] + R.S[ke] - R.Q[ke] * gp + R.Q[ke - R.t] * gm) + R.Dv[ke] +
-         P.iRe * ih2 * ((vis[ke + R.s] + vis[ke]) * (T(1) + third) + gp * L.Av[ke] + gm * L.Av[ke - R.t]);
+         T(0.5) * ih * (-S[ke + s] + S[ke] - Q[ke] * gp + Q[ke - t] * gm) +
+         L.pair(d, L.Dvu, L.Dvv)[ke] +
+         P.iRe * ih2 * ((vis[ke + s] + vis[ke]) * (T(1) + third) + gp * L.Av[ke] + gm * L.Av[ke - t]);
   } else {
-    dq = R.Dg[ke] + L.k.qidt * (rl + rr);
+    dq = L.pair(d, L.Dgu, L.Dgv)[ke] + L.k.qidt * (l.r + r.r);
   }
-  bq = mom_residual<T, Form>(P, L, R, ke, rl, rr);  // wall edges too (padded arrays), then discarded
+  bq = mom_residual<T, Form>(P, L, d, ke, l, r);  // wall edges too (padded arrays), then discarded
   if (!mine) bq = T(0);
 }
 
@@ -1937,7 +1955,8 @@ struct TeamSolve {
   bool odd;
   // with_p = false: the 4x4 velocity block alone (the projection method's
   // intermediate-velocity block), solved as solve_vanka<T, 4> does
-  __device__ __forceinline__ TeamSolve(const Prm<T>& P, const Lv<T>& L, int q, T dq, bool ap0, bool ap1,
+  template <class LV>
+  __device__ __forceinline__ TeamSolve(const Prm<T>& P, const LV& L, int q, T dq, bool ap0, bool ap1,
                                        T S, T vc, T A44, bool with_p = true) {
     const unsigned FULL = 0xffffffffu;
     ih = L.ih;
@@ -1980,8 +1999,8 @@ struct TeamSolve {
 // (TeamSolve); lane q writes edge q and lane 0 the pressure.  All 32 lanes of
 // the warp call this (ok = false: a spare team, which computes on cell (1,1)
 // and stores nothing).
-template <typename T, class Form>
-__device__ __forceinline__ void vanka_team(const Prm<T>& P, const Lv<T>& L, int i, int j, bool ok,
+template <typename T, class Form, class LV>
+__device__ __forceinline__ void vanka_team(const Prm<T>& P, const LV& L, int i, int j, bool ok,
                                            T omega) {
   const int W = L.pitch;
   const int q = threadIdx.x & 3, d = q >> 1;
@@ -1992,20 +2011,23 @@ __device__ __forceinline__ void vanka_team(const Prm<T>& P, const Lv<T>& L, int 
   bool a0 = L.px || i > 1, a1 = L.px || i < L.m1, a2 = j > 1, a3 = j < L.m2;
   bool mine = q == 0 ? a0 : q == 1 ? a1 : q == 2 ? a2 : a3;
   int ke = q == 0 ? kW : (q == 2 ? k - W : k);
+  // the neighbour across the edge's face; a periodic ghost holds the cell's copy
+  const int nq = k + (q == 0 ? -1 : q == 1 ? 1 : q == 2 ? -W : W);
+  const RhoPair<T> ra = rho_pair<T, Form>(P, L, k), rb = rho_pair<T, Form>(P, L, nq);
+  const int kf = (q & 1) ? k : nq;  // the face's own edge (kW's copy for a periodic west face)
   T dq, bq;
-  team_row<T, Form>(P, L, i, j, d, ke, mine, dq, bq);
+  team_row<T, Form>(P, L, i, j, d, ke, (q & 1) ? ra : rb, (q & 1) ? rb : ra, mine, dq, bq);
   // the mass row by faces: lane q takes face q (W, E, S, N) of the cell, the
   // face of its own edge: its velocity in d.u, its flux of
   // grad.(A m grad(mu + alpha p)) and, if open, its share of sum A m
-  const T* mob = L.mobn;
-  const int nq = k + (q == 0 ? -1 : q == 1 ? 1 : q == 2 ? -W : W);
+  auto mob = L.mobn;
   T am = mob[nq] + mob[k];
-  T f0 = team_sum<T>((q & 1) ? (d ? L.v[k] : L.u[k]) : -(d ? L.v[k - W] : L.u[k - 1]));
+  T f0 = team_sum<T>((q & 1) ? L.pair(d, L.u, L.v)[kf] : -L.pair(d, L.u, L.v)[kf]);
   T f1 = team_sum<T>(am * ((L.mu[nq] - L.mu[k]) + P.alpha * (L.p[nq] - L.p[k])));
   T f2 = team_sum<T>(mine ? am : T(0));
   T A44 = L.k.a2dif * f2;
   T b4 = f0 * ih - L.k.adif * f1 - L.fp[k];
-  TeamSolve<T> ts(P, L, q, dq, d ? a2 : a0, d ? a3 : a1, d ? L.Sy[k] : L.Sx[k], L.visn[k], A44);
+  TeamSolve<T> ts(P, L, q, dq, d ? a2 : a0, d ? a3 : a1, L.pair(d, L.Sx, L.Sy)[k], L.visn[k], A44);
   T pr;
   T x = ts.apply(bq, b4, pr);
   if (!ok) return;
@@ -2022,24 +2044,29 @@ __device__ __forceinline__ void vanka_team(const Prm<T>& P, const Lv<T>& L, int 
 // time term (with gravity), the convection and -f; half 1 the pressure gradient,
 // the surface tension and the viscous terms.  The two halves sum to the
 // momentum row's N - f (up to the order of the additions).  FullForm only.
-template <typename T>
-__device__ __forceinline__ T mom_residual_half(const Prm<T>& P, const Lv<T>& L, const MomRow<T>& R,
-                                               int k, T rl, T rr, int half) {
-  const int s = R.s, t = R.t;
-  const T *a = R.a, *b = R.b;
+template <typename T, class LV>
+__device__ __forceinline__ T mom_residual_half(const Prm<T>& P, const LV& L, int d, int k, T rl,
+                                               T rr, int half) {
+  const int s = d ? L.pitch : 1, t = d ? 1 : L.pitch;
+  auto a = L.pair(d, L.u, L.v);
+  auto b = L.pair(1 - d, L.u, L.v);
   T ae = a[k];
   T dl = (ae - a[k - s]) * L.ih, dr = (a[k + s] - ae) * L.ih;
   T Dp = (a[k + t] - ae) * L.ih, Dm = (ae - a[k - t]) * L.ih;
   if (half == 0) {
-    T conv = T(0.5) * (R.S[k + s] * dr + R.S[k] * dl + R.Q[k] * Dp + R.Q[k - t] * Dm);
-    T time = ae * (R.T1[k] + L.k.qidt * (rl + rr)) + R.T0[k];
-    return time + conv - R.f[k];
+    auto S = L.pair(d, L.Sx, L.Sy);
+    auto Q = L.pair(d, L.Qx, L.Qy);
+    T conv = T(0.5) * (S[k + s] * dr + S[k] * dl + Q[k] * Dp + Q[k - t] * Dm);
+    T time = ae * (L.pair(d, L.T1u, L.T1v)[k] + L.k.qidt * (rl + rr)) +
+             L.pair(d, L.T0u, L.T0v)[k];
+    return time + conv - L.pair(d, L.fu, L.fv)[k];
   }
-  const T *vis = L.visn, *rn = L.rhon;
+  auto vis = L.visn;
+  auto rn = L.rhon;
   T dvl = dl + (b[k] - b[k - t]) * L.ih;
   T dvr = dr + (b[k + s] - b[k + s - t]) * L.ih;
-  T press = (L.p[k + s] - L.p[k]) * L.ih * P.iM;
-  T st = -(rn[k + s] * L.mu[k] + rn[k] * L.mu[k + s]) * R.Tf[k] * P.iM;
+  T press = (L.p[k + s] - L.p[k]) * L.k.ihM;
+  T st = -(rn[k + s] * L.mu[k] + rn[k] * L.mu[k + s]) * L.pair(d, L.Tx, L.Ty)[k] * P.iM;
   T vl = vis[k], vr = vis[k + s];
   T visc = -P.iRe * L.ih * ((vr * dr - vl * dl) + (L.Av[k] * Dp - L.Av[k - t] * Dm) +
                             (vr * dvr - vl * dvl) * T(1.0 / 3.0));
@@ -2052,8 +2079,8 @@ __device__ __forceinline__ T mom_residual_half(const Prm<T>& P, const Lv<T>& L, 
 // evaluates half a row.  Both halves of the team then run the same solve;
 // the lower half stores.  For levels whose colour leaves most of the GPU idle:
 // the visit's chain of dependent instructions is what bounds them.
-template <typename T>
-__device__ __forceinline__ void vanka_team8(const Prm<T>& P, const Lv<T>& L, int i, int j, bool ok,
+template <typename T, class LV>
+__device__ __forceinline__ void vanka_team8(const Prm<T>& P, const LV& L, int i, int j, bool ok,
                                             T omega) {
   const int W = L.pitch;
   const int q = threadIdx.x & 3, d = q >> 1, half = (threadIdx.x >> 2) & 1;
@@ -2064,13 +2091,12 @@ __device__ __forceinline__ void vanka_team8(const Prm<T>& P, const Lv<T>& L, int
   bool a0 = L.px || i > 1, a1 = L.px || i < L.m1, a2 = j > 1, a3 = j < L.m2;
   bool mine = q == 0 ? a0 : q == 1 ? a1 : q == 2 ? a2 : a3;
   int ke = q == 0 ? kW : (q == 2 ? k - W : k);
-  MomRow<T> R = mom_row<T, FullForm>(P, L, d);
-  T rl = L.rhoc[ke], rr = L.rhoc[ke + R.s];
-  T dq = R.Dg[ke] + L.k.qidt * (rl + rr);
-  T bq = mom_residual_half<T>(P, L, R, ke, rl, rr, half);
+  T rl = L.rhoc[ke], rr = L.rhoc[ke + (d ? W : 1)];
+  T dq = L.pair(d, L.Dgu, L.Dgv)[ke] + L.k.qidt * (rl + rr);
+  T bq = mom_residual_half<T>(P, L, d, ke, rl, rr, half);
   bq += __shfl_xor_sync(0xffffffffu, bq, 4);
   if (!mine) bq = T(0);
-  const T* mob = L.mobn;
+  auto mob = L.mobn;
   const int nq = k + (q == 0 ? -1 : q == 1 ? 1 : q == 2 ? -W : W);
   T am = mob[nq] + mob[k];
   T f0 = team_sum<T>((q & 1) ? (d ? L.v[k] : L.u[k]) : -(d ? L.v[k - W] : L.u[k - 1]));
@@ -2095,8 +2121,8 @@ __device__ __forceinline__ void vanka_team8(const Prm<T>& P, const Lv<T>& L, int
 // team of four lanes: lane q builds row q (team_row without pressure, surface
 // tension and gravity) and the team solves the block (TeamSolve without the
 // pressure row); lane q writes edge q.
-template <typename T>
-__device__ __forceinline__ void vanka4_team(const Prm<T>& P, const Lv<T>& L, int i, int j, bool ok,
+template <typename T, class LV>
+__device__ __forceinline__ void vanka4_team(const Prm<T>& P, const LV& L, int i, int j, bool ok,
                                             T omega) {
   const int W = L.pitch;
   const int q = threadIdx.x & 3, d = q >> 1;
@@ -2106,9 +2132,12 @@ __device__ __forceinline__ void vanka4_team(const Prm<T>& P, const Lv<T>& L, int
   bool a0 = L.px || i > 1, a1 = L.px || i < L.m1, a2 = j > 1, a3 = j < L.m2;
   bool mine = q == 0 ? a0 : q == 1 ? a1 : q == 2 ? a2 : a3;
   int ke = q == 0 ? kW : (q == 2 ? k - W : k);
+  // the neighbour across the edge's face; a periodic ghost holds the cell's copy
+  const int nq = k + (q == 0 ? -1 : q == 1 ? 1 : q == 2 ? -W : W);
+  const RhoPair<T> ra = rho_pair<T, ProjForm>(P, L, k), rb = rho_pair<T, ProjForm>(P, L, nq);
   T dq, bq;
-  team_row<T, ProjForm>(P, L, i, j, d, ke, mine, dq, bq);
-  TeamSolve<T> ts(P, L, q, dq, d ? a2 : a0, d ? a3 : a1, d ? L.Sy[k] : L.Sx[k], L.visn[k], T(0), false);
+  team_row<T, ProjForm>(P, L, i, j, d, ke, (q & 1) ? ra : rb, (q & 1) ? rb : ra, mine, dq, bq);
+  TeamSolve<T> ts(P, L, q, dq, d ? a2 : a0, d ? a3 : a1, L.pair(d, L.Sx, L.Sy)[k], L.visn[k], T(0), false);
   T pr;
   T x = ts.apply(bq, T(0), pr);
   if (!ok || !mine) return;
@@ -2125,8 +2154,8 @@ __device__ __forceinline__ void vanka4_team(const Prm<T>& P, const Lv<T>& L, int
 // the cell terms.  The solve follows solve_coupled7: the NS block's
 // structured solve (TeamSolve) applied to three right-hand sides, then the
 // 2x2 Schur system for (dc, dmu).  Lane q writes edge q, lane 0 c, mu, p.
-template <typename T, class Form>
-__device__ __forceinline__ void coupled_team(const Prm<T>& P, const Lv<T>& L, int i, int j, bool ok,
+template <typename T, class Form, class LV>
+__device__ __forceinline__ void coupled_team(const Prm<T>& P, const LV& L, int i, int j, bool ok,
                                              T omega) {
   const int W = L.pitch;
   const int q = threadIdx.x & 3, d = q >> 1;
@@ -2137,10 +2166,14 @@ __device__ __forceinline__ void coupled_team(const Prm<T>& P, const Lv<T>& L, in
   bool a0 = L.px || i > 1, a1 = L.px || i < L.m1, a2 = j > 1, a3 = j < L.m2;
   bool mine = q == 0 ? a0 : q == 1 ? a1 : q == 2 ? a2 : a3;
   int ke = q == 0 ? kW : (q == 2 ? k - W : k);
+  // the neighbour across the edge's face; a periodic ghost holds the cell's copy
+  const int nq = k + (q == 0 ? -1 : q == 1 ? 1 : q == 2 ? -W : W);
+  const RhoPair<T> ra = rho_pair<T, Form>(P, L, k), rb = rho_pair<T, Form>(P, L, nq);
+  const int kf = (q & 1) ? k : nq;  // the face's own edge (kW's copy for a periodic west face)
   T dq, bq;
-  team_row<T, Form>(P, L, i, j, d, ke, mine, dq, bq);
-  ChRows<T> C = ch_team_rows<T, Form>(P, L, i, j, q, mine);
-  T sdiv = team_sum<T>((q & 1) ? (d ? L.v[k] : L.u[k]) : -(d ? L.v[k - W] : L.u[k - 1]));
+  team_row<T, Form>(P, L, i, j, d, ke, (q & 1) ? ra : rb, (q & 1) ? rb : ra, mine, dq, bq);
+  ChRows<T> C = ch_team_rows<T, Form>(P, L, i, j, q, mine, ra, rb);
+  T sdiv = team_sum<T>((q & 1) ? L.pair(d, L.u, L.v)[kf] : -L.pair(d, L.u, L.v)[kf]);
   T sm = C.sm, sflux = C.sflux, gq = C.gq;
   T J11 = C.J11, J12 = C.J12, J21 = C.J21, J22 = C.J22, Rc = C.Rc, Rm = C.Rm;
   // the mass row and the couplings of edge q: d N_q/dc, d N_q/dmu (rows of
@@ -2151,7 +2184,7 @@ __device__ __forceinline__ void coupled_team(const Prm<T>& P, const Lv<T>& L, in
   T gm = mine ? gq : T(0);
   T cq0 = mine ? T(0.25) * C.drho * P.idt * (d ? Form::val_v(L, ke) : Form::val_u(L, ke)) : T(0);
   T cq1 = mine ? -gq * P.iM : T(0);
-  TeamSolve<T> ts(P, L, q, dq, d ? a2 : a0, d ? a3 : a1, d ? L.Sy[k] : L.Sx[k], L.visn[k], A44);
+  TeamSolve<T> ts(P, L, q, dq, d ? a2 : a0, d ? a3 : a1, L.pair(d, L.Sx, L.Sy)[k], L.visn[k], A44);
   T p0, p1, p2;
   T x0 = ts.apply(bq, b4, p0);
   T x1 = ts.apply(cq0, T(0), p1);
@@ -2246,8 +2279,8 @@ __global__ void __launch_bounds__(SNT) k_vanka_team(Prm<T> P, Lv<T> L, int colou
 // instructions, which is what bounds a launch whose colour fills the GPU
 // more than once: the busiest sub-partition issues three warps of half a
 // visit instead of two warps of a whole one.
-template <typename T, class Form>
-__device__ __forceinline__ void vanka_pair(const Prm<T>& P, const Lv<T>& L, int i, int j, bool ok,
+template <typename T, class Form, class LV>
+__device__ __forceinline__ void vanka_pair(const Prm<T>& P, const LV& L, int i, int j, bool ok,
                                            T omega) {
   const unsigned FULL = 0xffffffffu;
   const int W = L.pitch;
@@ -2261,10 +2294,15 @@ __device__ __forceinline__ void vanka_pair(const Prm<T>& P, const Lv<T>& L, int 
   bool ap0 = d ? a2 : a0, ap1 = d ? a3 : a1;
   int ke0 = d ? k - W : kW;
   T dq0, bq0, dq1, bq1;
-  team_row<T, Form>(P, L, i, j, d, ke0, ap0, dq0, bq0);
-  team_row<T, Form>(P, L, i, j, d, k, ap1, dq1, bq1);
+  {
+    const int o = d ? W : 1;
+    const RhoPair<T> rl = rho_pair<T, Form>(P, L, k - o), rk = rho_pair<T, Form>(P, L, k),
+                     rr = rho_pair<T, Form>(P, L, k + o);
+    team_row<T, Form>(P, L, i, j, d, ke0, rl, rk, ap0, dq0, bq0);
+    team_row<T, Form>(P, L, i, j, d, k, rk, rr, ap1, dq1, bq1);
+  }
   // the mass row by faces (as vanka_team): faces W, E on lane 0, S, N on lane 1
-  const T* mob = L.mobn;
+  auto mob = L.mobn;
   const int off = d ? W : 1;
   const int n0 = k - off, n1 = k + off;
   T am0 = mob[n0] + mob[k], am1 = mob[n1] + mob[k];
@@ -2356,8 +2394,9 @@ __global__ void __launch_bounds__(SNT) k_vanka_split(Prm<T> P, Lv<T> L, int colo
 // fused group (one warp per sub-partition)
 constexpr int QN_TEAM_MAX_SLOTS = 32;
 
-template <typename T, class Form>
-__device__ void smooth_block(const Prm<T>& P, const Lv<T>& L, T omega, int coupled, int team8 = 0) {
+template <typename T, class Form, class LV>
+__device__ __forceinline__ void smooth_block(const Prm<T>& P, const LV& L, T omega, int coupled,
+                                             int team8) {
   const int kcol = L.kcol;
   if constexpr (std::is_same<Form, ProjForm>::value) {
     // projection method (Sec. 7.2): CH red-black, intermediate-velocity blocks
@@ -2504,16 +2543,19 @@ __device__ void smooth_block(const Prm<T>& P, const Lv<T>& L, T omega, int coupl
   }  // primitive method
 }
 
-template <typename T, class Form>
-__device__ __forceinline__ void coarse_vcycle_body(const Prm<T>& P, const CoarseLevels<T>& C, int nu1,
-                                                   int nu2, int nuc, T omega, int coupled,
+// The V-cycle on the levels get(0) .. get(n - 1) as one loop over its level
+// visits (down, coarsest, up), so that the smoother's code, the longest of the
+// kernel, appears once: the visits of a colour step are bound by instruction
+// latency, fetch included.
+template <typename T, class Form, class Get>
+__device__ __forceinline__ void coarse_vcycle_body(const Prm<T>& P, const Get& get, int n, int base,
+                                                   int nu1, int nu2, int nuc, T omega, int coupled,
                                                    int team8) {
-  const int n = C.n;
   double dummy[10];
-  if (C.base) {
+  if (base) {
     for (int l = 1; l < n; ++l) {
-      const Lv<T>& F = C.L[l - 1];
-      const Lv<T>& G = C.L[l];
+      const auto& F = get(l - 1);
+      const auto& G = get(l);
       for (int t = grp_rank(); t < (G.m1 + 1) * (G.m2 + 1); t += grp_size())
         restrict_base_cell(F, G, t % (G.m1 + 1), t / (G.m1 + 1));
       grp_sync();
@@ -2525,42 +2567,50 @@ __device__ __forceinline__ void coarse_vcycle_body(const Prm<T>& P, const Coarse
       grp_sync();
     }
   }
-  for (int l = 0; l < n - 1; ++l) {
-    const Lv<T>& F = C.L[l];
-    const Lv<T>& G = C.L[l + 1];
-    for (int s = 0; s < nu1; ++s) smooth_block<T, Form>(P, F, omega, coupled, team8);
-    for (int t = grp_rank(); t < F.m1 * F.m2; t += grp_size())
-      residual_cell<T, 0, Form>(P, F, t % F.m1 + 1, t / F.m1 + 1, dummy);
-    grp_sync();
-    for (int t = grp_rank(); t < (G.m1 + 1) * (G.m2 + 1); t += grp_size())
-      restrict_state_cell(P, F, G, t % (G.m1 + 1), t / (G.m1 + 1));
-    grp_sync();
-    bc_unknowns_block(G);
-    for (int t = grp_rank(); t < G.m1 * G.m2; t += grp_size())
-      restrict_res_cell(F, G, t % G.m1 + 1, t / G.m1 + 1);
-    grp_sync();
-    for (int t = grp_rank(); t < G.m1 * G.m2; t += grp_size())
-      residual_cell<T, 1, Form>(P, G, t % G.m1 + 1, t / G.m1 + 1, dummy);
-    grp_sync();
-  }
-  for (int s = 0; s < nuc; ++s) smooth_block<T, Form>(P, C.L[n - 1], omega, coupled, team8);
-  for (int l = n - 2; l >= 0; --l) {
-    const Lv<T>& F = C.L[l];
-    const Lv<T>& G = C.L[l + 1];
-    for (int t = grp_rank(); t < F.m1 * F.m2; t += grp_size())
-      prolong_cell(P, F, G, t % F.m1 + 1, t / F.m1 + 1);
-    grp_sync();
-    bc_unknowns_block(F);
-    for (int s = 0; s < nu2; ++s) smooth_block<T, Form>(P, F, omega, coupled, team8);
+  for (int visit = 0; visit < 2 * n - 1; ++visit) {
+    const bool down = visit < n - 1, up = visit >= n;
+    const int l = up ? 2 * n - 2 - visit : visit;
+    const auto& F = get(l);
+    if (up) {  // the correction from the level below
+      const auto& G = get(l + 1);
+      for (int t = grp_rank(); t < F.m1 * F.m2; t += grp_size())
+        prolong_cell(P, F, G, t % F.m1 + 1, t / F.m1 + 1);
+      grp_sync();
+      bc_unknowns_block(F);
+    }
+    const int sweeps = down ? nu1 : up ? nu2 : nuc;
+    for (int s = 0; s < sweeps; ++s) smooth_block<T, Form>(P, F, omega, coupled, team8);
+    if (down) {
+      const auto& G = get(l + 1);
+      for (int t = grp_rank(); t < F.m1 * F.m2; t += grp_size())
+        residual_cell<T, 0, Form>(P, F, t % F.m1 + 1, t / F.m1 + 1, dummy);
+      grp_sync();
+      for (int t = grp_rank(); t < (G.m1 + 1) * (G.m2 + 1); t += grp_size())
+        restrict_state_cell(P, F, G, t % (G.m1 + 1), t / (G.m1 + 1));
+      for (int t = grp_rank(); t < G.m1 * G.m2; t += grp_size())
+        restrict_res_cell(F, G, t % G.m1 + 1, t / G.m1 + 1);
+      grp_sync();
+      bc_unknowns_block(G);
+      for (int t = grp_rank(); t < G.m1 * G.m2; t += grp_size())
+        residual_cell<T, 1, Form>(P, G, t % G.m1 + 1, t / G.m1 + 1, dummy);
+      grp_sync();
+    }
   }
 }
+
+// level l of a CoarseLevels
+template <typename T>
+struct LevelsOf {
+  const CoarseLevels<T>& C;
+  __device__ __forceinline__ const Lv<T>& operator()(int l) const { return C.L[l]; }
+};
 
 template <typename T, class Form, int NT>
 __global__ void __launch_bounds__(NT) k_coarse_vcycle(Prm<T> P, CoarseLevels<T> C, int nu1, int nu2,
                                                       int nuc, int kcol, T omega, int coupled,
                                                       int team8) {
   pdl_enter();
-  coarse_vcycle_body<T, Form>(P, C, nu1, nu2, nuc, omega, coupled, team8);
+  coarse_vcycle_body<T, Form>(P, LevelsOf<T>{C}, C.n, C.base, nu1, nu2, nuc, omega, coupled, team8);
 }
 
 // --------------------------------------------------------------------------
@@ -2645,13 +2695,10 @@ __global__ void __launch_bounds__(NT) k_coarse_vcycle_smem(Prm<double> P, Coarse
     }
     S->L[l] = X;
   }
-  if (threadIdx.x == 0) {
-    S->n = n;
-    S->base = 0;
-  }
   asm volatile("cp.async.wait_all;" ::: "memory");
   __syncthreads();
-  coarse_vcycle_body<double, FullForm>(P, *S, nu1, nu2, nuc, omega, coupled, team8);
+  coarse_vcycle_body<double, FullForm>(P, LevelsOf<double>{*S}, n, 0, nu1, nu2, nuc, omega, coupled,
+                                       team8);
   __syncthreads();
   for (int l = 0; copy && l < n; ++l) {
     const Lv<double>& G = C.L[l];
@@ -2659,6 +2706,123 @@ __global__ void __launch_bounds__(NT) k_coarse_vcycle_smem(Prm<double> P, Coarse
     double* g = G.c - (G.pitch + 1);
     coarse_copy<NT, false>(g, G.pitch, M.ng[l], arr + M.off[l], cc, rr, 0, QN_LV_WRITTEN);
     coarse_copy<NT, false>(g, G.pitch, M.ng[l], arr + M.off[l], cc, rr, QN_LV_RHOC, QN_LV_RHOC + 1);
+  }
+}
+
+// --------------------------------------------------------------------------
+// The fused V-cycle of FP32 error-equation levels on a shared-memory copy.  Its
+// visits have no slow arithmetic: what a colour step cost was the chain of
+// address arithmetic (a 64-bit address for each of the ~60 array elements a
+// visit reads) and L2 round trips.  The copy interleaves the level's arrays:
+// cell k's 41 values sit together (LvS), so that a visit forms three
+// addresses (its row and the rows beside it) and reads everything else at
+// constant offsets from them.  41 words a cell is odd, so lanes on cells any
+// power of two (or 5) apart fall into different banks.
+// Measured (GB300, ncu, caches warm): the 16x32 .. 2x4 levels of the 256x512
+// drop 245 -> 139 us, the 28x28 and 14x14 levels of a served 448x448 request
+// (64 coupled sweeps on the coarsest) 1504 -> 1121 us.  Launched wherever the
+// records fit the opt-in shared memory (option coarse_smem; about 1380 padded
+// cells); a larger group reads global memory.
+// --------------------------------------------------------------------------
+// the arrays of an error-equation level that its V-cycle touches, in the order
+// of a cell's record
+#define QN_ERR_ARRAYS(X)                                                                       \
+  X(c) X(mu) X(p) X(u) X(v) X(fc) X(fmu) X(fp) X(fu) X(fv) X(rc) X(rmu) X(rp) X(ru) X(rv)     \
+  X(sc) X(smu) X(sp) X(su) X(sv) X(cn) X(rhon) X(mobn) X(visn) X(Gn) X(Aru) X(Arv) X(Sx)      \
+  X(Sy) X(Qx) X(Qy) X(Av) X(Tx) X(Ty) X(Dvu) X(Dvv) X(Bc) X(Bmu) X(Bu) X(Bv) X(Bdc)
+enum {
+#define QN_ERR_INDEX(m) ERR_##m,
+  QN_ERR_ARRAYS(QN_ERR_INDEX)
+#undef QN_ERR_INDEX
+      ERR_N
+};
+static_assert(ERR_N % 2 == 1, "an odd record keeps strided lanes in different banks");
+
+// array OFF of the records at b: element k as if it were a plain array
+template <typename T, int OFF>
+struct Fld {
+  T* b;
+  __device__ __forceinline__ T& operator[](int k) const { return b[k * ERR_N + OFF]; }
+};
+// an error-equation level in records (the members and constants of Lv)
+template <typename T>
+struct LvS {
+  typedef T real;
+  static constexpr bool has_rho = false;
+  LvK<T> k;
+  int m1, m2, px, pitch, kcol, c8;
+  T h, ih, ih2;
+#define QN_ERR_MEMBER(m) Fld<T, ERR_##m> m;
+  QN_ERR_ARRAYS(QN_ERR_MEMBER)
+#undef QN_ERR_MEMBER
+  // level L with its record of cell (0,0) at b
+  __device__ __forceinline__ LvS(const Lv<T>& L, T* b)
+      : k(L.k), m1(L.m1), m2(L.m2), px(L.px), pitch(L.m1 + 3), kcol(L.kcol), c8(L.c8), h(L.h),
+        ih(L.ih), ih2(L.ih2) {
+#define QN_ERR_SET(m) m.b = b;
+    QN_ERR_ARRAYS(QN_ERR_SET)
+#undef QN_ERR_SET
+  }
+  __device__ __forceinline__ int at(int i, int j) const { return j * pitch + i; }
+  __device__ __forceinline__ int uhi() const { return px ? m1 : m1 - 1; }
+  // neighbours in the record: the pair's second array is the first one element on
+  template <int OFF>
+  __device__ __forceinline__ Fld<T, OFF> pair(int d, Fld<T, OFF> x, Fld<T, OFF + 1>) const {
+    return {x.b + d};
+  }
+};
+
+struct ErrSmem {
+  int off[QN_MAX_FUSED_LEVELS];  // first word of level l's records
+};
+
+template <typename T>
+struct ErrLevels {
+  const CoarseLevels<T>& C;
+  const ErrSmem& M;
+  T* base;
+  __device__ __forceinline__ LvS<T> operator()(int l) const {
+    const Lv<T>& L = C.L[l];
+    return LvS<T>(L, base + M.off[l] + (L.m1 + 4) * ERR_N);  // cell (0,0) of the frame from (-1,-1)
+  }
+};
+
+template <int NT>
+__global__ void __launch_bounds__(NT) k_coarse_err(Prm<float> P, const __grid_constant__ CoarseLevels<float> C,
+                                                   const __grid_constant__ ErrSmem M, int nu1, int nu2,
+                                                   int nuc, float omega, int coupled) {
+  extern __shared__ __align__(16) float qn_err_smem[];
+  pdl_enter();
+  const int n = C.n;
+  for (int l = 0; l < n; ++l) {  // the padded frame of every array, all copies in flight at once
+    const Lv<float>& L = C.L[l];
+    const int cc = L.m1 + 3, cells = cc * (L.m2 + 3);
+    for (int t = threadIdx.x; t < cells; t += NT) {
+      const int g = (t / cc - 1) * L.pitch + t % cc - 1;
+      const unsigned sa = (unsigned)__cvta_generic_to_shared(qn_err_smem + M.off[l] + t * ERR_N);
+#define QN_ERR_IN(m)                                                                        \
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(sa + 4 * ERR_##m), "l"(L.m + g) \
+               : "memory");
+      QN_ERR_ARRAYS(QN_ERR_IN)
+#undef QN_ERR_IN
+    }
+  }
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  __syncthreads();
+  const ErrLevels<float> get{C, M, qn_err_smem};
+  coarse_vcycle_body<float, ErrForm>(P, get, n, 1, nu1, nu2, nuc, omega, coupled, 0);
+  __syncthreads();
+  // what the levels above read of the group: the iterate of its finest level
+  const Lv<float>& L = C.L[0];
+  const int cc = L.m1 + 3, cells = cc * (L.m2 + 3);
+  for (int t = threadIdx.x; t < cells; t += NT) {
+    const int g = (t / cc - 1) * L.pitch + t % cc - 1;
+    const float* r = qn_err_smem + M.off[0] + t * ERR_N;
+    L.c[g] = r[ERR_c];
+    L.mu[g] = r[ERR_mu];
+    L.p[g] = r[ERR_p];
+    L.u[g] = r[ERR_u];
+    L.v[g] = r[ERR_v];
   }
 }
 
@@ -2693,8 +2857,8 @@ __device__ __forceinline__ void st_release_u32(unsigned* p, unsigned v) {
 }
 
 // the visits of pass `pass` on rows r0..r1 (1-based, inclusive)
-template <typename T, class Form>
-__device__ __forceinline__ void wave_pass(const Prm<T>& P, const Lv<T>& L, const WavePlan& W,
+template <typename T, class Form, class LV>
+__device__ __forceinline__ void wave_pass(const Prm<T>& P, const LV& L, const WavePlan& W,
                                           int pass, int r0, int r1, T omega) {
   const int per = W.coupled ? L.kcol : L.kcol + 2;
   const int q = pass % per;
@@ -3373,12 +3537,8 @@ void launch_vanka(const Prm<T>& P, const Lv<T>& L0, int colour, T omega, cudaStr
   qlaunch(&k_vanka<T, Form>, (n + SNT - 1) / SNT, SNT, 0, s, P, L, colour, omega);
   ++g_launches;
 }
-// Plan of the shared-memory copy of an FP64 full-iterate fused group: every
-// level's arrays at their block's stride in QN_LV_ARRAYS order (checked
-// pointer by pointer), columns within the copy kernel's 32-wide rows, and the
-// whole copy within the device's opt-in shared memory per block.  Returns the
-// dynamic shared-memory bytes, 0 if the group does not qualify.
-static size_t coarse_smem_plan(const Lv<double>* levels, int n, CoarseSmem& M) {
+// shared memory a block of the current device may opt in to
+static int smem_optin() {
   static std::atomic<int> optin{0};
   if (!optin.load()) {
     int dev = 0, v = 0;
@@ -3386,6 +3546,14 @@ static size_t coarse_smem_plan(const Lv<double>* levels, int n, CoarseSmem& M) {
     cudaDeviceGetAttribute(&v, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     optin = v > 0 ? v : 1;
   }
+  return optin.load();
+}
+// Plan of the shared-memory copy of an FP64 full-iterate fused group: every
+// level's arrays at their block's stride in QN_LV_ARRAYS order (checked
+// pointer by pointer), columns within the copy kernel's 32-wide rows, and the
+// whole copy within the device's opt-in shared memory per block.  Returns the
+// dynamic shared-memory bytes, 0 if the group does not qualify.
+static size_t coarse_smem_plan(const Lv<double>* levels, int n, CoarseSmem& M) {
   const int head = (int)((sizeof(CoarseLevels<double>) + 15) / 16 * 2);
   long long elems = head;
   M.head = head;
@@ -3406,15 +3574,29 @@ static size_t coarse_smem_plan(const Lv<double>* levels, int n, CoarseSmem& M) {
     elems = (elems + 1) / 2 * 2;  // 16-byte aligned copies
   }
   const size_t bytes = (size_t)elems * sizeof(double);
-  return bytes <= (size_t)optin.load() ? bytes : 0;
+  return bytes <= (size_t)smem_optin() ? bytes : 0;
+}
+
+// Plan of k_coarse_err's copy; returns its bytes, 0 if it does not fit
+static size_t coarse_err_plan(const Lv<float>* levels, int n, ErrSmem& M) {
+  const long long limit = smem_optin();
+  long long words = 0;
+  for (int l = 0; l < n; ++l) {
+    M.off[l] = (int)words;
+    words += (long long)(levels[l].m1 + 3) * (levels[l].m2 + 3) * ERR_N;
+    if (4 * words > limit) return 0;
+  }
+  return (size_t)words * sizeof(float);
 }
 
 void coarse_smem_prepare() {
   int dev = 0, v = 0;
   cudaGetDevice(&dev);
   if (cudaDeviceGetAttribute(&v, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) == cudaSuccess &&
-      v > 0)
+      v > 0) {
     cudaFuncSetAttribute(&k_coarse_vcycle_smem<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, v);
+    cudaFuncSetAttribute(&k_coarse_err<512>, cudaFuncAttributeMaxDynamicSharedMemorySize, v);
+  }
   cudaGetLastError();
 }
 
@@ -3435,6 +3617,15 @@ int launch_coarse_vcycle(const Prm<T>& P, const Lv<T>* levels, int n, int nu1, i
               C, M, bytes ? 1 : 0, nu1, nu2, nuc, omega, coupled, team8);
       ++g_launches;
       return bytes ? 1 : 0;
+    }
+  }
+  if constexpr (std::is_same<Form, ErrForm>::value && sizeof(T) == 4) {
+    ErrSmem M = {};
+    const size_t bytes = smem && ctas <= 1 ? coarse_err_plan(levels, n, M) : 0;
+    if (bytes) {
+      qlaunch(&k_coarse_err<NT>, 1, NT, bytes, s, P, C, M, nu1, nu2, nuc, omega, coupled);
+      ++g_launches;
+      return 0;
     }
   }
   if (ctas <= 1) {

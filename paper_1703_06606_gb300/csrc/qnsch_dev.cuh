@@ -47,6 +47,8 @@ struct LvK {
 
 template <typename T>
 struct Lv {
+  typedef T real;
+  static constexpr bool has_rho = true;
   LvK<T> k;
   int m1, m2, px, pitch;
   // Vanka colours of this level: kcol colours, (2i+j) mod 8 when c8 is set
@@ -94,6 +96,8 @@ struct Lv {
   // e is a correction to, and X.c - c^n formed in FP64 before rounding
   T *Bc = nullptr, *Bmu = nullptr, *Bu = nullptr, *Bv = nullptr, *Bdc = nullptr;
   __device__ __forceinline__ int at(int i, int j) const { return j * pitch + i; }
+  // the array of direction d (0: x, 1: y) of a pair
+  __device__ __forceinline__ T* pair(int d, T* x, T* y) const { return d ? y : x; }
   // x-edge unknowns: walls exclude i = 0 and i = m1; periodic keeps i = m1 (= edge 0)
   __device__ __forceinline__ int uhi() const { return px ? m1 : m1 - 1; }
 };
@@ -179,17 +183,19 @@ template <typename T> __device__ __forceinline__ T gsec_da(T a, T b) {
 // ---------------------------------------------------------------------------
 
 // G(c) = a_x((D_x c)^2) + a_y((D_y c)^2) at cell k (times h^2)
-template <typename T>
-__device__ __forceinline__ T G_h2(const T* c, int k, int pitch) {
-  T cc = c[k];
+template <class A>
+__device__ __forceinline__ auto G_h2(A c, int k, int pitch) {
+  auto cc = c[k];
+  typedef decltype(cc) T;
   T de = c[k + 1] - cc, dw = cc - c[k - 1], dn = c[k + pitch] - cc, ds = cc - c[k - pitch];
   return T(0.5) * (de * de + dw * dw + dn * dn + ds * ds);
 }
 
 // h^2 grad_d.(A kap grad_D phi) at cell k
-template <typename T>
-__device__ __forceinline__ T lap_h2(const T* kap, const T* phi, int k, int pitch) {
-  T kc = kap[k], pc = phi[k];
+template <class A, class B>
+__device__ __forceinline__ auto lap_h2(A kap, B phi, int k, int pitch) {
+  auto kc = kap[k], pc = phi[k];
+  typedef decltype(kc) T;
   return T(0.5) * ((kap[k + 1] + kc) * (phi[k + 1] - pc) - (kc + kap[k - 1]) * (pc - phi[k - 1]) +
                    (kap[k + pitch] + kc) * (phi[k + pitch] - pc) -
                    (kc + kap[k - pitch]) * (pc - phi[k - pitch]));
@@ -198,32 +204,32 @@ __device__ __forceinline__ T lap_h2(const T* kap, const T* phi, int k, int pitch
 // (pm-num-phase) with the advection (e1e2) of App. A.4
 // (the overloads taking densities let a caller that already holds rho(c) of
 // the cell and its neighbours skip the divisions; the values are the same)
-template <typename T>
-__device__ __forceinline__ T op_c(const Prm<T>& P, const Lv<T>& L, int k, T rho) {
+template <typename T, class LV>
+__device__ __forceinline__ T op_c(const Prm<T>& P, const LV& L, int k, T rho) {
   const int W = L.pitch;
-  const T* cn = L.cn;
-  const T* rn = L.rhon;
+  auto cn = L.cn;
+  auto rn = L.rhon;
   T c = L.c[k], cnk = cn[k];
   T adv = rn[k + 1] * L.Tx[k] * L.u[k] + rn[k - 1] * L.Tx[k - 1] * L.u[k - 1] +
           rn[k + W] * L.Ty[k] * L.v[k] + rn[k - W] * L.Ty[k - W] * L.v[k - W];
   T diff = lap_h2(L.mobn, L.mu, k, W) + P.alpha * lap_h2(L.mobn, L.p, k, W);
   return rho * (c - cnk) * P.idt + adv - P.iPe * L.ih2 * diff;
 }
-template <typename T>
-__device__ __forceinline__ T op_c(const Prm<T>& P, const Lv<T>& L, int k) {
+template <typename T, class LV>
+__device__ __forceinline__ T op_c(const Prm<T>& P, const LV& L, int k) {
   return op_c(P, L, k, rho_of(P, L.c[k]));
 }
 
 // (pm-num-chem) with the time-averaged gradient term (pointwise G)
 // rq[f]: rho(c) of the neighbours k + 1, k - 1, k + W, k - W; rmu multiplies mu
 // (rho(c) in (pm-num-chem), rho^n in the projection method's (pj-num-chem))
-template <typename T>
-__device__ __forceinline__ T op_mu_r(const Prm<T>& P, const Lv<T>& L, int k, T rho, const T (&rq)[4],
+template <typename T, class LV>
+__device__ __forceinline__ T op_mu_r(const Prm<T>& P, const LV& L, int k, T rho, const T (&rq)[4],
                                      T rmu) {
   const int W = L.pitch;
-  const T* c = L.c;
-  const T* cn = L.cn;
-  const T* rn = L.rhon;
+  auto c = L.c;
+  auto cn = L.cn;
+  auto rn = L.rhon;
   T ck = c[k], cnk = cn[k];
   T rnk = rn[k];
   T rh = T(0.5) * (rho + rnk);
@@ -243,12 +249,12 @@ __device__ __forceinline__ T op_mu_r(const Prm<T>& P, const Lv<T>& L, int k, T r
   div *= T(0.25) * L.ih2;  // 1/2 (face average) * 1/2 (c^{n+1/2}) / h^2
   return rmu * L.mu[k] - P.K * bulk - grad + P.Lam * div;
 }
-template <typename T>
-__device__ __forceinline__ T op_mu(const Prm<T>& P, const Lv<T>& L, int k, T rho, const T (&rq)[4]) {
+template <typename T, class LV>
+__device__ __forceinline__ T op_mu(const Prm<T>& P, const LV& L, int k, T rho, const T (&rq)[4]) {
   return op_mu_r(P, L, k, rho, rq, rho);
 }
-template <typename T>
-__device__ __forceinline__ T op_mu(const Prm<T>& P, const Lv<T>& L, int k) {
+template <typename T, class LV>
+__device__ __forceinline__ T op_mu(const Prm<T>& P, const LV& L, int k) {
   const int W = L.pitch;
   const T rq[4] = {rho_of(P, L.c[k + 1]), rho_of(P, L.c[k - 1]), rho_of(P, L.c[k + W]),
                    rho_of(P, L.c[k - W])};
@@ -256,8 +262,8 @@ __device__ __forceinline__ T op_mu(const Prm<T>& P, const Lv<T>& L, int k) {
 }
 
 // (pm-num-mass)
-template <typename T>
-__device__ __forceinline__ T op_p(const Prm<T>& P, const Lv<T>& L, int k) {
+template <typename T, class LV>
+__device__ __forceinline__ T op_p(const Prm<T>& P, const LV& L, int k) {
   const int W = L.pitch;
   T dv = (L.u[k] - L.u[k - 1] + L.v[k] - L.v[k - W]) * L.ih;
   T diff = lap_h2(L.mobn, L.mu, k, W) + P.alpha * lap_h2(L.mobn, L.p, k, W);
@@ -269,13 +275,13 @@ __device__ __forceinline__ T op_p(const Prm<T>& P, const Lv<T>& L, int k) {
 // Cu.. / Cv.. of Lv): the same sum as op_u / op_v, term by term, regrouped by
 // unknown.  rs = the sum of rho(c) over the edge's two cells.  s is the stride
 // along the edge normal, t across it; a the row's own velocity, b the other one.
-template <typename T>
-__device__ __forceinline__ T mom_asm(const Lv<T>& L, int d, int k, T rs) {
+template <typename T, class LV>
+__device__ __forceinline__ T mom_asm(const LV& L, int d, int k, T rs) {
   const int s = d ? L.pitch : 1, t = d ? 1 : L.pitch;
-  const T *a = d ? L.v : L.u, *b = d ? L.u : L.v;
-  const T *C = d ? L.Cv : L.Cu, *aP = d ? L.aPv : L.aPu, *aM = d ? L.aMv : L.aMu;
-  const T *tP = d ? L.tPv : L.tPu, *tM = d ? L.tMv : L.tMu;
-  const T *M0 = d ? L.M0v : L.M0u, *M1 = d ? L.M1v : L.M1u;
+  auto a = d ? L.v : L.u; auto b = d ? L.u : L.v;
+  auto C = d ? L.Cv : L.Cu; auto aP = d ? L.aPv : L.aPu; auto aM = d ? L.aMv : L.aMu;
+  auto tP = d ? L.tPv : L.tPu; auto tM = d ? L.tMv : L.tMu;
+  auto M0 = d ? L.M0v : L.M0u; auto M1 = d ? L.M1v : L.M1u;
   T r = (d ? L.T0v : L.T0u)[k] + (C[k] + L.k.qidt * rs) * a[k];
   r += aP[k] * a[k + s] + aM[k] * a[k - s] + tP[k] * a[k + t] + tM[k] * a[k - t];
   // the grad-div term's cross derivative of the other velocity
@@ -290,11 +296,11 @@ __device__ __forceinline__ T mom_asm(const Lv<T>& L, int d, int k, T rs) {
 // (rs = rho(c_k) + rho(c_{k+1}), twice the density average on the edge).  PST =
 // false drops the pressure and surface-tension terms: the intermediate-velocity
 // row of the projection method (pj-num-mx).
-template <typename T, bool PST = true>
-__device__ __forceinline__ T op_u(const Prm<T>& P, const Lv<T>& L, int k, T rs) {
+template <typename T, bool PST = true, class LV>
+__device__ __forceinline__ T op_u(const Prm<T>& P, const LV& L, int k, T rs) {
   if constexpr (PST && sizeof(T) == 8) return mom_asm(L, 0, k, rs);  // FP64 primitive row
   const int W = L.pitch;
-  const T *u = L.u, *vis = L.visn, *rn = L.rhon;
+  auto u = L.u; auto vis = L.visn; auto rn = L.rhon;
   T ue = u[k];
   T dxl = (ue - u[k - 1]) * L.ih, dxr = (u[k + 1] - ue) * L.ih;
   T dvl = dxl + (L.v[k] - L.v[k - W]) * L.ih;
@@ -313,8 +319,8 @@ __device__ __forceinline__ T op_u(const Prm<T>& P, const Lv<T>& L, int k, T rs) 
                             (vr * dvr - vl * dvl) * T(1.0 / 3.0));
   return r + visc;
 }
-template <typename T>
-__device__ __forceinline__ T op_u(const Prm<T>& P, const Lv<T>& L, int k) {
+template <typename T, class LV>
+__device__ __forceinline__ T op_u(const Prm<T>& P, const LV& L, int k) {
   return op_u(P, L, k, rho_of(P, L.c[k]) + rho_of(P, L.c[k + 1]));
 }
 
@@ -322,11 +328,11 @@ __device__ __forceinline__ T op_u(const Prm<T>& P, const Lv<T>& L, int k) {
 // vertices k (east, (i+1/2, j+1/2)) and k-1 (west); gravity (1/Fr) A_y rho^n is in T0v
 // PST = false: the projection method's intermediate-velocity row, without
 // pressure, surface tension and gravity (those act in (pj-num-pjx))
-template <typename T, bool PST = true>
-__device__ __forceinline__ T op_v(const Prm<T>& P, const Lv<T>& L, int k, T rs) {
+template <typename T, bool PST = true, class LV>
+__device__ __forceinline__ T op_v(const Prm<T>& P, const LV& L, int k, T rs) {
   if constexpr (PST && sizeof(T) == 8) return mom_asm(L, 1, k, rs);  // FP64 primitive row
   const int W = L.pitch;
-  const T *v = L.v, *vis = L.visn, *rn = L.rhon;
+  auto v = L.v; auto vis = L.visn; auto rn = L.rhon;
   T ve = v[k];
   T dyb = (ve - v[k - W]) * L.ih, dyt = (v[k + W] - ve) * L.ih;
   T dvb = dyb + (L.u[k] - L.u[k - 1]) * L.ih;
@@ -345,8 +351,8 @@ __device__ __forceinline__ T op_v(const Prm<T>& P, const Lv<T>& L, int k, T rs) 
                             (vt * dvt - vb * dvb) * T(1.0 / 3.0));
   return r + visc;
 }
-template <typename T>
-__device__ __forceinline__ T op_v(const Prm<T>& P, const Lv<T>& L, int k) {
+template <typename T, class LV>
+__device__ __forceinline__ T op_v(const Prm<T>& P, const LV& L, int k) {
   return op_v(P, L, k, rho_of(P, L.c[k]) + rho_of(P, L.c[k + L.pitch]));
 }
 
@@ -358,8 +364,8 @@ __device__ __forceinline__ T op_v(const Prm<T>& P, const Lv<T>& L, int k) {
 // level n+1.  Gravity acts here, tested with u^{n+1} in the energy proof.
 // ---------------------------------------------------------------------------
 // u^{n+1} at edge (i+1/2, j), i = 0..m1; zero on no-slip walls
-template <typename T>
-__device__ __forceinline__ T proj_u(const Prm<T>& P, const Lv<T>& L, int i, int j) {
+template <typename T, class LV>
+__device__ __forceinline__ T proj_u(const Prm<T>& P, const LV& L, int i, int j) {
   if (!L.px && (i <= 0 || i >= L.m1)) return T(0);
   int k = L.at(i, j);
   T cl = L.c[k], cr = L.c[k + 1];
@@ -370,8 +376,8 @@ __device__ __forceinline__ T proj_u(const Prm<T>& P, const Lv<T>& L, int i, int 
   return L.u[k] + (st - dp) * P.iM / (Ar * P.idt);
 }
 // v^{n+1} at edge (i, j+1/2), j = 0..m2; zero on the walls in y
-template <typename T>
-__device__ __forceinline__ T proj_v(const Prm<T>& P, const Lv<T>& L, int i, int j) {
+template <typename T, class LV>
+__device__ __forceinline__ T proj_v(const Prm<T>& P, const LV& L, int i, int j) {
   if (j <= 0 || j >= L.m2) return T(0);
   const int W = L.pitch;
   int k = L.at(i, j);
@@ -385,15 +391,15 @@ __device__ __forceinline__ T proj_v(const Prm<T>& P, const Lv<T>& L, int i, int 
 // The four face velocities u^{n+1} of cell (i,j) (E, W, N, S), from rho(c) of the
 // cell (rk) and of its neighbours (rq[f] for k + 1, k - 1, k + W, k - W): the
 // same values as proj_u / proj_v without re-evaluating the densities.
-template <typename T>
-__device__ __forceinline__ void proj_faces(const Prm<T>& P, const Lv<T>& L, int i, int j, T rk,
+template <typename T, class LV>
+__device__ __forceinline__ void proj_faces(const Prm<T>& P, const LV& L, int i, int j, T rk,
                                            const T (&rq)[4], T (&w)[4]) {
   const int W = L.pitch;
   int k = L.at(i, j);
-  const T *c = L.c, *mu = L.mu, *p = L.p;
+  auto c = L.c; auto mu = L.mu; auto p = L.p;
   const T g = P.Fr_inv / P.idt;
   // face between cells a (left/below) and b = a + off, velocity array at a
-  auto face = [&](int a, int off, const T* vel, T ra, T rb, T grav) {
+  auto face = [&](int a, int off, auto vel, T ra, T rb, T grav) {
     T Ar = T(0.5) * (ra + rb);
     T dp = (p[a + off] - p[a]) * L.ih;
     T st = T(0.5) * (rb * mu[a] + ra * mu[a + off]) * (c[a + off] - c[a]) * L.ih;
@@ -409,11 +415,11 @@ __device__ __forceinline__ void proj_faces(const Prm<T>& P, const Lv<T>& L, int 
 // rho = rho(c^{n+1}) and c^{n+1} in the advection; and (pj-num-mass): d_x u^{n+1}
 // + d_y v^{n+1} - (alpha/Pe)(grad.(A m grad mu) + alpha grad.(A m grad p)).
 // Both from the shared densities rq and the face velocities w of proj_faces.
-template <typename T>
-__device__ __forceinline__ T opp_c_w(const Prm<T>& P, const Lv<T>& L, int k, const T (&rq)[4],
+template <typename T, class LV>
+__device__ __forceinline__ T opp_c_w(const Prm<T>& P, const LV& L, int k, const T (&rq)[4],
                                      const T (&w)[4]) {
   const int W = L.pitch;
-  const T* c = L.c;
+  auto c = L.c;
   T ck = c[k];
   T t = L.rhon[k] * (ck - L.cn[k]) * P.idt;
   T ax = T(0.5) * (rq[0] * (c[k + 1] - ck) * L.ih * w[0] + rq[1] * (ck - c[k - 1]) * L.ih * w[1]);
@@ -421,8 +427,8 @@ __device__ __forceinline__ T opp_c_w(const Prm<T>& P, const Lv<T>& L, int k, con
   T diff = lap_h2(L.mobn, L.mu, k, W) + P.alpha * lap_h2(L.mobn, L.p, k, W);
   return t + ax + ay - P.iPe * L.ih2 * diff;
 }
-template <typename T>
-__device__ __forceinline__ T opp_p_w(const Prm<T>& P, const Lv<T>& L, int k, const T (&w)[4]) {
+template <typename T, class LV>
+__device__ __forceinline__ T opp_p_w(const Prm<T>& P, const LV& L, int k, const T (&w)[4]) {
   const int W = L.pitch;
   T dv = (w[0] - w[1] + w[2] - w[3]) * L.ih;
   T diff = lap_h2(L.mobn, L.mu, k, W) + P.alpha * lap_h2(L.mobn, L.p, k, W);
@@ -430,27 +436,27 @@ __device__ __forceinline__ T opp_p_w(const Prm<T>& P, const Lv<T>& L, int k, con
 }
 
 // (pj-num-chem): as (pm-num-chem) with rho^n in front of mu
-template <typename T>
-__device__ __forceinline__ T opp_mu(const Prm<T>& P, const Lv<T>& L, int k) {
+template <typename T, class LV>
+__device__ __forceinline__ T opp_mu(const Prm<T>& P, const LV& L, int k) {
   const int W = L.pitch;
   const T rq[4] = {rho_of(P, L.c[k + 1]), rho_of(P, L.c[k - 1]), rho_of(P, L.c[k + W]),
                    rho_of(P, L.c[k - W])};
   return op_mu_r(P, L, k, rho_of(P, L.c[k]), rq, L.rhon[k]);
 }
-template <typename T>
-__device__ __forceinline__ T opp_u(const Prm<T>& P, const Lv<T>& L, int k) {
+template <typename T, class LV>
+__device__ __forceinline__ T opp_u(const Prm<T>& P, const LV& L, int k) {
   return op_u<T, false>(P, L, k, rho_of(P, L.c[k]) + rho_of(P, L.c[k + 1]));
 }
-template <typename T>
-__device__ __forceinline__ T opp_v(const Prm<T>& P, const Lv<T>& L, int k) {
+template <typename T, class LV>
+__device__ __forceinline__ T opp_v(const Prm<T>& P, const LV& L, int k) {
   return op_v<T, false>(P, L, k, rho_of(P, L.c[k]) + rho_of(P, L.c[k + L.pitch]));
 }
 
 // ---------------------------------------------------------------------------
 // stores that keep ghost copies consistent (App. A.6 boundary conditions)
 // ---------------------------------------------------------------------------
-template <typename T>
-__device__ __forceinline__ void store_cell(const Lv<T>& L, T* a, int i, int j, T x) {
+template <typename T, class LV, class A>
+__device__ __forceinline__ void store_cell(const LV& L, A a, int i, int j, T x) {
   const int W = L.pitch;
   int k = j * W + i;
   a[k] = x;
@@ -460,10 +466,10 @@ __device__ __forceinline__ void store_cell(const Lv<T>& L, T* a, int i, int j, T
   if (j == L.m2) a[k + W] = x;
 }
 
-template <typename T>
-__device__ __forceinline__ void store_u(const Lv<T>& L, int e, int j, T x) {
+template <typename T, class LV>
+__device__ __forceinline__ void store_u(const LV& L, int e, int j, T x) {
   const int W = L.pitch;
-  T* u = L.u;
+  auto u = L.u;
   int cols[3] = {e, e, e};
   int n = 1;
   if (L.px) {
@@ -479,10 +485,10 @@ __device__ __forceinline__ void store_u(const Lv<T>& L, int e, int j, T x) {
   }
 }
 
-template <typename T>
-__device__ __forceinline__ void store_v(const Lv<T>& L, int i, int e, T x) {
+template <typename T, class LV>
+__device__ __forceinline__ void store_v(const LV& L, int i, int e, T x) {
   const int W = L.pitch;
-  T* v = L.v;
+  auto v = L.v;
   int k = e * W + i;
   v[k] = x;
   if (L.px) {
@@ -512,11 +518,11 @@ template <typename T> __device__ __forceinline__ T dgsec(T a, T b, T e) {
   return T(0.25) * e * (a * (a - T(1)) + b * (b - T(1)) + (T(2) * a - T(1) + e) * (a + b - T(1) + e));
 }
 
-template <typename T>
-__device__ __forceinline__ T opd_c(const Prm<T>& P, const Lv<T>& L, int k) {
+template <typename T, class LV>
+__device__ __forceinline__ T opd_c(const Prm<T>& P, const LV& L, int k) {
   const int W = L.pitch;
-  const T* cn = L.cn;
-  const T* rn = L.rhon;
+  auto cn = L.cn;
+  auto rn = L.rhon;
   T e = L.c[k], C = L.Bc[k];
   T rp = rho_of(P, C + e), rC = rho_of(P, C);
   (void)cn;
@@ -526,10 +532,10 @@ __device__ __forceinline__ T opd_c(const Prm<T>& P, const Lv<T>& L, int k) {
   return e * (rp + rsec_(P, rp, rC) * L.Bdc[k]) * P.idt + adv - P.iPe * L.ih2 * diff;
 }
 
-template <typename T>
-__device__ __forceinline__ T opd_mu(const Prm<T>& P, const Lv<T>& L, int k) {
+template <typename T, class LV>
+__device__ __forceinline__ T opd_mu(const Prm<T>& P, const LV& L, int k) {
   const int W = L.pitch;
-  const T *e = L.c, *B = L.Bc, *cn = L.cn, *rn = L.rhon;
+  auto e = L.c; auto B = L.Bc; auto cn = L.cn; auto rn = L.rhon;
   T ek = e[k], Ck = B[k], cnk = cn[k], rnk = rn[k];
   T cp = Ck + ek;
   T rp = rho_of(P, cp), rC = rho_of(P, Ck);
@@ -563,15 +569,15 @@ __device__ __forceinline__ T opd_mu(const Prm<T>& P, const Lv<T>& L, int k) {
   return rp * L.mu[k] + dr * L.Bmu[k] - P.K * dbulk - dgrad + P.Lam * ddiv;
 }
 
-template <typename T>
-__device__ __forceinline__ T opd_p(const Prm<T>& P, const Lv<T>& L, int k) { return op_p(P, L, k); }
+template <typename T, class LV>
+__device__ __forceinline__ T opd_p(const Prm<T>& P, const LV& L, int k) { return op_p(P, L, k); }
 
 // x row: the terms of op_u that are linear in (u, v, p, mu), applied to e, plus
 // 1/2 (A_x rho(c') - A_x rho^n) e_u/dt + 1/2 A_x(rho(c') - rho(C)) U/dt
-template <typename T>
-__device__ __forceinline__ T opd_u(const Prm<T>& P, const Lv<T>& L, int k) {
+template <typename T, class LV>
+__device__ __forceinline__ T opd_u(const Prm<T>& P, const LV& L, int k) {
   const int W = L.pitch;
-  const T *u = L.u, *vis = L.visn, *rn = L.rhon;
+  auto u = L.u; auto vis = L.visn; auto rn = L.rhon;
   T ue = u[k];
   T cl = L.Bc[k] + L.c[k], cr = L.Bc[k + 1] + L.c[k + 1];
   T rpl = rho_of(P, cl), rpr = rho_of(P, cr);
@@ -594,10 +600,10 @@ __device__ __forceinline__ T opd_u(const Prm<T>& P, const Lv<T>& L, int k) {
   return time + conv + press + st + visc;
 }
 
-template <typename T>
-__device__ __forceinline__ T opd_v(const Prm<T>& P, const Lv<T>& L, int k) {
+template <typename T, class LV>
+__device__ __forceinline__ T opd_v(const Prm<T>& P, const LV& L, int k) {
   const int W = L.pitch;
-  const T *v = L.v, *vis = L.visn, *rn = L.rhon;
+  auto v = L.v; auto vis = L.visn; auto rn = L.rhon;
   T ve = v[k];
   T cb = L.Bc[k] + L.c[k], ct = L.Bc[k + W] + L.c[k + W];
   T rpb = rho_of(P, cb), rpt = rho_of(P, ct);
@@ -624,42 +630,82 @@ __device__ __forceinline__ T opd_v(const Prm<T>& P, const Lv<T>& L, int k) {
 // the base X of a defect-correction cycle).  val_c / val_mu return the full
 // value c, mu that the local Jacobians of the smoothers are evaluated at.
 struct FullForm {
-  template <typename T> static __device__ __forceinline__ T val_c(const Lv<T>& L, int k) { return L.c[k]; }
-  template <typename T> static __device__ __forceinline__ T rho(const Prm<T>&, const Lv<T>& L, int k) { return L.rhoc[k]; }
-  template <typename T> static __device__ __forceinline__ T val_u(const Lv<T>& L, int k) { return L.u[k]; }
-  template <typename T> static __device__ __forceinline__ T val_v(const Lv<T>& L, int k) { return L.v[k]; }
-  template <typename T> static __device__ __forceinline__ T val_mu(const Lv<T>& L, int k) { return L.mu[k]; }
-  template <typename T> static __device__ __forceinline__ T Nc(const Prm<T>& P, const Lv<T>& L, int k) { return op_c(P, L, k); }
-  template <typename T> static __device__ __forceinline__ T Nmu(const Prm<T>& P, const Lv<T>& L, int k) { return op_mu(P, L, k); }
-  template <typename T> static __device__ __forceinline__ T Np(const Prm<T>& P, const Lv<T>& L, int k) { return op_p(P, L, k); }
-  template <typename T> static __device__ __forceinline__ T Nu(const Prm<T>& P, const Lv<T>& L, int k) { return op_u(P, L, k); }
-  template <typename T> static __device__ __forceinline__ T Nv(const Prm<T>& P, const Lv<T>& L, int k) { return op_v(P, L, k); }
+  template <class LV>
+static __device__ __forceinline__ typename LV::real val_c(const LV& L, int k) {
+  typedef typename LV::real T; return L.c[k]; }
+  template <typename T, class LV>
+static __device__ __forceinline__ T rho(const Prm<T>&, const LV& L, int k) { return L.rhoc[k]; }
+  template <class LV>
+static __device__ __forceinline__ typename LV::real val_u(const LV& L, int k) {
+  typedef typename LV::real T; return L.u[k]; }
+  template <class LV>
+static __device__ __forceinline__ typename LV::real val_v(const LV& L, int k) {
+  typedef typename LV::real T; return L.v[k]; }
+  template <class LV>
+static __device__ __forceinline__ typename LV::real val_mu(const LV& L, int k) {
+  typedef typename LV::real T; return L.mu[k]; }
+  template <typename T, class LV>
+static __device__ __forceinline__ T Nc(const Prm<T>& P, const LV& L, int k) { return op_c(P, L, k); }
+  template <typename T, class LV>
+static __device__ __forceinline__ T Nmu(const Prm<T>& P, const LV& L, int k) { return op_mu(P, L, k); }
+  template <typename T, class LV>
+static __device__ __forceinline__ T Np(const Prm<T>& P, const LV& L, int k) { return op_p(P, L, k); }
+  template <typename T, class LV>
+static __device__ __forceinline__ T Nu(const Prm<T>& P, const LV& L, int k) { return op_u(P, L, k); }
+  template <typename T, class LV>
+static __device__ __forceinline__ T Nv(const Prm<T>& P, const LV& L, int k) { return op_v(P, L, k); }
 };
 // The projection method on the full iterate (u, v arrays hold the intermediate
 // velocity).  Its N_c and N_p need the cell's face velocities (proj_faces,
 // which needs the cell index for the wall edges), so the kernels call
 // opp_c_w / opp_p_w directly.
 struct ProjForm {
-  template <typename T> static __device__ __forceinline__ T val_c(const Lv<T>& L, int k) { return L.c[k]; }
-  template <typename T> static __device__ __forceinline__ T rho(const Prm<T>&, const Lv<T>& L, int k) { return L.rhoc[k]; }
-  template <typename T> static __device__ __forceinline__ T val_u(const Lv<T>& L, int k) { return L.u[k]; }
-  template <typename T> static __device__ __forceinline__ T val_v(const Lv<T>& L, int k) { return L.v[k]; }
-  template <typename T> static __device__ __forceinline__ T val_mu(const Lv<T>& L, int k) { return L.mu[k]; }
-  template <typename T> static __device__ __forceinline__ T Nmu(const Prm<T>& P, const Lv<T>& L, int k) { return opp_mu(P, L, k); }
-  template <typename T> static __device__ __forceinline__ T Nu(const Prm<T>& P, const Lv<T>& L, int k) { return opp_u(P, L, k); }
-  template <typename T> static __device__ __forceinline__ T Nv(const Prm<T>& P, const Lv<T>& L, int k) { return opp_v(P, L, k); }
+  template <class LV>
+static __device__ __forceinline__ typename LV::real val_c(const LV& L, int k) {
+  typedef typename LV::real T; return L.c[k]; }
+  template <typename T, class LV>
+static __device__ __forceinline__ T rho(const Prm<T>&, const LV& L, int k) { return L.rhoc[k]; }
+  template <class LV>
+static __device__ __forceinline__ typename LV::real val_u(const LV& L, int k) {
+  typedef typename LV::real T; return L.u[k]; }
+  template <class LV>
+static __device__ __forceinline__ typename LV::real val_v(const LV& L, int k) {
+  typedef typename LV::real T; return L.v[k]; }
+  template <class LV>
+static __device__ __forceinline__ typename LV::real val_mu(const LV& L, int k) {
+  typedef typename LV::real T; return L.mu[k]; }
+  template <typename T, class LV>
+static __device__ __forceinline__ T Nmu(const Prm<T>& P, const LV& L, int k) { return opp_mu(P, L, k); }
+  template <typename T, class LV>
+static __device__ __forceinline__ T Nu(const Prm<T>& P, const LV& L, int k) { return opp_u(P, L, k); }
+  template <typename T, class LV>
+static __device__ __forceinline__ T Nv(const Prm<T>& P, const LV& L, int k) { return opp_v(P, L, k); }
 };
 struct ErrForm {
-  template <typename T> static __device__ __forceinline__ T val_c(const Lv<T>& L, int k) { return L.Bc[k] + L.c[k]; }
-  template <typename T> static __device__ __forceinline__ T rho(const Prm<T>& P, const Lv<T>& L, int k) { return rho_of(P, val_c(L, k)); }
-  template <typename T> static __device__ __forceinline__ T val_u(const Lv<T>& L, int k) { return L.Bu[k] + L.u[k]; }
-  template <typename T> static __device__ __forceinline__ T val_v(const Lv<T>& L, int k) { return L.Bv[k] + L.v[k]; }
-  template <typename T> static __device__ __forceinline__ T val_mu(const Lv<T>& L, int k) { return L.Bmu[k] + L.mu[k]; }
-  template <typename T> static __device__ __forceinline__ T Nc(const Prm<T>& P, const Lv<T>& L, int k) { return opd_c(P, L, k); }
-  template <typename T> static __device__ __forceinline__ T Nmu(const Prm<T>& P, const Lv<T>& L, int k) { return opd_mu(P, L, k); }
-  template <typename T> static __device__ __forceinline__ T Np(const Prm<T>& P, const Lv<T>& L, int k) { return opd_p(P, L, k); }
-  template <typename T> static __device__ __forceinline__ T Nu(const Prm<T>& P, const Lv<T>& L, int k) { return opd_u(P, L, k); }
-  template <typename T> static __device__ __forceinline__ T Nv(const Prm<T>& P, const Lv<T>& L, int k) { return opd_v(P, L, k); }
+  template <class LV>
+static __device__ __forceinline__ typename LV::real val_c(const LV& L, int k) {
+  typedef typename LV::real T; return L.Bc[k] + L.c[k]; }
+  template <typename T, class LV>
+static __device__ __forceinline__ T rho(const Prm<T>& P, const LV& L, int k) { return rho_of(P, val_c(L, k)); }
+  template <class LV>
+static __device__ __forceinline__ typename LV::real val_u(const LV& L, int k) {
+  typedef typename LV::real T; return L.Bu[k] + L.u[k]; }
+  template <class LV>
+static __device__ __forceinline__ typename LV::real val_v(const LV& L, int k) {
+  typedef typename LV::real T; return L.Bv[k] + L.v[k]; }
+  template <class LV>
+static __device__ __forceinline__ typename LV::real val_mu(const LV& L, int k) {
+  typedef typename LV::real T; return L.Bmu[k] + L.mu[k]; }
+  template <typename T, class LV>
+static __device__ __forceinline__ T Nc(const Prm<T>& P, const LV& L, int k) { return opd_c(P, L, k); }
+  template <typename T, class LV>
+static __device__ __forceinline__ T Nmu(const Prm<T>& P, const LV& L, int k) { return opd_mu(P, L, k); }
+  template <typename T, class LV>
+static __device__ __forceinline__ T Np(const Prm<T>& P, const LV& L, int k) { return opd_p(P, L, k); }
+  template <typename T, class LV>
+static __device__ __forceinline__ T Nu(const Prm<T>& P, const LV& L, int k) { return opd_u(P, L, k); }
+  template <typename T, class LV>
+static __device__ __forceinline__ T Nv(const Prm<T>& P, const LV& L, int k) { return opd_v(P, L, k); }
 };
 
 }  // namespace qn
