@@ -17,6 +17,17 @@ namespace qn {
 
 constexpr int BX = 32, BY = 8, NT = BX * BY;
 
+// the type a kernel computes in for data of type T: the error equation's
+// kernels with their contraction fixed (Fused)
+template <typename T, class Form>
+using compute_t = typename std::conditional<std::is_same<Form, ErrForm>::value, Fused<T>, T>::type;
+// the same bits as data of the kernel's type
+template <typename R, template <typename> class S, typename T>
+static inline const S<R>& as_compute(const S<T>& x) {
+  static_assert(sizeof(S<T>) == sizeof(S<R>), "one layout");
+  return reinterpret_cast<const S<R>&>(x);
+}
+
 static inline dim3 grid2(int nx, int ny) { return dim3((nx + BX - 1) / BX, (ny + BY - 1) / BY); }
 
 // number of kernels issued by this library since load (host-side count;
@@ -69,15 +80,15 @@ __device__ __forceinline__ void warp_sum5(double& a, double& b, double& c, doubl
   // lanes 0..15 keep a, b, e, lanes 16..31 keep c, d (and a zero)
   double x = (b4 ? c : a) + __shfl_xor_sync(FULL, b4 ? a : c, 16);
   double y = (b4 ? d : b) + __shfl_xor_sync(FULL, b4 ? b : d, 16);
-  double z = e + __shfl_xor_sync(FULL, e, 16);  // the same on both halves
+  double z = e + shfl_xor(e, 16);  // the same on both halves
   // lanes with bit 3 clear keep x, the others y
   double w = (b3 ? y : x) + __shfl_xor_sync(FULL, b3 ? x : y, 8);
   // e on the lanes with bit 2 set in a register of its own: two values, three exchanges
   z += __shfl_xor_sync(FULL, z, 8);
   const bool b2 = lane & 4;
   double wz = (b2 ? z : w) + __shfl_xor_sync(FULL, b2 ? w : z, 4);
-  wz += __shfl_xor_sync(FULL, wz, 2);
-  wz += __shfl_xor_sync(FULL, wz, 1);
+  wz += shfl_xor(wz, 2);
+  wz += shfl_xor(wz, 1);
   a = __shfl_sync(FULL, wz, 0);
   b = __shfl_sync(FULL, wz, 8);
   c = __shfl_sync(FULL, wz, 16);
@@ -254,11 +265,13 @@ __device__ __forceinline__ void residual_cell(const Prm<T>& P, const LV& L, int 
     nu = op_u<T, false>(P, L, k, rk + rq[0]);  // also on boundary edges (padded arrays); masked below
     nv = op_v<T, false>(P, L, k, rk + rq[2]);  // also on boundary edges (padded arrays); masked below
   } else {
-    nc = Form::Nc(P, L, k);
-    nm = Form::Nmu(P, L, k);
-    np = Form::Np(P, L, k);
-    nu = Form::Nu(P, L, k);  // also on boundary edges (padded arrays); masked below
-    nv = Form::Nv(P, L, k);  // also on boundary edges (padded arrays); masked below
+    const ErrCell<T> X = err_cell(P, L, k);
+    T flux = flux_sum(P, L, k);
+    nc = err_c(P, L, k, X.r[0]) - L.k.dif * flux;
+    nm = err_mu(P, L, k, X);
+    np = (L.u[k] - L.u[k - 1] + L.v[k] - L.v[k - L.pitch]) * L.ih - L.k.adif * flux;
+    nu = err_row(P, L, 0, k, X.r[0] + X.r[1], X.dr[0] + X.dr[1]);  // wall edges too, as above
+    nv = err_row(P, L, 1, k, X.r[0] + X.r[3], X.dr[0] + X.dr[3]);
   }
   if (MODE == 0) {
     T r[5] = {L.fc[k] - nc, L.fmu[k] - nm, L.fp[k] - np, hu ? L.fu[k] - nu : T(0),
@@ -368,6 +381,44 @@ __device__ __forceinline__ void ch_system_full(const Prm<T>& P, const LV& L, int
   J[1][1] = rk;
 }
 
+// ch_system for the error equation: the residuals of err_c and err_mu, and
+// ch_system_full's Jacobian at the full values C + e, Mu + e_mu
+template <typename T, class LV>
+__device__ __forceinline__ void ch_system_err(const Prm<T>& P, const LV& L, int i, int j,
+                                              const ErrCell<T>& X, T (&J)[2][2], T (&R)[2]) {
+  const int W = L.pitch;
+  const int k = L.at(i, j);
+  const int off[5] = {0, 1, -1, W, -W};
+  const bool wall[5] = {false, !L.px && i == L.m1, !L.px && i == 1, j == L.m2, j == 1};
+  auto mob = L.mobn;
+  R[0] = err_c(P, L, k, X.r[0]) - L.k.dif * flux_sum(P, L, k) - L.fc[k];
+  R[1] = err_mu(P, L, k, X) - L.fmu[k];
+  T ck = X.B[0] + X.e[0], cnk = L.cn[k], rk = X.r[0], rnk = X.rn[0], mk = mob[k];
+  T muk = L.Bmu[k] + L.mu[k];
+  T S = rk + rnk, ch = ck + cnk;
+  T sm = T(0), G2 = T(0), sd = T(0), SD = T(0), SW = T(0);
+#pragma unroll
+  for (int f = 1; f < 5; ++f) {
+    T cq = X.B[f] + X.e[f], d = cq - ck;
+    G2 += d * d;
+    sd += d;
+    SD += (cq + L.cn[k + off[f]]) - ch;
+    sm += wall[f] ? T(0) : mk + mob[k + off[f]];
+    SW += wall[f] ? T(0) : S + (X.r[f] + X.rn[f]);
+  }
+  T dck = ck - cnk, ar = -P.alpha * rk, drho = ar * rk, r = ar * rnk;
+  T dr = -P.alpha * rnk * drho;
+  T A = ck * ck - ck, An = cnk * cnk - cnk, sA = A + An, t = ch - T(1), g4 = sA * t;
+  T Gs = L.k.hih2 * G2 + L.Gn[k];
+  T E = L.k.K8 * (A * A + An * An) + L.k.L4 * Gs;
+  T tc = T(2) * ck - T(1);
+  J[0][0] = (rk + drho * dck) * P.idt;
+  J[0][1] = L.k.dif * sm;
+  J[1][0] = drho * (muk + L.k.L8 * SD - L.k.K8 * g4) - L.k.K8 * (S * (tc * t + sA)) -
+            r * (L.k.K4 * (A * tc) - L.k.L4h * sd) - dr * E - L.k.L8 * SW;
+  J[1][1] = rk;
+}
+
 // The 2x2 CH system of cell (i,j): residuals R = N - f of (N_c, N_mu) and their
 // Jacobian J in (c, mu), neighbours frozen, at the full values c, mu
 template <typename T, class Form, class LV>
@@ -378,6 +429,10 @@ __device__ __forceinline__ void ch_system(const Prm<T>& P, const LV& L, int i, i
   const int off[4] = {1, -1, W, -W};
   if constexpr (std::is_same<Form, FullForm>::value) {
     ch_system_full(P, L, i, j, J, R);
+    return;
+  }
+  if constexpr (std::is_same<Form, ErrForm>::value) {
+    ch_system_err(P, L, i, j, err_cell(P, L, k), J, R);
     return;
   }
   // rho(c) of the cell and its four neighbours, shared by N_c, N_mu and J
@@ -392,8 +447,7 @@ __device__ __forceinline__ void ch_system(const Prm<T>& P, const LV& L, int i, i
     Rc = opp_c_w(P, L, k, rq4, wf) - L.fc[k];
     Rm = op_mu_r(P, L, k, rho, rq4, L.rhon[k]) - L.fmu[k];
   } else {
-    Rc = Form::Nc(P, L, k) - L.fc[k];
-    Rm = Form::Nmu(P, L, k) - L.fmu[k];
+    Rc = Rm = T(0);
   }
   auto cn = L.cn; auto rn = L.rhon; auto mob = L.mobn;
   // full values c, mu at which the local Jacobian is evaluated
@@ -452,30 +506,85 @@ __device__ __forceinline__ void ch_cell(const Prm<T>& P, const LV& L, int i, int
   T dc = (J[1][1] * R[0] - J[0][1] * R[1]) * idet;
   T dm = (J[0][0] * R[1] - J[1][0] * R[0]) * idet;
   int k = L.at(i, j);
-  T cnew = L.c[k] - dc;
-  store_cell(L, L.c, i, j, cnew);
-  if constexpr (!std::is_same<Form, ErrForm>::value) store_cell(L, L.rhoc, i, j, rho_of(P, cnew));
-  store_cell(L, L.mu, i, j, L.mu[k] - dm);
+  const bool ghosts = has_ghosts(L, i, j);
+  const T cnew = L.c[k] - dc, mnew = L.mu[k] - dm;
+  put_cell(L, L.c, i, j, ghosts, cnew);
+  if constexpr (!std::is_same<Form, ErrForm>::value)
+    put_cell(L, L.rhoc, i, j, ghosts, rho_of(P, cnew));
+  put_cell(L, L.mu, i, j, ghosts, mnew);
+}
+
+// first cell i0 >= 1 of colour `colour` in row j and the stride between cells
+// of that colour in the row; false if the row has none
+template <class LV>
+__device__ __forceinline__ bool colour_row(const LV& L, int colour, int j, int& i0, int& stride) {
+  if (L.c8) {
+    int d = (colour - j) & 7;
+    if (d & 1) return false;
+    i0 = d >> 1;
+    if (i0 == 0) i0 = 4;
+    stride = 4;
+  } else {
+    const int K = L.kcol;
+    int y = colour + 2 * (K - (j - K * L.kdiv.div(j)));  // (colour - 2j) mod K, plus at most 2K
+    y = y >= 2 * K ? y - 2 * K : y;
+    y = y >= K ? y - K : y;
+    i0 = y == 0 ? K : y;
+    stride = K;
+  }
+  return true;
+}
+
+// slots of Vanka colour `col`: slot t -> row j0 + rstep * (t / mpr), t % mpr-th
+// cell of that row's colour
+struct ColourSlots {
+  int j0, rstep, mpr, n;
+};
+
+template <class LV>
+__host__ __device__ __forceinline__ ColourSlots vanka_slots(const LV& L, int col) {
+  ColourSlots cs;
+  cs.j0 = L.c8 && ((col - 1) & 1) ? 2 : 1;  // eight colours: rows with (col - j) even
+  cs.rstep = L.c8 ? 2 : 1;
+  cs.mpr = L.vrow.d;
+  cs.n = cs.j0 > L.m2 ? 0 : (((L.m2 - cs.j0) >> (cs.rstep - 1)) + 1) * cs.mpr;
+  return cs;
+}
+
+template <class LV>
+__device__ __forceinline__ bool vanka_slot_cell(const LV& L, int col, const ColourSlots& cs, int t,
+                                                int& i, int& j) {
+  const int r = L.vrow.div(t);
+  j = cs.j0 + cs.rstep * r;
+  int i0, stride;
+  if (!colour_row(L, col, j, i0, stride)) return false;
+  i = i0 + stride * (t - r * cs.mpr);
+  return i <= L.m1;
+}
+
+// cell of slot t of CH colour `colour` ((i + j) % 2, rows packed); false past the row's end
+template <class LV>
+__device__ __forceinline__ bool ch_slot_cell(const LV& L, int colour, int t, int& i, int& j) {
+  const int r = L.crow.div(t);
+  j = r + 1;
+  i = (((colour - j) & 1) ? 1 : 2) + 2 * (t - r * L.crow.d);
+  return i <= L.m1;
 }
 
 // cells of CH colour `colour` ((i + j) % 2), packed: slot t -> row t / mpr + 1
 template <typename T, class Form>
 __global__ void __launch_bounds__(64) k_ch(Prm<T> P, Lv<T> L, int colour) {
   pdl_enter();
-  int mpr = (L.m1 + 1) / 2;
-  int t = blockIdx.x * 64 + threadIdx.x;
-  if (t >= mpr * L.m2) return;
-  int j = t / mpr + 1;
-  int i = (((colour - j) & 1) ? 1 : 2) + 2 * (t % mpr);
-  if (i > L.m1) return;
+  int t = blockIdx.x * 64 + threadIdx.x, i, j;
+  if (t >= L.crow.d * L.m2 || !ch_slot_cell(L, colour, t, i, j)) return;
   ch_cell<T, Form>(P, L, i, j);
 }
 
 // sum over the four lanes of a team (lanes 4t .. 4t+3)
 template <typename T>
 __device__ __forceinline__ T team_sum(T v) {
-  v += __shfl_xor_sync(0xffffffffu, v, 1);
-  return v + __shfl_xor_sync(0xffffffffu, v, 2);
+  v += shfl_xor(v, 1);
+  return v + shfl_xor(v, 2);
 }
 
 // u^{n+1} at face q (W, E, S, N) of cell k (0 on a wall face), as proj_faces
@@ -495,18 +604,17 @@ __device__ __forceinline__ T proj_face_team(const Prm<T>& P, const LV& L, int k,
   return open ? vel[a] + (st - dp) * P.iM / (Ar * P.idt) - grav : T(0);
 }
 
-// rho(c) of the full value at cell k and, on error levels, of the base: what
-// the rows of a team's lane need of a cell
+// rho(c) of the full value at cell k and, on error levels, its difference to
+// the base's: what the rows of a team's lane need of a cell
 template <typename T>
 struct RhoPair {
-  T r, b;
+  T r, d;
 };
 template <typename T, class Form, class LV>
 __device__ __forceinline__ RhoPair<T> rho_pair(const Prm<T>& P, const LV& L, int k) {
-  if constexpr (std::is_same<Form, ErrForm>::value)
-    return {Form::rho(P, L, k), rho_of(P, L.Bc[k])};
-  else
-    return {Form::rho(P, L, k), T(0)};
+  const T r = Form::rho(P, L, k);
+  if constexpr (std::is_same<Form, ErrForm>::value) return {r, rsec_(P, r, L.rB[k]) * L.c[k]};
+  else return {r, T(0)};
 }
 
 // sums over the four lanes of a team of eight values each lane holds, every
@@ -521,12 +629,12 @@ __device__ __forceinline__ void team_sum8(double (&v)[8]) {
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     double send = b0 ? v[i] : v[i + 4], keep = b0 ? v[i + 4] : v[i];
-    r[i] = keep + __shfl_xor_sync(FULL, send, 1);
+    r[i] = keep + shfl_xor(send, 1);
   }
 #pragma unroll
   for (int i = 0; i < 2; ++i) {
     double send = b1 ? r[i] : r[i + 2], keep = b1 ? r[i + 2] : r[i];
-    t[i] = keep + __shfl_xor_sync(FULL, send, 2);
+    t[i] = keep + shfl_xor(send, 2);
   }
 #pragma unroll
   for (int m = 0; m < 8; ++m)
@@ -641,12 +749,10 @@ __device__ __forceinline__ ChRows<T> ch_team_rows(const Prm<T>& P, const LV& L, 
   } else if constexpr (std::is_same<Form, ErrForm>::value) {
     auto e = L.c; auto B = L.Bc;
     T ek = e[k], Ck = B[k];
-    T rC = ra.b;
-    Nc = ek * (rho + rsec_(P, rho, rC) * L.Bdc[k]) * P.idt + sadv - L.k.dif * sflux;
+    Nc = ek * (rho + rsec_(P, rho, L.rB[k]) * L.Bdc[k]) * P.idt + sadv - L.k.dif * sflux;
     T dC = B[nq] - Ck, de = e[nq] - ek;
-    T rCq = rb.b;
-    T dr = rsec_(P, rho, rC) * ek;
-    T drq = rsec_(P, rq, rCq) * e[nq];
+    T dr = ra.d;
+    T drq = rb.d;
     T chP = Ck + cnk;
     T sdGe = team_sum<T>(de * (T(2) * dC + de));
     T sGC = team_sum<T>(dC * dC);
@@ -709,10 +815,12 @@ __device__ __forceinline__ void ch_team(const Prm<T>& P, const LV& L, int i, int
   T dm = (R.J11 * R.Rm - R.J21 * R.Rc) * idet;
   if (ok && q == 0) {
     int k = L.at(i, j);
-    T cnew = L.c[k] - dc;
-    store_cell(L, L.c, i, j, cnew);
-    if constexpr (!std::is_same<Form, ErrForm>::value) store_cell(L, L.rhoc, i, j, rho_of(P, cnew));
-    store_cell(L, L.mu, i, j, L.mu[k] - dm);
+    const bool ghosts = has_ghosts(L, i, j);
+    const T cnew = L.c[k] - dc, mnew = L.mu[k] - dm;
+    put_cell(L, L.c, i, j, ghosts, cnew);
+    if constexpr (!std::is_same<Form, ErrForm>::value)
+      put_cell(L, L.rhoc, i, j, ghosts, rho_of(P, cnew));
+    put_cell(L, L.mu, i, j, ghosts, mnew);
   }
 }
 
@@ -720,18 +828,11 @@ __device__ __forceinline__ void ch_team(const Prm<T>& P, const LV& L, int i, int
 template <typename T, class Form>
 __global__ void __launch_bounds__(64) k_ch_team(Prm<T> P, Lv<T> L, int colour) {
   pdl_enter();
-  int mpr = (L.m1 + 1) / 2;
-  int n = mpr * L.m2;
+  int n = L.crow.d * L.m2;
   int t = blockIdx.x * 64 + threadIdx.x;
   if ((t & ~31) >= 4 * n) return;  // warp-uniform
-  int s = t >> 2;
-  int j = 1, i = 1;
-  bool ok = false;
-  if (s < n) {
-    j = s / mpr + 1;
-    i = (((colour - j) & 1) ? 1 : 2) + 2 * (s % mpr);
-    ok = i <= L.m1;
-  }
+  int i = 1, j = 1;
+  bool ok = (t >> 2) < n && ch_slot_cell(L, colour, t >> 2, i, j);
   if (!ok) i = j = 1;
   ch_team<T, Form>(P, L, i, j, ok);
 }
@@ -743,12 +844,14 @@ __global__ void __launch_bounds__(64) k_ch_team(Prm<T> P, Lv<T> L, int colour) {
 // --------------------------------------------------------------------------
 // The 5x5 Vanka system of cell (i,j): A = Jacobian of (N_u W, N_u E, N_v S,
 // N_v N, N_p) in (u_W, u_E, v_S, v_N, p), b = residuals N - f; rows and
-// columns of wall edges (act = false) replaced by the identity
+// columns of wall edges (act = false) replaced by the identity.  X: the cell's
+// densities on an error level (else unused)
 template <typename T, class Form, class LV>
 __device__ __forceinline__ void vanka_system(const Prm<T>& P, const LV& L, int i, int j,
-                                             T (&A)[5][5], T (&b)[5], bool (&act)[5]) {
+                                             const ErrCell<T>* X, T (&A)[5][5], T (&b)[5],
+                                             bool (&act)[5]) {
   const int W = L.pitch;
-  const T ih = L.ih, ih2 = L.ih2;
+  const T ih = L.ih;
   auto vis = L.visn;
   int k = L.at(i, j);
   int eW = (L.px && i == 1) ? L.m1 : i - 1;
@@ -762,72 +865,54 @@ __device__ __forceinline__ void vanka_system(const Prm<T>& P, const LV& L, int i
   for (int r = 0; r < 5; ++r)
 #pragma unroll
     for (int c = 0; c < 5; ++c) A[r][c] = T(0);
-  const T third = T(1.0 / 3.0);
-  // density sums on the four edges from rho(c) of the cell and its four
-  // neighbours (c at kW + 1 is c at k, exactly: ghosts are copies)
-  T Arq[4];
-  {
-    T rk = Form::rho(P, L, k);
-    Arq[0] = Form::rho(P, L, kW) + rk;
-    Arq[1] = rk + Form::rho(P, L, k + 1);
-    Arq[2] = Form::rho(P, L, k - W) + rk;
-    Arq[3] = rk + Form::rho(P, L, k + W);
-  }
-  // x-edge rows: q = 0 (west edge, index kW), q = 1 (east edge, index k)
+  // The rows W, E, S, N sit at these edges.  A periodic cell of column 1 has its
+  // west edge as unknown m1, at kW; edge 0 holds its copy, of the coefficients
+  // too, and at k - 1 the row shares its values with the other rows.  Only the
+  // right-hand side is kept on kW alone.
+  const int ke[4] = {k - 1, k, k - W, k};
+  const T f[4] = {L.fu[kW], L.fu[k], L.fv[k - W], L.fv[k]};
+  const T gt = (j == L.m2) ? T(2) : T(1), gb = (j == 1) ? T(2) : T(1);
+  const T ge = (!L.px && i == L.m1) ? T(2) : T(1), gw = (!L.px && i == 1) ? T(2) : T(1);
+  const T v3 = vis[k] * L.k.v3;
+  T rows[4];  // N of each row, evaluated on wall edges too (padded arrays), then discarded
+  if constexpr (std::is_same<Form, ErrForm>::value) {
+    const int nb[4] = {2, 1, 4, 3};  // the edge's other cell
 #pragma unroll
-  for (int q = 0; q < 2; ++q) {
-    int ke = q == 0 ? kW : k;
-    T Arn = L.Aru[ke];
-    T Ar = T(0.5) * Arq[q];
-    T gt = (j == L.m2) ? T(2) : T(1), gb = (j == 1) ? T(2) : T(1);
-    if constexpr (!std::is_same<Form, ErrForm>::value) {  // per-step coefficients
-      A[q][q] = L.Dgu[ke] + L.k.qidt * Arq[q];
-      continue;
+    for (int q = 0; q < 4; ++q) {
+      const T rs = X->r[0] + X->r[nb[q]], ds = X->dr[0] + X->dr[nb[q]];
+      A[q][q] = err_diag(L, q >> 1, ke[q], rs, q < 2 ? gt : ge, q < 2 ? gb : gw);
+      rows[q] = err_row(P, L, q >> 1, ke[q], rs, ds);
     }
-    A[q][q] = Arn * P.idt + T(0.5) * (Ar - Arn) * P.idt +
-              T(0.5) * ih * (-L.Sx[ke + 1] + L.Sx[ke] - L.Qx[ke] * gt + L.Qx[ke - W] * gb) +
-              L.Dvu[ke] +
-              P.iRe * ih2 * ((vis[ke + 1] + vis[ke]) * (T(1) + third) + gt * L.Av[ke] +
-                             gb * L.Av[ke - W]);
-  }
-  {
-    T v3 = vis[k] * L.k.v3, v1 = vis[k] * L.k.v1, sc = L.k.hih * L.Sx[k];
-    A[0][1] = sc - v1 - v3;
-    A[1][0] = -sc - v1 - v3;
-    A[0][2] = v3;
-    A[0][3] = -v3;
-    A[1][2] = -v3;
-    A[1][3] = v3;
-    A[0][4] = L.k.ihM;
-    A[1][4] = -L.k.ihM;
-  }
-  // y-edge rows: q = 2 (south edge, index k - W), q = 3 (north edge, index k)
+    // the coupling of a pair's edges is the stencil's entry for the other one
+    A[0][1] = L.aPu[ke[0]];
+    A[1][0] = L.aMu[ke[1]];
+    A[2][3] = L.aPv[ke[2]];
+    A[3][2] = L.aMv[ke[3]];
+  } else {
+    // density sums on the four edges
+    const T rk = Form::rho(P, L, k);
+    const T rs[4] = {Form::rho(P, L, k - 1) + rk, rk + Form::rho(P, L, k + 1),
+                     Form::rho(P, L, k - W) + rk, rk + Form::rho(P, L, k + W)};
+    constexpr bool PST = std::is_same<Form, FullForm>::value;
 #pragma unroll
-  for (int q = 2; q < 4; ++q) {
-    int ke = q == 2 ? k - W : k;
-    T Arn = L.Arv[ke];
-    T Ar = T(0.5) * Arq[q];
-    T ge = (!L.px && i == L.m1) ? T(2) : T(1), gw = (!L.px && i == 1) ? T(2) : T(1);
-    if constexpr (!std::is_same<Form, ErrForm>::value) {  // per-step coefficients
-      A[q][q] = L.Dgv[ke] + L.k.qidt * Arq[q];
-      continue;
+    for (int q = 0; q < 4; ++q) {
+      A[q][q] = (q < 2 ? L.Dgu : L.Dgv)[ke[q]] + L.k.qidt * rs[q];  // per-step coefficients
+      if (q < 2) rows[q] = op_u<T, PST>(P, L, ke[q], rs[q]);
+      else rows[q] = op_v<T, PST>(P, L, ke[q], rs[q]);
     }
-    A[q][q] = Arn * P.idt + T(0.5) * (Ar - Arn) * P.idt +
-              T(0.5) * ih * (-L.Qy[ke] * ge + L.Qy[ke - 1] * gw - L.Sy[ke + W] + L.Sy[ke]) +
-              L.Dvv[ke] +
-              P.iRe * ih2 * (ge * L.Av[ke] + gw * L.Av[ke - 1] +
-                             (vis[ke + W] + vis[ke]) * (T(1) + third));
+    const T v1 = vis[k] * L.k.v1, sx = L.k.hih * L.Sx[k], sy = L.k.hih * L.Sy[k];
+    A[0][1] = sx - v1 - v3;
+    A[1][0] = -sx - v1 - v3;
+    A[2][3] = sy - v1 - v3;
+    A[3][2] = -sy - v1 - v3;
   }
-  {
-    T v3 = vis[k] * L.k.v3, v1 = vis[k] * L.k.v1, sc = L.k.hih * L.Sy[k];
-    A[2][3] = sc - v1 - v3;
-    A[3][2] = -sc - v1 - v3;
-    A[2][0] = v3;
-    A[2][1] = -v3;
-    A[3][0] = -v3;
-    A[3][1] = v3;
-    A[2][4] = L.k.ihM;
-    A[3][4] = -L.k.ihM;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    b[q] = act[q] ? rows[q] - f[q] : T(0);
+    const int o = q < 2 ? 2 : 0;  // the couplings to the other direction's edges
+    A[q][o] = (q & 1) ? -v3 : v3;
+    A[q][o + 1] = (q & 1) ? v3 : -v3;
+    A[q][4] = (q & 1) ? -L.k.ihM : L.k.ihM;
   }
   {
     auto mob = L.mobn;
@@ -842,58 +927,6 @@ __device__ __forceinline__ void vanka_system(const Prm<T>& P, const LV& L, int i
     A[4][2] = -ih;
     A[4][3] = ih;
     A[4][4] = L.k.a2dif * sm;
-  }
-  if constexpr (std::is_same<Form, FullForm>::value) {
-    {
-      T nq = op_u(P, L, kW, Arq[0]);  // evaluated on wall edges too (padded arrays), then discarded
-      b[0] = act[0] ? nq - L.fu[kW] : T(0);
-    }
-    {
-      T nq = op_u(P, L, k, Arq[1]);  // evaluated on wall edges too (padded arrays), then discarded
-      b[1] = act[1] ? nq - L.fu[k] : T(0);
-    }
-    {
-      T nq = op_v(P, L, k - W, Arq[2]);  // evaluated on wall edges too (padded arrays), then discarded
-      b[2] = act[2] ? nq - L.fv[k - W] : T(0);
-    }
-    {
-      T nq = op_v(P, L, k, Arq[3]);  // evaluated on wall edges too (padded arrays), then discarded
-      b[3] = act[3] ? nq - L.fv[k] : T(0);
-    }
-  } else if constexpr (std::is_same<Form, ProjForm>::value) {
-    {
-      T nq = op_u<T, false>(P, L, kW, Arq[0]);  // evaluated on wall edges too (padded arrays), then discarded
-      b[0] = act[0] ? nq - L.fu[kW] : T(0);
-    }
-    {
-      T nq = op_u<T, false>(P, L, k, Arq[1]);  // evaluated on wall edges too (padded arrays), then discarded
-      b[1] = act[1] ? nq - L.fu[k] : T(0);
-    }
-    {
-      T nq = op_v<T, false>(P, L, k - W, Arq[2]);  // evaluated on wall edges too (padded arrays), then discarded
-      b[2] = act[2] ? nq - L.fv[k - W] : T(0);
-    }
-    {
-      T nq = op_v<T, false>(P, L, k, Arq[3]);  // evaluated on wall edges too (padded arrays), then discarded
-      b[3] = act[3] ? nq - L.fv[k] : T(0);
-    }
-  } else {
-    {
-      T nq = Form::Nu(P, L, kW);  // evaluated on wall edges too (padded arrays), then discarded
-      b[0] = act[0] ? nq - L.fu[kW] : T(0);
-    }
-    {
-      T nq = Form::Nu(P, L, k);  // evaluated on wall edges too (padded arrays), then discarded
-      b[1] = act[1] ? nq - L.fu[k] : T(0);
-    }
-    {
-      T nq = Form::Nv(P, L, k - W);  // evaluated on wall edges too (padded arrays), then discarded
-      b[2] = act[2] ? nq - L.fv[k - W] : T(0);
-    }
-    {
-      T nq = Form::Nv(P, L, k);  // evaluated on wall edges too (padded arrays), then discarded
-      b[3] = act[3] ? nq - L.fv[k] : T(0);
-    }
   }
   if constexpr (std::is_same<Form, ProjForm>::value) b[4] = T(0);  // the 4x4 block has no p row
   else b[4] = (L.u[k] - L.u[k - 1] + L.v[k] - L.v[k - W]) * ih - L.k.adif * flux_sum(P, L, k) - L.fp[k];
@@ -957,17 +990,21 @@ template <typename T, class Form, class LV>
 __device__ __forceinline__ void vanka_cell(const Prm<T>& P, const LV& L, int i, int j, T omega) {
   T A[5][5], b[5];
   bool act[5];
-  vanka_system<T, Form>(P, L, i, j, A, b, act);
+  ErrCell<T> X;
+  if constexpr (std::is_same<Form, ErrForm>::value) X = err_cell(P, L, L.at(i, j));
+  vanka_system<T, Form>(P, L, i, j, &X, A, b, act);
   const int W = L.pitch;
   int k = L.at(i, j);
   solve_vanka<T, 5>(A, b, act, L.visn[k] * L.k.v3, L.k.ihM, L.ih, L.k.ihaM);
   int eW = (L.px && i == 1) ? L.m1 : i - 1;
   int kW = L.at(eW, j);
-  if (act[0]) store_u(L, eW, j, L.u[kW] - omega * b[0]);
-  if (act[1]) store_u(L, i, j, L.u[k] - omega * b[1]);
-  if (act[2]) store_v(L, i, j - 1, L.v[k - W] - omega * b[2]);
-  if (act[3]) store_v(L, i, j, L.v[k] - omega * b[3]);
-  store_cell(L, L.p, i, j, L.p[k] - omega * b[4]);
+  // every old value is read before the first store: a load behind a store that
+  // may alias it waits its full latency, once per value
+  const bool ghosts = has_ghosts(L, i, j);
+  const T w = L.u[kW] - omega * b[0], e = L.u[k] - omega * b[1], so = L.v[k - W] - omega * b[2],
+          n = L.v[k] - omega * b[3], pn = L.p[k] - omega * b[4];
+  put_edges(L, i, j, ghosts, act, w, e, so, n);
+  put_cell(L, L.p, i, j, ghosts, pn);
 }
 
 // Exact solve of the coupled 7x7 system of coupled_cell by blocks.  Its NS part
@@ -1051,8 +1088,14 @@ template <typename T, class Form, class LV>
 __device__ __forceinline__ void coupled_cell(const Prm<T>& P, const LV& L, int i, int j, T omega) {
   T A5[5][5], b5[5], J2[2][2], R2[2];
   bool act[5];
-  vanka_system<T, Form>(P, L, i, j, A5, b5, act);
-  ch_system<T, Form>(P, L, i, j, J2, R2);
+  ErrCell<T> X;
+  if constexpr (std::is_same<Form, ErrForm>::value) {
+    X = err_cell(P, L, L.at(i, j));
+    ch_system_err(P, L, i, j, X, J2, R2);
+  } else {
+    ch_system<T, Form>(P, L, i, j, J2, R2);
+  }
+  vanka_system<T, Form>(P, L, i, j, &X, A5, b5, act);
   T A[7][7], b[7];
 #pragma unroll
   for (int r = 0; r < 7; ++r)
@@ -1081,7 +1124,7 @@ __device__ __forceinline__ void coupled_cell(const Prm<T>& P, const LV& L, int i
 #pragma unroll
   for (int f = 0; f < 4; ++f)
     if (!wall[f]) sm += mob[k] + mob[k + off[f]];
-  T rho = Form::rho(P, L, k), drho = -P.alpha * rho * rho;
+  const T rho = J2[1][1], drho = -P.alpha * rho * rho;  // d N_mu / d mu is rho(c)
   // rho^n D c^n / 2 at the four faces of the cell, as in (e1e2) and (e1e1)
   T gW = rn[k - 1] * L.Tx[k - 1];
   T gE = rn[k + 1] * L.Tx[k];
@@ -1094,7 +1137,7 @@ __device__ __forceinline__ void coupled_cell(const Prm<T>& P, const LV& L, int i
   A[0][5] = gN;
   A[0][6] = diffc;
   T half_idt = T(0.25) * drho * P.idt;  // d/dc of (A rho(c) - A rho^n) x / (2 dt), per edge
-  A[2][0] = half_idt * Form::val_u(L, kW);
+  A[2][0] = half_idt * Form::val_u(L, k - 1);
   A[3][0] = half_idt * Form::val_u(L, k);
   A[4][0] = half_idt * Form::val_v(L, k - W);
   A[5][0] = half_idt * Form::val_v(L, k);
@@ -1113,16 +1156,17 @@ __device__ __forceinline__ void coupled_cell(const Prm<T>& P, const LV& L, int i
       }
       A[2 + q][2 + q] = T(1);
     }
-  solve_coupled7(A, b, act, L.visn[k] * L.k.v3, L.k.ihM, L.ih, L.k.ihaM);
-  T cnew = L.c[k] - omega * b[0];
-  store_cell(L, L.c, i, j, cnew);
-  if constexpr (!std::is_same<Form, ErrForm>::value) store_cell(L, L.rhoc, i, j, rho_of(P, cnew));
-  store_cell(L, L.mu, i, j, L.mu[k] - omega * b[1]);
-  if (act[0]) store_u(L, eW, j, L.u[kW] - omega * b[2]);
-  if (act[1]) store_u(L, i, j, L.u[k] - omega * b[3]);
-  if (act[2]) store_v(L, i, j - 1, L.v[k - W] - omega * b[4]);
-  if (act[3]) store_v(L, i, j, L.v[k] - omega * b[5]);
-  store_cell(L, L.p, i, j, L.p[k] - omega * b[6]);
+  solve_coupled7<T>(A, b, act, L.visn[k] * L.k.v3, L.k.ihM, L.ih, L.k.ihaM);
+  const bool ghosts = has_ghosts(L, i, j);  // (old values first, as in vanka_cell)
+  const T cnew = L.c[k] - omega * b[0], mnew = L.mu[k] - omega * b[1];
+  const T w = L.u[kW] - omega * b[2], e = L.u[k] - omega * b[3], so = L.v[k - W] - omega * b[4],
+          n = L.v[k] - omega * b[5], pn = L.p[k] - omega * b[6];
+  put_cell(L, L.c, i, j, ghosts, cnew);
+  if constexpr (!std::is_same<Form, ErrForm>::value)
+    put_cell(L, L.rhoc, i, j, ghosts, rho_of(P, cnew));
+  put_cell(L, L.mu, i, j, ghosts, mnew);
+  put_edges(L, i, j, ghosts, act, w, e, so, n);
+  put_cell(L, L.p, i, j, ghosts, pn);
 }
 
 // Vanka colour of cell (i,j): (2i + j) mod 8 (periodic x, m1 = 0 mod 4) or
@@ -1131,60 +1175,6 @@ template <class LV>
 __device__ __forceinline__ int vanka_colour(const LV& L, int i, int j) {
   typedef typename LV::real T;
   return L.c8 ? (2 * i + j) & 7 : (i + 2 * j) % L.kcol;
-}
-
-// first cell i0 >= 1 of colour `colour` in row j and the stride between cells
-// of that colour in the row; false if the row has none
-template <class LV>
-__device__ __forceinline__ bool colour_row(const LV& L, int colour, int j, int& i0, int& stride) {
-  typedef typename LV::real T;
-  if (L.c8) {
-    int d = (colour - j) & 7;
-    if (d & 1) return false;
-    i0 = d >> 1;
-    if (i0 == 0) i0 = 4;
-    stride = 4;
-  } else {
-    int K = L.kcol;
-    i0 = ((colour - 2 * j) % K + K) % K;
-    if (i0 == 0) i0 = K;
-    stride = K;
-  }
-  return true;
-}
-
-// slots of Vanka colour `col`: slot t -> row j0 + rstep * (t / mpr), t % mpr-th
-// cell of that row's colour
-struct ColourSlots {
-  int j0, rstep, mpr, n;
-};
-
-template <class LV>
-__host__ __device__ __forceinline__ ColourSlots vanka_slots(const LV& L, int col) {
-  typedef typename LV::real T;
-  ColourSlots cs;
-  if (L.c8) {
-    cs.j0 = ((col - 1) & 1) ? 2 : 1;  // rows with (col - j) even
-    cs.rstep = 2;
-    cs.mpr = (L.m1 + 3) / 4;
-  } else {
-    cs.j0 = 1;
-    cs.rstep = 1;
-    cs.mpr = (L.m1 + L.kcol - 1) / L.kcol;
-  }
-  cs.n = cs.j0 > L.m2 ? 0 : ((L.m2 - cs.j0) / cs.rstep + 1) * cs.mpr;
-  return cs;
-}
-
-template <class LV>
-__device__ __forceinline__ bool vanka_slot_cell(const LV& L, int col, const ColourSlots& cs, int t,
-                                                int& i, int& j) {
-  typedef typename LV::real T;
-  j = cs.j0 + cs.rstep * (t / cs.mpr);
-  int i0, stride;
-  if (!colour_row(L, col, j, i0, stride)) return false;
-  i = i0 + stride * (t % cs.mpr);
-  return i <= L.m1;
 }
 
 // per-level smoother launches: one thread per cell of the colour, packed into
@@ -1222,17 +1212,17 @@ template <typename T, class Form, class LV>
 __device__ __forceinline__ void vanka4_cell(const Prm<T>& P, const LV& L, int i, int j, T omega) {
   T A5[5][5], b5[5];
   bool act[5];
-  vanka_system<T, Form>(P, L, i, j, A5, b5, act);
+  vanka_system<T, Form>(P, L, i, j, (const ErrCell<T>*)nullptr, A5, b5, act);
   const int W = L.pitch;
   int k = L.at(i, j);
   solve_vanka<T, 4>(A5, b5, act, L.visn[k] * L.k.v3, L.k.ihM, L.ih, L.k.ihaM);
   const T(&b)[5] = b5;
   int eW = (L.px && i == 1) ? L.m1 : i - 1;
   int kW = L.at(eW, j);
-  if (act[0]) store_u(L, eW, j, L.u[kW] - omega * b[0]);
-  if (act[1]) store_u(L, i, j, L.u[k] - omega * b[1]);
-  if (act[2]) store_v(L, i, j - 1, L.v[k - W] - omega * b[2]);
-  if (act[3]) store_v(L, i, j, L.v[k] - omega * b[3]);
+  const bool ghosts = has_ghosts(L, i, j);
+  const T w = L.u[kW] - omega * b[0], e = L.u[k] - omega * b[1], so = L.v[k - W] - omega * b[2],
+          n = L.v[k] - omega * b[3];
+  put_edges(L, i, j, ghosts, act, w, e, so, n);
 }
 
 template <typename T, class Form>
@@ -1295,18 +1285,11 @@ __device__ __forceinline__ void pgs_team(const Prm<T>& P, const LV& L, int i, in
 template <typename T>
 __global__ void __launch_bounds__(64) k_pgs_team(Prm<T> P, Lv<T> L, int colour) {
   pdl_enter();
-  int mpr = (L.m1 + 1) / 2;
-  int n = mpr * L.m2;
+  int n = L.crow.d * L.m2;
   int t = blockIdx.x * 64 + threadIdx.x;
   if ((t & ~31) >= 4 * n) return;  // warp-uniform
-  int s = t >> 2;
-  int j = 1, i = 1;
-  bool ok = false;
-  if (s < n) {
-    j = s / mpr + 1;
-    i = (((colour - j) & 1) ? 1 : 2) + 2 * (s % mpr);
-    ok = i <= L.m1;
-  }
+  int i = 1, j = 1;
+  bool ok = (t >> 2) < n && ch_slot_cell(L, colour, t >> 2, i, j);
   if (!ok) i = j = 1;
   pgs_team<T>(P, L, i, j, ok);
 }
@@ -1315,12 +1298,8 @@ __global__ void __launch_bounds__(64) k_pgs_team(Prm<T> P, Lv<T> L, int colour) 
 template <typename T>
 __global__ void __launch_bounds__(64) k_pgs(Prm<T> P, Lv<T> L, int colour) {
   pdl_enter();
-  int mpr = (L.m1 + 1) / 2;
-  int t = blockIdx.x * 64 + threadIdx.x;
-  if (t >= mpr * L.m2) return;
-  int j = t / mpr + 1;
-  int i = (((colour - j) & 1) ? 1 : 2) + 2 * (t % mpr);
-  if (i > L.m1) return;
+  int t = blockIdx.x * 64 + threadIdx.x, i, j;
+  if (t >= L.crow.d * L.m2 || !ch_slot_cell(L, colour, t, i, j)) return;
   pgs_cell<T>(P, L, i, j);
 }
 
@@ -1369,15 +1348,15 @@ __device__ __forceinline__ int xsrc_cell(int I, int m1, int px) {
 __device__ __forceinline__ bool frame_pos(int t, int m1, int m2, int& I, int& J) {
   int NX = m1 + 3, NY = m2 + 3;
   if (t < 4 * NX) {
-    int r = t / NX;
-    I = t % NX - 1;
+    int r = (t >= NX) + (t >= 2 * NX) + (t >= 3 * NX);
+    I = t - r * NX - 1;
     J = r < 2 ? r - 1 : m2 + r - 2;  // rows -1, 0, m2, m2+1
     return true;
   }
   t -= 4 * NX;
   if (t < 4 * NY) {
-    int cidx = t / NY;
-    J = t % NY - 1;
+    int cidx = (t >= NY) + (t >= 2 * NY) + (t >= 3 * NY);
+    J = t - cidx * NY - 1;
     I = cidx < 2 ? cidx - 1 : m1 + cidx - 2;  // columns -1, 0, m1, m1+1
     return true;
   }
@@ -1774,13 +1753,15 @@ __global__ void k_prolong(Prm<T> P, Lv<T> F, Lv<T> C) {
 // kernels above, in the same colour order, so the results are the same.
 // --------------------------------------------------------------------------
 // coarse base X_H = R X_h (cells: 4-mean; edges: 2 coincident fine edges), one entry
-template <class LV>
-__device__ __forceinline__ void restrict_base_cell(const LV& F, const LV& C, int I, int J) {
-  typedef typename LV::real T;
+template <typename T, class LV>
+__device__ __forceinline__ void restrict_base_cell(const Prm<T>& P, const LV& F, const LV& C, int I,
+                                                   int J) {
   int kc = C.at(I, J);
   if (I >= 1 && J >= 1) {
     int kf = F.at(2 * I - 1, 2 * J - 1), W = F.pitch;
-    C.Bc[kc] = T(0.25) * (F.Bc[kf] + F.Bc[kf + 1] + F.Bc[kf + W] + F.Bc[kf + W + 1]);
+    const T B = T(0.25) * (F.Bc[kf] + F.Bc[kf + 1] + F.Bc[kf + W] + F.Bc[kf + W + 1]);
+    C.Bc[kc] = B;
+    C.rB[kc] = rho_of(P, B);
     C.Bmu[kc] = T(0.25) * (F.Bmu[kf] + F.Bmu[kf + 1] + F.Bmu[kf + W] + F.Bmu[kf + W + 1]);
     C.Bdc[kc] = T(0.25) * (F.Bdc[kf] + F.Bdc[kf + 1] + F.Bdc[kf + W] + F.Bdc[kf + W + 1]);
   }
@@ -1799,6 +1780,7 @@ template <class LV>
 __device__ __forceinline__ void bc_base_cell(const LV& L, int I, int J) {
   typedef typename LV::real T;
   fill_cell_ghost(L, L.Bc, I, J);
+  fill_cell_ghost(L, L.rB, I, J);
   fill_cell_ghost(L, L.Bmu, I, J);
   fill_cell_ghost(L, L.Bdc, I, J);
   fill_u_ghost(L, L.Bu, I, J);
@@ -1863,82 +1845,71 @@ __device__ __forceinline__ void bc_unknowns_block(const LV& L) {
 // --------------------------------------------------------------------------
 // N - f of the momentum row in direction d (0: the x row, op_u, unknown u; 1:
 // the y row, op_v, unknown v; opd_u / opd_v for ErrForm) at edge index k, from
-// rho(c) of the edge's two cells.  Both directions run the same instructions
-// on different arrays and strides (s along the edge normal, t across it).
-// FullForm uses the per-step row coefficients; ErrForm (the error equation of
-// the defect correction) has none of them and adds the base-state term of the
-// time derivative.
+// rho(c) of the edge's two cells; kf is the index of its right-hand side.  Both
+// directions run the same instructions on different arrays and strides (s
+// along the edge normal, t across it).
 template <typename T, class Form, class LV>
-__device__ __forceinline__ T mom_residual(const Prm<T>& P, const LV& L, int d, int k,
+__device__ __forceinline__ T mom_residual(const Prm<T>& P, const LV& L, int d, int k, int kf,
                                           RhoPair<T> l, RhoPair<T> r) {
-  const T f = L.pair(d, L.fu, L.fv)[k];
-  // FP64 primitive rows: the per-step assembled stencil
+  const T f = L.pair(d, L.fu, L.fv)[kf];
   if constexpr (std::is_same<Form, FullForm>::value && sizeof(T) == 8) {
     return mom_asm(L, d, k, l.r + r.r) - f;
-  } else {
-    T Ar = T(0.5) * (l.r + r.r);
+  } else if constexpr (std::is_same<Form, ErrForm>::value) {
+    return err_row(P, L, d, k, l.r + r.r, l.d + r.d) - f;
+  } else {  // the projection method's intermediate-velocity row
     const int s = d ? L.pitch : 1, t = d ? 1 : L.pitch;
     auto a = L.pair(d, L.u, L.v);
     auto b = L.pair(1 - d, L.u, L.v);
     auto S = L.pair(d, L.Sx, L.Sy);
     auto Q = L.pair(d, L.Qx, L.Qy);
     auto vis = L.visn;
-    auto rn = L.rhon;
     T ae = a[k];
     T dl = (ae - a[k - s]) * L.ih, dr = (a[k + s] - ae) * L.ih;
     T dvl = dl + (b[k] - b[k - t]) * L.ih;
     T dvr = dr + (b[k + s] - b[k + s - t]) * L.ih;
     T Dp = (a[k + t] - ae) * L.ih, Dm = (ae - a[k - t]) * L.ih;
     T conv = T(0.5) * (S[k + s] * dr + S[k] * dl + Q[k] * Dp + Q[k - t] * Dm);
-    T time;
-    if constexpr (std::is_same<Form, ErrForm>::value) {
-      // rho(X + e) - rho(X) of the two cells by the secant of rho, times the base velocity
-      T dAr = T(0.5) * (rsec_(P, l.r, l.b) * L.c[k] + rsec_(P, r.r, r.b) * L.c[k + s]);
-      T Arn = L.pair(d, L.Aru, L.Arv)[k];
-      time = Arn * ae * P.idt + T(0.5) * (Ar - Arn) * P.idt * ae +
-             T(0.5) * dAr * P.idt * L.pair(d, L.Bu, L.Bv)[k] + L.pair(d, L.Dvu, L.Dvv)[k] * ae;
-    } else {
-      time = ae * (L.pair(d, L.T1u, L.T1v)[k] + L.k.qidt * (l.r + r.r)) +
+    T time = ae * (L.pair(d, L.T1u, L.T1v)[k] + L.k.qidt * (l.r + r.r)) +
              L.pair(d, L.T0u, L.T0v)[k];
-    }
-    T press = T(0), st = T(0);  // the projection method's intermediate-velocity row has neither
-    if constexpr (!std::is_same<Form, ProjForm>::value) {
-      press = (L.p[k + s] - L.p[k]) * L.k.ihM;
-      st = -(rn[k + s] * L.mu[k] + rn[k] * L.mu[k + s]) * L.pair(d, L.Tx, L.Ty)[k] * P.iM;
-    }
     T vl = vis[k], vr = vis[k + s];
     T visc = -P.iRe * L.ih * ((vr * dr - vl * dl) + (L.Av[k] * Dp - L.Av[k - t] * Dm) +
                               (vr * dvr - vl * dvl) * T(1.0 / 3.0));
-    return time + conv + press + st + visc - f;
+    return time + conv + visc - f;
   }
 }
 
 // Diagonal entry dq and residual bq = N - f (0 on a wall edge) of momentum row
 // q of the Vanka block of cell (i,j), for lane q of a team: direction d (0:
-// x-edge, 1: y-edge), edge index ke, rho(c) of the edge's cells l and r.
+// x-edge, 1: y-edge), edge index ke of the row (its copy at column 0 for a
+// periodic west edge) and kf of its right-hand side, rho(c) of the edge's
+// cells l and r.
 template <typename T, class Form, class LV>
 __device__ __forceinline__ void team_row(const Prm<T>& P, const LV& L, int i, int j, int d, int ke,
-                                         RhoPair<T> l, RhoPair<T> r, bool mine, T& dq, T& bq) {
+                                         int kf, RhoPair<T> l, RhoPair<T> r, bool mine, T& dq,
+                                         T& bq) {
   if constexpr (std::is_same<Form, ErrForm>::value) {
-    const T ih = L.ih, ih2 = L.ih2, third = T(1.0 / 3.0);
-    const int s = d ? L.pitch : 1, t = d ? 1 : L.pitch;
-    auto vis = L.visn;
-    auto S = L.pair(d, L.Sx, L.Sy);
-    auto Q = L.pair(d, L.Qx, L.Qy);
-    T Ar = T(0.5) * (l.r + r.r);
-    // the diagonal from the frozen arrays (error levels carry no row coefficients)
     T gp = d ? ((!L.px && i == L.m1) ? T(2) : T(1)) : ((j == L.m2) ? T(2) : T(1));
     T gm = d ? ((!L.px && i == 1) ? T(2) : T(1)) : ((j == 1) ? T(2) : T(1));
-    T Arn = L.pair(d, L.Aru, L.Arv)[ke];
-    dq = Arn * P.idt + T(0.5) * (Ar - Arn) * P.idt +
-         T(0.5) * ih * (-S[ke + s] + S[ke] - Q[ke] * gp + Q[ke - t] * gm) +
-         L.pair(d, L.Dvu, L.Dvv)[ke] +
-         P.iRe * ih2 * ((vis[ke + s] + vis[ke]) * (T(1) + third) + gp * L.Av[ke] + gm * L.Av[ke - t]);
+    dq = err_diag(L, d, ke, l.r + r.r, gp, gm);
   } else {
     dq = L.pair(d, L.Dgu, L.Dgv)[ke] + L.k.qidt * (l.r + r.r);
   }
-  bq = mom_residual<T, Form>(P, L, d, ke, l, r);  // wall edges too (padded arrays), then discarded
+  bq = mom_residual<T, Form>(P, L, d, ke, kf, l, r);  // wall edges too (padded arrays), then discarded
   if (!mine) bq = T(0);
+}
+// the couplings b01, b10 of the two edges of direction d of cell k within B
+// (the block without its v3 part): (first row, second edge) and the converse
+template <typename T, class Form, class LV>
+__device__ __forceinline__ void pair_couplings(const LV& L, int d, int k, T vc, T& b01, T& b10) {
+  if constexpr (std::is_same<Form, ErrForm>::value) {
+    const T v3 = vc * L.k.v3;
+    b01 = L.pair(d, L.aPu, L.aPv)[k - (d ? L.pitch : 1)] + v3;
+    b10 = L.pair(d, L.aMu, L.aMv)[k] + v3;
+  } else {
+    const T v1 = vc * L.k.v1, sc = L.k.hih * L.pair(d, L.Sx, L.Sy)[k];
+    b01 = sc - v1;
+    b10 = -sc - v1;
+  }
 }
 
 // The structured solve of solve_vanka, split over a team of four lanes.  The
@@ -1956,37 +1927,36 @@ struct TeamSolve {
   // with_p = false: the 4x4 velocity block alone (the projection method's
   // intermediate-velocity block), solved as solve_vanka<T, 4> does
   template <class LV>
-  __device__ __forceinline__ TeamSolve(const Prm<T>& P, const LV& L, int q, T dq, bool ap0, bool ap1,
-                                       T S, T vc, T A44, bool with_p = true) {
+  __device__ __forceinline__ TeamSolve(const LV& L, int q, T dq, bool ap0, bool ap1, T b01, T b10,
+                                       T vc, T A44, bool with_p = true) {
     const unsigned FULL = 0xffffffffu;
     ih = L.ih;
     v3 = vc * L.k.v3;
     odd = q & 1;
-    T dqo = __shfl_xor_sync(FULL, dq, 1);
+    T dqo = shfl_xor(dq, 1);
     T D0 = odd ? dqo : dq, D1 = odd ? dq : dqo;
     B00 = ap0 ? D0 - v3 : T(1);
     B11 = ap1 ? D1 - v3 : T(1);
-    const T v1 = vc * L.k.v1, sc = L.k.hih * S;
-    B01 = (ap0 && ap1) ? sc - v1 : T(0);
-    B10 = (ap0 && ap1) ? -sc - v1 : T(0);
+    B01 = (ap0 && ap1) ? b01 : T(0);
+    B10 = (ap0 && ap1) ? b10 : T(0);
     idet = qrcp(B00 * B11 - B01 * B10);
     T zn = odd ? ((ap1 ? B00 : T(0)) + (ap0 ? B10 : T(0))) : ((ap0 ? B11 : T(0)) + (ap1 ? B01 : T(0)));
     z = (odd ? -zn : zn) * idet;
     T sdot = odd ? -z : z;
-    sdot += __shfl_xor_sync(FULL, sdot, 1);
-    sdot += __shfl_xor_sync(FULL, sdot, 2);
+    sdot += shfl_xor(sdot, 1);
+    sdot += shfl_xor(sdot, 2);
     g = qrcp(T(1) + v3 * sdot);
     iden = with_p ? qrcp(A44 + L.k.ihaM * (sdot * g)) : T(0);
     ga = with_p ? g * L.k.ihM : T(0);
   }
   __device__ __forceinline__ T apply(T rq, T r4, T& pr) const {
     const unsigned FULL = 0xffffffffu;
-    T rqo = __shfl_xor_sync(FULL, rq, 1);
+    T rqo = shfl_xor(rq, 1);
     T r0 = odd ? rqo : rq, r1 = odd ? rq : rqo;
     T y = ((odd ? B00 : B11) * (odd ? r1 : r0) - (odd ? B10 : B01) * (odd ? r0 : r1)) * idet;
     T tdot = odd ? -y : y;
-    tdot += __shfl_xor_sync(FULL, tdot, 1);
-    tdot += __shfl_xor_sync(FULL, tdot, 2);
+    tdot += shfl_xor(tdot, 1);
+    tdot += shfl_xor(tdot, 2);
     const T tg = tdot * g;
     pr = (r4 + ih * tg) * iden;
     return y - z * (v3 * tg + ga * pr);
@@ -2016,7 +1986,7 @@ __device__ __forceinline__ void vanka_team(const Prm<T>& P, const LV& L, int i, 
   const RhoPair<T> ra = rho_pair<T, Form>(P, L, k), rb = rho_pair<T, Form>(P, L, nq);
   const int kf = (q & 1) ? k : nq;  // the face's own edge (kW's copy for a periodic west face)
   T dq, bq;
-  team_row<T, Form>(P, L, i, j, d, ke, (q & 1) ? ra : rb, (q & 1) ? rb : ra, mine, dq, bq);
+  team_row<T, Form>(P, L, i, j, d, kf, ke, (q & 1) ? ra : rb, (q & 1) ? rb : ra, mine, dq, bq);
   // the mass row by faces: lane q takes face q (W, E, S, N) of the cell, the
   // face of its own edge: its velocity in d.u, its flux of
   // grad.(A m grad(mu + alpha p)) and, if open, its share of sum A m
@@ -2027,17 +1997,17 @@ __device__ __forceinline__ void vanka_team(const Prm<T>& P, const LV& L, int i, 
   T f2 = team_sum<T>(mine ? am : T(0));
   T A44 = L.k.a2dif * f2;
   T b4 = f0 * ih - L.k.adif * f1 - L.fp[k];
-  TeamSolve<T> ts(P, L, q, dq, d ? a2 : a0, d ? a3 : a1, L.pair(d, L.Sx, L.Sy)[k], L.visn[k], A44);
+  const T vc = L.visn[k];
+  T b01, b10;
+  pair_couplings<T, Form>(L, d, k, vc, b01, b10);
+  TeamSolve<T> ts(L, q, dq, d ? a2 : a0, d ? a3 : a1, b01, b10, vc, A44);
   T pr;
   T x = ts.apply(bq, b4, pr);
   if (!ok) return;
-  if (mine) {
-    if (q == 0) store_u(L, eW, j, L.u[kW] - omega * x);
-    else if (q == 1) store_u(L, i, j, L.u[k] - omega * x);
-    else if (q == 2) store_v(L, i, j - 1, L.v[k - W] - omega * x);
-    else store_v(L, i, j, L.v[k] - omega * x);
-  }
-  if (q == 0) store_cell(L, L.p, i, j, L.p[k] - omega * pr);
+  const bool ghosts = has_ghosts(L, i, j);
+  const T xn = L.pair(d, L.u, L.v)[ke] - omega * x, pn = L.p[k] - omega * pr;
+  if (mine) put_edge(L, i, j, q, ghosts, xn);
+  if (q == 0) put_cell(L, L.p, i, j, ghosts, pn);
 }
 
 // One half of mom_residual for a lane pair of an eight-lane team: half 0 the
@@ -2094,7 +2064,7 @@ __device__ __forceinline__ void vanka_team8(const Prm<T>& P, const LV& L, int i,
   T rl = L.rhoc[ke], rr = L.rhoc[ke + (d ? W : 1)];
   T dq = L.pair(d, L.Dgu, L.Dgv)[ke] + L.k.qidt * (rl + rr);
   T bq = mom_residual_half<T>(P, L, d, ke, rl, rr, half);
-  bq += __shfl_xor_sync(0xffffffffu, bq, 4);
+  bq += shfl_xor(bq, 4);
   if (!mine) bq = T(0);
   auto mob = L.mobn;
   const int nq = k + (q == 0 ? -1 : q == 1 ? 1 : q == 2 ? -W : W);
@@ -2104,17 +2074,17 @@ __device__ __forceinline__ void vanka_team8(const Prm<T>& P, const LV& L, int i,
   T f2 = team_sum<T>(mine ? am : T(0));
   T A44 = L.k.a2dif * f2;
   T b4 = f0 * ih - L.k.adif * f1 - L.fp[k];
-  TeamSolve<T> ts(P, L, q, dq, d ? a2 : a0, d ? a3 : a1, d ? L.Sy[k] : L.Sx[k], L.visn[k], A44);
+  const T vc = L.visn[k];
+  T b01, b10;
+  pair_couplings<T, FullForm>(L, d, k, vc, b01, b10);
+  TeamSolve<T> ts(L, q, dq, d ? a2 : a0, d ? a3 : a1, b01, b10, vc, A44);
   T pr;
   T x = ts.apply(bq, b4, pr);
   if (!ok || half) return;
-  if (mine) {
-    if (q == 0) store_u(L, eW, j, L.u[kW] - omega * x);
-    else if (q == 1) store_u(L, i, j, L.u[k] - omega * x);
-    else if (q == 2) store_v(L, i, j - 1, L.v[k - W] - omega * x);
-    else store_v(L, i, j, L.v[k] - omega * x);
-  }
-  if (q == 0) store_cell(L, L.p, i, j, L.p[k] - omega * pr);
+  const bool ghosts = has_ghosts(L, i, j);
+  const T xn = L.pair(d, L.u, L.v)[ke] - omega * x, pn = L.p[k] - omega * pr;
+  if (mine) put_edge(L, i, j, q, ghosts, xn);
+  if (q == 0) put_cell(L, L.p, i, j, ghosts, pn);
 }
 
 // The projection method's 4x4 intermediate-velocity block (vanka4_cell) by a
@@ -2135,16 +2105,17 @@ __device__ __forceinline__ void vanka4_team(const Prm<T>& P, const LV& L, int i,
   // the neighbour across the edge's face; a periodic ghost holds the cell's copy
   const int nq = k + (q == 0 ? -1 : q == 1 ? 1 : q == 2 ? -W : W);
   const RhoPair<T> ra = rho_pair<T, ProjForm>(P, L, k), rb = rho_pair<T, ProjForm>(P, L, nq);
+  const int kf = (q & 1) ? k : nq;  // the face's own edge (kW's copy for a periodic west face)
   T dq, bq;
-  team_row<T, ProjForm>(P, L, i, j, d, ke, (q & 1) ? ra : rb, (q & 1) ? rb : ra, mine, dq, bq);
-  TeamSolve<T> ts(P, L, q, dq, d ? a2 : a0, d ? a3 : a1, L.pair(d, L.Sx, L.Sy)[k], L.visn[k], T(0), false);
+  team_row<T, ProjForm>(P, L, i, j, d, kf, ke, (q & 1) ? ra : rb, (q & 1) ? rb : ra, mine, dq, bq);
+  const T vc = L.visn[k];
+  T b01, b10;
+  pair_couplings<T, ProjForm>(L, d, k, vc, b01, b10);
+  TeamSolve<T> ts(L, q, dq, d ? a2 : a0, d ? a3 : a1, b01, b10, vc, T(0), false);
   T pr;
   T x = ts.apply(bq, T(0), pr);
   if (!ok || !mine) return;
-  if (q == 0) store_u(L, eW, j, L.u[kW] - omega * x);
-  else if (q == 1) store_u(L, i, j, L.u[k] - omega * x);
-  else if (q == 2) store_v(L, i, j - 1, L.v[k - W] - omega * x);
-  else store_v(L, i, j, L.v[k] - omega * x);
+  put_edge(L, i, j, q, has_ghosts(L, i, j), L.pair(d, L.u, L.v)[ke] - omega * x);
 }
 
 // Coupled 7x7 block of coupled_cell by a team of four lanes (lane & 3 = q:
@@ -2171,7 +2142,7 @@ __device__ __forceinline__ void coupled_team(const Prm<T>& P, const LV& L, int i
   const RhoPair<T> ra = rho_pair<T, Form>(P, L, k), rb = rho_pair<T, Form>(P, L, nq);
   const int kf = (q & 1) ? k : nq;  // the face's own edge (kW's copy for a periodic west face)
   T dq, bq;
-  team_row<T, Form>(P, L, i, j, d, ke, (q & 1) ? ra : rb, (q & 1) ? rb : ra, mine, dq, bq);
+  team_row<T, Form>(P, L, i, j, d, kf, ke, (q & 1) ? ra : rb, (q & 1) ? rb : ra, mine, dq, bq);
   ChRows<T> C = ch_team_rows<T, Form>(P, L, i, j, q, mine, ra, rb);
   T sdiv = team_sum<T>((q & 1) ? L.pair(d, L.u, L.v)[kf] : -L.pair(d, L.u, L.v)[kf]);
   T sm = C.sm, sflux = C.sflux, gq = C.gq;
@@ -2184,7 +2155,10 @@ __device__ __forceinline__ void coupled_team(const Prm<T>& P, const LV& L, int i
   T gm = mine ? gq : T(0);
   T cq0 = mine ? T(0.25) * C.drho * P.idt * (d ? Form::val_v(L, ke) : Form::val_u(L, ke)) : T(0);
   T cq1 = mine ? -gq * P.iM : T(0);
-  TeamSolve<T> ts(P, L, q, dq, d ? a2 : a0, d ? a3 : a1, L.pair(d, L.Sx, L.Sy)[k], L.visn[k], A44);
+  const T vc = L.visn[k];
+  T b01, b10;
+  pair_couplings<T, Form>(L, d, k, vc, b01, b10);
+  TeamSolve<T> ts(L, q, dq, d ? a2 : a0, d ? a3 : a1, b01, b10, vc, A44);
   T p0, p1, p2;
   T x0 = ts.apply(bq, b4, p0);
   T x1 = ts.apply(cq0, T(0), p1);
@@ -2198,18 +2172,16 @@ __device__ __forceinline__ void coupled_team(const Prm<T>& P, const LV& L, int i
   T x = x0 - x1 * dc - x2 * dm;
   T pr = p0 - p1 * dc - p2 * dm;
   if (!ok) return;
-  if (mine) {
-    if (q == 0) store_u(L, eW, j, L.u[kW] - omega * x);
-    else if (q == 1) store_u(L, i, j, L.u[k] - omega * x);
-    else if (q == 2) store_v(L, i, j - 1, L.v[k - W] - omega * x);
-    else store_v(L, i, j, L.v[k] - omega * x);
-  }
+  const bool ghosts = has_ghosts(L, i, j);
+  const T xn = L.pair(d, L.u, L.v)[ke] - omega * x, pn = L.p[k] - omega * pr;
+  const T cnew = L.c[k] - omega * dc, mnew = L.mu[k] - omega * dm;
+  if (mine) put_edge(L, i, j, q, ghosts, xn);
   if (q == 0) {
-    T cnew = L.c[k] - omega * dc;
-    store_cell(L, L.c, i, j, cnew);
-    if constexpr (!std::is_same<Form, ErrForm>::value) store_cell(L, L.rhoc, i, j, rho_of(P, cnew));
-    store_cell(L, L.mu, i, j, L.mu[k] - omega * dm);
-    store_cell(L, L.p, i, j, L.p[k] - omega * pr);
+    put_cell(L, L.c, i, j, ghosts, cnew);
+    if constexpr (!std::is_same<Form, ErrForm>::value)
+      put_cell(L, L.rhoc, i, j, ghosts, rho_of(P, cnew));
+    put_cell(L, L.mu, i, j, ghosts, mnew);
+    put_cell(L, L.p, i, j, ghosts, pn);
   }
 }
 
@@ -2298,8 +2270,8 @@ __device__ __forceinline__ void vanka_pair(const Prm<T>& P, const LV& L, int i, 
     const int o = d ? W : 1;
     const RhoPair<T> rl = rho_pair<T, Form>(P, L, k - o), rk = rho_pair<T, Form>(P, L, k),
                      rr = rho_pair<T, Form>(P, L, k + o);
-    team_row<T, Form>(P, L, i, j, d, ke0, rl, rk, ap0, dq0, bq0);
-    team_row<T, Form>(P, L, i, j, d, k, rk, rr, ap1, dq1, bq1);
+    team_row<T, Form>(P, L, i, j, d, k - o, ke0, rl, rk, ap0, dq0, bq0);
+    team_row<T, Form>(P, L, i, j, d, k, k, rk, rr, ap1, dq1, bq1);
   }
   // the mass row by faces (as vanka_team): faces W, E on lane 0, S, N on lane 1
   auto mob = L.mobn;
@@ -2310,9 +2282,9 @@ __device__ __forceinline__ void vanka_pair(const Prm<T>& P, const LV& L, int i, 
   T fs1 = am0 * ((L.mu[n0] - L.mu[k]) + P.alpha * (L.p[n0] - L.p[k])) +
           am1 * ((L.mu[n1] - L.mu[k]) + P.alpha * (L.p[n1] - L.p[k]));
   T fs2 = (ap0 ? am0 : T(0)) + (ap1 ? am1 : T(0));
-  fs0 += __shfl_xor_sync(FULL, fs0, 1);
-  fs1 += __shfl_xor_sync(FULL, fs1, 1);
-  fs2 += __shfl_xor_sync(FULL, fs2, 1);
+  fs0 += shfl_xor(fs0, 1);
+  fs1 += shfl_xor(fs1, 1);
+  fs2 += shfl_xor(fs2, 1);
   T A44 = L.k.a2dif * fs2;
   T b4 = fs0 * ih - L.k.adif * fs1 - L.fp[k];
   // this pair's block B = A_vv - v3 w w^T (TeamSolve, both rows on one lane)
@@ -2327,13 +2299,13 @@ __device__ __forceinline__ void vanka_pair(const Prm<T>& P, const LV& L, int i, 
   T z0 = ((ap0 ? B11 : T(0)) + (ap1 ? B01 : T(0))) * idet;
   T z1 = -((ap1 ? B00 : T(0)) + (ap0 ? B10 : T(0))) * idet;
   T sdot = z0 + -z1;
-  sdot += __shfl_xor_sync(FULL, sdot, 1);
+  sdot += shfl_xor(sdot, 1);
   T g = qrcp(T(1) + v3 * sdot);
   T iden = qrcp(A44 + L.k.ihaM * (sdot * g));
   T y0 = (B11 * bq0 - B01 * bq1) * idet;
   T y1 = (B00 * bq1 - B10 * bq0) * idet;
   T tdot = y0 + -y1;
-  tdot += __shfl_xor_sync(FULL, tdot, 1);
+  tdot += shfl_xor(tdot, 1);
   T tg = tdot * g;
   T pr = (b4 + ih * tg) * iden;
   T f = v3 * tg + (g * L.k.ihM) * pr;
@@ -2401,25 +2373,19 @@ __device__ __forceinline__ void smooth_block(const Prm<T>& P, const LV& L, T ome
   if constexpr (std::is_same<Form, ProjForm>::value) {
     // projection method (Sec. 7.2): CH red-black, intermediate-velocity blocks
     // over the Vanka colours, pressure Gauss-Seidel red-black
-    const int mpr = (L.m1 + 1) / 2;
+    const int mpr = L.crow.d;
     // four lanes per cell while a colour fits the block in one pass
     const bool cteam = 4 * mpr * L.m2 <= grp_size();
     for (int col = 0; col < 2; ++col) {
       if (cteam) {
-        int t = grp_rank(), sl = t >> 2, j = 1, i = 1;
-        bool ok = false;
-        if (sl < mpr * L.m2) {
-          j = sl / mpr + 1;
-          i = (((col - j) & 1) ? 1 : 2) + 2 * (sl % mpr);
-          ok = i <= L.m1;
-        }
+        int t = grp_rank(), i = 1, j = 1;
+        bool ok = (t >> 2) < mpr * L.m2 && ch_slot_cell(L, col, t >> 2, i, j);
         if (!ok) i = j = 1;
         if ((t & ~31) < 4 * mpr * L.m2) ch_team<T, Form>(P, L, i, j, ok);  // warp-uniform
       } else {
         for (int t = grp_rank(); t < mpr * L.m2; t += grp_size()) {
-          int j = t / mpr + 1;
-          int i = (((col - j) & 1) ? 1 : 2) + 2 * (t % mpr);
-          if (i <= L.m1) ch_cell<T, Form>(P, L, i, j);
+          int i, j;
+          if (ch_slot_cell(L, col, t, i, j)) ch_cell<T, Form>(P, L, i, j);
         }
       }
       grp_sync();
@@ -2444,20 +2410,14 @@ __device__ __forceinline__ void smooth_block(const Prm<T>& P, const LV& L, T ome
     }
     for (int col = 0; col < 2; ++col) {
       if (cteam) {
-        int t = grp_rank(), sl = t >> 2, j = 1, i = 1;
-        bool ok = false;
-        if (sl < mpr * L.m2) {
-          j = sl / mpr + 1;
-          i = (((col - j) & 1) ? 1 : 2) + 2 * (sl % mpr);
-          ok = i <= L.m1;
-        }
+        int t = grp_rank(), i = 1, j = 1;
+        bool ok = (t >> 2) < mpr * L.m2 && ch_slot_cell(L, col, t >> 2, i, j);
         if (!ok) i = j = 1;
         if ((t & ~31) < 4 * mpr * L.m2) pgs_team<T>(P, L, i, j, ok);  // warp-uniform
       } else {
         for (int t = grp_rank(); t < mpr * L.m2; t += grp_size()) {
-          int j = t / mpr + 1;
-          int i = (((col - j) & 1) ? 1 : 2) + 2 * (t % mpr);
-          if (i <= L.m1) pgs_cell<T>(P, L, i, j);
+          int i, j;
+          if (ch_slot_cell(L, col, t, i, j)) pgs_cell<T>(P, L, i, j);
         }
       }
       grp_sync();
@@ -2485,28 +2445,22 @@ __device__ __forceinline__ void smooth_block(const Prm<T>& P, const LV& L, T ome
     }
     return;
   }
-  const int mpr = (L.m1 + 1) / 2;
+  const int mpr = L.crow.d;
   constexpr bool team_ok = std::is_same<Form, FullForm>::value && sizeof(T) == 8;
   constexpr bool vteam_ok = team_ok || std::is_same<Form, ErrForm>::value;
   for (int col = 0; col < 2; ++col) {
     if (vteam_ok && 4 * mpr * L.m2 <= grp_size()) {
       int t = grp_rank();
       if ((t & ~31) < 4 * mpr * L.m2) {  // warp-uniform
-        int sl = t >> 2, j = 1, i = 1;
-        bool ok = false;
-        if (sl < mpr * L.m2) {
-          j = sl / mpr + 1;
-          i = (((col - j) & 1) ? 1 : 2) + 2 * (sl % mpr);
-          ok = i <= L.m1;
-        }
+        int i = 1, j = 1;
+        bool ok = (t >> 2) < mpr * L.m2 && ch_slot_cell(L, col, t >> 2, i, j);
         if (!ok) i = j = 1;
         ch_team<T, Form>(P, L, i, j, ok);
       }
     } else {
       for (int t = grp_rank(); t < mpr * L.m2; t += grp_size()) {
-        int j = t / mpr + 1;
-        int i = (((col - j) & 1) ? 1 : 2) + 2 * (t % mpr);
-        if (i <= L.m1) ch_cell<T, Form>(P, L, i, j);
+        int i, j;
+        if (ch_slot_cell(L, col, t, i, j)) ch_cell<T, Form>(P, L, i, j);
       }
     }
     grp_sync();
@@ -2557,7 +2511,7 @@ __device__ __forceinline__ void coarse_vcycle_body(const Prm<T>& P, const Get& g
       const auto& F = get(l - 1);
       const auto& G = get(l);
       for (int t = grp_rank(); t < (G.m1 + 1) * (G.m2 + 1); t += grp_size())
-        restrict_base_cell(F, G, t % (G.m1 + 1), t / (G.m1 + 1));
+        restrict_base_cell(P, F, G, t % (G.m1 + 1), t / (G.m1 + 1));
       grp_sync();
       const int nf = 4 * (G.m1 + 3) + 4 * (G.m2 + 3);
       for (int t = grp_rank(); t < nf; t += grp_size()) {
@@ -2692,6 +2646,7 @@ __global__ void __launch_bounds__(NT) k_coarse_vcycle_smem(Prm<double> P, Coarse
       QN_LV_ARRAYS(QN_REBASE)
 #undef QN_REBASE
       X.pitch = cc;
+      X.nst = ns;
     }
     S->L[l] = X;
   }
@@ -2714,22 +2669,23 @@ __global__ void __launch_bounds__(NT) k_coarse_vcycle_smem(Prm<double> P, Coarse
 // visits have no slow arithmetic: what a colour step cost was the chain of
 // address arithmetic (a 64-bit address for each of the ~60 array elements a
 // visit reads) and L2 round trips.  The copy interleaves the level's arrays:
-// cell k's 41 values sit together (LvS), so that a visit forms three
+// cell k's 43 values sit together (LvS), so that a visit forms three
 // addresses (its row and the rows beside it) and reads everything else at
-// constant offsets from them.  41 words a cell is odd, so lanes on cells any
+// constant offsets from them.  43 words a cell is odd, so lanes on cells any
 // power of two (or 5) apart fall into different banks.
 // Measured (GB300, ncu, caches warm): the 16x32 .. 2x4 levels of the 256x512
 // drop 245 -> 139 us, the 28x28 and 14x14 levels of a served 448x448 request
 // (64 coupled sweeps on the coarsest) 1504 -> 1121 us.  Launched wherever the
-// records fit the opt-in shared memory (option coarse_smem; about 1380 padded
+// records fit the opt-in shared memory (option coarse_smem; about 1350 padded
 // cells); a larger group reads global memory.
 // --------------------------------------------------------------------------
 // the arrays of an error-equation level that its V-cycle touches, in the order
 // of a cell's record
 #define QN_ERR_ARRAYS(X)                                                                       \
   X(c) X(mu) X(p) X(u) X(v) X(fc) X(fmu) X(fp) X(fu) X(fv) X(rc) X(rmu) X(rp) X(ru) X(rv)     \
-  X(sc) X(smu) X(sp) X(su) X(sv) X(cn) X(rhon) X(mobn) X(visn) X(Gn) X(Aru) X(Arv) X(Sx)      \
-  X(Sy) X(Qx) X(Qy) X(Av) X(Tx) X(Ty) X(Dvu) X(Dvv) X(Bc) X(Bmu) X(Bu) X(Bv) X(Bdc)
+  X(sc) X(smu) X(sp) X(su) X(sv) X(cn) X(rhon) X(mobn) X(visn) X(Gn) X(T1u) X(T1v) X(aPu)    \
+  X(aPv) X(aMu) X(aMv) X(tPu) X(tPv) X(tMu) X(tMv) X(Tx) X(Ty) X(Bc) X(Bmu) X(Bu) X(Bv)       \
+  X(Bdc) X(rB)
 enum {
 #define QN_ERR_INDEX(m) ERR_##m,
   QN_ERR_ARRAYS(QN_ERR_INDEX)
@@ -2750,6 +2706,7 @@ struct LvS {
   typedef T real;
   static constexpr bool has_rho = false;
   LvK<T> k;
+  FastDiv vrow, crow, kdiv;
   int m1, m2, px, pitch, kcol, c8;
   T h, ih, ih2;
 #define QN_ERR_MEMBER(m) Fld<T, ERR_##m> m;
@@ -2757,7 +2714,7 @@ struct LvS {
 #undef QN_ERR_MEMBER
   // level L with its record of cell (0,0) at b
   __device__ __forceinline__ LvS(const Lv<T>& L, T* b)
-      : k(L.k), m1(L.m1), m2(L.m2), px(L.px), pitch(L.m1 + 3), kcol(L.kcol), c8(L.c8), h(L.h),
+      : k(L.k), vrow(L.vrow), crow(L.crow), kdiv(L.kdiv), m1(L.m1), m2(L.m2), px(L.px), pitch(L.m1 + 3), kcol(L.kcol), c8(L.c8), h(L.h),
         ih(L.ih), ih2(L.ih2) {
 #define QN_ERR_SET(m) m.b = b;
     QN_ERR_ARRAYS(QN_ERR_SET)
@@ -2788,14 +2745,15 @@ struct ErrLevels {
 };
 
 template <int NT>
-__global__ void __launch_bounds__(NT) k_coarse_err(Prm<float> P, const __grid_constant__ CoarseLevels<float> C,
+__global__ void __launch_bounds__(NT) k_coarse_err(Prm<rf32> P, const __grid_constant__ CoarseLevels<rf32> C,
                                                    const __grid_constant__ ErrSmem M, int nu1, int nu2,
-                                                   int nuc, float omega, int coupled) {
-  extern __shared__ __align__(16) float qn_err_smem[];
+                                                   int nuc, rf32 omega, int coupled) {
+  extern __shared__ __align__(16) float qn_err_words[];
+  rf32* qn_err_smem = reinterpret_cast<rf32*>(qn_err_words);
   pdl_enter();
   const int n = C.n;
   for (int l = 0; l < n; ++l) {  // the padded frame of every array, all copies in flight at once
-    const Lv<float>& L = C.L[l];
+    const Lv<rf32>& L = C.L[l];
     const int cc = L.m1 + 3, cells = cc * (L.m2 + 3);
     for (int t = threadIdx.x; t < cells; t += NT) {
       const int g = (t / cc - 1) * L.pitch + t % cc - 1;
@@ -2809,15 +2767,15 @@ __global__ void __launch_bounds__(NT) k_coarse_err(Prm<float> P, const __grid_co
   }
   asm volatile("cp.async.wait_all;" ::: "memory");
   __syncthreads();
-  const ErrLevels<float> get{C, M, qn_err_smem};
-  coarse_vcycle_body<float, ErrForm>(P, get, n, 1, nu1, nu2, nuc, omega, coupled, 0);
+  const ErrLevels<rf32> get{C, M, qn_err_smem};
+  coarse_vcycle_body<rf32, ErrForm>(P, get, n, 1, nu1, nu2, nuc, omega, coupled, 0);
   __syncthreads();
   // what the levels above read of the group: the iterate of its finest level
-  const Lv<float>& L = C.L[0];
+  const Lv<rf32>& L = C.L[0];
   const int cc = L.m1 + 3, cells = cc * (L.m2 + 3);
   for (int t = threadIdx.x; t < cells; t += NT) {
     const int g = (t / cc - 1) * L.pitch + t % cc - 1;
-    const float* r = qn_err_smem + M.off[0] + t * ERR_N;
+    const rf32* r = qn_err_smem + M.off[0] + t * ERR_N;
     L.c[g] = r[ERR_c];
     L.mu[g] = r[ERR_mu];
     L.p[g] = r[ERR_p];
@@ -2864,26 +2822,20 @@ __device__ __forceinline__ void wave_pass(const Prm<T>& P, const LV& L, const Wa
   const int q = pass % per;
   const int tid = threadIdx.x, nt = blockDim.x;
   if (!W.coupled && q < 2) {  // CH colour q: packed as in k_ch
-    const int mpr = (L.m1 + 1) / 2;
+    const int mpr = L.crow.d;
     const int t_lo = (r0 - 1) * mpr, t_hi = r1 * mpr;
     if (mpr * L.m2 <= W.ch_team_max) {
       for (int base = t_lo; base < t_hi; base += nt / 4) {
         if (base + ((tid & ~31) >> 2) >= t_hi) continue;  // warp-uniform
         int t = base + (tid >> 2), i = 1, j = 1;
-        bool ok = t < t_hi;
-        if (ok) {
-          j = t / mpr + 1;
-          i = (((q - j) & 1) ? 1 : 2) + 2 * (t % mpr);
-          ok = i <= L.m1;
-        }
+        bool ok = t < t_hi && ch_slot_cell(L, q, t, i, j);
         if (!ok) i = j = 1;
         ch_team<T, Form>(P, L, i, j, ok);
       }
     } else {
       for (int t = t_lo + tid; t < t_hi; t += nt) {
-        int j = t / mpr + 1;
-        int i = (((q - j) & 1) ? 1 : 2) + 2 * (t % mpr);
-        if (i <= L.m1) ch_cell<T, Form>(P, L, i, j);
+        int i, j;
+        if (ch_slot_cell(L, q, t, i, j)) ch_cell<T, Form>(P, L, i, j);
       }
     }
     return;
@@ -2987,10 +2939,9 @@ __global__ void __launch_bounds__(SNT) k_skew(Prm<T> P, Lv<T> L, SkewTasks S, T 
   const int q = S.q[k];
   if constexpr (!COUPLED) {
     if (q < 2) {  // CH colour q, slots as in k_ch
-      const int mpr = (L.m1 + 1) / 2;
-      const int j = t / mpr + 1;
-      const int i = (((q - j) & 1) ? 1 : 2) + 2 * (t % mpr);
-      if (i <= L.m1) ch_cell<T, Form>(P, L, i, j);
+      const int mpr = L.crow.d;
+      int i, j;
+      if (ch_slot_cell(L, q, t, i, j)) ch_cell<T, Form>(P, L, i, j);
       return;
     }
   }
@@ -3033,34 +2984,34 @@ __global__ void k_cast_frozen(Lv<double> D, Lv<T> E, long long n, int off) {
   if (t >= n) return;
   long long q = t - off;  // origin-relative index
   E.cn[q] = (T)D.cn[q];
-  E.un[q] = (T)D.un[q];
-  E.vn[q] = (T)D.vn[q];
   E.rhon[q] = (T)D.rhon[q];
   E.mobn[q] = (T)D.mobn[q];
   E.visn[q] = (T)D.visn[q];
   E.Gn[q] = (T)D.Gn[q];
-  E.Aru[q] = (T)D.Aru[q];
-  E.Arv[q] = (T)D.Arv[q];
-  E.Sx[q] = (T)D.Sx[q];
-  E.Sy[q] = (T)D.Sy[q];
-  E.Qx[q] = (T)D.Qx[q];
-  E.Qy[q] = (T)D.Qy[q];
-  E.Av[q] = (T)D.Av[q];
+  E.T1u[q] = (T)D.T1u[q];
+  E.T1v[q] = (T)D.T1v[q];
+  E.aPu[q] = (T)D.aPu[q];
+  E.aPv[q] = (T)D.aPv[q];
+  E.aMu[q] = (T)D.aMu[q];
+  E.aMv[q] = (T)D.aMv[q];
+  E.tPu[q] = (T)D.tPu[q];
+  E.tPv[q] = (T)D.tPv[q];
+  E.tMu[q] = (T)D.tMu[q];
+  E.tMv[q] = (T)D.tMv[q];
   E.Tx[q] = (T)D.Tx[q];
   E.Ty[q] = (T)D.Ty[q];
-  E.Dvu[q] = (T)D.Dvu[q];
-  E.Dvv[q] = (T)D.Dvv[q];
 }
 
 // base X = x (rounded), X.c - c^n formed in FP64, right-hand side = FP64 residual
 // (rounded), correction e = 0
 template <typename T>
-__global__ void k_start_correction(Lv<double> D, Lv<T> E, long long n, int off) {
+__global__ void k_start_correction(Prm<T> P, Lv<double> D, Lv<T> E, long long n, int off) {
   pdl_enter();
   long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= n) return;
   long long q = t - off;
   E.Bc[q] = (T)D.c[q];
+  E.rB[q] = rho_of(P, E.Bc[q]);
   E.Bmu[q] = (T)D.mu[q];
   E.Bu[q] = (T)D.u[q];
   E.Bv[q] = (T)D.v[q];
@@ -3104,12 +3055,12 @@ __global__ void k_rho_fill(Prm<double> P, Lv<double> L, long long n, int off) {
 
 // coarse base X_H = R X_h (cells: 4-mean; edges: 2 coincident fine edges)
 template <typename T>
-__global__ void k_restrict_base(Lv<T> F, Lv<T> C) {
+__global__ void k_restrict_base(Prm<T> P, Lv<T> F, Lv<T> C) {
   pdl_enter();
   int I = blockIdx.x * BX + threadIdx.x;
   int J = blockIdx.y * BY + threadIdx.y;
   if (I > C.m1 || J > C.m2) return;
-  restrict_base_cell(F, C, I, J);
+  restrict_base_cell(P, F, C, I, J);
 }
 
 template <typename T>
@@ -3425,36 +3376,42 @@ int nparts_cells(const Lv<T>& L) {
 }
 
 template <typename T, class Form>
-void launch_residual(const Prm<T>& P, const Lv<T>& L0, double* part, cudaStream_t s) {
-  const Lv<T> L = level_consts(P, L0);
+void launch_residual(const Prm<T>& P0, const Lv<T>& L0, double* part, cudaStream_t s) {
+  typedef compute_t<T, Form> R;
+  const Prm<R>& P = as_compute<R>(P0);
+  const Lv<R> L = as_compute<R>(level_consts(P0, L0));
   if (residual_rows(L) == 2)
-    qlaunch(&k_residual<T, 0, Form, 2>, grid2(L.m1, (L.m2 + 1) / 2), dim3(BX, BY), 0, s, P, L, part);
+    qlaunch(&k_residual<R, 0, Form, 2>, grid2(L.m1, (L.m2 + 1) / 2), dim3(BX, BY), 0, s, P, L, part);
   else
-    qlaunch(&k_residual<T, 0, Form, 1>, grid2(L.m1, L.m2), dim3(BX, BY), 0, s, P, L, part);
+    qlaunch(&k_residual<R, 0, Form, 1>, grid2(L.m1, L.m2), dim3(BX, BY), 0, s, P, L, part);
   ++g_launches;
 }
 template <typename T, class Form>
-void launch_add_op(const Prm<T>& P, const Lv<T>& L0, cudaStream_t s) {
-  const Lv<T> L = level_consts(P, L0);
+void launch_add_op(const Prm<T>& P0, const Lv<T>& L0, cudaStream_t s) {
+  typedef compute_t<T, Form> R;
+  const Prm<R>& P = as_compute<R>(P0);
+  const Lv<R> L = as_compute<R>(level_consts(P0, L0));
   if (residual_rows(L) == 2)
-    qlaunch(&k_residual<T, 1, Form, 2>, grid2(L.m1, (L.m2 + 1) / 2), dim3(BX, BY), 0, s, P, L, nullptr);
+    qlaunch(&k_residual<R, 1, Form, 2>, grid2(L.m1, (L.m2 + 1) / 2), dim3(BX, BY), 0, s, P, L, nullptr);
   else
-    qlaunch(&k_residual<T, 1, Form, 1>, grid2(L.m1, L.m2), dim3(BX, BY), 0, s, P, L, nullptr);
+    qlaunch(&k_residual<R, 1, Form, 1>, grid2(L.m1, L.m2), dim3(BX, BY), 0, s, P, L, nullptr);
   ++g_launches;
 }
 template <typename T, class Form>
-void launch_ch(const Prm<T>& P, const Lv<T>& L0, int colour, cudaStream_t s, int team_max) {
-  const Lv<T> L = level_consts(P, L0);
+void launch_ch(const Prm<T>& P0, const Lv<T>& L0, int colour, cudaStream_t s, int team_max) {
+  typedef compute_t<T, Form> R;
+  const Prm<R>& P = as_compute<R>(P0);
+  const Lv<R> L = as_compute<R>(level_consts(P0, L0));
   int n = (L.m1 + 1) / 2 * L.m2;
   if (n <= 0) return;
   if constexpr (sizeof(T) == 8 || std::is_same<Form, ErrForm>::value) {
     if (n <= team_max) {  // four lanes per cell: shorter critical path per visit
-      qlaunch(&k_ch_team<T, Form>, (4 * n + 63) / 64, 64, 0, s, P, L, colour);
+      qlaunch(&k_ch_team<R, Form>, (4 * n + 63) / 64, 64, 0, s, P, L, colour);
       ++g_launches;
       return;
     }
   }
-  qlaunch(&k_ch<T, Form>, (n + 63) / 64, 64, 0, s, P, L, colour);
+  qlaunch(&k_ch<R, Form>, (n + 63) / 64, 64, 0, s, P, L, colour);
   ++g_launches;
 }
 // SM sub-partitions of the current device (4 per SM)
@@ -3499,9 +3456,11 @@ int vanka_split_single(int n, int split) {
 }
 
 template <typename T, class Form>
-void launch_vanka(const Prm<T>& P, const Lv<T>& L0, int colour, T omega, cudaStream_t s,
+void launch_vanka(const Prm<T>& P0, const Lv<T>& L0, int colour, T omega, cudaStream_t s,
                   int team_max, int team8_max, int pair_max, int split) {
-  const Lv<T> L = level_consts(P, L0);
+  typedef compute_t<T, Form> R;
+  const Prm<R>& P = as_compute<R>(P0);
+  const Lv<R> L = as_compute<R>(level_consts(P0, L0));
   int n = vanka_slots(L, colour).n;
   if (n <= 0) return;
   if constexpr (std::is_same<Form, FullForm>::value && sizeof(T) == 8) {
@@ -3514,27 +3473,27 @@ void launch_vanka(const Prm<T>& P, const Lv<T>& L0, int colour, T omega, cudaStr
   if constexpr ((std::is_same<Form, FullForm>::value && sizeof(T) == 8) ||
                 std::is_same<Form, ErrForm>::value) {
     if (n <= team_max) {  // four lanes per block: shorter critical path per visit
-      qlaunch(&k_vanka_team<T, Form>, (4 * n + SNT - 1) / SNT, SNT, 0, s, P, L, colour, omega);
+      qlaunch(&k_vanka_team<R, Form>, (4 * n + SNT - 1) / SNT, SNT, 0, s, P, L, colour, omega);
       ++g_launches;
       return;
     }
   }
   if constexpr (std::is_same<Form, FullForm>::value && sizeof(T) == 8) {
     if (n <= pair_max) {  // a lane pair per block: half the FP64 instructions per lane
-      qlaunch(&k_vanka_pair<T, Form>, (2 * n + SNT - 1) / SNT, SNT, 0, s, P, L, colour, omega);
+      qlaunch(&k_vanka_pair<R, Form>, (2 * n + SNT - 1) / SNT, SNT, 0, s, P, L, colour, omega);
       ++g_launches;
       return;
     }
     const int ns = split > 0 ? vanka_split_single(n, split) : n;
     if (ns < n) {  // one lane per block for slots [0, ns), a lane pair for the rest
       const long long threads = (long long)ns + 2LL * (n - ns);
-      qlaunch(&k_vanka_split<T, Form>, (int)((threads + SNT - 1) / SNT), SNT, 0, s, P, L, colour,
+      qlaunch(&k_vanka_split<R, Form>, (int)((threads + SNT - 1) / SNT), SNT, 0, s, P, L, colour,
               omega, ns);
       ++g_launches;
       return;
     }
   }
-  qlaunch(&k_vanka<T, Form>, (n + SNT - 1) / SNT, SNT, 0, s, P, L, colour, omega);
+  qlaunch(&k_vanka<R, Form>, (n + SNT - 1) / SNT, SNT, 0, s, P, L, colour, omega);
   ++g_launches;
 }
 // shared memory a block of the current device may opt in to
@@ -3601,13 +3560,15 @@ void coarse_smem_prepare() {
 }
 
 template <typename T, class Form>
-int launch_coarse_vcycle(const Prm<T>& P, const Lv<T>* levels, int n, int nu1, int nu2, int nuc,
+int launch_coarse_vcycle(const Prm<T>& P0, const Lv<T>* levels, int n, int nu1, int nu2, int nuc,
                          int kcol, T omega, int coupled, cudaStream_t s, int team8, int ctas,
                          int smem) {
-  CoarseLevels<T> C;
+  typedef compute_t<T, Form> R;
+  const Prm<R>& P = as_compute<R>(P0);
+  CoarseLevels<R> C;
   C.n = n;
   C.base = std::is_same<Form, ErrForm>::value;
-  for (int l = 0; l < n; ++l) C.L[l] = level_consts(P, levels[l]);
+  for (int l = 0; l < n; ++l) C.L[l] = as_compute<R>(level_consts(P0, levels[l]));
   constexpr int NT = sizeof(T) == 8 ? 256 : 512;
   if constexpr (std::is_same<Form, FullForm>::value && sizeof(T) == 8) {
     if (ctas <= 1) {
@@ -3629,7 +3590,7 @@ int launch_coarse_vcycle(const Prm<T>& P, const Lv<T>* levels, int n, int nu1, i
     }
   }
   if (ctas <= 1) {
-    qlaunch(&k_coarse_vcycle<T, Form, NT>, 1, NT, 0, s, P, C, nu1, nu2, nuc, kcol, omega, coupled,
+    qlaunch(&k_coarse_vcycle<R, Form, NT>, 1, NT, 0, s, P, C, nu1, nu2, nuc, kcol, omega, coupled,
             team8);
   } else {  // one cluster of ctas blocks (a size coarse_cluster_blocks accepted)
     cudaLaunchConfig_t cfg = {};
@@ -3645,7 +3606,7 @@ int launch_coarse_vcycle(const Prm<T>& P, const Lv<T>* levels, int n, int nu1, i
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = g_pdl ? 2 : 1;
-    cudaLaunchKernelEx(&cfg, &k_coarse_vcycle<T, Form, NT>, P, C, nu1, nu2, nuc, kcol, omega,
+    cudaLaunchKernelEx(&cfg, &k_coarse_vcycle<R, Form, NT>, P, C, nu1, nu2, nuc, kcol, omega,
                        coupled, team8);
   }
   ++g_launches;
@@ -3659,7 +3620,7 @@ int launch_coarse_vcycle(const Prm<T>& P, const Lv<T>* levels, int n, int nu1, i
 template <typename T, class Form>
 static int cluster_fit(int ctas) {
   constexpr int NT = sizeof(T) == 8 ? 256 : 512;
-  auto kern = &k_coarse_vcycle<T, Form, NT>;
+  auto kern = &k_coarse_vcycle<compute_t<T, Form>, Form, NT>;
   if (ctas > 8 &&
       cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
     cudaGetLastError();
@@ -3696,32 +3657,36 @@ int coarse_cluster_blocks(int ctas) {
 }
 
 template <typename T, class Form>
-void launch_vanka4(const Prm<T>& P, const Lv<T>& L0, int colour, T omega, cudaStream_t s,
+void launch_vanka4(const Prm<T>& P0, const Lv<T>& L0, int colour, T omega, cudaStream_t s,
                    int team_max) {
-  const Lv<T> L = level_consts(P, L0);
+  typedef compute_t<T, Form> R;
+  const Prm<R>& P = as_compute<R>(P0);
+  const Lv<R> L = as_compute<R>(level_consts(P0, L0));
   int n = vanka_slots(L, colour).n;
   if (n <= 0) return;
   if constexpr (std::is_same<Form, ProjForm>::value && sizeof(T) == 8) {
     if (n <= team_max) {  // four lanes per block: shorter critical path per visit
-      qlaunch(&k_vanka4_team<T>, (4 * n + SNT - 1) / SNT, SNT, 0, s, P, L, colour, omega);
+      qlaunch(&k_vanka4_team<R>, (4 * n + SNT - 1) / SNT, SNT, 0, s, P, L, colour, omega);
       ++g_launches;
       return;
     }
   }
-  qlaunch(&k_vanka4<T, Form>, (n + SNT - 1) / SNT, SNT, 0, s, P, L, colour, omega);
+  qlaunch(&k_vanka4<R, Form>, (n + SNT - 1) / SNT, SNT, 0, s, P, L, colour, omega);
   ++g_launches;
 }
 template <typename T>
-void launch_pgs(const Prm<T>& P, const Lv<T>& L0, int colour, cudaStream_t s, int team_max) {
-  const Lv<T> L = level_consts(P, L0);
+void launch_pgs(const Prm<T>& P0, const Lv<T>& L0, int colour, cudaStream_t s, int team_max) {
+  typedef compute_t<T, ProjForm> R;
+  const Prm<R>& P = as_compute<R>(P0);
+  const Lv<R> L = as_compute<R>(level_consts(P0, L0));
   int n = (L.m1 + 1) / 2 * L.m2;
   if (n <= 0) return;
   if (n <= team_max) {  // four lanes per cell: shorter critical path per visit
-    qlaunch(&k_pgs_team<T>, (4 * n + 63) / 64, 64, 0, s, P, L, colour);
+    qlaunch(&k_pgs_team<R>, (4 * n + 63) / 64, 64, 0, s, P, L, colour);
     ++g_launches;
     return;
   }
-  qlaunch(&k_pgs<T>, (n + 63) / 64, 64, 0, s, P, L, colour);
+  qlaunch(&k_pgs<R>, (n + 63) / 64, 64, 0, s, P, L, colour);
   ++g_launches;
 }
 template <typename T>
@@ -3738,17 +3703,19 @@ void launch_proj_diss(const Prm<T>& P, const Lv<T>& L, const T* uo, const T* vo,
   ++g_launches;
 }
 template <typename T, class Form>
-void launch_coupled(const Prm<T>& P, const Lv<T>& L0, int colour, T omega, cudaStream_t s,
+void launch_coupled(const Prm<T>& P0, const Lv<T>& L0, int colour, T omega, cudaStream_t s,
                     int team_max) {
-  const Lv<T> L = level_consts(P, L0);
+  typedef compute_t<T, Form> R;
+  const Prm<R>& P = as_compute<R>(P0);
+  const Lv<R> L = as_compute<R>(level_consts(P0, L0));
   int n = vanka_slots(L, colour).n;
   if (n <= 0) return;
   if (n <= team_max) {  // four lanes per block: shorter critical path per visit
-    qlaunch(&k_coupled_team<T, Form>, (4 * n + SNT - 1) / SNT, SNT, 0, s, P, L, colour, omega);
+    qlaunch(&k_coupled_team<R, Form>, (4 * n + SNT - 1) / SNT, SNT, 0, s, P, L, colour, omega);
     ++g_launches;
     return;
   }
-  qlaunch(&k_coupled<T, Form>, (n + SNT - 1) / SNT, SNT, 0, s, P, L, colour, omega);
+  qlaunch(&k_coupled<R, Form>, (n + SNT - 1) / SNT, SNT, 0, s, P, L, colour, omega);
   ++g_launches;
 }
 
@@ -3763,9 +3730,9 @@ void launch_cast_frozen(const Lv<double>& D, const Lv<T>& E, cudaStream_t s) {
   ++g_launches;
 }
 template <typename T>
-void launch_start_correction(const Lv<double>& D, const Lv<T>& E, cudaStream_t s) {
+void launch_start_correction(const Prm<T>& P, const Lv<double>& D, const Lv<T>& E, cudaStream_t s) {
   long long n = padded_n(D.m1, D.m2);
-  qlaunch(&k_start_correction<T>, (unsigned)((n + 255) / 256), 256, 0, s, D, E, n, D.pitch + 1);
+  qlaunch(&k_start_correction<T>, (unsigned)((n + 255) / 256), 256, 0, s, P, D, E, n, D.pitch + 1);
   ++g_launches;
 }
 template <typename T>
@@ -3781,8 +3748,8 @@ void launch_rho_fill(const Prm<double>& P, const Lv<double>& L, cudaStream_t s) 
   ++g_launches;
 }
 template <typename T>
-void launch_restrict_base(const Lv<T>& F, const Lv<T>& C, cudaStream_t s) {
-  qlaunch(&k_restrict_base<T>, grid2(C.m1 + 1, C.m2 + 1), dim3(BX, BY), 0, s, F, C);
+void launch_restrict_base(const Prm<T>& P, const Lv<T>& F, const Lv<T>& C, cudaStream_t s) {
+  qlaunch(&k_restrict_base<T>, grid2(C.m1 + 1, C.m2 + 1), dim3(BX, BY), 0, s, P, F, C);
   ++g_launches;
   int n = frame_threads(C.m1, C.m2);
   qlaunch(&k_bc_base<T>, (n + 255) / 256, 256, 0, s, C);
@@ -3903,9 +3870,11 @@ void launch_pack_out(const Lv<T>& L, double* dst, const T* src, int kind, cudaSt
 }
 
 template <typename T, class Form>
-void launch_wave(const Prm<T>& P, const Lv<T>& L0, const WavePlan& W, T omega, unsigned* ctr,
+void launch_wave(const Prm<T>& P0, const Lv<T>& L0, const WavePlan& W, T omega, unsigned* ctr,
                  double* flag, cudaStream_t s) {
-  const Lv<T> L = level_consts(P, L0);
+  typedef compute_t<T, Form> R;
+  const Prm<R>& P = as_compute<R>(P0);
+  const Lv<R> L = as_compute<R>(level_consts(P0, L0));
   static std::atomic<int> blocks_per_sm{0};
   static std::atomic<int> sms{0};
   if (!sms.load()) {
@@ -3916,20 +3885,22 @@ void launch_wave(const Prm<T>& P, const Lv<T>& L0, const WavePlan& W, T omega, u
   }
   if (!blocks_per_sm.load()) {
     int b = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_wave<T, Form>, WAVE_NT, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_wave<R, Form>, WAVE_NT, 0);
     blocks_per_sm = b > 0 ? b : 1;
   }
   const long long tasks = (long long)W.nbands * W.npass;
   const int grid = (int)std::min<long long>((long long)sms.load() * blocks_per_sm.load(), tasks);
   cudaMemsetAsync(ctr, 0, (size_t)(1 + W.nbands) * sizeof(unsigned), s);
-  qlaunch(&k_wave<T, Form>, grid, WAVE_NT, 0, s, P, L, W, omega, ctr, flag);
+  qlaunch(&k_wave<R, Form>, grid, WAVE_NT, 0, s, P, L, W, omega, ctr, flag);
   ++g_launches;
 }
 
 template <typename T, class Form>
-int launch_skew(const Prm<T>& P, const Lv<T>& L0, int nsteps, int coupled, int rows, T omega,
+int launch_skew(const Prm<T>& P0, const Lv<T>& L0, int nsteps, int coupled, int rows, T omega,
                 cudaStream_t s) {
-  const Lv<T> L = level_consts(P, L0);
+  typedef compute_t<T, Form> R;
+  const Prm<R>& P = as_compute<R>(P0);
+  const Lv<R> L = as_compute<R>(level_consts(P0, L0));
   const int per = coupled ? L.kcol : L.kcol + 2;
   const int H = std::max(rows, 1);
   const int group = std::max(1, SKEW_MAX_TASKS / per);  // steps per schedule
@@ -3949,7 +3920,7 @@ int launch_skew(const Prm<T>& P, const Lv<T>& L0, int nsteps, int coupled, int r
         const int q = p % per;
         int t_lo, t_hi;
         if (!coupled && q < 2) {
-          const int mpr = (L.m1 + 1) / 2;
+          const int mpr = L.crow.d;
           t_lo = (lo - 1) * mpr;
           t_hi = (hi - 1) * mpr;
         } else {
@@ -3971,8 +3942,8 @@ int launch_skew(const Prm<T>& P, const Lv<T>& L0, int nsteps, int coupled, int r
       }
       S.boff[S.n] = nb;
       if (S.n == 0) continue;
-      if (coupled) qlaunch(&k_skew<T, Form, true>, nb, SNT, 0, s, P, L, S, omega);
-      else qlaunch(&k_skew<T, Form, false>, nb, SNT, 0, s, P, L, S, omega);
+      if (coupled) qlaunch(&k_skew<R, Form, true>, nb, SNT, 0, s, P, L, S, omega);
+      else qlaunch(&k_skew<R, Form, false>, nb, SNT, 0, s, P, L, S, omega);
       ++g_launches;
       ++launches;
     }
@@ -4022,10 +3993,11 @@ int partial_rows_needed(int m1, int m2) {
 
 #define QN_INSTANTIATE(T)                                                                        \
   template void launch_cast_frozen<T>(const Lv<double>&, const Lv<T>&, cudaStream_t);            \
-  template void launch_start_correction<T>(const Lv<double>&, const Lv<T>&, cudaStream_t);       \
+  template void launch_start_correction<T>(const Prm<T>&, const Lv<double>&, const Lv<T>&,       \
+                                           cudaStream_t);                                        \
   template void launch_apply_correction<T>(const Prm<double>&, const Lv<double>&, const Lv<T>&,    \
                                             cudaStream_t);                                          \
-  template void launch_restrict_base<T>(const Lv<T>&, const Lv<T>&, cudaStream_t);               \
+  template void launch_restrict_base<T>(const Prm<T>&, const Lv<T>&, const Lv<T>&, cudaStream_t); \
   template void launch_bc_unknowns<T>(const Lv<T>&, cudaStream_t);                               \
   template void launch_frozen<T>(const Prm<T>&, const Lv<T>&, cudaStream_t);                     \
   template void launch_restrict_state<T>(const Prm<T>&, const Lv<T>&, const Lv<T>&, cudaStream_t); \

@@ -109,12 +109,14 @@ void launch_proj_diss(const Prm<T>& P, const Lv<T>& L, const T* uo, const T* vo,
                       double* out1, cudaStream_t s);
 // defect correction: E (error-equation level) from the FP64 level D
 template <typename T> void launch_cast_frozen(const Lv<double>& D, const Lv<T>& E, cudaStream_t s);
-template <typename T> void launch_start_correction(const Lv<double>& D, const Lv<T>& E, cudaStream_t s);
+template <typename T>
+void launch_start_correction(const Prm<T>& P, const Lv<double>& D, const Lv<T>& E, cudaStream_t s);
 template <typename T>
 void launch_apply_correction(const Prm<double>& P, const Lv<double>& D, const Lv<T>& E, cudaStream_t s);
 // rho(c) of the iterate over the whole padded arrays of an FP64 full-iterate level
 void launch_rho_fill(const Prm<double>& P, const Lv<double>& L, cudaStream_t s);
-template <typename T> void launch_restrict_base(const Lv<T>& F, const Lv<T>& C, cudaStream_t s);
+template <typename T>
+void launch_restrict_base(const Prm<T>& P, const Lv<T>& F, const Lv<T>& C, cudaStream_t s);
 template <typename T> void launch_bc_unknowns(const Lv<T>& L, cudaStream_t s);
 template <typename T> void launch_frozen(const Prm<T>& P, const Lv<T>& L, cudaStream_t s);
 template <typename T> void launch_restrict_state(const Prm<T>& P, const Lv<T>& F, const Lv<T>& C, cudaStream_t s);

@@ -13,7 +13,79 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <type_traits>
+
 namespace qn {
+
+// FP32 and FP64 numbers whose multiply-adds are fused by the way an expression
+// is written.  The compiler contracts a * b + c as it sees fit in each kernel
+// it inlines a function into; two kernels that run the same visits (a colour
+// launch, the wavefront, the skewed chunks, the fused coarse V-cycle) then
+// differ by rounding.  Here a product is held as its two factors until it is
+// added (fused) or used (rounded): product + product fuses the left one.
+template <typename F>
+struct Fused {
+  F v;
+  Fused() = default;
+  __host__ __device__ constexpr Fused(float x) : v((F)x) {}
+  __host__ __device__ constexpr Fused(double x) : v((F)x) {}
+  __host__ __device__ constexpr Fused(int x) : v((F)x) {}
+  __host__ __device__ explicit operator float() const { return (float)v; }
+  __host__ __device__ explicit operator double() const { return (double)v; }
+};
+typedef Fused<float> rf32;
+typedef Fused<double> rf64;
+static_assert(sizeof(rf32) == 4 && sizeof(rf64) == 8 && std::is_trivially_copyable<rf32>::value &&
+                  std::is_trivially_copyable<rf64>::value,
+              "the bits of a float and a double");
+#ifdef __CUDACC__
+#define QN_F __device__ __forceinline__
+QN_F float rn_add(float x, float y) { return __fadd_rn(x, y); }
+QN_F float rn_mul(float x, float y) { return __fmul_rn(x, y); }
+QN_F float rn_fma(float x, float y, float z) { return __fmaf_rn(x, y, z); }
+QN_F double rn_add(double x, double y) { return __dadd_rn(x, y); }
+QN_F double rn_mul(double x, double y) { return __dmul_rn(x, y); }
+QN_F double rn_fma(double x, double y, double z) { return __fma_rn(x, y, z); }
+template <typename F>
+struct Product {
+  F a, b;
+  QN_F operator Fused<F>() const { return rn_mul(a, b); }
+};
+#define QN_T template <typename F> QN_F
+QN_T Fused<F> operator+(Fused<F> x, Fused<F> y) { return rn_add(x.v, y.v); }
+QN_T Fused<F> operator-(Fused<F> x, Fused<F> y) { return rn_add(x.v, -y.v); }
+QN_T Fused<F> operator-(Fused<F> x) { return -x.v; }
+QN_T Product<F> operator*(Fused<F> x, Fused<F> y) { return {x.v, y.v}; }
+QN_T Product<F> operator*(Product<F> x, Fused<F> y) { return {rn_mul(x.a, x.b), y.v}; }
+QN_T Product<F> operator*(Fused<F> x, Product<F> y) { return {x.v, rn_mul(y.a, y.b)}; }
+QN_T Product<F> operator*(Product<F> x, Product<F> y) {
+  return {rn_mul(x.a, x.b), rn_mul(y.a, y.b)};
+}
+QN_T Product<F> operator-(Product<F> x) { return {-x.a, x.b}; }
+QN_T Fused<F> operator+(Product<F> x, Fused<F> y) { return rn_fma(x.a, x.b, y.v); }
+QN_T Fused<F> operator+(Fused<F> x, Product<F> y) { return rn_fma(y.a, y.b, x.v); }
+QN_T Fused<F> operator-(Product<F> x, Fused<F> y) { return rn_fma(x.a, x.b, -y.v); }
+QN_T Fused<F> operator-(Fused<F> x, Product<F> y) { return rn_fma(-y.a, y.b, x.v); }
+QN_T Fused<F> operator+(Product<F> x, Product<F> y) { return rn_fma(x.a, x.b, rn_mul(y.a, y.b)); }
+QN_T Fused<F> operator-(Product<F> x, Product<F> y) { return rn_fma(x.a, x.b, -rn_mul(y.a, y.b)); }
+QN_T Fused<F>& operator+=(Fused<F>& x, Fused<F> y) { return x = x + y; }
+QN_T Fused<F>& operator-=(Fused<F>& x, Fused<F> y) { return x = x - y; }
+QN_T Fused<F>& operator+=(Fused<F>& x, Product<F> y) { return x = x + y; }
+QN_T Fused<F>& operator-=(Fused<F>& x, Product<F> y) { return x = x - y; }
+QN_T Fused<F>& operator*=(Fused<F>& x, Fused<F> y) { return x = x * y; }
+QN_T Fused<F> operator/(Fused<F> x, Fused<F> y) { return x.v / y.v; }
+#undef QN_T
+// the value of the lane whose index differs from this one's by the bits o
+template <typename T>
+QN_F T shfl_xor(T x, int o) {
+  return __shfl_xor_sync(0xffffffffu, x, o);
+}
+template <typename F>
+QN_F Fused<F> shfl_xor(Fused<F> x, int o) {
+  return __shfl_xor_sync(0xffffffffu, x.v, o);
+}
+#undef QN_F
+#endif
 
 template <typename T>
 struct Prm {
@@ -26,6 +98,27 @@ struct Prm {
   T eps_m;         // mobility regularisation, m(c) = sqrt(c^2 (1-c)^2 + eps_m)
   T idt;           // 1/dt
 };
+
+// n / d for 0 <= n < 2^31 by one multiply-high and a shift: with s = ceil(log2
+// d) - 1 and m = ceil(2^(32+s) / d), m d exceeds 2^(32+s) by less than d <=
+// 2^(s+1), so the quotient's error n (m d - 2^(32+s)) / (d 2^(32+s)) stays
+// below 1/d.  A run-time division takes about 25 dependent instructions, and a
+// visit's slot-to-cell mapping needs three.
+struct FastDiv {
+  unsigned m;
+  int s, d;
+#ifdef __CUDACC__
+  __device__ __forceinline__ int div(int n) const {
+    return d == 1 ? n : (int)(__umulhi((unsigned)n, m) >> s);
+  }
+#endif
+};
+inline FastDiv fast_div(int d) {
+  int s = -1;
+  while ((1LL << (s + 1)) < d) ++s;
+  if (s < 0) return {0u, 0, 1};
+  return {(unsigned)(((1ULL << (32 + s)) + (unsigned)d - 1) / (unsigned)d), s, d};
+}
 
 // Products of the parameters and a level's spacing that the operators multiply
 // by (level_consts, on the host at each launch).  A warp's FP64 instruction
@@ -50,6 +143,10 @@ struct Lv {
   typedef T real;
   static constexpr bool has_rho = true;
   LvK<T> k;
+  // slot-to-cell mapping: cells of a Vanka colour in one of its rows, of a CH
+  // colour in a row, and the number of Vanka colours
+  FastDiv vrow, crow, kdiv;
+  long long nst;  // elements from one array of the level to the next
   int m1, m2, px, pitch;
   // Vanka colours of this level: kcol colours, (2i+j) mod 8 when c8 is set
   // (periodic x with m1 = 0 mod 4), else (i+2j) mod kcol
@@ -68,11 +165,11 @@ struct Lv {
   // the divergence corrections 1/2[D_x(rho a_x u) + Dfrak_y(..)] (x-edges)
   // and 1/2[Dfrak_x(..) + D_y(rho a_y v)] (y-edges) of (e1e1-2)
   T *Aru, *Arv, *Sx, *Sy, *Qx, *Qy, *Av, *Tx, *Ty, *Dvu, *Dvv;
-  // FP64 full-iterate levels only, built per step (they depend on dt): for each
+  // built per step (they depend on dt): for each
   // momentum row (x-edges *u, y-edges *v) the time-term coefficients, time =
   // x T1 + T0 + (dt^-1/2) A rho(c) x with T1 = A rho^n/(2dt) + Dv and T0 =
   // -A rho^n x^n/dt (plus, in the primitive method's y rows, gravity
-  // (1/Fr) A_y rho^n), and Dg, the part of the row's diagonal entry that does not
+  // (1/Fr) A_y rho^n), and, on the full-iterate levels, Dg, the part of the row's diagonal entry that does not
   // depend on the iterate (the whole diagonal is Dg + A rho(c)/(2dt))
   T *T1u = nullptr, *T1v = nullptr, *T0u = nullptr, *T0v = nullptr, *Dgu = nullptr, *Dgv = nullptr;
   // FP64 full-iterate levels only: rho(c) of the iterate, ghosts included.
@@ -95,9 +192,14 @@ struct Lv {
   // error-equation (defect-correction) levels only: base state X the iterate
   // e is a correction to, and X.c - c^n formed in FP64 before rounding
   T *Bc = nullptr, *Bmu = nullptr, *Bu = nullptr, *Bv = nullptr, *Bdc = nullptr;
+  T* rB = nullptr;  // rho(Bc)
   __device__ __forceinline__ int at(int i, int j) const { return j * pitch + i; }
   // the array of direction d (0: x, 1: y) of a pair
-  __device__ __forceinline__ T* pair(int d, T* x, T* y) const { return d ? y : x; }
+  // (the pairs' arrays are neighbours, the assembled rows' seven apart): an
+  // offset, where selecting between two kernel parameters is an indexed
+  // constant load that the array's own load has to wait for
+  __device__ __forceinline__ T* pair(int d, T* x, T*) const { return x + (d ? nst : 0); }
+  __device__ __forceinline__ T* row_pair(int d, T* x, T*) const { return x + (d ? 7 * nst : 0); }
   // x-edge unknowns: walls exclude i = 0 and i = m1; periodic keeps i = m1 (= edge 0)
   __device__ __forceinline__ int uhi() const { return px ? m1 : m1 - 1; }
 };
@@ -111,6 +213,9 @@ inline Lv<T> level_consts(const Prm<T>& P, const Lv<T>& L) {
          T(0.5 * ih),     T(dif),           T(al * dif),            T(al * al * dif),
          T(ih * ih * iM), T(0.5 * ih2),     T(0.125 * P.K),         T(0.25 * P.K),
          T(0.25 * P.Lam), T(0.125 * P.Lam * ih2), T(0.25 * P.Lam * ih2)};
+  X.vrow = fast_div(L.c8 ? (L.m1 + 3) / 4 : (L.m1 + L.kcol - 1) / L.kcol);
+  X.crow = fast_div((L.m1 + 1) / 2);
+  X.kdiv = fast_div(L.kcol);
   return X;
 }
 
@@ -134,6 +239,7 @@ template <typename T> __device__ __forceinline__ T rho_of(const Prm<T>& P, T c) 
 // ulp, whose rounding the FP64 defect correction absorbs; IEEE division in FP64
 template <typename T> __device__ __forceinline__ T qdiv(T a, T b) { return a / b; }
 template <> __device__ __forceinline__ float qdiv(float a, float b) { return __fdividef(a, b); }
+template <> __device__ __forceinline__ rf32 qdiv(rf32 a, rf32 b) { return __fdividef(a.v, b.v); }
 // 1/x for the pivots of the local block solves.  FP32: the fast division, as
 // qdiv.  FP64: one step of the third-order iteration r <- r + r (e + e^2),
 // e = 1 - x r, which is Newton's for the zero of 1/r - x with the next term of
@@ -148,15 +254,22 @@ template <typename T> __device__ __forceinline__ T qrcp(T x) { return qdiv(T(1),
 template <> __device__ __forceinline__ double qrcp(double x) {
   double r;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-  double e = fma(-x, r, 1.0);
-  e = fma(e, e, e);
-  return fma(r, e, r);
+  double e = __fma_rn(-x, r, 1.0);
+  e = __fma_rn(e, e, e);
+  return __fma_rn(r, e, r);
 }
+template <> __device__ __forceinline__ rf64 qrcp(rf64 x) { return qrcp(x.v); }
 template <> __device__ __forceinline__ double rho_of(const Prm<double>& P, double c) {
   return qrcp(P.ia * c + P.ib);
 }
+template <> __device__ __forceinline__ rf64 rho_of(const Prm<rf64>& P, rf64 c) {
+  return qrcp<rf64>(P.ia * c + P.ib);
+}
 template <> __device__ __forceinline__ float rho_of(const Prm<float>& P, float c) {
   return qdiv(1.0f, P.ia * c + P.ib);
+}
+template <> __device__ __forceinline__ rf32 rho_of(const Prm<rf32>& P, rf32 c) {
+  return qdiv(rf32(1.0f), P.ia * c + P.ib);
 }
 template <typename T> __device__ __forceinline__ T visc_of(const Prm<T>& P, T c) {
   return T(1) / (P.va * c + P.vb);
@@ -184,18 +297,20 @@ template <typename T> __device__ __forceinline__ T gsec_da(T a, T b) {
 
 // G(c) = a_x((D_x c)^2) + a_y((D_y c)^2) at cell k (times h^2)
 template <class A>
-__device__ __forceinline__ auto G_h2(A c, int k, int pitch) {
-  auto cc = c[k];
-  typedef decltype(cc) T;
+__device__ __forceinline__ auto G_h2(A c, int k, int pitch) ->
+    typename std::decay<decltype(c[k])>::type {
+  typedef typename std::decay<decltype(c[k])>::type T;
+  T cc = c[k];
   T de = c[k + 1] - cc, dw = cc - c[k - 1], dn = c[k + pitch] - cc, ds = cc - c[k - pitch];
   return T(0.5) * (de * de + dw * dw + dn * dn + ds * ds);
 }
 
 // h^2 grad_d.(A kap grad_D phi) at cell k
 template <class A, class B>
-__device__ __forceinline__ auto lap_h2(A kap, B phi, int k, int pitch) {
-  auto kc = kap[k], pc = phi[k];
-  typedef decltype(kc) T;
+__device__ __forceinline__ auto lap_h2(A kap, B phi, int k, int pitch) ->
+    typename std::decay<decltype(kap[k])>::type {
+  typedef typename std::decay<decltype(kap[k])>::type T;
+  T kc = kap[k], pc = phi[k];
   return T(0.5) * ((kap[k + 1] + kc) * (phi[k + 1] - pc) - (kc + kap[k - 1]) * (pc - phi[k - 1]) +
                    (kap[k + pitch] + kc) * (phi[k + pitch] - pc) -
                    (kc + kap[k - pitch]) * (pc - phi[k - pitch]));
@@ -278,11 +393,16 @@ __device__ __forceinline__ T op_p(const Prm<T>& P, const LV& L, int k) {
 template <typename T, class LV>
 __device__ __forceinline__ T mom_asm(const LV& L, int d, int k, T rs) {
   const int s = d ? L.pitch : 1, t = d ? 1 : L.pitch;
-  auto a = d ? L.v : L.u; auto b = d ? L.u : L.v;
-  auto C = d ? L.Cv : L.Cu; auto aP = d ? L.aPv : L.aPu; auto aM = d ? L.aMv : L.aMu;
-  auto tP = d ? L.tPv : L.tPu; auto tM = d ? L.tMv : L.tMu;
-  auto M0 = d ? L.M0v : L.M0u; auto M1 = d ? L.M1v : L.M1u;
-  T r = (d ? L.T0v : L.T0u)[k] + (C[k] + L.k.qidt * rs) * a[k];
+  auto a = L.pair(d, L.u, L.v);
+  auto b = L.pair(1 - d, L.u, L.v);
+  auto C = L.row_pair(d, L.Cu, L.Cv);
+  auto aP = L.row_pair(d, L.aPu, L.aPv);
+  auto aM = L.row_pair(d, L.aMu, L.aMv);
+  auto tP = L.row_pair(d, L.tPu, L.tPv);
+  auto tM = L.row_pair(d, L.tMu, L.tMv);
+  auto M0 = L.row_pair(d, L.M0u, L.M0v);
+  auto M1 = L.row_pair(d, L.M1u, L.M1v);
+  T r = L.pair(d, L.T0u, L.T0v)[k] + (C[k] + L.k.qidt * rs) * a[k];
   r += aP[k] * a[k + s] + aM[k] * a[k - s] + tP[k] * a[k + t] + tM[k] * a[k - t];
   // the grad-div term's cross derivative of the other velocity
   T vl = L.visn[k], vr = L.visn[k + s];
@@ -500,6 +620,46 @@ __device__ __forceinline__ void store_v(const LV& L, int i, int e, T x) {
   }
 }
 
+// Whether any value that a block on cell (i,j) writes has a ghost copy: only
+// then do its stores go through store_cell, store_u and store_v.
+template <class LV>
+__device__ __forceinline__ bool has_ghosts(const LV& L, int i, int j) {
+  return i <= 2 || i >= L.m1 - 1 || j == 1 || j == L.m2;
+}
+template <typename T, class LV, class A>
+__device__ __forceinline__ void put_cell(const LV& L, A a, int i, int j, bool ghosts, T x) {
+  if (ghosts) store_cell(L, a, i, j, x);
+  else a[L.at(i, j)] = x;
+}
+// the four edges (W, E, S, N) of cell (i,j); act: the ones that hold an unknown
+template <typename T, class LV>
+__device__ __forceinline__ void put_edges(const LV& L, int i, int j, bool ghosts,
+                                          const bool* act, T w, T e, T so, T n) {
+  if (ghosts) {
+    if (act[0]) store_u(L, (L.px && i == 1) ? L.m1 : i - 1, j, w);
+    if (act[1]) store_u(L, i, j, e);
+    if (act[2]) store_v(L, i, j - 1, so);
+    if (act[3]) store_v(L, i, j, n);
+  } else {
+    const int k = L.at(i, j);
+    L.u[k - 1] = w;
+    L.u[k] = e;
+    L.v[k - L.pitch] = so;
+    L.v[k] = n;
+  }
+}
+// edge q (W, E, S, N) of cell (i,j), which holds an unknown, by one lane of a team
+template <typename T, class LV>
+__device__ __forceinline__ void put_edge(const LV& L, int i, int j, int q, bool ghosts, T x) {
+  if (ghosts) {
+    if (q < 2) store_u(L, q ? i : (L.px && i == 1) ? L.m1 : i - 1, j, x);
+    else store_v(L, i, q == 3 ? j : j - 1, x);
+  } else {
+    const int k = L.at(i, j);
+    L.pair(q >> 1, L.u, L.v)[q == 0 ? k - 1 : q == 2 ? k - L.pitch : k] = x;
+  }
+}
+
 // ---------------------------------------------------------------------------
 // error equation for defect correction: N_e(e) = N(X + e) - N(X) for the
 // iterate e stored in c, mu, p, u, v of the level and the base X in Bc, Bmu, Bu,
@@ -518,112 +678,104 @@ template <typename T> __device__ __forceinline__ T dgsec(T a, T b, T e) {
   return T(0.25) * e * (a * (a - T(1)) + b * (b - T(1)) + (T(2) * a - T(1) + e) * (a + b - T(1) + e));
 }
 
+// What the rows of the error equation at a cell share, at the cell and its east,
+// west, north and south neighbours: e and the base's c and rho^n, rho at the
+// full value and the difference rho(C + e) - rho(C).
+template <typename T>
+struct ErrCell {
+  T e[5], B[5], rn[5], r[5], dr[5];
+};
 template <typename T, class LV>
-__device__ __forceinline__ T opd_c(const Prm<T>& P, const LV& L, int k) {
-  const int W = L.pitch;
-  auto cn = L.cn;
-  auto rn = L.rhon;
-  T e = L.c[k], C = L.Bc[k];
-  T rp = rho_of(P, C + e), rC = rho_of(P, C);
-  (void)cn;
-  T adv = rn[k + 1] * L.Tx[k] * L.u[k] + rn[k - 1] * L.Tx[k - 1] * L.u[k - 1] +
-          rn[k + W] * L.Ty[k] * L.v[k] + rn[k - W] * L.Ty[k - W] * L.v[k - W];
-  T diff = lap_h2(L.mobn, L.mu, k, W) + P.alpha * lap_h2(L.mobn, L.p, k, W);
-  return e * (rp + rsec_(P, rp, rC) * L.Bdc[k]) * P.idt + adv - P.iPe * L.ih2 * diff;
+__device__ __forceinline__ ErrCell<T> err_cell(const Prm<T>& P, const LV& L, int k) {
+  const int off[5] = {0, 1, -1, L.pitch, -L.pitch};
+  ErrCell<T> X;
+#pragma unroll
+  for (int q = 0; q < 5; ++q) {
+    X.e[q] = L.c[k + off[q]];
+    X.B[q] = L.Bc[k + off[q]];
+    X.rn[q] = L.rhon[k + off[q]];
+    X.dr[q] = L.rB[k + off[q]];
+  }
+#pragma unroll
+  for (int q = 0; q < 5; ++q) {
+    X.r[q] = rho_of(P, X.B[q] + X.e[q]);
+    X.dr[q] = rsec_(P, X.r[q], X.dr[q]) * X.e[q];
+  }
+  return X;
 }
 
+// N_c of the error equation without its diffusion: (pm-num-phase) applied to e
 template <typename T, class LV>
-__device__ __forceinline__ T opd_mu(const Prm<T>& P, const LV& L, int k) {
+__device__ __forceinline__ T err_c(const Prm<T>& P, const LV& L, int k, T rp) {
+  auto rn = L.rhon;
   const int W = L.pitch;
-  auto e = L.c; auto B = L.Bc; auto cn = L.cn; auto rn = L.rhon;
-  T ek = e[k], Ck = B[k], cnk = cn[k], rnk = rn[k];
+  T adv = rn[k + 1] * L.Tx[k] * L.u[k] + rn[k - 1] * L.Tx[k - 1] * L.u[k - 1] +
+          rn[k + W] * L.Ty[k] * L.v[k] + rn[k - W] * L.Ty[k - W] * L.v[k - W];
+  return L.c[k] * (rp + rsec_(P, rp, L.rB[k]) * L.Bdc[k]) * P.idt + adv;
+}
+
+// N_mu of the error equation
+template <typename T, class LV>
+__device__ __forceinline__ T err_mu(const Prm<T>& P, const LV& L, int k, const ErrCell<T>& X) {
+  const int off[5] = {0, 1, -1, L.pitch, -L.pitch};
+  T ek = X.e[0], Ck = X.B[0], cnk = L.cn[k], rnk = X.rn[0], rp = X.r[0];
   T cp = Ck + ek;
-  T rp = rho_of(P, cp), rC = rho_of(P, Ck);
-  T dr = rsec_(P, rp, rC) * ek;             // rho(c') - rho(C)
+  T dr = X.dr[0];                           // rho(c') - rho(C)
   T rhp = T(0.5) * (rp + rnk);              // rho^{n+1/2} at c'
   T r_new = rsec_(P, rp, rnk);              // r(c', c^n)
   T d_r = -P.alpha * rnk * dr;              // r(c', c^n) - r(C, c^n)
   T dF = gsec(cp, Ck) * ek;                 // F(c') - F(C)
   T dbulk = rhp * dgsec(Ck, cnk, ek) + T(0.5) * dr * gsec(Ck, cnk) + T(0.5) * dF * r_new +
             T(0.5) * (Fdw(Ck) + Fdw(cnk)) * d_r;
-  // G(c') - G(C) and G(C), both times h^2
-  const int off[4] = {1, -1, W, -W};
+  // G(c') - G(C) and G(C), both times 2 h^2
   T dG = T(0), GC = T(0), ddiv = T(0);
   T chP = Ck + cnk;  // 2 c^{n+1/2} at C
 #pragma unroll
-  for (int f = 0; f < 4; ++f) {
-    int q = k + off[f];
-    T dC = B[q] - Ck, de = e[q] - ek;
+  for (int f = 1; f < 5; ++f) {
+    T dC = X.B[f] - Ck, de = X.e[f] - ek;
     dG += de * (T(2) * dC + de);
     GC += dC * dC;
-    T rq = rho_of(P, B[q] + e[q]), rCq = rho_of(P, B[q]);
-    T rhq = T(0.5) * (rq + rn[q]);
-    T drq = rsec_(P, rq, rCq) * e[q];
     // div(A rho_h(c') grad(e/2)) + div(A d rho_h grad c^{n+1/2}(C)), per face
-    ddiv += (rhp + rhq) * de + T(0.5) * (dr + drq) * ((B[q] + cn[q]) - chP);
+    ddiv += (rhp + T(0.5) * (X.r[f] + X.rn[f])) * de +
+            T(0.5) * (dr + X.dr[f]) * ((X.B[f] + L.cn[k + off[f]]) - chP);
   }
-  dG *= T(0.5);
-  GC *= T(0.5);
-  T dgrad = T(0.25) * P.Lam * (dG * L.ih2 * r_new + (GC * L.ih2 + L.Gn[k]) * d_r);
-  ddiv *= T(0.25) * L.ih2;
-  return rp * L.mu[k] + dr * L.Bmu[k] - P.K * dbulk - dgrad + P.Lam * ddiv;
+  T dgrad = L.k.L4 * (L.k.hih2 * dG * r_new + (L.k.hih2 * GC + L.Gn[k]) * d_r);
+  return rp * L.mu[k] + dr * L.Bmu[k] - P.K * dbulk - dgrad + L.k.L4h * ddiv;
 }
 
+// momentum row d (0: x, 1: y) at edge k of the error equation: the terms of the
+// row that are linear in (u, v, p, mu) from the per-step coefficients, over
+// differences to the edge's own velocity (so that a smooth e keeps its relative
+// accuracy in FP32), plus 1/2 (A rho(c') - A rho^n) e/dt and 1/2 A (rho(c') -
+// rho(C)) U/dt.  rs and ds: the sums of rho(c') and of rho(c') - rho(C) over
+// the edge's two cells.
 template <typename T, class LV>
-__device__ __forceinline__ T opd_p(const Prm<T>& P, const LV& L, int k) { return op_p(P, L, k); }
-
-// x row: the terms of op_u that are linear in (u, v, p, mu), applied to e, plus
-// 1/2 (A_x rho(c') - A_x rho^n) e_u/dt + 1/2 A_x(rho(c') - rho(C)) U/dt
-template <typename T, class LV>
-__device__ __forceinline__ T opd_u(const Prm<T>& P, const LV& L, int k) {
-  const int W = L.pitch;
-  auto u = L.u; auto vis = L.visn; auto rn = L.rhon;
-  T ue = u[k];
-  T cl = L.Bc[k] + L.c[k], cr = L.Bc[k + 1] + L.c[k + 1];
-  T rpl = rho_of(P, cl), rpr = rho_of(P, cr);
-  T Arp = T(0.5) * (rpl + rpr);
-  T dAr = T(0.5) * (rsec_(P, rpl, rho_of(P, L.Bc[k])) * L.c[k] +
-                    rsec_(P, rpr, rho_of(P, L.Bc[k + 1])) * L.c[k + 1]);
-  T dxl = (ue - u[k - 1]) * L.ih, dxr = (u[k + 1] - ue) * L.ih;
-  T dvl = dxl + (L.v[k] - L.v[k - W]) * L.ih;
-  T dvr = dxr + (L.v[k + 1] - L.v[k + 1 - W]) * L.ih;
-  T Dt = (u[k + W] - ue) * L.ih, Db = (ue - u[k - W]) * L.ih;
-  T Arn = L.Aru[k];
-  T conv = T(0.5) * (L.Sx[k + 1] * dxr + L.Sx[k] * dxl + L.Qx[k] * Dt + L.Qx[k - W] * Db);
-  T time = Arn * ue * P.idt + T(0.5) * (Arp - Arn) * P.idt * ue + T(0.5) * dAr * P.idt * L.Bu[k] +
-           L.Dvu[k] * ue;
-  T press = (L.p[k + 1] - L.p[k]) * L.ih * P.iM;
-  T st = -(rn[k + 1] * L.mu[k] + rn[k] * L.mu[k + 1]) * L.Tx[k] * P.iM;
-  T vl = vis[k], vr = vis[k + 1];
-  T visc = -P.iRe * L.ih * ((vr * dxr - vl * dxl) + (L.Av[k] * Dt - L.Av[k - W] * Db) +
-                            (vr * dvr - vl * dvl) * T(1.0 / 3.0));
-  return time + conv + press + st + visc;
+__device__ __forceinline__ T err_row(const Prm<T>& P, const LV& L, int d, int k, T rs, T ds) {
+  const int s = d ? L.pitch : 1, t = d ? 1 : L.pitch;
+  auto a = L.pair(d, L.u, L.v);
+  auto b = L.pair(1 - d, L.u, L.v);
+  auto rn = L.rhon;
+  auto mu = L.mu;
+  T ae = a[k];
+  T r = (L.pair(d, L.T1u, L.T1v)[k] + L.k.qidt * rs) * ae +
+        L.k.qidt * ds * L.pair(d, L.Bu, L.Bv)[k];
+  r += L.pair(d, L.aPu, L.aPv)[k] * (a[k + s] - ae);
+  r += L.pair(d, L.aMu, L.aMv)[k] * (a[k - s] - ae);
+  r += L.pair(d, L.tPu, L.tPv)[k] * (a[k + t] - ae);
+  r += L.pair(d, L.tMu, L.tMv)[k] * (a[k - t] - ae);
+  T vl = L.visn[k], vr = L.visn[k + s];
+  r -= L.k.v3 * (vr * (b[k + s] - b[k + s - t]) - vl * (b[k] - b[k - t]));
+  r += (L.p[k + s] - L.p[k]) * L.k.ihM;
+  r -= (rn[k + s] * mu[k] + rn[k] * mu[k + s]) * (L.pair(d, L.Tx, L.Ty)[k] * P.iM);
+  return r;
 }
-
+// the row's diagonal entry in its own velocity; gp, gm: 2 where the neighbour
+// across on that side is a wall's reflected ghost, else 1
 template <typename T, class LV>
-__device__ __forceinline__ T opd_v(const Prm<T>& P, const LV& L, int k) {
-  const int W = L.pitch;
-  auto v = L.v; auto vis = L.visn; auto rn = L.rhon;
-  T ve = v[k];
-  T cb = L.Bc[k] + L.c[k], ct = L.Bc[k + W] + L.c[k + W];
-  T rpb = rho_of(P, cb), rpt = rho_of(P, ct);
-  T Arp = T(0.5) * (rpb + rpt);
-  T dAr = T(0.5) * (rsec_(P, rpb, rho_of(P, L.Bc[k])) * L.c[k] +
-                    rsec_(P, rpt, rho_of(P, L.Bc[k + W])) * L.c[k + W]);
-  T dyb = (ve - v[k - W]) * L.ih, dyt = (v[k + W] - ve) * L.ih;
-  T dvb = dyb + (L.u[k] - L.u[k - 1]) * L.ih;
-  T dvt = dyt + (L.u[k + W] - L.u[k + W - 1]) * L.ih;
-  T De = (v[k + 1] - ve) * L.ih, Dw = (ve - v[k - 1]) * L.ih;
-  T Arn = L.Arv[k];
-  T conv = T(0.5) * (L.Qy[k] * De + L.Qy[k - 1] * Dw + L.Sy[k + W] * dyt + L.Sy[k] * dyb);
-  T time = Arn * ve * P.idt + T(0.5) * (Arp - Arn) * P.idt * ve + T(0.5) * dAr * P.idt * L.Bv[k] +
-           L.Dvv[k] * ve;
-  T press = (L.p[k + W] - L.p[k]) * L.ih * P.iM;
-  T st = -(rn[k + W] * L.mu[k] + rn[k] * L.mu[k + W]) * L.Ty[k] * P.iM;
-  T vb = vis[k], vt = vis[k + W];
-  T visc = -P.iRe * L.ih * ((L.Av[k] * De - L.Av[k - 1] * Dw) + (vt * dyt - vb * dyb) +
-                            (vt * dvt - vb * dvb) * T(1.0 / 3.0));
-  return time + conv + press + st + visc;
+__device__ __forceinline__ T err_diag(const LV& L, int d, int k, T rs, T gp, T gm) {
+  return L.pair(d, L.T1u, L.T1v)[k] + L.k.qidt * rs - L.pair(d, L.aPu, L.aPv)[k] -
+         L.pair(d, L.aMu, L.aMv)[k] - gp * L.pair(d, L.tPu, L.tPv)[k] -
+         gm * L.pair(d, L.tMu, L.tMv)[k];
 }
 
 // Two forms of the iterate: Full (x itself, Sec. 6.1) and Err (correction e to

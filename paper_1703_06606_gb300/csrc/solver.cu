@@ -399,6 +399,7 @@ int alloc_all(qnsch_s* s) {
     L.kcol = colours_of(a, s->px);
     L.c8 = s->px && a % 4 == 0;
     L.pitch = pitch;
+    L.nst = (long long)n;
     L.h = h;
     L.ih = 1.0 / h;
     L.ih2 = 1.0 / (h * h);
@@ -454,11 +455,11 @@ int alloc_all(qnsch_s* s) {
   return sync(s);
 }
 
-// error-equation levels: the 38 arrays of a level without the per-step row
-// coefficients, the assembled momentum stencils and rho(c) of the iterate
-// (their operators use none of them), plus the base Bc, Bmu, Bu, Bv, Bdc
-constexpr int NFIELD_ERR = NFIELD - 7 - 14 + 5;
-static_assert(NFIELD_ERR == 43, "error-level arrays");
+// error-equation levels: the unknowns, right-hand sides, residuals and kept
+// iterate (20 arrays), c^n and its four derived cell fields, the momentum rows
+// as T1 and their four neighbour coefficients (10), D c^n / 2 (2), and the
+// base Bc, Bmu, Bu, Bv, Bdc with rho(Bc)
+constexpr int NFIELD_ERR = 43;
 
 template <typename T>
 int alloc_err_levels(qnsch_s* s, std::vector<Lv<T>>& E) {
@@ -492,15 +493,16 @@ int alloc_err_levels(qnsch_s* s, std::vector<Lv<T>>& E) {
     L.kcol = D.kcol;
     L.c8 = D.c8;
     L.pitch = D.pitch;
+    L.nst = (long long)n;
     L.h = (T)D.h;
     L.ih = (T)D.ih;
     L.ih2 = (T)D.ih2;
     T** f[NFIELD_ERR] = {&L.c,   &L.mu,  &L.p,   &L.u,   &L.v,    &L.fc,  &L.fmu, &L.fp,
                          &L.fu,  &L.fv,  &L.rc,  &L.rmu, &L.rp,   &L.ru,  &L.rv,  &L.sc,
-                         &L.smu, &L.sp,  &L.su,  &L.sv,  &L.cn,   &L.un,  &L.vn,  &L.rhon,
-                         &L.mobn, &L.visn, &L.Gn, &L.Aru, &L.Arv, &L.Sx,  &L.Sy,  &L.Qx,
-                         &L.Qy,  &L.Av,  &L.Tx,  &L.Ty,  &L.Dvu,  &L.Dvv, &L.Bc,  &L.Bmu,
-                         &L.Bu,  &L.Bv,  &L.Bdc};
+                         &L.smu, &L.sp,  &L.su,  &L.sv,  &L.cn,   &L.rhon, &L.mobn, &L.visn,
+                         &L.Gn,  &L.T1u, &L.T1v, &L.aPu, &L.aPv, &L.aMu, &L.aMv, &L.tPu,
+                         &L.tPv, &L.tMu, &L.tMv, &L.Tx,  &L.Ty,  &L.Bc,  &L.Bmu, &L.Bu,
+                         &L.Bv,  &L.Bdc, &L.rB};
     for (int q = 0; q < NFIELD_ERR; ++q) *f[q] = base + (size_t)q * n + D.pitch + 1;
   }
   s->blocks.insert(s->blocks.end(), got.begin(), got.end());
@@ -977,11 +979,11 @@ template <typename T>
 void correction_cycle(qnsch_s* s, std::vector<Lv<T>>& E) {
   Prm<double> P64 = make_prm(s);
   Prm<T> P = cast_prm<T>(P64);
-  qn::launch_start_correction(s->L[0], E[0], s->stream);
+  qn::launch_start_correction(P, s->L[0], E[0], s->stream);
   // the base state on every level; the single-block V-cycle restricts it to
   // the levels below its first one itself
   int f = fused_from(s, E);
-  for (int l = 1; l < s->nlev && l <= f; ++l) qn::launch_restrict_base(E[l - 1], E[l], s->stream);
+  for (int l = 1; l < s->nlev && l <= f; ++l) qn::launch_restrict_base(P, E[l - 1], E[l], s->stream);
   vcycle<T, ErrForm>(s, E, P, 0);
   qn::launch_apply_correction(P64, s->L[0], E[0], s->stream);
 }

@@ -54,8 +54,11 @@ def test_one_cycle_matches_the_global_memory_launch(qn, name, m1, m2, px, opts):
         x0 = s.get_iterate()
         s.vcycle()
         out.append(s.get_iterate())
-    for k in x0:
-        size = np.max(np.abs(out[1][k] - x0[k]))
+    sizes = {k: np.max(np.abs(out[1][k] - x0[k])) for k in x0}
+    # u and v are the components of one vector: a component that is zero by
+    # symmetry (u on the 2 x 2 grid) holds only the rounding of the other's rows
+    sizes["u"] = sizes["v"] = max(sizes["u"], sizes["v"])
+    for k, size in sizes.items():
         assert np.max(np.abs(out[0][k] - out[1][k])) <= 1e-4 * size + 1e-300, k
 
 
