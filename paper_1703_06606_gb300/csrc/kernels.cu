@@ -300,7 +300,7 @@ __device__ __forceinline__ void residual_cell(const Prm<T>& P, const LV& L, int 
 // 2 BY rows, so that a 256x512 grid fits the GPU in one round of blocks and
 // the norms' reduction is shared by two cells.
 template <typename T, int MODE, class Form, int ROWS>
-__global__ void k_residual(Prm<T> P, Lv<T> L, double* part) {
+__global__ void __launch_bounds__(NT, 2) k_residual(Prm<T> P, Lv<T> L, double* part) {
   pdl_enter();
   int i = blockIdx.x * BX + threadIdx.x + 1;
   int j = blockIdx.y * (ROWS * BY) + threadIdx.y + 1;
@@ -573,7 +573,7 @@ __device__ __forceinline__ bool ch_slot_cell(const LV& L, int colour, int t, int
 
 // cells of CH colour `colour` ((i + j) % 2), packed: slot t -> row t / mpr + 1
 template <typename T, class Form>
-__global__ void __launch_bounds__(64) k_ch(Prm<T> P, Lv<T> L, int colour) {
+__global__ void __launch_bounds__(64, 4) k_ch(Prm<T> P, Lv<T> L, int colour) {
   pdl_enter();
   int t = blockIdx.x * 64 + threadIdx.x, i, j;
   if (t >= L.crow.d * L.m2 || !ch_slot_cell(L, colour, t, i, j)) return;
@@ -616,6 +616,17 @@ __device__ __forceinline__ RhoPair<T> rho_pair(const Prm<T>& P, const LV& L, int
   if constexpr (std::is_same<Form, ErrForm>::value) return {r, rsec_(P, r, L.rB[k]) * L.c[k]};
   else return {r, T(0)};
 }
+
+// Whether small launches in T give a visit four lanes.  In FP64 a warp's
+// instruction holds its pipe for 64 cycles or more whatever its lanes do, so a
+// visit split over four lanes is a shorter chain.  In FP32 the chain is loads
+// and their latency, and one lane that has all of them in flight at once
+// (launch bounds that leave it the registers) is as fast on the smallest level
+// and twice as fast on the largest: coupled visits 4.4 us a colour on 14x14 to
+// 56x56 levels and 6.1 us on 448x448 with one lane, 4.5 and 12.5 us (512x512)
+// with four.
+template <typename T>
+constexpr bool lane_teams = sizeof(T) == 8;
 
 // sums over the four lanes of a team of eight values each lane holds, every
 // lane receiving all eight: the first exchange halves what a lane adds up
@@ -826,7 +837,7 @@ __device__ __forceinline__ void ch_team(const Prm<T>& P, const LV& L, int i, int
 
 // per-level CH launch with four lanes per cell (colour (i + j) % 2, packed)
 template <typename T, class Form>
-__global__ void __launch_bounds__(64) k_ch_team(Prm<T> P, Lv<T> L, int colour) {
+__global__ void __launch_bounds__(64, 4) k_ch_team(Prm<T> P, Lv<T> L, int colour) {
   pdl_enter();
   int n = L.crow.d * L.m2;
   int t = blockIdx.x * 64 + threadIdx.x;
@@ -1183,7 +1194,7 @@ __device__ __forceinline__ int vanka_colour(const LV& L, int i, int j) {
 constexpr int SNT = 64;
 
 template <typename T, class Form>
-__global__ void __launch_bounds__(SNT) k_vanka(Prm<T> P, Lv<T> L, int colour, T omega) {
+__global__ void __launch_bounds__(SNT, 4) k_vanka(Prm<T> P, Lv<T> L, int colour, T omega) {
   pdl_enter();
   ColourSlots cs = vanka_slots(L, colour);
   int t = blockIdx.x * SNT + threadIdx.x;
@@ -1193,7 +1204,7 @@ __global__ void __launch_bounds__(SNT) k_vanka(Prm<T> P, Lv<T> L, int colour, T 
 }
 
 template <typename T, class Form>
-__global__ void __launch_bounds__(SNT) k_coupled(Prm<T> P, Lv<T> L, int colour, T omega) {
+__global__ void __launch_bounds__(SNT, 4) k_coupled(Prm<T> P, Lv<T> L, int colour, T omega) {
   pdl_enter();
   ColourSlots cs = vanka_slots(L, colour);
   int t = blockIdx.x * SNT + threadIdx.x;
@@ -1226,7 +1237,7 @@ __device__ __forceinline__ void vanka4_cell(const Prm<T>& P, const LV& L, int i,
 }
 
 template <typename T, class Form>
-__global__ void __launch_bounds__(SNT) k_vanka4(Prm<T> P, Lv<T> L, int colour, T omega) {
+__global__ void __launch_bounds__(SNT, 4) k_vanka4(Prm<T> P, Lv<T> L, int colour, T omega) {
   pdl_enter();
   ColourSlots cs = vanka_slots(L, colour);
   int t = blockIdx.x * SNT + threadIdx.x;
@@ -1283,7 +1294,7 @@ __device__ __forceinline__ void pgs_team(const Prm<T>& P, const LV& L, int i, in
 }
 
 template <typename T>
-__global__ void __launch_bounds__(64) k_pgs_team(Prm<T> P, Lv<T> L, int colour) {
+__global__ void __launch_bounds__(64, 4) k_pgs_team(Prm<T> P, Lv<T> L, int colour) {
   pdl_enter();
   int n = L.crow.d * L.m2;
   int t = blockIdx.x * 64 + threadIdx.x;
@@ -1296,7 +1307,7 @@ __global__ void __launch_bounds__(64) k_pgs_team(Prm<T> P, Lv<T> L, int colour) 
 
 // cells of colour (i + j) % 2 == colour, packed as in k_ch
 template <typename T>
-__global__ void __launch_bounds__(64) k_pgs(Prm<T> P, Lv<T> L, int colour) {
+__global__ void __launch_bounds__(64, 4) k_pgs(Prm<T> P, Lv<T> L, int colour) {
   pdl_enter();
   int t = blockIdx.x * 64 + threadIdx.x, i, j;
   if (t >= L.crow.d * L.m2 || !ch_slot_cell(L, colour, t, i, j)) return;
@@ -1429,7 +1440,7 @@ __device__ __forceinline__ void fill_v_ghost(const LV& L, A a, int I, int J) {
 }
 
 template <typename T>
-__global__ void k_bc_unknowns(Lv<T> L) {
+__global__ void __launch_bounds__(NT, 2) k_bc_unknowns(Lv<T> L) {
   pdl_enter();
   int t = blockIdx.x * blockDim.x + threadIdx.x;
   int I, J;
@@ -1443,7 +1454,7 @@ __global__ void k_bc_unknowns(Lv<T> L) {
 }
 
 template <typename T>
-__global__ void k_bc_frozen(Lv<T> L) {
+__global__ void __launch_bounds__(NT, 2) k_bc_frozen(Lv<T> L) {
   pdl_enter();
   int t = blockIdx.x * blockDim.x + threadIdx.x;
   int I, J;
@@ -1455,7 +1466,7 @@ __global__ void k_bc_frozen(Lv<T> L) {
 
 // rho(c^n), m(c^n), mu(c^n) on the whole ghosted cell range; G(c^n) inside
 template <typename T>
-__global__ void k_frozen_derived(Prm<T> P, Lv<T> L) {
+__global__ void __launch_bounds__(NT, 2) k_frozen_derived(Prm<T> P, Lv<T> L) {
   pdl_enter();
   int i = blockIdx.x * BX + threadIdx.x;
   int j = blockIdx.y * BY + threadIdx.y;
@@ -1470,7 +1481,7 @@ __global__ void k_frozen_derived(Prm<T> P, Lv<T> L) {
 
 // frozen coefficients of (pm-num-mx): cells and vertices (needs rho^n, mu(c^n), ghosts)
 template <typename T>
-__global__ void k_frozen_coef1(Lv<T> L) {
+__global__ void __launch_bounds__(NT, 2) k_frozen_coef1(Lv<T> L) {
   pdl_enter();
   int i = blockIdx.x * BX + threadIdx.x;
   int j = blockIdx.y * BY + threadIdx.y;
@@ -1494,7 +1505,7 @@ __global__ void k_frozen_coef1(Lv<T> L) {
 
 // divergence corrections of (e1e1-2) on edges (needs k_frozen_coef1)
 template <typename T>
-__global__ void k_frozen_coef2(Lv<T> L) {
+__global__ void __launch_bounds__(NT, 2) k_frozen_coef2(Lv<T> L) {
   pdl_enter();
   int i = blockIdx.x * BX + threadIdx.x;
   int j = blockIdx.y * BY + threadIdx.y;
@@ -1542,7 +1553,7 @@ __device__ __forceinline__ void assemble_row(const Prm<T>& P, const LV& L, int k
 // diagonal entry (the whole entry is Dg + A rho(c)/(2dt)), with the reflected
 // no-slip ghosts doubling the tangential wall terms (g = 2)
 template <typename T>
-__global__ void k_frozen_coef3(Prm<T> P, Lv<T> L) {
+__global__ void __launch_bounds__(NT, 2) k_frozen_coef3(Prm<T> P, Lv<T> L) {
   pdl_enter();
   int i = blockIdx.x * BX + threadIdx.x;
   int j = blockIdx.y * BY + threadIdx.y;
@@ -1610,7 +1621,7 @@ __device__ __forceinline__ void restrict_state_cell(const Prm<T>& P, const LV& F
 // coarse iterate = R x_h (cells: 4-mean; edges: mean of the 2 coincident fine edges),
 // and a copy kept for the correction
 template <typename T>
-__global__ void k_restrict_state(Prm<T> P, Lv<T> F, Lv<T> C) {
+__global__ void __launch_bounds__(NT, 2) k_restrict_state(Prm<T> P, Lv<T> F, Lv<T> C) {
   pdl_enter();
   int I = blockIdx.x * BX + threadIdx.x;
   int J = blockIdx.y * BY + threadIdx.y;
@@ -1669,7 +1680,7 @@ __device__ __forceinline__ void restrict_res_cell(const LV& F, const LV& C, int 
 }
 
 template <typename T>
-__global__ void k_restrict_res(Lv<T> F, Lv<T> C) {
+__global__ void __launch_bounds__(NT, 2) k_restrict_res(Lv<T> F, Lv<T> C) {
   pdl_enter();
   int I = blockIdx.x * BX + threadIdx.x + 1;
   int J = blockIdx.y * BY + threadIdx.y + 1;
@@ -1678,7 +1689,7 @@ __global__ void k_restrict_res(Lv<T> F, Lv<T> C) {
 }
 
 template <typename T>
-__global__ void k_restrict_frozen(Lv<T> F, Lv<T> C) {
+__global__ void __launch_bounds__(NT, 2) k_restrict_frozen(Lv<T> F, Lv<T> C) {
   pdl_enter();
   int I = blockIdx.x * BX + threadIdx.x;
   int J = blockIdx.y * BY + threadIdx.y;
@@ -1736,7 +1747,7 @@ __device__ __forceinline__ void prolong_cell(const Prm<T>& P, const LV& F, const
 }
 
 template <typename T>
-__global__ void k_prolong(Prm<T> P, Lv<T> F, Lv<T> C) {
+__global__ void __launch_bounds__(NT, 2) k_prolong(Prm<T> P, Lv<T> F, Lv<T> C) {
   pdl_enter();
   int i = blockIdx.x * BX + threadIdx.x + 1;
   int j = blockIdx.y * BY + threadIdx.y + 1;
@@ -2190,7 +2201,7 @@ __device__ __forceinline__ void coupled_team(const Prm<T>& P, const LV& L, int i
 // split over four lanes.  Whole warps past the last team return together, so
 // every warp that calls vanka_team has all 32 lanes in it.
 template <typename T>
-__global__ void __launch_bounds__(SNT) k_vanka4_team(Prm<T> P, Lv<T> L, int colour, T omega) {
+__global__ void __launch_bounds__(SNT, 4) k_vanka4_team(Prm<T> P, Lv<T> L, int colour, T omega) {
   pdl_enter();
   ColourSlots cs = vanka_slots(L, colour);
   int t = blockIdx.x * SNT + threadIdx.x;
@@ -2202,7 +2213,7 @@ __global__ void __launch_bounds__(SNT) k_vanka4_team(Prm<T> P, Lv<T> L, int colo
 }
 
 template <typename T, class Form>
-__global__ void __launch_bounds__(SNT) k_coupled_team(Prm<T> P, Lv<T> L, int colour, T omega) {
+__global__ void __launch_bounds__(SNT, 4) k_coupled_team(Prm<T> P, Lv<T> L, int colour, T omega) {
   pdl_enter();
   ColourSlots cs = vanka_slots(L, colour);
   int t = blockIdx.x * SNT + threadIdx.x;
@@ -2215,7 +2226,7 @@ __global__ void __launch_bounds__(SNT) k_coupled_team(Prm<T> P, Lv<T> L, int col
 
 // per-level launch with eight lanes per Vanka block (vanka_team8; FP64 full
 // iterate)
-__global__ void __launch_bounds__(SNT) k_vanka_team8(Prm<double> P, Lv<double> L, int colour,
+__global__ void __launch_bounds__(SNT, 4) k_vanka_team8(Prm<double> P, Lv<double> L, int colour,
                                                      double omega) {
   pdl_enter();
   ColourSlots cs = vanka_slots(L, colour);
@@ -2228,7 +2239,7 @@ __global__ void __launch_bounds__(SNT) k_vanka_team8(Prm<double> P, Lv<double> L
 }
 
 template <typename T, class Form>
-__global__ void __launch_bounds__(SNT) k_vanka_team(Prm<T> P, Lv<T> L, int colour, T omega) {
+__global__ void __launch_bounds__(SNT, 4) k_vanka_team(Prm<T> P, Lv<T> L, int colour, T omega) {
   pdl_enter();
   ColourSlots cs = vanka_slots(L, colour);
   int t = blockIdx.x * SNT + threadIdx.x;
@@ -2324,7 +2335,7 @@ __device__ __forceinline__ void vanka_pair(const Prm<T>& P, const LV& L, int i, 
 // per-level launch with a lane pair per Vanka block (vanka_pair; FP64 full
 // iterate).  Whole warps past the last pair return together.
 template <typename T, class Form>
-__global__ void __launch_bounds__(SNT) k_vanka_pair(Prm<T> P, Lv<T> L, int colour, T omega) {
+__global__ void __launch_bounds__(SNT, 4) k_vanka_pair(Prm<T> P, Lv<T> L, int colour, T omega) {
   pdl_enter();
   ColourSlots cs = vanka_slots(L, colour);
   int t = blockIdx.x * SNT + threadIdx.x;
@@ -2344,7 +2355,7 @@ __global__ void __launch_bounds__(SNT) k_vanka_pair(Prm<T> P, Lv<T> L, int colou
 // round of pair warps for the remainder issues fewer FP64 instructions on the
 // busiest sub-partition than a second, mostly empty single-lane round.
 template <typename T, class Form>
-__global__ void __launch_bounds__(SNT) k_vanka_split(Prm<T> P, Lv<T> L, int colour, T omega,
+__global__ void __launch_bounds__(SNT, 4) k_vanka_split(Prm<T> P, Lv<T> L, int colour, T omega,
                                                      int nsingle) {
   pdl_enter();
   ColourSlots cs = vanka_slots(L, colour);
@@ -2427,13 +2438,13 @@ __device__ __forceinline__ void smooth_block(const Prm<T>& P, const LV& L, T ome
     for (int col = 0; col < kcol; ++col) {
       ColourSlots cs = vanka_slots(L, col);
       // four lanes per block while the colour fits the block in one pass
-      if (4 * cs.n <= grp_size()) {
+      if (lane_teams<T> && 4 * cs.n <= grp_size()) {
         int t = grp_rank();
         if ((t & ~31) < 4 * cs.n) {  // warp-uniform: the warp holds at least one team
           int i = 1, j = 1;
           bool ok = (t >> 2) < cs.n && vanka_slot_cell(L, col, cs, t >> 2, i, j);
           if (!ok) i = j = 1;
-          coupled_team<T, Form>(P, L, i, j, ok, omega);
+          if constexpr (lane_teams<T>) coupled_team<T, Form>(P, L, i, j, ok, omega);
         }
       } else {
         for (int t = grp_rank(); t < cs.n; t += grp_size()) {
@@ -2447,7 +2458,7 @@ __device__ __forceinline__ void smooth_block(const Prm<T>& P, const LV& L, T ome
   }
   const int mpr = L.crow.d;
   constexpr bool team_ok = std::is_same<Form, FullForm>::value && sizeof(T) == 8;
-  constexpr bool vteam_ok = team_ok || std::is_same<Form, ErrForm>::value;
+  constexpr bool vteam_ok = lane_teams<T>;
   for (int col = 0; col < 2; ++col) {
     if (vteam_ok && 4 * mpr * L.m2 <= grp_size()) {
       int t = grp_rank();
@@ -2455,7 +2466,7 @@ __device__ __forceinline__ void smooth_block(const Prm<T>& P, const LV& L, T ome
         int i = 1, j = 1;
         bool ok = (t >> 2) < mpr * L.m2 && ch_slot_cell(L, col, t >> 2, i, j);
         if (!ok) i = j = 1;
-        ch_team<T, Form>(P, L, i, j, ok);
+        if constexpr (vteam_ok) ch_team<T, Form>(P, L, i, j, ok);
       }
     } else {
       for (int t = grp_rank(); t < mpr * L.m2; t += grp_size()) {
@@ -2467,8 +2478,8 @@ __device__ __forceinline__ void smooth_block(const Prm<T>& P, const LV& L, T ome
   }
   for (int col = 0; col < kcol; ++col) {
     ColourSlots cs = vanka_slots(L, col);
-    // FP64: while the colour fits one warp per sub-partition of the group; the
-    // latency-bound FP32 error levels: while it fits the group in one pass
+    // while the colour fits one warp per sub-partition of the group (full
+    // iterate), or the group in one pass (FP64 error levels)
     const int team_slots = team_ok ? QN_TEAM_MAX_SLOTS * (int)gridDim.x : grp_size() / 4;
     if (team_ok && team8 && 8 * cs.n <= grp_size()) {  // eight lanes per block
       int t = grp_rank();
@@ -2484,7 +2495,7 @@ __device__ __forceinline__ void smooth_block(const Prm<T>& P, const LV& L, T ome
         int i = 1, j = 1;
         bool ok = (t >> 2) < cs.n && vanka_slot_cell(L, col, cs, t >> 2, i, j);
         if (!ok) i = j = 1;
-        vanka_team<T, Form>(P, L, i, j, ok, omega);
+        if constexpr (vteam_ok) vanka_team<T, Form>(P, L, i, j, ok, omega);
       }
     } else {
       for (int t = grp_rank(); t < cs.n; t += grp_size()) {
@@ -2560,7 +2571,7 @@ struct LevelsOf {
 };
 
 template <typename T, class Form, int NT>
-__global__ void __launch_bounds__(NT) k_coarse_vcycle(Prm<T> P, CoarseLevels<T> C, int nu1, int nu2,
+__global__ void __launch_bounds__(NT, 1) k_coarse_vcycle(Prm<T> P, CoarseLevels<T> C, int nu1, int nu2,
                                                       int nuc, int kcol, T omega, int coupled,
                                                       int team8) {
   pdl_enter();
@@ -2620,7 +2631,7 @@ __device__ __forceinline__ void coarse_copy(double* __restrict__ g, int pg, long
 }
 
 template <int NT>
-__global__ void __launch_bounds__(NT) k_coarse_vcycle_smem(Prm<double> P, CoarseLevels<double> C,
+__global__ void __launch_bounds__(NT, 1) k_coarse_vcycle_smem(Prm<double> P, CoarseLevels<double> C,
                                                            CoarseSmem M, int copy, int nu1, int nu2,
                                                            int nuc, double omega, int coupled,
                                                            int team8) {
@@ -2745,7 +2756,7 @@ struct ErrLevels {
 };
 
 template <int NT>
-__global__ void __launch_bounds__(NT) k_coarse_err(Prm<rf32> P, const __grid_constant__ CoarseLevels<rf32> C,
+__global__ void __launch_bounds__(NT, 1) k_coarse_err(Prm<rf32> P, const __grid_constant__ CoarseLevels<rf32> C,
                                                    const __grid_constant__ ErrSmem M, int nu1, int nu2,
                                                    int nuc, rf32 omega, int coupled) {
   extern __shared__ __align__(16) float qn_err_words[];
@@ -2824,13 +2835,13 @@ __device__ __forceinline__ void wave_pass(const Prm<T>& P, const LV& L, const Wa
   if (!W.coupled && q < 2) {  // CH colour q: packed as in k_ch
     const int mpr = L.crow.d;
     const int t_lo = (r0 - 1) * mpr, t_hi = r1 * mpr;
-    if (mpr * L.m2 <= W.ch_team_max) {
+    if (lane_teams<T> && mpr * L.m2 <= W.ch_team_max) {
       for (int base = t_lo; base < t_hi; base += nt / 4) {
         if (base + ((tid & ~31) >> 2) >= t_hi) continue;  // warp-uniform
         int t = base + (tid >> 2), i = 1, j = 1;
         bool ok = t < t_hi && ch_slot_cell(L, q, t, i, j);
         if (!ok) i = j = 1;
-        ch_team<T, Form>(P, L, i, j, ok);
+        if constexpr (lane_teams<T>) ch_team<T, Form>(P, L, i, j, ok);
       }
     } else {
       for (int t = t_lo + tid; t < t_hi; t += nt) {
@@ -2847,14 +2858,16 @@ __device__ __forceinline__ void wave_pass(const Prm<T>& P, const LV& L, const Wa
   const int qlo = r0 > cs.j0 ? (r0 - cs.j0 + cs.rstep - 1) / cs.rstep : 0;
   const int qhi = (r1 - cs.j0) / cs.rstep;
   const int t_lo = qlo * cs.mpr, t_hi = min((qhi + 1) * cs.mpr, cs.n);
-  if (cs.n <= W.vanka_team_max) {
+  if (lane_teams<T> && cs.n <= W.vanka_team_max) {
     for (int base = t_lo; base < t_hi; base += nt / 4) {
       if (base + ((tid & ~31) >> 2) >= t_hi) continue;  // warp-uniform
       int t = base + (tid >> 2), i = 1, j = 1;
       bool ok = t < t_hi && vanka_slot_cell(L, col, cs, t, i, j);
       if (!ok) i = j = 1;
-      if (W.coupled) coupled_team<T, Form>(P, L, i, j, ok, omega);
-      else vanka_team<T, Form>(P, L, i, j, ok, omega);
+      if constexpr (lane_teams<T>) {
+        if (W.coupled) coupled_team<T, Form>(P, L, i, j, ok, omega);
+        else vanka_team<T, Form>(P, L, i, j, ok, omega);
+      }
     }
   } else {
     for (int t = t_lo + tid; t < t_hi; t += nt) {
@@ -2929,7 +2942,7 @@ __global__ void __launch_bounds__(WAVE_NT) k_wave(Prm<T> P, Lv<T> L, WavePlan W,
 // No block waits for another; stream order orders the launches.
 // --------------------------------------------------------------------------
 template <typename T, class Form, bool COUPLED>
-__global__ void __launch_bounds__(SNT) k_skew(Prm<T> P, Lv<T> L, SkewTasks S, T omega) {
+__global__ void __launch_bounds__(SNT, 4) k_skew(Prm<T> P, Lv<T> L, SkewTasks S, T omega) {
   pdl_enter();
   const int b = blockIdx.x;
   int k = 0;
@@ -2963,7 +2976,7 @@ struct FiveArrays {
   double* p[5];
 };
 
-__global__ void k_predict(FiveArrays X, FiveArrays A, FiveArrays B, FiveArrays C, double w0,
+__global__ void __launch_bounds__(NT, 2) k_predict(FiveArrays X, FiveArrays A, FiveArrays B, FiveArrays C, double w0,
                           double w1, double w2, long long n, int off) {
   pdl_enter();
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -2978,7 +2991,7 @@ __global__ void k_predict(FiveArrays X, FiveArrays A, FiveArrays B, FiveArrays C
 // --------------------------------------------------------------------------
 // error-equation frozen data = rounded FP64 frozen data (whole padded arrays)
 template <typename T>
-__global__ void k_cast_frozen(Lv<double> D, Lv<T> E, long long n, int off) {
+__global__ void __launch_bounds__(NT, 2) k_cast_frozen(Lv<double> D, Lv<T> E, long long n, int off) {
   pdl_enter();
   long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= n) return;
@@ -3005,7 +3018,7 @@ __global__ void k_cast_frozen(Lv<double> D, Lv<T> E, long long n, int off) {
 // base X = x (rounded), X.c - c^n formed in FP64, right-hand side = FP64 residual
 // (rounded), correction e = 0
 template <typename T>
-__global__ void k_start_correction(Prm<T> P, Lv<double> D, Lv<T> E, long long n, int off) {
+__global__ void __launch_bounds__(NT, 2) k_start_correction(Prm<T> P, Lv<double> D, Lv<T> E, long long n, int off) {
   pdl_enter();
   long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= n) return;
@@ -3030,7 +3043,7 @@ __global__ void k_start_correction(Prm<T> P, Lv<double> D, Lv<T> E, long long n,
 
 // x += e on the whole padded arrays (ghost rules are linear, so ghosts stay valid)
 template <typename T>
-__global__ void k_apply_correction(Prm<double> P, Lv<double> D, Lv<T> E, long long n, int off) {
+__global__ void __launch_bounds__(NT, 2) k_apply_correction(Prm<double> P, Lv<double> D, Lv<T> E, long long n, int off) {
   pdl_enter();
   long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= n) return;
@@ -3045,7 +3058,7 @@ __global__ void k_apply_correction(Prm<double> P, Lv<double> D, Lv<T> E, long lo
 
 // rho(c) of the iterate over the whole padded array, after c was written in
 // bulk (a new step's start, fields set from the host)
-__global__ void k_rho_fill(Prm<double> P, Lv<double> L, long long n, int off) {
+__global__ void __launch_bounds__(NT, 2) k_rho_fill(Prm<double> P, Lv<double> L, long long n, int off) {
   pdl_enter();
   long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= n) return;
@@ -3055,7 +3068,7 @@ __global__ void k_rho_fill(Prm<double> P, Lv<double> L, long long n, int off) {
 
 // coarse base X_H = R X_h (cells: 4-mean; edges: 2 coincident fine edges)
 template <typename T>
-__global__ void k_restrict_base(Prm<T> P, Lv<T> F, Lv<T> C) {
+__global__ void __launch_bounds__(NT, 2) k_restrict_base(Prm<T> P, Lv<T> F, Lv<T> C) {
   pdl_enter();
   int I = blockIdx.x * BX + threadIdx.x;
   int J = blockIdx.y * BY + threadIdx.y;
@@ -3064,7 +3077,7 @@ __global__ void k_restrict_base(Prm<T> P, Lv<T> F, Lv<T> C) {
 }
 
 template <typename T>
-__global__ void k_bc_base(Lv<T> L) {
+__global__ void __launch_bounds__(NT, 2) k_bc_base(Lv<T> L) {
   pdl_enter();
   int t = blockIdx.x * blockDim.x + threadIdx.x;
   int I, J;
@@ -3077,7 +3090,7 @@ __global__ void k_bc_base(Lv<T> L) {
 // reductions
 // --------------------------------------------------------------------------
 template <typename T>
-__global__ void k_sum_p(Lv<T> L, double* part) {
+__global__ void __launch_bounds__(NT, 2) k_sum_p(Lv<T> L, double* part) {
   pdl_enter();
   int i = blockIdx.x * BX + threadIdx.x + 1;
   int j = blockIdx.y * BY + threadIdx.y + 1;
@@ -3087,7 +3100,7 @@ __global__ void k_sum_p(Lv<T> L, double* part) {
 }
 
 template <typename T>
-__global__ void k_sub_mean_p(Lv<T> L, const double* sum, double inv_n) {
+__global__ void __launch_bounds__(NT, 2) k_sub_mean_p(Lv<T> L, const double* sum, double inv_n) {
   pdl_enter();
   int i = blockIdx.x * BX + threadIdx.x;
   int j = blockIdx.y * BY + threadIdx.y;
@@ -3097,7 +3110,7 @@ __global__ void k_sub_mean_p(Lv<T> L, const double* sum, double inv_n) {
 
 // mass: sum rho(c), sum rho(c) c over the cells (Thm. 6.1)
 template <typename T>
-__global__ void k_mass(Prm<T> P, Lv<T> L, const T* c, double* part) {
+__global__ void __launch_bounds__(NT, 2) k_mass(Prm<T> P, Lv<T> L, const T* c, double* part) {
   pdl_enter();
   int i = blockIdx.x * BX + threadIdx.x + 1;
   int j = blockIdx.y * BY + threadIdx.y + 1;
@@ -3134,7 +3147,7 @@ __device__ __forceinline__ double diag_div(const Lv<double>& L, const double* u,
 
 // per cell: [0] |div|, [1] max(div, 0), [2] max(-div, 0) (block maxima), then
 // the sums [3] c, [4] c a_y(v), [5] c y, [6] div^2
-__global__ void k_diag_cells(Lv<double> L, const double* c, const double* u, const double* v,
+__global__ void __launch_bounds__(NT, 2) k_diag_cells(Lv<double> L, const double* c, const double* u, const double* v,
                              double* part) {
   pdl_enter();
   int i = blockIdx.x * BX + threadIdx.x + 1;
@@ -3204,7 +3217,7 @@ __global__ void k_div_field(Lv<double> L, const double* u, const double* v, doub
 // energy E_h (Thm. 6.2): per cell rho [a_x(u^2) + a_y(v^2)]/2 + (eps eta/(2We)) rho G(c)
 // + (eta/(eps We)) rho F(c) + rho y / Fr; weights passed in w[0..2]
 template <typename T>
-__global__ void k_energy(Prm<T> P, Lv<T> L, const T* c, const T* u, const T* v, double w_grad,
+__global__ void __launch_bounds__(NT, 2) k_energy(Prm<T> P, Lv<T> L, const T* c, const T* u, const T* v, double w_grad,
                          double w_bulk, double w_pot, double* part) {
   pdl_enter();
   int i = blockIdx.x * BX + threadIdx.x + 1;
@@ -3231,7 +3244,7 @@ __global__ void k_energy(Prm<T> P, Lv<T> L, const T* c, const T* u, const T* v, 
 // thread (i,j) with i = 0..m1, j = 0..m2 handles vertex (i+1/2, j+1/2) and, for
 // i, j >= 1, cell (i,j) and its east / north faces.  w: [dt/Re, dt/(3Re), dt/(M Pe)]
 template <typename T>
-__global__ void k_dissipation(Prm<T> P, Lv<T> L, double w_visc, double w_div, double w_ch,
+__global__ void __launch_bounds__(NT, 2) k_dissipation(Prm<T> P, Lv<T> L, double w_visc, double w_div, double w_ch,
                               double* part) {
   pdl_enter();
   int i = blockIdx.x * BX + threadIdx.x;
@@ -3404,7 +3417,7 @@ void launch_ch(const Prm<T>& P0, const Lv<T>& L0, int colour, cudaStream_t s, in
   const Lv<R> L = as_compute<R>(level_consts(P0, L0));
   int n = (L.m1 + 1) / 2 * L.m2;
   if (n <= 0) return;
-  if constexpr (sizeof(T) == 8 || std::is_same<Form, ErrForm>::value) {
+  if constexpr (lane_teams<T>) {
     if (n <= team_max) {  // four lanes per cell: shorter critical path per visit
       qlaunch(&k_ch_team<R, Form>, (4 * n + 63) / 64, 64, 0, s, P, L, colour);
       ++g_launches;
@@ -3470,8 +3483,7 @@ void launch_vanka(const Prm<T>& P0, const Lv<T>& L0, int colour, T omega, cudaSt
       return;
     }
   }
-  if constexpr ((std::is_same<Form, FullForm>::value && sizeof(T) == 8) ||
-                std::is_same<Form, ErrForm>::value) {
+  if constexpr (lane_teams<T>) {
     if (n <= team_max) {  // four lanes per block: shorter critical path per visit
       qlaunch(&k_vanka_team<R, Form>, (4 * n + SNT - 1) / SNT, SNT, 0, s, P, L, colour, omega);
       ++g_launches;
@@ -3554,7 +3566,7 @@ void coarse_smem_prepare() {
   if (cudaDeviceGetAttribute(&v, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) == cudaSuccess &&
       v > 0) {
     cudaFuncSetAttribute(&k_coarse_vcycle_smem<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, v);
-    cudaFuncSetAttribute(&k_coarse_err<512>, cudaFuncAttributeMaxDynamicSharedMemorySize, v);
+    cudaFuncSetAttribute(&k_coarse_err<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, v);
   }
   cudaGetLastError();
 }
@@ -3584,7 +3596,7 @@ int launch_coarse_vcycle(const Prm<T>& P0, const Lv<T>* levels, int n, int nu1, 
     ErrSmem M = {};
     const size_t bytes = smem && ctas <= 1 ? coarse_err_plan(levels, n, M) : 0;
     if (bytes) {
-      qlaunch(&k_coarse_err<NT>, 1, NT, bytes, s, P, C, M, nu1, nu2, nuc, omega, coupled);
+      qlaunch(&k_coarse_err<256>, 1, 256, bytes, s, P, C, M, nu1, nu2, nuc, omega, coupled);
       ++g_launches;
       return 0;
     }
@@ -3710,10 +3722,12 @@ void launch_coupled(const Prm<T>& P0, const Lv<T>& L0, int colour, T omega, cuda
   const Lv<R> L = as_compute<R>(level_consts(P0, L0));
   int n = vanka_slots(L, colour).n;
   if (n <= 0) return;
-  if (n <= team_max) {  // four lanes per block: shorter critical path per visit
-    qlaunch(&k_coupled_team<R, Form>, (4 * n + SNT - 1) / SNT, SNT, 0, s, P, L, colour, omega);
-    ++g_launches;
-    return;
+  if constexpr (lane_teams<T>) {
+    if (n <= team_max) {  // four lanes per block: shorter critical path per visit
+      qlaunch(&k_coupled_team<R, Form>, (4 * n + SNT - 1) / SNT, SNT, 0, s, P, L, colour, omega);
+      ++g_launches;
+      return;
+    }
   }
   qlaunch(&k_coupled<R, Form>, (n + SNT - 1) / SNT, SNT, 0, s, P, L, colour, omega);
   ++g_launches;
