@@ -70,6 +70,14 @@ static void qlaunch(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, 
 // --------------------------------------------------------------------------
 // block reduction helpers (fixed order: deterministic for a fixed launch shape)
 // --------------------------------------------------------------------------
+// fmax of non-negative values or NaN (which the other operand replaces), by
+// their bit patterns: off the FP64 pipe
+__device__ __forceinline__ double max_bits(double x, double y) {
+  const long long inf = 0x7ff0000000000000LL;
+  const long long a = __double_as_longlong(x), b = __double_as_longlong(y);
+  return a > inf ? y : b > inf ? x : a > b ? x : y;
+}
+
 // sums over a warp of five values each lane holds; lane 0 receives them.  Two
 // exchanges first split the values over the lanes (4 + 2 additions), so the
 // warp issues 10 FP64 additions instead of 25.
@@ -125,43 +133,50 @@ __device__ __forceinline__ void block_sum_store(double (&val)[NV], double* part,
 #pragma unroll
     for (int q = 0; q < NV; ++q) {
       double x = sh[lane & (NT / 32 - 1)][q];  // lane 0 reduces the values of lanes 0 .. NT/32 - 1
-      if (q < nmax_first) {
-        long long b = __double_as_longlong(x);
-        for (int o = NT / 64; o > 0; o >>= 1) {
-          long long c = __shfl_down_sync(0xffffffffu, b, o);
-          b = c > b ? c : b;
-        }
-        x = __longlong_as_double(b);
-      } else {
-        for (int o = NT / 64; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
+      for (int o = NT / 64; o > 0; o >>= 1) {
+        const double y = __shfl_down_sync(0xffffffffu, x, o);
+        x = q < nmax_first ? max_bits(x, y) : x + y;
       }
       if (lane == 0) part[(blockIdx.y * gridDim.x + blockIdx.x) * NV + q] = x;
     }
   }
 }
 
-// Sum (or max) nparts rows of NV partials in a fixed order; one block of 256.
-__global__ void k_finalize(const double* part, int nparts, int nv, int nmax_first, double scale_sum,
-                           double* out) {
+// Sum (or max) nparts rows of nv <= 32 partials in a fixed order, in one block:
+// consecutive threads read consecutive partials (a thread's all of one
+// column), and a warp then adds each column's share.
+constexpr int FIN_NT = 1024;
+__global__ void __launch_bounds__(FIN_NT) k_finalize(const double* part, int nparts, int nv,
+                                                     int nmax_first, double scale_sum, double* out) {
   pdl_enter();
-  __shared__ double sh[256];
-  for (int q = 0; q < nv; ++q) {
-    bool mx = q < nmax_first;
-    double acc = 0.0;
-    for (int p = threadIdx.x; p < nparts; p += 256) {
-      double x = part[p * nv + q];
-      acc = mx ? fmax(acc, x) : acc + x;
+  __shared__ double sh[FIN_NT];
+  const int stride = FIN_NT / nv * nv, q = threadIdx.x % nv;
+  const bool mx = q < nmax_first;
+  double acc = 0.0;
+  if ((int)threadIdx.x < stride) {
+    const long long n = (long long)nparts * nv;
+#pragma unroll 4
+    for (long long p = threadIdx.x; p < n; p += stride) {
+      const double x = part[p];
+      if (mx) acc = max_bits(acc, x);
+      else acc += x;
     }
-    sh[threadIdx.x] = acc;
-    __syncthreads();
-    for (int s = 128; s > 0; s >>= 1) {
-      if (threadIdx.x < s) sh[threadIdx.x] = mx ? fmax(sh[threadIdx.x], sh[threadIdx.x + s])
-                                                 : sh[threadIdx.x] + sh[threadIdx.x + s];
-      __syncthreads();
-    }
-    if (threadIdx.x == 0) out[q] = mx ? sh[0] : sh[0] * scale_sum;
-    __syncthreads();
   }
+  sh[threadIdx.x] = acc;
+  __syncthreads();
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (w >= nv) return;
+  const bool wmx = w < nmax_first;
+  double x = 0.0;
+  for (int p = w + lane * nv; p < stride; p += 32 * nv) {
+    if (wmx) x = max_bits(x, sh[p]);
+    else x += sh[p];
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    const double y = __shfl_down_sync(0xffffffffu, x, o);
+    x = wmx ? max_bits(x, y) : x + y;
+  }
+  if (lane == 0) out[w] = wmx ? x : x * scale_sum;
 }
 
 // --------------------------------------------------------------------------
@@ -231,13 +246,16 @@ __device__ __forceinline__ T chem_full(const Prm<T>& P, const LV& L, int k, T rk
          P.alpha * rk * rnk * E;
 }
 
-// r = f - N(x) (MODE 0; val receives |r| and r^2 per family) or f += N(x) (MODE 1)
+// the residual's five rows at one cell: r = f - N(x) (MODE 0) or f + N(x) (MODE 1)
+template <typename T>
+struct Rows5 {
+  T r[5];
+};
 // at thread (i,j): cell families at (i,j), u-edge (i,j) and v-edge (i,j)
 template <typename T, int MODE, class Form, class LV>
-__device__ __forceinline__ void residual_cell(const Prm<T>& P, const LV& L, int i, int j,
-                                              double (&val)[10]) {
+__device__ __forceinline__ Rows5<T> residual_rows5(const Prm<T>& P, const LV& L, int i, int j) {
   int k = L.at(i, j);
-  bool hu = i <= L.uhi(), hv = j < L.m2;
+  const T f[5] = {L.fc[k], L.fmu[k], L.fp[k], L.fu[k], L.fv[k]};
   T nc, nm, np, nu, nv;
   if constexpr (std::is_same<Form, FullForm>::value) {
     // rho(c) of the cell and its neighbours, shared by the five rows, and the
@@ -273,58 +291,80 @@ __device__ __forceinline__ void residual_cell(const Prm<T>& P, const LV& L, int 
     nu = err_row(P, L, 0, k, X.r[0] + X.r[1], X.dr[0] + X.dr[1]);  // wall edges too, as above
     nv = err_row(P, L, 1, k, X.r[0] + X.r[3], X.dr[0] + X.dr[3]);
   }
+  const T n[5] = {nc, nm, np, nu, nv};
+  Rows5<T> X;
+#pragma unroll
+  for (int q = 0; q < 5; ++q) X.r[q] = MODE == 0 ? f[q] - n[q] : f[q] + n[q];
+  return X;
+}
+// stores them (MODE 0: into r, MODE 1: into f) and adds to val: the largest |r|
+// and the sum of r^2 per family (MODE 0)
+template <typename T, int MODE, class LV>
+__device__ __forceinline__ void residual_store(const LV& L, int i, int j, const Rows5<T>& X,
+                                               double (&val)[10]) {
+  const int k = L.at(i, j);
+  const bool own[5] = {true, true, true, i <= L.uhi(), j < L.m2};
   if (MODE == 0) {
-    T r[5] = {L.fc[k] - nc, L.fmu[k] - nm, L.fp[k] - np, hu ? L.fu[k] - nu : T(0),
-              hv ? L.fv[k] - nv : T(0)};
-    L.rc[k] = r[0];
-    L.rmu[k] = r[1];
-    L.rp[k] = r[2];
-    if (hu) L.ru[k] = r[3];
-    if (hv) L.rv[k] = r[4];
+    L.rc[k] = X.r[0];
+    L.rmu[k] = X.r[1];
+    L.rp[k] = X.r[2];
+    if (own[3]) L.ru[k] = X.r[3];
+    if (own[4]) L.rv[k] = X.r[4];
 #pragma unroll
     for (int q = 0; q < 5; ++q) {
-      double a = (double)r[q];
-      val[q] = fabs(a);
-      val[5 + q] = a * a;
+      const double a = own[q] ? (double)X.r[q] : 0.0;
+      // |r| >= 0 or NaN: the bit patterns order as the values
+      const long long b = __double_as_longlong(fabs(a)), m = __double_as_longlong(val[q]);
+      val[q] = __longlong_as_double(b > m ? b : m);
+      val[5 + q] += a * a;
     }
   } else {
-    L.fc[k] += nc;
-    L.fmu[k] += nm;
-    L.fp[k] += np;
-    if (hu) L.fu[k] += nu;
-    if (hv) L.fv[k] += nv;
+    L.fc[k] = X.r[0];
+    L.fmu[k] = X.r[1];
+    L.fp[k] = X.r[2];
+    if (own[3]) L.fu[k] = X.r[3];
+    if (own[4]) L.fv[k] = X.r[4];
   }
 }
+template <typename T, int MODE, class Form, class LV>
+__device__ __forceinline__ void residual_cell(const Prm<T>& P, const LV& L, int i, int j,
+                                              double (&val)[10]) {
+  residual_store<T, MODE>(L, i, j, residual_rows5<T, MODE, Form>(P, L, i, j), val);
+}
 
-// ROWS = 2 (large levels): each thread takes rows j and j + BY of a block of
-// 2 BY rows, so that a 256x512 grid fits the GPU in one round of blocks and
-// the norms' reduction is shared by two cells.
+// ROWS > 1 (large levels): each thread takes ROWS / 2 pairs of rows BY apart, so
+// that the norms' reduction is shared by ROWS cells.  Both rows of a pair are
+// evaluated before either is stored: the second's loads would wait behind
+// stores they might alias.
 template <typename T, int MODE, class Form, int ROWS>
 __global__ void __launch_bounds__(NT, 2) k_residual(Prm<T> P, Lv<T> L, double* part) {
   pdl_enter();
   int i = blockIdx.x * BX + threadIdx.x + 1;
   int j = blockIdx.y * (ROWS * BY) + threadIdx.y + 1;
   double val[10] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};  // max x5 then sum of squares x5
-  if (i <= L.m1 && j <= L.m2) residual_cell<T, MODE, Form>(P, L, i, j, val);
-  if (ROWS == 2 && i <= L.m1 && j + BY <= L.m2) {
-    double v2[10];
-    residual_cell<T, MODE, Form>(P, L, i, j + BY, v2);
-    if (MODE == 0) {
-#pragma unroll
-      for (int q = 0; q < 5; ++q) {  // |r| >= 0 or NaN: the bit patterns order as the values
-        long long a = __double_as_longlong(val[q]), b = __double_as_longlong(v2[q]);
-        val[q] = __longlong_as_double(a > b ? a : b);
-        val[5 + q] += v2[5 + q];
-      }
+  if (ROWS == 1) {
+    if (i <= L.m1 && j <= L.m2) residual_cell<T, MODE, Form>(P, L, i, j, val);
+  } else {
+#pragma unroll 1
+    for (int r = 0; r < ROWS; r += 2, j += 2 * BY) {
+      if (i > L.m1 || j > L.m2) break;
+      const bool two = j + BY <= L.m2;
+      const Rows5<T> A = residual_rows5<T, MODE, Form>(P, L, i, j);
+      const Rows5<T> B = residual_rows5<T, MODE, Form>(P, L, i, two ? j + BY : j);
+      residual_store<T, MODE>(L, i, j, A, val);
+      if (two) residual_store<T, MODE>(L, i, j + BY, B, val);
     }
   }
   if (MODE == 0 && part) block_sum_store<10>(val, part, 5);
 }
 
-// rows per residual thread on level L: two on levels of at least 65536 cells
+// rows per residual thread on level L: two on levels of at least 65536 cells,
+// eight where that still leaves the GPU several blocks an SM (2^21 cells: 1024
+// blocks), so that one block sums a quarter of the partials
 template <typename T>
 static int residual_rows(const Lv<T>& L) {
-  return (long long)L.m1 * L.m2 >= 65536 ? 2 : 1;
+  const long long n = (long long)L.m1 * L.m2;
+  return n >= (1LL << 21) ? 8 : n >= 65536 ? 2 : 1;
 }
 
 // --------------------------------------------------------------------------
@@ -3393,7 +3433,10 @@ void launch_residual(const Prm<T>& P0, const Lv<T>& L0, double* part, cudaStream
   typedef compute_t<T, Form> R;
   const Prm<R>& P = as_compute<R>(P0);
   const Lv<R> L = as_compute<R>(level_consts(P0, L0));
-  if (residual_rows(L) == 2)
+  const int rows = residual_rows(L);
+  if (rows == 8)
+    qlaunch(&k_residual<R, 0, Form, 8>, grid2(L.m1, (L.m2 + 7) / 8), dim3(BX, BY), 0, s, P, L, part);
+  else if (rows == 2)
     qlaunch(&k_residual<R, 0, Form, 2>, grid2(L.m1, (L.m2 + 1) / 2), dim3(BX, BY), 0, s, P, L, part);
   else
     qlaunch(&k_residual<R, 0, Form, 1>, grid2(L.m1, L.m2), dim3(BX, BY), 0, s, P, L, part);
@@ -3404,7 +3447,10 @@ void launch_add_op(const Prm<T>& P0, const Lv<T>& L0, cudaStream_t s) {
   typedef compute_t<T, Form> R;
   const Prm<R>& P = as_compute<R>(P0);
   const Lv<R> L = as_compute<R>(level_consts(P0, L0));
-  if (residual_rows(L) == 2)
+  const int rows = residual_rows(L);
+  if (rows == 8)
+    qlaunch(&k_residual<R, 1, Form, 8>, grid2(L.m1, (L.m2 + 7) / 8), dim3(BX, BY), 0, s, P, L, nullptr);
+  else if (rows == 2)
     qlaunch(&k_residual<R, 1, Form, 2>, grid2(L.m1, (L.m2 + 1) / 2), dim3(BX, BY), 0, s, P, L, nullptr);
   else
     qlaunch(&k_residual<R, 1, Form, 1>, grid2(L.m1, L.m2), dim3(BX, BY), 0, s, P, L, nullptr);
@@ -3711,7 +3757,7 @@ void launch_proj_diss(const Prm<T>& P, const Lv<T>& L, const T* uo, const T* vo,
                       double* out1, cudaStream_t s) {
   qlaunch(&k_proj_diss<T>, grid2(L.m1, L.m2), dim3(BX, BY), 0, s, P, L, uo, vo, part);
   ++g_launches;
-  qlaunch(&k_finalize, 1, 256, 0, s, part, nparts_cells(L), 1, 0, 0.5 * (double)L.h * (double)L.h, out1);
+  qlaunch(&k_finalize, 1, FIN_NT, 0, s, part, nparts_cells(L), 1, 0, 0.5 * (double)L.h * (double)L.h, out1);
   ++g_launches;
 }
 template <typename T, class Form>
@@ -3815,7 +3861,7 @@ template <typename T>
 void launch_gauge(const Lv<T>& L, double* part, double* scal, cudaStream_t s) {
   qlaunch(&k_sum_p<T>, grid2(L.m1, L.m2), dim3(BX, BY), 0, s, L, part);
   ++g_launches;
-  qlaunch(&k_finalize, 1, 256, 0, s, part, nparts_cells(L), 1, 0, 1.0, scal);
+  qlaunch(&k_finalize, 1, FIN_NT, 0, s, part, nparts_cells(L), 1, 0, 1.0, scal);
   ++g_launches;
   qlaunch(&k_sub_mean_p<T>, grid2(L.m1 + 2, L.m2 + 2), dim3(BX, BY), 0, s, L, scal,
                                                                      1.0 / ((double)L.m1 * L.m2));
@@ -3826,16 +3872,16 @@ void launch_norms_finalize(const Lv<T>& L, double* part, double* out10, cudaStre
   // part rows are [max x5, sum of squares x5]; out10 = [l2 x5, max x5] after the
   // host applies sqrt(h^2 *) to the sums; here: out[0..4] = max, out[5..9] = h^2 sum
   dim3 g = grid2(L.m1, (L.m2 + residual_rows(L) - 1) / residual_rows(L));  // k_residual's blocks
-  qlaunch(&k_finalize, 1, 256, 0, s, part, (int)(g.x * g.y), 10, 5, (double)L.h * (double)L.h, out10);
+  qlaunch(&k_finalize, 1, FIN_NT, 0, s, part, (int)(g.x * g.y), 10, 5, (double)L.h * (double)L.h, out10);
   ++g_launches;
 }
 void launch_diag(const Lv<double>& L, const double* c, const double* u, const double* v,
                  double* part, double* out11, cudaStream_t s) {
   qlaunch(&k_diag_cells, grid2(L.m1, L.m2), dim3(BX, BY), 0, s, L, c, u, v, part);
-  qlaunch(&k_finalize, 1, 256, 0, s, part, nparts_cells(L), 7, 3, 1.0, out11);
+  qlaunch(&k_finalize, 1, FIN_NT, 0, s, part, nparts_cells(L), 7, 3, 1.0, out11);
   int nb = (L.m1 + NT - 1) / NT;
   qlaunch(&k_diag_cols, nb, NT, 0, s, L, c, part);
-  qlaunch(&k_finalize, 1, 256, 0, s, part, nb, 4, 2, 1.0, out11 + 7);
+  qlaunch(&k_finalize, 1, FIN_NT, 0, s, part, nb, 4, 2, 1.0, out11 + 7);
   g_launches += 4;
 }
 void launch_div_field(const Lv<double>& L, const double* u, const double* v, double* out,
@@ -3848,7 +3894,7 @@ void launch_mass(const Prm<T>& P, const Lv<T>& L, const T* c, double* part, doub
                  cudaStream_t s) {
   qlaunch(&k_mass<T>, grid2(L.m1, L.m2), dim3(BX, BY), 0, s, P, L, c, part);
   ++g_launches;
-  qlaunch(&k_finalize, 1, 256, 0, s, part, nparts_cells(L), 2, 0, (double)L.h * (double)L.h, out2);
+  qlaunch(&k_finalize, 1, FIN_NT, 0, s, part, nparts_cells(L), 2, 0, (double)L.h * (double)L.h, out2);
   ++g_launches;
 }
 template <typename T>
@@ -3858,7 +3904,7 @@ void launch_energy(const Prm<T>& P, const Lv<T>& L, const T* c, const T* u, cons
   qlaunch(&k_energy<T>, grid2(L.m1, L.m2), dim3(BX, BY), 0, s, P, L, c, u, v, w_grad, w_bulk, w_pot,
                                                           part);
   ++g_launches;
-  qlaunch(&k_finalize, 1, 256, 0, s, part, nparts_cells(L), 1, 0, (double)L.h * (double)L.h, out1);
+  qlaunch(&k_finalize, 1, FIN_NT, 0, s, part, nparts_cells(L), 1, 0, (double)L.h * (double)L.h, out1);
   ++g_launches;
 }
 template <typename T>
@@ -3867,7 +3913,7 @@ void launch_dissipation(const Prm<T>& P, const Lv<T>& L, double w_visc, double w
   dim3 g = grid2(L.m1 + 1, L.m2 + 1);
   qlaunch(&k_dissipation<T>, g, dim3(BX, BY), 0, s, P, L, w_visc, w_div, w_ch, part);
   ++g_launches;
-  qlaunch(&k_finalize, 1, 256, 0, s, part, g.x * g.y, 1, 0, (double)L.h * (double)L.h, out1);
+  qlaunch(&k_finalize, 1, FIN_NT, 0, s, part, g.x * g.y, 1, 0, (double)L.h * (double)L.h, out1);
   ++g_launches;
 }
 template <typename T>
