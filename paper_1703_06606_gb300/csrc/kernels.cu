@@ -219,7 +219,7 @@ __device__ __forceinline__ typename LV::real adv_sum(const LV& L, int k) {
   return rn[k + 1] * L.Tx[k] * L.u[k] + rn[k - 1] * L.Tx[k - 1] * L.u[k - 1] +
          rn[k + W] * L.Ty[k] * L.v[k] + rn[k - W] * L.Ty[k - W] * L.v[k - W];
 }
-// (pm-num-chem) (op_mu with its constants folded): with S = rho + rho^n, A(c) =
+// (pm-num-chem) with its constants folded: with S = rho + rho^n, A(c) =
 // c (c - 1), 8 rho^{n+1/2} g = S (A + A^n)(c + c^n - 1) and 8 (F + F^n)/2 =
 // A^2 + (A^n)^2
 template <typename T, class LV>
@@ -268,8 +268,8 @@ __device__ __forceinline__ Rows5<T> residual_rows5(const Prm<T>& P, const LV& L,
     nc = rk * (L.c[k] - L.cn[k]) * P.idt + adv_sum(L, k) - L.k.dif * flux;
     nm = chem_full(P, L, k, rk, rq);
     np = (L.u[k] - L.u[k - 1] + L.v[k] - L.v[k - W]) * L.ih - L.k.adif * flux;
-    nu = op_u(P, L, k, rk + rq[0]);  // also on boundary edges (padded arrays); masked below
-    nv = op_v(P, L, k, rk + rq[2]);  // also on boundary edges (padded arrays); masked below
+    nu = mom_asm<true>(L, 0, k, rk + rq[0]);  // also on boundary edges (padded arrays); masked below
+    nv = mom_asm<true>(L, 1, k, rk + rq[2]);
   } else if constexpr (std::is_same<Form, ProjForm>::value) {
     const int W = L.pitch;
     auto rc = L.rhoc;
@@ -277,11 +277,12 @@ __device__ __forceinline__ Rows5<T> residual_rows5(const Prm<T>& P, const LV& L,
     const T rq[4] = {rc[k + 1], rc[k - 1], rc[k + W], rc[k - W]};
     T w[4];
     proj_faces(P, L, i, j, rk, rq, w);
-    nc = opp_c_w(P, L, k, rq, w);
-    nm = op_mu_r(P, L, k, rk, rq, L.rhon[k]);
-    np = opp_p_w(P, L, k, w);
-    nu = op_u<T, false>(P, L, k, rk + rq[0]);  // also on boundary edges (padded arrays); masked below
-    nv = op_v<T, false>(P, L, k, rk + rq[2]);  // also on boundary edges (padded arrays); masked below
+    T flux = flux_sum(P, L, k);
+    nc = opp_c_w(P, L, k, rq, w, flux);
+    nm = chem_full(P, L, k, rk, rq) + (L.rhon[k] - rk) * L.mu[k];  // rho^n in front of mu
+    np = opp_p_w(L, w, flux);
+    nu = mom_asm<false>(L, 0, k, rk + rq[0]);
+    nv = mom_asm<false>(L, 1, k, rk + rq[2]);
   } else {
     const ErrCell<T> X = err_cell(P, L, k);
     T flux = flux_sum(P, L, k);
@@ -372,13 +373,14 @@ static int residual_rows(const Lv<T>& L) {
 // of each cell with (i + j) % 2 == colour; neighbours frozen.  Faces on
 // Neumann walls do not contribute (their ghost follows the cell).
 // --------------------------------------------------------------------------
-// ch_system for the FP64 primitive form, with the constants and the terms
+// ch_system for the full iterate (PROJ: the projection method's form), with the
+// constants and the terms
 // common to the residuals and the Jacobian folded (chem_full's notation; E =
 // K ((F + F^n)/2) + (Lam/4) Gbar): about 115 FP64 instructions where the
 // unfolded sums take about 190.  On a wall face the ghost's c and c^n are the
 // cell's own, so its differences vanish and only the coefficients of c (2 rho
 // sums) and the mobilities need the face left out.
-template <typename T, class LV>
+template <bool PROJ, typename T, class LV>
 __device__ __forceinline__ void ch_system_full(const Prm<T>& P, const LV& L, int i, int j,
                                                T (&J)[2][2], T (&R)[2]) {
   const int W = L.pitch;
@@ -411,14 +413,27 @@ __device__ __forceinline__ void ch_system_full(const Prm<T>& P, const LV& L, int
   T A = ck * ck - ck, An = cnk * cnk - cnk, sA = A + An, t = ch - T(1), g4 = sA * t;
   T Gs = L.k.hih2 * G2 + L.Gn[k];
   T E = L.k.K8 * (A * A + An * An) + L.k.L4 * Gs;
-  R[0] = rk * dck * P.idt - L.fc[k] + adv_sum(L, k) - L.k.dif * flux;
-  R[1] = rk * muk - L.fmu[k] + L.k.L8 * div - L.k.K8 * (S * g4) - r * E;
+  R[1] = (PROJ ? rnk : rk) * muk - L.fmu[k] + L.k.L8 * div - L.k.K8 * (S * g4) - r * E;
   T tc = T(2) * ck - T(1);
-  J[0][0] = (rk + drho * dck) * P.idt;
   J[0][1] = L.k.dif * sm;
-  J[1][0] = drho * (muk + L.k.L8 * SD - L.k.K8 * g4) - L.k.K8 * (S * (tc * t + sA)) -
+  J[1][0] = drho * ((PROJ ? T(0) : muk) + L.k.L8 * SD - L.k.K8 * g4) - L.k.K8 * (S * (tc * t + sA)) -
             r * (L.k.K4 * (A * tc) - L.k.L4h * sd) - dr * E - L.k.L8 * SW;
-  J[1][1] = rk;
+  if constexpr (PROJ) {
+    // projection method: rho^n in the time derivative and in front of mu; the
+    // advection a(rho(c) D c u^{n+1}) differentiated in c_ij through D c only,
+    // with rho(c) of the neighbours and u^{n+1} at the iterate (the smoother's
+    // choice; the fixed point is the scheme's)
+    const T rq[4] = {rc[k + 1], rc[k - 1], rc[k + W], rc[k - W]};
+    T w[4];  // the face velocities u^{n+1} (E, W, N, S)
+    proj_faces(P, L, i, j, rk, rq, w);
+    R[0] = opp_c_w(P, L, k, rq, w, flux) - L.fc[k];
+    J[0][0] = rnk * P.idt + L.k.hih * (rq[1] * w[1] - rq[0] * w[0] + rq[3] * w[3] - rq[2] * w[2]);
+    J[1][1] = rnk;
+  } else {
+    R[0] = rk * dck * P.idt - L.fc[k] + adv_sum(L, k) - L.k.dif * flux;
+    J[0][0] = (rk + drho * dck) * P.idt;
+    J[1][1] = rk;
+  }
 }
 
 // ch_system for the error equation: the residuals of err_c and err_mu, and
@@ -464,78 +479,10 @@ __device__ __forceinline__ void ch_system_err(const Prm<T>& P, const LV& L, int 
 template <typename T, class Form, class LV>
 __device__ __forceinline__ void ch_system(const Prm<T>& P, const LV& L, int i, int j,
                                           T (&J)[2][2], T (&R)[2]) {
-  const int W = L.pitch;
-  int k = L.at(i, j);
-  const int off[4] = {1, -1, W, -W};
-  if constexpr (std::is_same<Form, FullForm>::value) {
-    ch_system_full(P, L, i, j, J, R);
-    return;
-  }
-  if constexpr (std::is_same<Form, ErrForm>::value) {
-    ch_system_err(P, L, i, j, err_cell(P, L, k), J, R);
-    return;
-  }
-  // rho(c) of the cell and its four neighbours, shared by N_c, N_mu and J
-  T rho, rq4[4];
-  rho = Form::rho(P, L, k);
-#pragma unroll
-  for (int f = 0; f < 4; ++f) rq4[f] = Form::rho(P, L, k + off[f]);
-  T Rc, Rm;
-  T wf[4];  // projection method: the face velocities u^{n+1} (E, W, N, S)
-  if constexpr (std::is_same<Form, ProjForm>::value) {
-    proj_faces(P, L, i, j, rho, rq4, wf);
-    Rc = opp_c_w(P, L, k, rq4, wf) - L.fc[k];
-    Rm = op_mu_r(P, L, k, rho, rq4, L.rhon[k]) - L.fmu[k];
-  } else {
-    Rc = Rm = T(0);
-  }
-  auto cn = L.cn; auto rn = L.rhon; auto mob = L.mobn;
-  // full values c, mu at which the local Jacobian is evaluated
-  T ck = Form::val_c(L, k), cnk = cn[k], mk = Form::val_mu(L, k);
-  T drho = -P.alpha * rho * rho;
-  T rnk = rn[k];
-  T rh = T(0.5) * (rho + rnk);
-  T chk = ck + cnk;  // 2 c^{n+1/2}
-  T r = -P.alpha * rho * rnk, dr = -P.alpha * drho * rnk;
-  bool wall[4] = {!L.px && i == L.m1, !L.px && i == 1, j == L.m2, j == 1};
-  T sm = 0, dG = 0, dd = 0, G2 = 0;
-#pragma unroll
-  for (int f = 0; f < 4; ++f) {
-    int q = k + off[f];
-    T cq = Form::val_c(L, q);
-    T d = cq - ck;
-    G2 += d * d;
-    if (wall[f]) continue;
-    sm += mob[k] + mob[q];
-    dG -= d;
-    T rq = T(0.5) * (rq4[f] + rn[q]);
-    dd += T(0.5) * drho * ((cq + cn[q]) - chk) - (rh + rq);
-  }
-  // sm = 2 sum A m; dG = h^2 dG/dc; dd = 4 h^2 d(div)/dc; G2 = 2 h^2 G(c)
-  T J11 = (rho + drho * (ck - cnk)) * P.idt;
-  T J12 = T(0.5) * sm * P.iPe * L.ih2;
-  T Gs = T(0.5) * G2 * L.ih2 + L.Gn[k];
-  T dbulk = T(0.5) * drho * gsec(ck, cnk) + rh * gsec_da(ck, cnk) + T(0.5) * fdw(ck) * r +
-            T(0.5) * (Fdw(ck) + Fdw(cnk)) * dr;
-  T dgrad = T(0.25) * P.Lam * (dG * L.ih2 * r + Gs * dr);
-  T J21 = drho * mk - P.K * dbulk - dgrad + P.Lam * T(0.25) * L.ih2 * dd;
-  T J22 = rho;
-  if constexpr (std::is_same<Form, ProjForm>::value) {
-    // projection method: rho^n in the time derivative and in front of mu; the
-    // advection a(rho(c) D c u^{n+1}) differentiated in c_ij through D c only,
-    // with rho(c) of the neighbours and u^{n+1} at the iterate (the smoother's
-    // choice; the fixed point is the scheme's)
-    J11 = rnk * P.idt + T(0.5) * (-rq4[0] * wf[0] + rq4[1] * wf[1]) * L.ih +
-          T(0.5) * (-rq4[2] * wf[2] + rq4[3] * wf[3]) * L.ih;
-    J21 = -P.K * dbulk - dgrad + P.Lam * T(0.25) * L.ih2 * dd;
-    J22 = rnk;
-  }
-  J[0][0] = J11;
-  J[0][1] = J12;
-  J[1][0] = J21;
-  J[1][1] = J22;
-  R[0] = Rc;
-  R[1] = Rm;
+  if constexpr (std::is_same<Form, ErrForm>::value)
+    ch_system_err(P, L, i, j, err_cell(P, L, L.at(i, j)), J, R);
+  else
+    ch_system_full<std::is_same<Form, ProjForm>::value>(P, L, i, j, J, R);
 }
 
 template <typename T, class Form, class LV>
@@ -637,11 +584,9 @@ __device__ __forceinline__ T proj_face_team(const Prm<T>& P, const LV& L, int k,
   const int a = hi ? k : k - off;
   auto vel = d ? L.v : L.u; auto c = L.c; auto mu = L.mu; auto p = L.p;
   T ra = hi ? rk : rn, rb = hi ? rn : rk;
-  T Ar = T(0.5) * (ra + rb);
-  T dp = (p[a + off] - p[a]) * L.ih;
-  T st = T(0.5) * (rb * mu[a] + ra * mu[a + off]) * (c[a + off] - c[a]) * L.ih;
-  T grav = d ? P.Fr_inv / P.idt : T(0);
-  return open ? vel[a] + (st - dp) * P.iM / (Ar * P.idt) - grav : T(0);
+  return open ? vel[a] + proj_kick(L, ra, rb, mu[a], mu[a + off], c[a + off] - c[a], p[a + off] - p[a]) -
+                    (d ? L.k.gdt : T(0))
+              : T(0);
 }
 
 // rho(c) of the full value at cell k and, on error levels, its difference to
@@ -696,8 +641,8 @@ __device__ __forceinline__ void team_sum8(double (&v)[8]) {
 // E, S, N; open = face q is not a wall): residuals Rc = N_c - f_c,
 // Rm = N_mu - f_mu and the 2x2 Jacobian of ch_system, and for the coupled
 // block the open-face sum of A m, the diffusion flux sum, d rho/dc and face
-// q's rho^n D c^n / 2.  Lane q evaluates face q's terms of N_c, N_mu (op_c and
-// op_mu, or opd_c and opd_mu on error levels) and of the Jacobian's face
+// q's rho^n D c^n / 2.  Lane q evaluates face q's terms of N_c, N_mu (err_c
+// and err_mu on error levels) and of the Jacobian's face
 // sums; butterflies add them and every lane forms the cell terms.
 template <typename T>
 struct ChRows {
@@ -705,7 +650,8 @@ struct ChRows {
   T sm, sflux, drho, gq;
 };
 
-// ch_team_rows for the FP64 primitive form: ch_system_full's sums, a face a lane
+// ch_team_rows for the full iterate: ch_system_full's sums, a face a lane
+template <bool PROJ>
 __device__ __forceinline__ ChRows<double> ch_team_rows_full(const Prm<double>& P,
                                                             const Lv<double>& L, int i, int j,
                                                             int q, bool open, double rk, double rq) {
@@ -721,9 +667,15 @@ __device__ __forceinline__ ChRows<double> ch_team_rows_full(const Prm<double>& P
   T gq = rnq * L.pair(d, L.Tx, L.Ty)[kf];  // rho^n D c^n / 2 at face q
   T m = mob[k] + mob[nq];
   T S = rk + rnk, ch = ck + cnk, dq = cq - ck, D = (cq + cn[nq]) - ch, H = rq + rnq;
+  // the projection method advects rho(c) c with u^{n+1} at the face
+  T wq = T(0), rw = T(0);
+  if constexpr (PROJ) {
+    wq = proj_face_team(P, L, k, q, open, rk, rq);
+    rw = rq * wq;
+  }
   T v[8] = {m * (L.mu[nq] + P.alpha * L.p[nq] - (muk + P.alpha * L.p[k])),
             open ? m : T(0),
-            gq * L.pair(d, L.u, L.v)[kf],
+            PROJ ? rw * ((q & 1) ? dq : -dq) : gq * L.pair(d, L.u, L.v)[kf],
             dq * dq,
             dq,
             (H + S) * D,
@@ -739,13 +691,19 @@ __device__ __forceinline__ ChRows<double> ch_team_rows_full(const Prm<double>& P
   T E = L.k.K8 * (A * A + An * An) + L.k.L4 * Gs;
   T tc = T(2) * ck - T(1);
   ChRows<T> R;
-  R.Rc = rk * dck * P.idt - L.fc[k] + adv - L.k.dif * flux;
-  R.Rm = rk * muk - L.fmu[k] + L.k.L8 * div - L.k.K8 * (S * g4) - r * E;
-  R.J11 = (rk + drho * dck) * P.idt;
+  if constexpr (PROJ) {
+    R.Rc = rnk * dck * P.idt - L.fc[k] + L.k.hih * adv - L.k.dif * flux;
+    R.J11 = rnk * P.idt + L.k.hih * team_sum<T>((q & 1) ? -rw : rw);
+    R.J22 = rnk;
+  } else {
+    R.Rc = rk * dck * P.idt - L.fc[k] + adv - L.k.dif * flux;
+    R.J11 = (rk + drho * dck) * P.idt;
+    R.J22 = rk;
+  }
+  R.Rm = (PROJ ? rnk : rk) * muk - L.fmu[k] + L.k.L8 * div - L.k.K8 * (S * g4) - r * E;
   R.J12 = L.k.dif * sm;
-  R.J21 = drho * (muk + L.k.L8 * SD - L.k.K8 * g4) - L.k.K8 * (S * (tc * t + sA)) -
+  R.J21 = drho * ((PROJ ? T(0) : muk) + L.k.L8 * SD - L.k.K8 * g4) - L.k.K8 * (S * (tc * t + sA)) -
           r * (L.k.K4 * (A * tc) - L.k.L4h * sd) - dr * E - L.k.L8 * SW;
-  R.J22 = rk;
   R.sm = sm;
   R.sflux = flux;
   R.drho = drho;
@@ -756,51 +714,37 @@ __device__ __forceinline__ ChRows<double> ch_team_rows_full(const Prm<double>& P
 template <typename T, class Form, class LV>
 __device__ __forceinline__ ChRows<T> ch_team_rows(const Prm<T>& P, const LV& L, int i, int j, int q,
                                                   bool open, RhoPair<T> ra, RhoPair<T> rb) {
-  if constexpr (std::is_same<Form, FullForm>::value) {
-    return ch_team_rows_full(P, L, i, j, q, open, ra.r, rb.r);
+  if constexpr (!std::is_same<Form, ErrForm>::value) {
+    return ch_team_rows_full<std::is_same<Form, ProjForm>::value>(P, L, i, j, q, open, ra.r, rb.r);
   } else {
-  const int W = L.pitch;
-  const int d = q >> 1;
-  const T ih2 = L.ih2;
-  int k = L.at(i, j);
-  auto mob = L.mobn; auto cn = L.cn; auto rn = L.rhon;
-  const int nq = k + (q == 0 ? -1 : q == 1 ? 1 : q == 2 ? -W : W);
-  const int kf = q == 0 ? k - 1 : (q == 2 ? k - W : k);  // edge of face q
-  // full values at the cell and at the face's neighbour
-  T ck = Form::val_c(L, k), cnk = cn[k], mk = Form::val_mu(L, k), rnk = rn[k];
-  T rho = ra.r;
-  T cq = Form::val_c(L, nq), rq = rb.r;
-  T drho = -P.alpha * rho * rho;
-  T rh = T(0.5) * (rho + rnk);
-  T chk = ck + cnk;
-  T am = mob[nq] + mob[k];
-  T gq = rn[nq] * L.pair(d, L.Tx, L.Ty)[kf];  // rho^n D c^n / 2 at face q
-  T dlt = cq - ck;
-  // face sums: diffusion flux (N_c and the mass row), sum A m over open faces,
-  // advection of N_c, and the Jacobian's G, dG/dc and d(div)/dc terms
-  T sflux = team_sum<T>(am * ((L.mu[nq] - L.mu[k]) + P.alpha * (L.p[nq] - L.p[k])));
-  T sm = team_sum<T>(open ? am : T(0));
-  T sadv = team_sum<T>(gq * L.pair(d, L.u, L.v)[kf]);
-  T G2 = team_sum<T>(dlt * dlt);
-  T dG = team_sum<T>(open ? -dlt : T(0));
-  T dd = team_sum<T>(open ? T(0.5) * drho * ((cq + cn[nq]) - chk) - (rh + T(0.5) * (rq + rn[nq])) : T(0));
-  T Nc, Nm;
-  T wq = T(0), sJ11 = T(0);  // projection method: u^{n+1} at face q, its advection Jacobian
-  if constexpr (std::is_same<Form, ProjForm>::value) {
-    wq = proj_face_team(P, L, k, q, open, rho, rq);
-    // advection a(rho(c) D c u^{n+1}) of (pj-num-phase) by faces
-    T sadvp = team_sum<T>(T(0.5) * rq * ((q & 1) ? (cq - ck) : (ck - cq)) * L.ih * wq);
-    Nc = rnk * (ck - cnk) * P.idt + sadvp - L.k.dif * sflux;
-    T sdv = team_sum<T>((rh + T(0.5) * (rq + rn[nq])) * ((cq + cn[nq]) - chk));
-    T r = -P.alpha * rho * rnk;
-    T bulk = rh * gsec(ck, cnk) + T(0.5) * (Fdw(ck) + Fdw(cnk)) * r;
-    T grad = T(0.25) * P.Lam * (T(0.5) * G2 * ih2 + L.Gn[k]) * r;
-    Nm = rnk * mk - P.K * bulk - grad + P.Lam * T(0.25) * ih2 * sdv;
-    sJ11 = team_sum<T>(T(0.5) * ((q & 1) ? -rq * wq : rq * wq) * L.ih);
-  } else if constexpr (std::is_same<Form, ErrForm>::value) {
+    const int W = L.pitch;
+    const int d = q >> 1;
+    const T ih2 = L.ih2;
+    int k = L.at(i, j);
+    auto mob = L.mobn; auto cn = L.cn; auto rn = L.rhon;
+    const int nq = k + (q == 0 ? -1 : q == 1 ? 1 : q == 2 ? -W : W);
+    const int kf = q == 0 ? k - 1 : (q == 2 ? k - W : k);  // edge of face q
+    // full values at the cell and at the face's neighbour
+    T ck = Form::val_c(L, k), cnk = cn[k], mk = Form::val_mu(L, k), rnk = rn[k];
+    T rho = ra.r;
+    T cq = Form::val_c(L, nq), rq = rb.r;
+    T drho = -P.alpha * rho * rho;
+    T rh = T(0.5) * (rho + rnk);
+    T chk = ck + cnk;
+    T am = mob[nq] + mob[k];
+    T gq = rn[nq] * L.pair(d, L.Tx, L.Ty)[kf];  // rho^n D c^n / 2 at face q
+    T dlt = cq - ck;
+    // face sums: diffusion flux (N_c and the mass row), sum A m over open faces,
+    // advection of N_c, and the Jacobian's G, dG/dc and d(div)/dc terms
+    T sflux = team_sum<T>(am * ((L.mu[nq] - L.mu[k]) + P.alpha * (L.p[nq] - L.p[k])));
+    T sm = team_sum<T>(open ? am : T(0));
+    T sadv = team_sum<T>(gq * L.pair(d, L.u, L.v)[kf]);
+    T G2 = team_sum<T>(dlt * dlt);
+    T dG = team_sum<T>(open ? -dlt : T(0));
+    T dd = team_sum<T>(open ? T(0.5) * drho * ((cq + cn[nq]) - chk) - (rh + T(0.5) * (rq + rn[nq])) : T(0));
     auto e = L.c; auto B = L.Bc;
     T ek = e[k], Ck = B[k];
-    Nc = ek * (rho + rsec_(P, rho, L.rB[k]) * L.Bdc[k]) * P.idt + sadv - L.k.dif * sflux;
+    T Nc = ek * (rho + rsec_(P, rho, L.rB[k]) * L.Bdc[k]) * P.idt + sadv - L.k.dif * sflux;
     T dC = B[nq] - Ck, de = e[nq] - ek;
     T dr = ra.d;
     T drq = rb.d;
@@ -814,39 +758,24 @@ __device__ __forceinline__ ChRows<T> ch_team_rows(const Prm<T>& P, const LV& L, 
     T dbulk = rh * dgsec(Ck, cnk, ek) + T(0.5) * dr * gsec(Ck, cnk) + T(0.5) * dF * r_new +
               T(0.5) * (Fdw(Ck) + Fdw(cnk)) * d_r;
     T dgrad = T(0.25) * P.Lam * (T(0.5) * sdGe * ih2 * r_new + (T(0.5) * sGC * ih2 + L.Gn[k]) * d_r);
-    Nm = rho * L.mu[k] + dr * L.Bmu[k] - P.K * dbulk - dgrad + P.Lam * T(0.25) * ih2 * sddiv;
-  } else {
-    Nc = rho * (ck - cnk) * P.idt + sadv - L.k.dif * sflux;
-    T sdv = team_sum<T>((rh + T(0.5) * (rq + rn[nq])) * ((cq + cn[nq]) - chk));
-    T r = -P.alpha * rho * rnk;
-    T bulk = rh * gsec(ck, cnk) + T(0.5) * (Fdw(ck) + Fdw(cnk)) * r;
-    T grad = T(0.25) * P.Lam * (T(0.5) * G2 * ih2 + L.Gn[k]) * r;
-    Nm = rho * mk - P.K * bulk - grad + P.Lam * T(0.25) * ih2 * sdv;
-  }
-  ChRows<T> R;
-  R.Rc = Nc - L.fc[k];
-  R.Rm = Nm - L.fmu[k];
-  T r = -P.alpha * rho * rnk, drr = -P.alpha * drho * rnk;
-  R.J11 = (rho + drho * (ck - cnk)) * P.idt;
-  R.J12 = L.k.dif * sm;
-  T Gs = T(0.5) * G2 * ih2 + L.Gn[k];
-  T dbulkJ = T(0.5) * drho * gsec(ck, cnk) + rh * gsec_da(ck, cnk) + T(0.5) * fdw(ck) * r +
-             T(0.5) * (Fdw(ck) + Fdw(cnk)) * drr;
-  T dgradJ = T(0.25) * P.Lam * (dG * ih2 * r + Gs * drr);
-  R.J21 = drho * mk - P.K * dbulkJ - dgradJ + P.Lam * T(0.25) * ih2 * dd;
-  R.J22 = rho;
-  if constexpr (std::is_same<Form, ProjForm>::value) {
-    // ch_system's projection branch: rho^n in the time derivative and in front
-    // of mu; the advection differentiated through D c only
-    R.J11 = rnk * P.idt + sJ11;
-    R.J21 = -P.K * dbulkJ - dgradJ + P.Lam * T(0.25) * ih2 * dd;
-    R.J22 = rnk;
-  }
-  R.sm = sm;
-  R.sflux = sflux;
-  R.drho = drho;
-  R.gq = gq;
-  return R;
+    T Nm = rho * L.mu[k] + dr * L.Bmu[k] - P.K * dbulk - dgrad + P.Lam * T(0.25) * ih2 * sddiv;
+    ChRows<T> R;
+    R.Rc = Nc - L.fc[k];
+    R.Rm = Nm - L.fmu[k];
+    T r = -P.alpha * rho * rnk, drr = -P.alpha * drho * rnk;
+    R.J11 = (rho + drho * (ck - cnk)) * P.idt;
+    R.J12 = L.k.dif * sm;
+    T Gs = T(0.5) * G2 * ih2 + L.Gn[k];
+    T dbulkJ = T(0.5) * drho * gsec(ck, cnk) + rh * gsec_da(ck, cnk) + T(0.5) * fdw(ck) * r +
+               T(0.5) * (Fdw(ck) + Fdw(cnk)) * drr;
+    T dgradJ = T(0.25) * P.Lam * (dG * ih2 * r + Gs * drr);
+    R.J21 = drho * mk - P.K * dbulkJ - dgradJ + P.Lam * T(0.25) * ih2 * dd;
+    R.J22 = rho;
+    R.sm = sm;
+    R.sflux = sflux;
+    R.drho = drho;
+    R.gq = gq;
+    return R;
   }
 }
 
@@ -948,8 +877,7 @@ __device__ __forceinline__ void vanka_system(const Prm<T>& P, const LV& L, int i
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       A[q][q] = (q < 2 ? L.Dgu : L.Dgv)[ke[q]] + L.k.qidt * rs[q];  // per-step coefficients
-      if (q < 2) rows[q] = op_u<T, PST>(P, L, ke[q], rs[q]);
-      else rows[q] = op_v<T, PST>(P, L, ke[q], rs[q]);
+      rows[q] = mom_asm<PST>(L, q >> 1, ke[q], rs[q]);
     }
     const T v1 = vis[k] * L.k.v1, sx = L.k.hih * L.Sx[k], sy = L.k.hih * L.Sy[k];
     A[0][1] = sx - v1 - v3;
@@ -1298,7 +1226,7 @@ __device__ __forceinline__ void pgs_cell(const Prm<T>& P, const LV& L, int i, in
   const T rq[4] = {rc[k + 1], rc[k - 1], rc[k + W], rc[k - W]};
   T w[4];
   proj_faces(P, L, i, j, rk, rq, w);
-  T R = opp_p_w(P, L, k, w) - L.fp[k];
+  T R = opp_p_w(L, w, flux_sum(P, L, k)) - L.fp[k];
   const bool wall[4] = {!L.px && i == L.m1, !L.px && i == 1, j == L.m2, j == 1};
   const int off[4] = {1, -1, W, -W};
   T d = T(0);
@@ -1306,10 +1234,9 @@ __device__ __forceinline__ void pgs_cell(const Prm<T>& P, const LV& L, int i, in
   for (int f = 0; f < 4; ++f) {
     if (wall[f]) continue;
     int q = k + off[f];
-    T Ar = T(0.5) * (rk + rq[f]);
-    d += P.iM / (Ar * P.idt) * L.ih2 + P.alpha * P.alpha * P.iPe * T(0.5) * (L.mobn[k] + L.mobn[q]) * L.ih2;
+    d += L.k.pdiv * qrcp(rk + rq[f]) + L.k.a2dif * (L.mobn[k] + L.mobn[q]);
   }
-  store_cell(L, L.p, i, j, L.p[k] - R / d);
+  put_cell(L, L.p, i, j, has_ghosts(L, i, j), L.p[k] - R * qrcp(d));
 }
 
 // pgs_cell by a team of four lanes (lane & 3 = q: face W, E, S, N): lane q
@@ -1326,11 +1253,11 @@ __device__ __forceinline__ void pgs_team(const Prm<T>& P, const LV& L, int i, in
   T wq = proj_face_team(P, L, k, q, open, rk, rq);
   T am = L.mobn[nq] + L.mobn[k];
   T sdiv = team_sum<T>((q & 1) ? wq : -wq);
-  T sflux = team_sum<T>(T(0.5) * am * ((L.mu[nq] - L.mu[k]) + P.alpha * (L.p[nq] - L.p[k])));
-  T Ar = T(0.5) * (rk + rq);
-  T sd = team_sum<T>(open ? P.iM / (Ar * P.idt) * L.ih2 + P.alpha * P.alpha * P.iPe * T(0.5) * am * L.ih2 : T(0));
-  T R = sdiv * L.ih - P.alpha * P.iPe * L.ih2 * sflux - L.fp[k];
-  if (ok && q == 0) store_cell(L, L.p, i, j, L.p[k] - R / sd);
+  T sflux = team_sum<T>(am * ((L.mu[nq] - L.mu[k]) + P.alpha * (L.p[nq] - L.p[k])));
+  T sd = team_sum<T>(open ? L.k.pdiv * qrcp(rk + rq) + L.k.a2dif * am : T(0));
+  T R = sdiv * L.ih - L.k.adif * sflux - L.fp[k];
+  const T pn = L.p[k] - R * qrcp(sd);
+  if (ok && q == 0) put_cell(L, L.p, i, j, has_ghosts(L, i, j), pn);
 }
 
 template <typename T>
@@ -1894,8 +1821,8 @@ __device__ __forceinline__ void bc_unknowns_block(const LV& L) {
 // the cells of the colour, and on the smallest levels four lanes share one
 // Vanka block (one edge row each).
 // --------------------------------------------------------------------------
-// N - f of the momentum row in direction d (0: the x row, op_u, unknown u; 1:
-// the y row, op_v, unknown v; opd_u / opd_v for ErrForm) at edge index k, from
+// N - f of the momentum row in direction d (0: the x row, unknown u; 1:
+// the y row, unknown v) at edge index k: mom_asm, or err_row for ErrForm, from
 // rho(c) of the edge's two cells; kf is the index of its right-hand side.  Both
 // directions run the same instructions on different arrays and strides (s
 // along the edge normal, t across it).
@@ -1903,30 +1830,10 @@ template <typename T, class Form, class LV>
 __device__ __forceinline__ T mom_residual(const Prm<T>& P, const LV& L, int d, int k, int kf,
                                           RhoPair<T> l, RhoPair<T> r) {
   const T f = L.pair(d, L.fu, L.fv)[kf];
-  if constexpr (std::is_same<Form, FullForm>::value && sizeof(T) == 8) {
-    return mom_asm(L, d, k, l.r + r.r) - f;
-  } else if constexpr (std::is_same<Form, ErrForm>::value) {
+  if constexpr (std::is_same<Form, ErrForm>::value)
     return err_row(P, L, d, k, l.r + r.r, l.d + r.d) - f;
-  } else {  // the projection method's intermediate-velocity row
-    const int s = d ? L.pitch : 1, t = d ? 1 : L.pitch;
-    auto a = L.pair(d, L.u, L.v);
-    auto b = L.pair(1 - d, L.u, L.v);
-    auto S = L.pair(d, L.Sx, L.Sy);
-    auto Q = L.pair(d, L.Qx, L.Qy);
-    auto vis = L.visn;
-    T ae = a[k];
-    T dl = (ae - a[k - s]) * L.ih, dr = (a[k + s] - ae) * L.ih;
-    T dvl = dl + (b[k] - b[k - t]) * L.ih;
-    T dvr = dr + (b[k + s] - b[k + s - t]) * L.ih;
-    T Dp = (a[k + t] - ae) * L.ih, Dm = (ae - a[k - t]) * L.ih;
-    T conv = T(0.5) * (S[k + s] * dr + S[k] * dl + Q[k] * Dp + Q[k - t] * Dm);
-    T time = ae * (L.pair(d, L.T1u, L.T1v)[k] + L.k.qidt * (l.r + r.r)) +
-             L.pair(d, L.T0u, L.T0v)[k];
-    T vl = vis[k], vr = vis[k + s];
-    T visc = -P.iRe * L.ih * ((vr * dr - vl * dl) + (L.Av[k] * Dp - L.Av[k - t] * Dm) +
-                              (vr * dvr - vl * dvl) * T(1.0 / 3.0));
-    return time + conv + visc - f;
-  }
+  else
+    return mom_asm<std::is_same<Form, FullForm>::value>(L, d, k, l.r + r.r) - f;
 }
 
 // Diagonal entry dq and residual bq = N - f (0 on a wall edge) of momentum row
@@ -3157,7 +3064,7 @@ __global__ void __launch_bounds__(NT, 2) k_mass(Prm<T> P, Lv<T> L, const T* c, d
   double val[2] = {0.0, 0.0};
   if (i <= L.m1 && j <= L.m2) {
     double cc = (double)c[L.at(i, j)];
-    double r = 1.0 / ((double)P.ia * cc + (double)P.ib);
+    double r = rcp_any((double)P.ia * cc + (double)P.ib);
     val[0] = r;
     val[1] = r * cc;
   }
@@ -3181,8 +3088,8 @@ __device__ __forceinline__ double diag_v(const Lv<double>& L, const double* v, i
 // d_x u + d_y v of cell (i,j)
 __device__ __forceinline__ double diag_div(const Lv<double>& L, const double* u, const double* v,
                                            int i, int j) {
-  return (diag_u(L, u, i, j) - diag_u(L, u, i - 1, j)) / L.h +
-         (diag_v(L, v, i, j) - diag_v(L, v, i, j - 1)) / L.h;
+  return (diag_u(L, u, i, j) - diag_u(L, u, i - 1, j)) * L.ih +
+         (diag_v(L, v, i, j) - diag_v(L, v, i, j - 1)) * L.ih;
 }
 
 // per cell: [0] |div|, [1] max(div, 0), [2] max(-div, 0) (block maxima), then
@@ -3208,38 +3115,34 @@ __global__ void __launch_bounds__(NT, 2) k_diag_cells(Lv<double> L, const double
   block_sum_store<7>(val, part, 3);
 }
 
-// one thread per column i: eta_i = h sum_j c_ij and the upward crossings
-// c_j >= 1/2 > c_{j+1} (linear between cell centres); [0] highest crossing,
-// [1] Ly - lowest crossing (block maxima), then the sums [2] eta_i cos(2 pi
-// x_i / Lx) and [3] columns with a crossing
+// per cell: the upward crossing c_j >= 1/2 > c_{j+1} above it (linear between
+// cell centres); [0] highest crossing, [1] Ly - lowest crossing (block maxima),
+// then the sums [2] h c cos(2 pi x_i / Lx), whose column sums are eta_i = h
+// sum_j c_ij, and [3] crossings.  A thread a cell: one thread a column walked
+// its rows one load behind the other (row 1's block took 75 us on 256x512).
+// The block's 32 cosines are formed once, by its first warp.
 __global__ void __launch_bounds__(NT) k_diag_cols(Lv<double> L, const double* c, double* part) {
   pdl_enter();
-  int i = blockIdx.x * NT + threadIdx.x + 1;
-  double val[4] = {0.0, 0.0, 0.0, 0.0};
-  if (i <= L.m1) {
-    const double h = L.h, Ly = L.m2 * h, Lx = L.m1 * h;
+  __shared__ double cosx[BX];
+  const int i = blockIdx.x * BX + threadIdx.x + 1, j = blockIdx.y * BY + threadIdx.y + 1;
+  const double h = L.h, Ly = L.m2 * h, Lx = L.m1 * h;
+  if (threadIdx.y == 0) {
     const double pi = 3.14159265358979323846;
-    double eta = 0.0, ytop = 0.0, ybot = Ly;
-    bool found = false;
-    double a = c[L.at(i, 1)];
-    eta += a;
-    for (int j = 1; j < L.m2; ++j) {
-      double b = c[L.at(i, j + 1)];
-      eta += b;
+    cosx[threadIdx.x] = cos(2.0 * pi * ((i - 0.5) * h) / Lx);
+  }
+  __syncthreads();
+  double val[4] = {0.0, 0.0, 0.0, 0.0};
+  if (i <= L.m1 && j <= L.m2) {
+    const double a = c[L.at(i, j)];
+    val[2] = h * a * cosx[threadIdx.x];
+    if (j < L.m2) {
+      const double b = c[L.at(i, j + 1)];
       if (a >= 0.5 && b < 0.5) {
-        double y = (j - 0.5) * h + h * (a - 0.5) / (a - b);
-        if (!found || y > ytop) ytop = y;
-        if (!found || y < ybot) ybot = y;
-        found = true;
+        const double y = (j - 0.5) * h + h * (a - 0.5) / (a - b);
+        val[0] = y;
+        val[1] = Ly - y;
+        val[3] = 1.0;
       }
-      a = b;
-    }
-    eta *= h;
-    val[2] = eta * cos(2.0 * pi * ((i - 0.5) * h) / Lx);
-    if (found) {
-      val[0] = ytop;
-      val[1] = Ly - ybot;
-      val[3] = 1.0;
     }
   }
   block_sum_store<4>(val, part, 2);
@@ -3267,15 +3170,15 @@ __global__ void __launch_bounds__(NT, 2) k_energy(Prm<T> P, Lv<T> L, const T* c,
     const int W = L.pitch;
     int k = L.at(i, j);
     double cc = (double)c[k];
-    double r = 1.0 / ((double)P.ia * cc + (double)P.ib);
+    double r = rcp_any((double)P.ia * cc + (double)P.ib);
     double u0 = u[k], u1 = u[k - 1], v0 = v[k], v1 = v[k - W];
     double kin = 0.25 * (u0 * u0 + u1 * u1 + v0 * v0 + v1 * v1);
     double de = (double)c[k + 1] - cc, dw = cc - (double)c[k - 1];
     double dn = (double)c[k + W] - cc, ds = cc - (double)c[k - W];
-    double G = 0.5 * (de * de + dw * dw + dn * dn + ds * ds) / ((double)L.h * (double)L.h);
-    double F = 0.25 * cc * cc * (cc - 1.0) * (cc - 1.0);
+    // (w_grad carries 1 / (2 h^2), w_bulk 1/4)
+    double A = cc * (cc - 1.0);
     double y = (j - 0.5) * (double)L.h;
-    val[0] = r * (kin + w_grad * G + w_bulk * F + w_pot * y);
+    val[0] = r * (kin + w_grad * (de * de + dw * dw + dn * dn + ds * ds) + w_bulk * (A * A) + w_pot * y);
   }
   block_sum_store<1>(val, part, 0);
 }
@@ -3748,7 +3651,8 @@ void launch_pgs(const Prm<T>& P0, const Lv<T>& L0, int colour, cudaStream_t s, i
   ++g_launches;
 }
 template <typename T>
-void launch_proj_velocity(const Prm<T>& P, const Lv<T>& L, T* uo, T* vo, cudaStream_t s) {
+void launch_proj_velocity(const Prm<T>& P, const Lv<T>& L0, T* uo, T* vo, cudaStream_t s) {
+  const Lv<T> L = level_consts(P, L0);
   qlaunch(&k_proj_velocity<T>, grid2(L.m1 + 1, L.m2 + 1), dim3(BX, BY), 0, s, P, L, uo, vo);
   ++g_launches;
 }
@@ -3879,9 +3783,8 @@ void launch_diag(const Lv<double>& L, const double* c, const double* u, const do
                  double* part, double* out11, cudaStream_t s) {
   qlaunch(&k_diag_cells, grid2(L.m1, L.m2), dim3(BX, BY), 0, s, L, c, u, v, part);
   qlaunch(&k_finalize, 1, FIN_NT, 0, s, part, nparts_cells(L), 7, 3, 1.0, out11);
-  int nb = (L.m1 + NT - 1) / NT;
-  qlaunch(&k_diag_cols, nb, NT, 0, s, L, c, part);
-  qlaunch(&k_finalize, 1, FIN_NT, 0, s, part, nb, 4, 2, 1.0, out11 + 7);
+  qlaunch(&k_diag_cols, grid2(L.m1, L.m2), dim3(BX, BY), 0, s, L, c, part);
+  qlaunch(&k_finalize, 1, FIN_NT, 0, s, part, nparts_cells(L), 4, 2, 1.0, out11 + 7);
   g_launches += 4;
 }
 void launch_div_field(const Lv<double>& L, const double* u, const double* v, double* out,
@@ -3901,8 +3804,9 @@ template <typename T>
 void launch_energy(const Prm<T>& P, const Lv<T>& L, const T* c, const T* u, const T* v,
                    double w_grad, double w_bulk, double w_pot, double* part, double* out1,
                    cudaStream_t s) {
-  qlaunch(&k_energy<T>, grid2(L.m1, L.m2), dim3(BX, BY), 0, s, P, L, c, u, v, w_grad, w_bulk, w_pot,
-                                                          part);
+  const double h = L.h;
+  qlaunch(&k_energy<T>, grid2(L.m1, L.m2), dim3(BX, BY), 0, s, P, L, c, u, v, w_grad * 0.5 / (h * h),
+          0.25 * w_bulk, w_pot, part);
   ++g_launches;
   qlaunch(&k_finalize, 1, FIN_NT, 0, s, part, nparts_cells(L), 1, 0, (double)L.h * (double)L.h, out1);
   ++g_launches;

@@ -15,6 +15,7 @@
 #include <mutex>
 
 #include "qnsch.h"
+#include "qnsch_dev.cuh"
 
 namespace {
 
@@ -56,6 +57,10 @@ int partials_address(void** out) {
   return QNSCH_OK;
 }
 
+// The FP64 pipe bounds the kernel (a warp's FP64 instruction takes 19 cycles of
+// an SM, and 2048 x 4096 cells are 1724 warps an SM: 15.8 us an instruction),
+// not HBM (67 MB, 10 us): a division's ten FP64 instructions were two thirds
+// of it.  With rcp_any 152 -> 100 us at that size.
 // rho(c) = 1 / (ia c + ib) with ia = (rho2 - rho1)/(rho1 rho2), ib = 1/rho2 (Sec. 2.1)
 __global__ void k_mass_partials(const double* __restrict__ c, long long n, double ia, double ib,
                                 double* __restrict__ part) {
@@ -67,7 +72,7 @@ __global__ void k_mass_partials(const double* __restrict__ c, long long n, doubl
     long long k = base + (long long)q * NA_THREADS + threadIdx.x;
     if (k < n) {
       double cc = c[k];
-      double r = 1.0 / (ia * cc + ib);
+      double r = qn::rcp_any(ia * cc + ib);
       a += r;
       b += r * cc;
     }

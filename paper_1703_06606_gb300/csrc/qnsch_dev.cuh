@@ -136,6 +136,8 @@ struct LvK {
   T hih2;              // 1/(2 h^2)
   T K8, K4;            // K/8, K/4
   T L4, L8, L4h;       // Lam/4, Lam/(8 h^2), Lam/(4 h^2)
+  T kick, hkick, gdt;  // 2 dt/(M h), half of it, dt/Fr: the projection equation
+  T pdiv;              // 2 dt/(M h^2): its derivative in the pressure
 };
 
 template <typename T>
@@ -212,7 +214,9 @@ inline Lv<T> level_consts(const Prm<T>& P, const Lv<T>& L) {
   X.k = {T(0.25 * P.idt), T(ih * iM),       T(P.iRe * ih2),         T(P.iRe * ih2 / 3.0),
          T(0.5 * ih),     T(dif),           T(al * dif),            T(al * al * dif),
          T(ih * ih * iM), T(0.5 * ih2),     T(0.125 * P.K),         T(0.25 * P.K),
-         T(0.25 * P.Lam), T(0.125 * P.Lam * ih2), T(0.25 * P.Lam * ih2)};
+         T(0.25 * P.Lam), T(0.125 * P.Lam * ih2), T(0.25 * P.Lam * ih2),
+         T(2.0 * ih * iM / P.idt), T(ih * iM / P.idt), T(P.Fr_inv / P.idt),
+         T(2.0 * ih2 * iM / P.idt)};
   X.vrow = fast_div(L.c8 ? (L.m1 + 3) / 4 : (L.m1 + L.kcol - 1) / L.kcol);
   X.crow = fast_div((L.m1 + 1) / 2);
   X.kdiv = fast_div(L.kcol);
@@ -259,6 +263,12 @@ template <> __device__ __forceinline__ double qrcp(double x) {
   return __fma_rn(r, e, r);
 }
 template <> __device__ __forceinline__ rf64 qrcp(rf64 x) { return qrcp(x.v); }
+// 1/x for any x: qrcp where the iteration's numbers stay normal, else the
+// division (zero, infinity, NaN, the ends of the exponent range)
+__device__ __forceinline__ double rcp_any(double x) {
+  const unsigned e = (unsigned)__double2hiint(x) & 0x7ff00000u;
+  return e - 0x01000000u < 0x7d000000u ? qrcp(x) : 1.0 / x;
+}
 template <> __device__ __forceinline__ double rho_of(const Prm<double>& P, double c) {
   return qrcp(P.ia * c + P.ib);
 }
@@ -305,92 +315,15 @@ __device__ __forceinline__ auto G_h2(A c, int k, int pitch) ->
   return T(0.5) * (de * de + dw * dw + dn * dn + ds * ds);
 }
 
-// h^2 grad_d.(A kap grad_D phi) at cell k
-template <class A, class B>
-__device__ __forceinline__ auto lap_h2(A kap, B phi, int k, int pitch) ->
-    typename std::decay<decltype(kap[k])>::type {
-  typedef typename std::decay<decltype(kap[k])>::type T;
-  T kc = kap[k], pc = phi[k];
-  return T(0.5) * ((kap[k + 1] + kc) * (phi[k + 1] - pc) - (kc + kap[k - 1]) * (pc - phi[k - 1]) +
-                   (kap[k + pitch] + kc) * (phi[k + pitch] - pc) -
-                   (kc + kap[k - pitch]) * (pc - phi[k - pitch]));
-}
-
-// (pm-num-phase) with the advection (e1e2) of App. A.4
-// (the overloads taking densities let a caller that already holds rho(c) of
-// the cell and its neighbours skip the divisions; the values are the same)
-template <typename T, class LV>
-__device__ __forceinline__ T op_c(const Prm<T>& P, const LV& L, int k, T rho) {
-  const int W = L.pitch;
-  auto cn = L.cn;
-  auto rn = L.rhon;
-  T c = L.c[k], cnk = cn[k];
-  T adv = rn[k + 1] * L.Tx[k] * L.u[k] + rn[k - 1] * L.Tx[k - 1] * L.u[k - 1] +
-          rn[k + W] * L.Ty[k] * L.v[k] + rn[k - W] * L.Ty[k - W] * L.v[k - W];
-  T diff = lap_h2(L.mobn, L.mu, k, W) + P.alpha * lap_h2(L.mobn, L.p, k, W);
-  return rho * (c - cnk) * P.idt + adv - P.iPe * L.ih2 * diff;
-}
-template <typename T, class LV>
-__device__ __forceinline__ T op_c(const Prm<T>& P, const LV& L, int k) {
-  return op_c(P, L, k, rho_of(P, L.c[k]));
-}
-
-// (pm-num-chem) with the time-averaged gradient term (pointwise G)
-// rq[f]: rho(c) of the neighbours k + 1, k - 1, k + W, k - W; rmu multiplies mu
-// (rho(c) in (pm-num-chem), rho^n in the projection method's (pj-num-chem))
-template <typename T, class LV>
-__device__ __forceinline__ T op_mu_r(const Prm<T>& P, const LV& L, int k, T rho, const T (&rq)[4],
-                                     T rmu) {
-  const int W = L.pitch;
-  auto c = L.c;
-  auto cn = L.cn;
-  auto rn = L.rhon;
-  T ck = c[k], cnk = cn[k];
-  T rnk = rn[k];
-  T rh = T(0.5) * (rho + rnk);
-  T r = -P.alpha * rho * rnk;
-  T bulk = rh * gsec(ck, cnk) + T(0.5) * (Fdw(ck) + Fdw(cnk)) * r;
-  T grad = T(0.25) * P.Lam * (G_h2(c, k, W) * L.ih2 + L.Gn[k]) * r;
-  // grad_d.(A rho^{n+1/2} grad_D c^{n+1/2})
-  T chk = ck + cnk;
-  T div = T(0);
-  const int off[4] = {1, -1, W, -W};
-#pragma unroll
-  for (int f = 0; f < 4; ++f) {
-    int q = k + off[f];
-    T rf = T(0.5) * (rq[f] + rn[q]);
-    div += (rh + rf) * ((c[q] + cn[q]) - chk);
-  }
-  div *= T(0.25) * L.ih2;  // 1/2 (face average) * 1/2 (c^{n+1/2}) / h^2
-  return rmu * L.mu[k] - P.K * bulk - grad + P.Lam * div;
-}
-template <typename T, class LV>
-__device__ __forceinline__ T op_mu(const Prm<T>& P, const LV& L, int k, T rho, const T (&rq)[4]) {
-  return op_mu_r(P, L, k, rho, rq, rho);
-}
-template <typename T, class LV>
-__device__ __forceinline__ T op_mu(const Prm<T>& P, const LV& L, int k) {
-  const int W = L.pitch;
-  const T rq[4] = {rho_of(P, L.c[k + 1]), rho_of(P, L.c[k - 1]), rho_of(P, L.c[k + W]),
-                   rho_of(P, L.c[k - W])};
-  return op_mu(P, L, k, rho_of(P, L.c[k]), rq);
-}
-
-// (pm-num-mass)
-template <typename T, class LV>
-__device__ __forceinline__ T op_p(const Prm<T>& P, const LV& L, int k) {
-  const int W = L.pitch;
-  T dv = (L.u[k] - L.u[k - 1] + L.v[k] - L.v[k - W]) * L.ih;
-  T diff = lap_h2(L.mobn, L.mu, k, W) + P.alpha * lap_h2(L.mobn, L.p, k, W);
-  return dv - P.alpha * P.iPe * L.ih2 * diff;
-}
-
 // Momentum row d (0: x row at x-edge k, unknown u; 1: y row at y-edge k,
-// unknown v) of (pm-num-mx) from the per-step assembled stencil (the arrays
-// Cu.. / Cv.. of Lv): the same sum as op_u / op_v, term by term, regrouped by
-// unknown.  rs = the sum of rho(c) over the edge's two cells.  s is the stride
-// along the edge normal, t across it; a the row's own velocity, b the other one.
-template <typename T, class LV>
+// unknown v) of (pm-num-mx), with (e1e1-1), (e1e1-2) and (e1e1), from the
+// per-step assembled stencil (the arrays Cu.. / Cv.. of Lv): the row's terms
+// regrouped by unknown.  rs = the sum of rho(c) over the edge's two cells.  s
+// is the stride along the edge normal, t across it; a the row's own velocity, b
+// the other one.  PST = false drops the pressure and surface-tension terms:
+// the intermediate-velocity row of the projection method (pj-num-mx), whose
+// T0 holds no gravity either (that acts in the projection equation).
+template <bool PST, typename T, class LV>
 __device__ __forceinline__ T mom_asm(const LV& L, int d, int k, T rs) {
   const int s = d ? L.pitch : 1, t = d ? 1 : L.pitch;
   auto a = L.pair(d, L.u, L.v);
@@ -400,80 +333,15 @@ __device__ __forceinline__ T mom_asm(const LV& L, int d, int k, T rs) {
   auto aM = L.row_pair(d, L.aMu, L.aMv);
   auto tP = L.row_pair(d, L.tPu, L.tPv);
   auto tM = L.row_pair(d, L.tMu, L.tMv);
-  auto M0 = L.row_pair(d, L.M0u, L.M0v);
-  auto M1 = L.row_pair(d, L.M1u, L.M1v);
   T r = L.pair(d, L.T0u, L.T0v)[k] + (C[k] + L.k.qidt * rs) * a[k];
   r += aP[k] * a[k + s] + aM[k] * a[k - s] + tP[k] * a[k + t] + tM[k] * a[k - t];
   // the grad-div term's cross derivative of the other velocity
   T vl = L.visn[k], vr = L.visn[k + s];
   r -= L.k.v3 * (vr * (b[k + s] - b[k + s - t]) - vl * (b[k] - b[k - t]));
-  r += (L.p[k + s] - L.p[k]) * L.k.ihM + M0[k] * L.mu[k] + M1[k] * L.mu[k + s];
+  if constexpr (PST)
+    r += (L.p[k + s] - L.p[k]) * L.k.ihM + L.row_pair(d, L.M0u, L.M0v)[k] * L.mu[k] +
+         L.row_pair(d, L.M1u, L.M1v)[k] * L.mu[k + s];
   return r;
-}
-
-// x row of (pm-num-mx) at edge u_{i+1/2,j} (array index k = at(i,j)); cells k (left), k+1 (right),
-// vertices k (top, (i+1/2, j+1/2)) and k-W (bottom); (e1e1-1), (e1e1-2) and (e1e1)
-// (rs = rho(c_k) + rho(c_{k+1}), twice the density average on the edge).  PST =
-// false drops the pressure and surface-tension terms: the intermediate-velocity
-// row of the projection method (pj-num-mx).
-template <typename T, bool PST = true, class LV>
-__device__ __forceinline__ T op_u(const Prm<T>& P, const LV& L, int k, T rs) {
-  if constexpr (PST && sizeof(T) == 8) return mom_asm(L, 0, k, rs);  // FP64 primitive row
-  const int W = L.pitch;
-  auto u = L.u; auto vis = L.visn; auto rn = L.rhon;
-  T ue = u[k];
-  T dxl = (ue - u[k - 1]) * L.ih, dxr = (u[k + 1] - ue) * L.ih;
-  T dvl = dxl + (L.v[k] - L.v[k - W]) * L.ih;
-  T dvr = dxr + (L.v[k + 1] - L.v[k + 1 - W]) * L.ih;
-  T Dt = (u[k + W] - ue) * L.ih, Db = (ue - u[k - W]) * L.ih;
-  T conv = T(0.5) * (L.Sx[k + 1] * dxr + L.Sx[k] * dxl + L.Qx[k] * Dt + L.Qx[k - W] * Db);
-  T time = ue * (L.T1u[k] + L.k.qidt * rs) + L.T0u[k];
-  T r = time + conv;
-  if constexpr (PST) {
-    T press = (L.p[k + 1] - L.p[k]) * L.ih * P.iM;
-    T st = -(rn[k + 1] * L.mu[k] + rn[k] * L.mu[k + 1]) * L.Tx[k] * P.iM;
-    r = r + press + st;
-  }
-  T vl = vis[k], vr = vis[k + 1];
-  T visc = -P.iRe * L.ih * ((vr * dxr - vl * dxl) + (L.Av[k] * Dt - L.Av[k - W] * Db) +
-                            (vr * dvr - vl * dvl) * T(1.0 / 3.0));
-  return r + visc;
-}
-template <typename T, class LV>
-__device__ __forceinline__ T op_u(const Prm<T>& P, const LV& L, int k) {
-  return op_u(P, L, k, rho_of(P, L.c[k]) + rho_of(P, L.c[k + 1]));
-}
-
-// y row of (pm-num-mx) at edge v_{i,j+1/2} (index k = at(i,j)); cells k (bottom), k+W (top),
-// vertices k (east, (i+1/2, j+1/2)) and k-1 (west); gravity (1/Fr) A_y rho^n is in T0v
-// PST = false: the projection method's intermediate-velocity row, without
-// pressure, surface tension and gravity (those act in (pj-num-pjx))
-template <typename T, bool PST = true, class LV>
-__device__ __forceinline__ T op_v(const Prm<T>& P, const LV& L, int k, T rs) {
-  if constexpr (PST && sizeof(T) == 8) return mom_asm(L, 1, k, rs);  // FP64 primitive row
-  const int W = L.pitch;
-  auto v = L.v; auto vis = L.visn; auto rn = L.rhon;
-  T ve = v[k];
-  T dyb = (ve - v[k - W]) * L.ih, dyt = (v[k + W] - ve) * L.ih;
-  T dvb = dyb + (L.u[k] - L.u[k - 1]) * L.ih;
-  T dvt = dyt + (L.u[k + W] - L.u[k + W - 1]) * L.ih;
-  T De = (v[k + 1] - ve) * L.ih, Dw = (ve - v[k - 1]) * L.ih;
-  T conv = T(0.5) * (L.Qy[k] * De + L.Qy[k - 1] * Dw + L.Sy[k + W] * dyt + L.Sy[k] * dyb);
-  T time = ve * (L.T1v[k] + L.k.qidt * rs) + L.T0v[k];
-  T r = time + conv;
-  if constexpr (PST) {
-    T press = (L.p[k + W] - L.p[k]) * L.ih * P.iM;
-    T st = -(rn[k + W] * L.mu[k] + rn[k] * L.mu[k + W]) * L.Ty[k] * P.iM;
-    r = r + press + st;
-  }
-  T vb = vis[k], vt = vis[k + W];
-  T visc = -P.iRe * L.ih * ((L.Av[k] * De - L.Av[k - 1] * Dw) + (vt * dyt - vb * dyb) +
-                            (vt * dvt - vb * dvb) * T(1.0 / 3.0));
-  return r + visc;
-}
-template <typename T, class LV>
-__device__ __forceinline__ T op_v(const Prm<T>& P, const LV& L, int k) {
-  return op_v(P, L, k, rho_of(P, L.c[k]) + rho_of(P, L.c[k + L.pitch]));
 }
 
 // ---------------------------------------------------------------------------
@@ -483,17 +351,21 @@ __device__ __forceinline__ T op_v(const Prm<T>& P, const LV& L, int k) {
 // [- (1/Fr) A_y rho(c) in y], ST the surface-tension pairing of (e1e1) at
 // level n+1.  Gravity acts here, tested with u^{n+1} in the energy proof.
 // ---------------------------------------------------------------------------
+// what the projection adds to the velocity of the face between cells a and b,
+// without gravity: (ST - D p) dt / (M A rho), from both cells' rho and mu, the
+// differences of c and p, with the constants folded and one reciprocal
+template <typename T, class LV>
+__device__ __forceinline__ T proj_kick(const LV& L, T ra, T rb, T mua, T mub, T dc, T dp) {
+  return (L.k.hkick * ((rb * mua + ra * mub) * dc) - L.k.kick * dp) * qrcp(ra + rb);
+}
 // u^{n+1} at edge (i+1/2, j), i = 0..m1; zero on no-slip walls
 template <typename T, class LV>
 __device__ __forceinline__ T proj_u(const Prm<T>& P, const LV& L, int i, int j) {
   if (!L.px && (i <= 0 || i >= L.m1)) return T(0);
   int k = L.at(i, j);
   T cl = L.c[k], cr = L.c[k + 1];
-  T rl = rho_of(P, cl), rr = rho_of(P, cr);
-  T Ar = T(0.5) * (rl + rr);
-  T dp = (L.p[k + 1] - L.p[k]) * L.ih;
-  T st = T(0.5) * (rr * L.mu[k] + rl * L.mu[k + 1]) * (cr - cl) * L.ih;
-  return L.u[k] + (st - dp) * P.iM / (Ar * P.idt);
+  return L.u[k] + proj_kick(L, rho_of(P, cl), rho_of(P, cr), L.mu[k], L.mu[k + 1], cr - cl,
+                            L.p[k + 1] - L.p[k]);
 }
 // v^{n+1} at edge (i, j+1/2), j = 0..m2; zero on the walls in y
 template <typename T, class LV>
@@ -502,11 +374,8 @@ __device__ __forceinline__ T proj_v(const Prm<T>& P, const LV& L, int i, int j) 
   const int W = L.pitch;
   int k = L.at(i, j);
   T cb = L.c[k], ct = L.c[k + W];
-  T rb = rho_of(P, cb), rt = rho_of(P, ct);
-  T Ar = T(0.5) * (rb + rt);
-  T dp = (L.p[k + W] - L.p[k]) * L.ih;
-  T st = T(0.5) * (rt * L.mu[k] + rb * L.mu[k + W]) * (ct - cb) * L.ih;
-  return L.v[k] + (st - dp) * P.iM / (Ar * P.idt) - P.Fr_inv / P.idt;
+  return L.v[k] + proj_kick(L, rho_of(P, cb), rho_of(P, ct), L.mu[k], L.mu[k + W], ct - cb,
+                            L.p[k + W] - L.p[k]) - L.k.gdt;
 }
 // The four face velocities u^{n+1} of cell (i,j) (E, W, N, S), from rho(c) of the
 // cell (rk) and of its neighbours (rq[f] for k + 1, k - 1, k + W, k - W): the
@@ -516,60 +385,37 @@ __device__ __forceinline__ void proj_faces(const Prm<T>& P, const LV& L, int i, 
                                            const T (&rq)[4], T (&w)[4]) {
   const int W = L.pitch;
   int k = L.at(i, j);
-  auto c = L.c; auto mu = L.mu; auto p = L.p;
-  const T g = P.Fr_inv / P.idt;
+  auto c = L.c;
+  auto mu = L.mu;
+  auto p = L.p;
   // face between cells a (left/below) and b = a + off, velocity array at a
-  auto face = [&](int a, int off, auto vel, T ra, T rb, T grav) {
-    T Ar = T(0.5) * (ra + rb);
-    T dp = (p[a + off] - p[a]) * L.ih;
-    T st = T(0.5) * (rb * mu[a] + ra * mu[a + off]) * (c[a + off] - c[a]) * L.ih;
-    return vel[a] + (st - dp) * P.iM / (Ar * P.idt) - grav;
+  auto face = [&](int a, int off, auto vel, T ra, T rb) {
+    return vel[a] + proj_kick(L, ra, rb, mu[a], mu[a + off], c[a + off] - c[a], p[a + off] - p[a]);
   };
-  w[0] = (!L.px && i == L.m1) ? T(0) : face(k, 1, L.u, rk, rq[0], T(0));
-  w[1] = (!L.px && i == 1) ? T(0) : face(k - 1, 1, L.u, rq[1], rk, T(0));
-  w[2] = (j == L.m2) ? T(0) : face(k, W, L.v, rk, rq[2], g);
-  w[3] = (j == 1) ? T(0) : face(k - W, W, L.v, rq[3], rk, g);
+  w[0] = (!L.px && i == L.m1) ? T(0) : face(k, 1, L.u, rk, rq[0]);
+  w[1] = (!L.px && i == 1) ? T(0) : face(k - 1, 1, L.u, rq[1], rk);
+  w[2] = (j == L.m2) ? T(0) : face(k, W, L.v, rk, rq[2]) - L.k.gdt;
+  w[3] = (j == 1) ? T(0) : face(k - W, W, L.v, rq[3], rk) - L.k.gdt;
 }
 // (pj-num-phase): rho^n (c - c^n)/dt + a_x(rho_ew D_x c u^{n+1}) + a_y(...)
 // - (1/Pe) grad_d.(A m^n grad_D mu) - (alpha/Pe) grad_d.(A m^n grad_D p), with
 // rho = rho(c^{n+1}) and c^{n+1} in the advection; and (pj-num-mass): d_x u^{n+1}
 // + d_y v^{n+1} - (alpha/Pe)(grad.(A m grad mu) + alpha grad.(A m grad p)).
 // Both from the shared densities rq and the face velocities w of proj_faces.
+// flux: the face sum of (m(c^n) of both cells) (d mu + alpha d p)
 template <typename T, class LV>
 __device__ __forceinline__ T opp_c_w(const Prm<T>& P, const LV& L, int k, const T (&rq)[4],
-                                     const T (&w)[4]) {
+                                     const T (&w)[4], T flux) {
   const int W = L.pitch;
   auto c = L.c;
   T ck = c[k];
-  T t = L.rhon[k] * (ck - L.cn[k]) * P.idt;
-  T ax = T(0.5) * (rq[0] * (c[k + 1] - ck) * L.ih * w[0] + rq[1] * (ck - c[k - 1]) * L.ih * w[1]);
-  T ay = T(0.5) * (rq[2] * (c[k + W] - ck) * L.ih * w[2] + rq[3] * (ck - c[k - W]) * L.ih * w[3]);
-  T diff = lap_h2(L.mobn, L.mu, k, W) + P.alpha * lap_h2(L.mobn, L.p, k, W);
-  return t + ax + ay - P.iPe * L.ih2 * diff;
+  T adv = rq[0] * (c[k + 1] - ck) * w[0] + rq[1] * (ck - c[k - 1]) * w[1] +
+          rq[2] * (c[k + W] - ck) * w[2] + rq[3] * (ck - c[k - W]) * w[3];
+  return L.rhon[k] * (ck - L.cn[k]) * P.idt + L.k.hih * adv - L.k.dif * flux;
 }
 template <typename T, class LV>
-__device__ __forceinline__ T opp_p_w(const Prm<T>& P, const LV& L, int k, const T (&w)[4]) {
-  const int W = L.pitch;
-  T dv = (w[0] - w[1] + w[2] - w[3]) * L.ih;
-  T diff = lap_h2(L.mobn, L.mu, k, W) + P.alpha * lap_h2(L.mobn, L.p, k, W);
-  return dv - P.alpha * P.iPe * L.ih2 * diff;
-}
-
-// (pj-num-chem): as (pm-num-chem) with rho^n in front of mu
-template <typename T, class LV>
-__device__ __forceinline__ T opp_mu(const Prm<T>& P, const LV& L, int k) {
-  const int W = L.pitch;
-  const T rq[4] = {rho_of(P, L.c[k + 1]), rho_of(P, L.c[k - 1]), rho_of(P, L.c[k + W]),
-                   rho_of(P, L.c[k - W])};
-  return op_mu_r(P, L, k, rho_of(P, L.c[k]), rq, L.rhon[k]);
-}
-template <typename T, class LV>
-__device__ __forceinline__ T opp_u(const Prm<T>& P, const LV& L, int k) {
-  return op_u<T, false>(P, L, k, rho_of(P, L.c[k]) + rho_of(P, L.c[k + 1]));
-}
-template <typename T, class LV>
-__device__ __forceinline__ T opp_v(const Prm<T>& P, const LV& L, int k) {
-  return op_v<T, false>(P, L, k, rho_of(P, L.c[k]) + rho_of(P, L.c[k + L.pitch]));
+__device__ __forceinline__ T opp_p_w(const LV& L, const T (&w)[4], T flux) {
+  return (w[0] - w[1] + w[2] - w[3]) * L.ih - L.k.adif * flux;
 }
 
 // ---------------------------------------------------------------------------
@@ -778,86 +624,41 @@ __device__ __forceinline__ T err_diag(const LV& L, int d, int k, T rs, T gp, T g
          gm * L.pair(d, L.tMu, L.tMv)[k];
 }
 
-// Two forms of the iterate: Full (x itself, Sec. 6.1) and Err (correction e to
-// the base X of a defect-correction cycle).  val_c / val_mu return the full
-// value c, mu that the local Jacobians of the smoothers are evaluated at.
+// The forms of the iterate: Full (x itself, Sec. 6.1), Proj (the projection
+// method on the full iterate; its u, v arrays hold the intermediate velocity)
+// and Err (a correction e to the base X of a defect-correction cycle).  val_c
+// .. return the full values that the local Jacobians of the smoothers are
+// evaluated at, rho the density there.
 struct FullForm {
-  template <class LV>
-static __device__ __forceinline__ typename LV::real val_c(const LV& L, int k) {
-  typedef typename LV::real T; return L.c[k]; }
+  template <class LV> static __device__ __forceinline__ typename LV::real val_u(const LV& L, int k) {
+    return L.u[k];
+  }
+  template <class LV> static __device__ __forceinline__ typename LV::real val_v(const LV& L, int k) {
+    return L.v[k];
+  }
   template <typename T, class LV>
-static __device__ __forceinline__ T rho(const Prm<T>&, const LV& L, int k) { return L.rhoc[k]; }
-  template <class LV>
-static __device__ __forceinline__ typename LV::real val_u(const LV& L, int k) {
-  typedef typename LV::real T; return L.u[k]; }
-  template <class LV>
-static __device__ __forceinline__ typename LV::real val_v(const LV& L, int k) {
-  typedef typename LV::real T; return L.v[k]; }
-  template <class LV>
-static __device__ __forceinline__ typename LV::real val_mu(const LV& L, int k) {
-  typedef typename LV::real T; return L.mu[k]; }
-  template <typename T, class LV>
-static __device__ __forceinline__ T Nc(const Prm<T>& P, const LV& L, int k) { return op_c(P, L, k); }
-  template <typename T, class LV>
-static __device__ __forceinline__ T Nmu(const Prm<T>& P, const LV& L, int k) { return op_mu(P, L, k); }
-  template <typename T, class LV>
-static __device__ __forceinline__ T Np(const Prm<T>& P, const LV& L, int k) { return op_p(P, L, k); }
-  template <typename T, class LV>
-static __device__ __forceinline__ T Nu(const Prm<T>& P, const LV& L, int k) { return op_u(P, L, k); }
-  template <typename T, class LV>
-static __device__ __forceinline__ T Nv(const Prm<T>& P, const LV& L, int k) { return op_v(P, L, k); }
+  static __device__ __forceinline__ T rho(const Prm<T>&, const LV& L, int k) {
+    return L.rhoc[k];
+  }
 };
-// The projection method on the full iterate (u, v arrays hold the intermediate
-// velocity).  Its N_c and N_p need the cell's face velocities (proj_faces,
-// which needs the cell index for the wall edges), so the kernels call
-// opp_c_w / opp_p_w directly.
-struct ProjForm {
-  template <class LV>
-static __device__ __forceinline__ typename LV::real val_c(const LV& L, int k) {
-  typedef typename LV::real T; return L.c[k]; }
-  template <typename T, class LV>
-static __device__ __forceinline__ T rho(const Prm<T>&, const LV& L, int k) { return L.rhoc[k]; }
-  template <class LV>
-static __device__ __forceinline__ typename LV::real val_u(const LV& L, int k) {
-  typedef typename LV::real T; return L.u[k]; }
-  template <class LV>
-static __device__ __forceinline__ typename LV::real val_v(const LV& L, int k) {
-  typedef typename LV::real T; return L.v[k]; }
-  template <class LV>
-static __device__ __forceinline__ typename LV::real val_mu(const LV& L, int k) {
-  typedef typename LV::real T; return L.mu[k]; }
-  template <typename T, class LV>
-static __device__ __forceinline__ T Nmu(const Prm<T>& P, const LV& L, int k) { return opp_mu(P, L, k); }
-  template <typename T, class LV>
-static __device__ __forceinline__ T Nu(const Prm<T>& P, const LV& L, int k) { return opp_u(P, L, k); }
-  template <typename T, class LV>
-static __device__ __forceinline__ T Nv(const Prm<T>& P, const LV& L, int k) { return opp_v(P, L, k); }
-};
+struct ProjForm : FullForm {};
 struct ErrForm {
-  template <class LV>
-static __device__ __forceinline__ typename LV::real val_c(const LV& L, int k) {
-  typedef typename LV::real T; return L.Bc[k] + L.c[k]; }
+  template <class LV> static __device__ __forceinline__ typename LV::real val_c(const LV& L, int k) {
+    return L.Bc[k] + L.c[k];
+  }
+  template <class LV> static __device__ __forceinline__ typename LV::real val_u(const LV& L, int k) {
+    return L.Bu[k] + L.u[k];
+  }
+  template <class LV> static __device__ __forceinline__ typename LV::real val_v(const LV& L, int k) {
+    return L.Bv[k] + L.v[k];
+  }
+  template <class LV> static __device__ __forceinline__ typename LV::real val_mu(const LV& L, int k) {
+    return L.Bmu[k] + L.mu[k];
+  }
   template <typename T, class LV>
-static __device__ __forceinline__ T rho(const Prm<T>& P, const LV& L, int k) { return rho_of(P, val_c(L, k)); }
-  template <class LV>
-static __device__ __forceinline__ typename LV::real val_u(const LV& L, int k) {
-  typedef typename LV::real T; return L.Bu[k] + L.u[k]; }
-  template <class LV>
-static __device__ __forceinline__ typename LV::real val_v(const LV& L, int k) {
-  typedef typename LV::real T; return L.Bv[k] + L.v[k]; }
-  template <class LV>
-static __device__ __forceinline__ typename LV::real val_mu(const LV& L, int k) {
-  typedef typename LV::real T; return L.Bmu[k] + L.mu[k]; }
-  template <typename T, class LV>
-static __device__ __forceinline__ T Nc(const Prm<T>& P, const LV& L, int k) { return opd_c(P, L, k); }
-  template <typename T, class LV>
-static __device__ __forceinline__ T Nmu(const Prm<T>& P, const LV& L, int k) { return opd_mu(P, L, k); }
-  template <typename T, class LV>
-static __device__ __forceinline__ T Np(const Prm<T>& P, const LV& L, int k) { return opd_p(P, L, k); }
-  template <typename T, class LV>
-static __device__ __forceinline__ T Nu(const Prm<T>& P, const LV& L, int k) { return opd_u(P, L, k); }
-  template <typename T, class LV>
-static __device__ __forceinline__ T Nv(const Prm<T>& P, const LV& L, int k) { return opd_v(P, L, k); }
+  static __device__ __forceinline__ T rho(const Prm<T>& P, const LV& L, int k) {
+    return rho_of(P, val_c(L, k));
+  }
 };
 
 }  // namespace qn
