@@ -1556,44 +1556,55 @@ __global__ void __launch_bounds__(NT, 2) k_frozen_coef3(Prm<T> P, Lv<T> L) {
 // --------------------------------------------------------------------------
 // FAS transfers
 // --------------------------------------------------------------------------
-// coarse iterate = R x_h (cells: 4-mean; edges: mean of the 2 coincident fine edges),
-// and a copy kept for the correction
+// coarse iterate = R x_h (cells: 4-mean; edges: mean of the 2 coincident fine edges)
+// with its ghosts, and a copy kept for the correction.  The stores that keep
+// ghosts cover all of them but the cells' corners, which no operator reads:
+// wall edges and what lies beyond them are zero from the start.
 template <typename T, class LV>
 __device__ __forceinline__ void restrict_state_cell(const Prm<T>& P, const LV& F, const LV& C,
                                                     int I, int J) {
   int kc = C.at(I, J);
-  if (I >= 1 && J >= 1) {
+  const bool cell = I >= 1 && J >= 1;
+  T a = T(0), b = T(0), d = T(0), u = T(0), v = T(0);
+  if (cell) {
     int kf = F.at(2 * I - 1, 2 * J - 1), W = F.pitch;
-    T a = T(0.25) * (F.c[kf] + F.c[kf + 1] + F.c[kf + W] + F.c[kf + W + 1]);
-    T b = T(0.25) * (F.mu[kf] + F.mu[kf + 1] + F.mu[kf + W] + F.mu[kf + W + 1]);
-    T d = T(0.25) * (F.p[kf] + F.p[kf + 1] + F.p[kf + W] + F.p[kf + W + 1]);
-    C.c[kc] = a; C.sc[kc] = a;
-    if constexpr (LV::has_rho)
-      if (C.rhoc) C.rhoc[kc] = rho_of(P, a);
-    C.mu[kc] = b; C.smu[kc] = b;
-    C.p[kc] = d; C.sp[kc] = d;
+    a = T(0.25) * (F.c[kf] + F.c[kf + 1] + F.c[kf + W] + F.c[kf + W + 1]);
+    b = T(0.25) * (F.mu[kf] + F.mu[kf + 1] + F.mu[kf + W] + F.mu[kf + W + 1]);
+    d = T(0.25) * (F.p[kf] + F.p[kf + 1] + F.p[kf + W] + F.p[kf + W + 1]);
   }
   if (J >= 1) {  // u edge (I, J), I = 0..M1
     int kf = F.at(2 * I, 2 * J - 1);
-    T a = T(0.5) * (F.u[kf] + F.u[kf + F.pitch]);
-    C.u[kc] = a; C.su[kc] = a;
+    u = T(0.5) * (F.u[kf] + F.u[kf + F.pitch]);
   }
   if (I >= 1) {  // v edge (I, J), J = 0..M2
     int kf = F.at(2 * I - 1, 2 * J);
-    T a = T(0.5) * (F.v[kf] + F.v[kf + 1]);
-    C.v[kc] = a; C.sv[kc] = a;
+    v = T(0.5) * (F.v[kf] + F.v[kf + 1]);
   }
-}
-
-// coarse iterate = R x_h (cells: 4-mean; edges: mean of the 2 coincident fine edges),
-// and a copy kept for the correction
-template <typename T>
-__global__ void __launch_bounds__(NT, 2) k_restrict_state(Prm<T> P, Lv<T> F, Lv<T> C) {
-  pdl_enter();
-  int I = blockIdx.x * BX + threadIdx.x;
-  int J = blockIdx.y * BY + threadIdx.y;
-  if (I > C.m1 || J > C.m2) return;
-  restrict_state_cell(P, F, C, I, J);
+  const bool ghosts = has_ghosts(C, I, J);
+  if (cell) {
+    put_cell(C, C.c, I, J, ghosts, a);
+    if constexpr (LV::has_rho)
+      if (C.rhoc) put_cell(C, C.rhoc, I, J, ghosts, rho_of(P, a));
+    put_cell(C, C.mu, I, J, ghosts, b);
+    put_cell(C, C.p, I, J, ghosts, d);
+    C.sc[kc] = a;
+    C.smu[kc] = b;
+    C.sp[kc] = d;
+  }
+  if (J >= 1) {
+    if (I >= 1 && I <= C.uhi()) {
+      if (ghosts) store_u(C, I, J, u);
+      else C.u[kc] = u;
+    }
+    C.su[kc] = u;
+  }
+  if (I >= 1) {
+    if (J >= 1 && J < C.m2) {
+      if (ghosts) store_v(C, I, J, v);
+      else C.v[kc] = v;
+    }
+    C.sv[kc] = v;
+  }
 }
 
 template <class LV>
@@ -1621,38 +1632,42 @@ __device__ __forceinline__ void restrict_res_cell(const LV& F, const LV& C, int 
   typedef typename LV::real T;
   int kc = C.at(I, J);
   int kf = F.at(2 * I - 1, 2 * J - 1), W = F.pitch;
-  C.fc[kc] = T(0.25) * (F.rc[kf] + F.rc[kf + 1] + F.rc[kf + W] + F.rc[kf + W + 1]);
-  C.fmu[kc] = T(0.25) * (F.rmu[kf] + F.rmu[kf + 1] + F.rmu[kf + W] + F.rmu[kf + W + 1]);
-  C.fp[kc] = T(0.25) * (F.rp[kf] + F.rp[kf + 1] + F.rp[kf + W] + F.rp[kf + W + 1]);
+  const T c = T(0.25) * (F.rc[kf] + F.rc[kf + 1] + F.rc[kf + W] + F.rc[kf + W + 1]);
+  const T m = T(0.25) * (F.rmu[kf] + F.rmu[kf + 1] + F.rmu[kf + W] + F.rmu[kf + W + 1]);
+  const T p = T(0.25) * (F.rp[kf] + F.rp[kf + 1] + F.rp[kf + W] + F.rp[kf + W + 1]);
+  T u = T(0), v = T(0);
   if (I <= C.uhi()) {
-    T s = T(0);
 #pragma unroll
     for (int jj = 0; jj < 2; ++jj) {
       int jf = 2 * J - 1 + jj;
-      s += T(0.25) * ru_at(F, 2 * I - 1, jf) + T(0.5) * ru_at(F, 2 * I, jf) +
+      u += T(0.25) * ru_at(F, 2 * I - 1, jf) + T(0.5) * ru_at(F, 2 * I, jf) +
            T(0.25) * ru_at(F, 2 * I + 1, jf);
     }
-    C.fu[kc] = T(0.5) * s;
   }
   if (J < C.m2) {
-    T s = T(0);
 #pragma unroll
     for (int ii = 0; ii < 2; ++ii) {
       int ifn = 2 * I - 1 + ii;
-      s += T(0.25) * rv_at(F, ifn, 2 * J - 1) + T(0.5) * rv_at(F, ifn, 2 * J) +
+      v += T(0.25) * rv_at(F, ifn, 2 * J - 1) + T(0.5) * rv_at(F, ifn, 2 * J) +
            T(0.25) * rv_at(F, ifn, 2 * J + 1);
     }
-    C.fv[kc] = T(0.5) * s;
   }
+  C.fc[kc] = c;
+  C.fmu[kc] = m;
+  C.fp[kc] = p;
+  if (I <= C.uhi()) C.fu[kc] = T(0.5) * u;
+  if (J < C.m2) C.fv[kc] = T(0.5) * v;
 }
 
+// the coarse level's iterate (restrict_state_cell) and right-hand side R r_h in one launch
 template <typename T>
-__global__ void __launch_bounds__(NT, 2) k_restrict_res(Lv<T> F, Lv<T> C) {
+__global__ void __launch_bounds__(NT, 2) k_restrict(Prm<T> P, Lv<T> F, Lv<T> C) {
   pdl_enter();
-  int I = blockIdx.x * BX + threadIdx.x + 1;
-  int J = blockIdx.y * BY + threadIdx.y + 1;
+  int I = blockIdx.x * BX + threadIdx.x;
+  int J = blockIdx.y * BY + threadIdx.y;
   if (I > C.m1 || J > C.m2) return;
-  restrict_res_cell(F, C, I, J);
+  if (I >= 1 && J >= 1) restrict_res_cell(F, C, I, J);
+  restrict_state_cell(P, F, C, I, J);
 }
 
 template <typename T>
@@ -1676,20 +1691,20 @@ __global__ void __launch_bounds__(NT, 2) k_restrict_frozen(Lv<T> F, Lv<T> C) {
   }
 }
 
-// x_h += P(x_H - saved_H): cells piecewise constant; edges coincident or linear
-// in the normal direction, constant in the tangential direction
+// x_h += P(x_H - saved_H), with the ghosts (as restrict_state_cell): cells
+// piecewise constant; edges coincident or linear in the normal direction,
+// constant in the tangential direction
 template <typename T, class LV>
 __device__ __forceinline__ void prolong_cell(const Prm<T>& P, const LV& F, const LV& C, int i,
                                              int j) {
   int k = F.at(i, j);
   int I = (i + 1) >> 1, J = (j + 1) >> 1;
   int kc = C.at(I, J);
-  F.c[k] += C.c[kc] - C.sc[kc];
-  if constexpr (LV::has_rho)
-    if (F.rhoc) F.rhoc[k] = rho_of(P, F.c[k]);
-  F.mu[k] += C.mu[kc] - C.smu[kc];
-  F.p[k] += C.p[kc] - C.sp[kc];
-  if (i <= F.uhi()) {
+  const T c = F.c[k] + (C.c[kc] - C.sc[kc]), mu = F.mu[k] + (C.mu[kc] - C.smu[kc]),
+          p = F.p[k] + (C.p[kc] - C.sp[kc]);
+  const bool hu = i <= F.uhi(), hv = j < F.m2;
+  T u = T(0), v = T(0);
+  if (hu) {
     T e;
     if ((i & 1) == 0) {
       int q = C.at(i >> 1, J);
@@ -1698,9 +1713,9 @@ __device__ __forceinline__ void prolong_cell(const Prm<T>& P, const LV& F, const
       int q0 = C.at((i - 1) >> 1, J), q1 = C.at((i + 1) >> 1, J);
       e = T(0.5) * ((C.u[q0] - C.su[q0]) + (C.u[q1] - C.su[q1]));
     }
-    F.u[k] += e;
+    u = F.u[k] + e;
   }
-  if (j < F.m2) {
+  if (hv) {
     T e;
     if ((j & 1) == 0) {
       int q = C.at(I, j >> 1);
@@ -1709,7 +1724,21 @@ __device__ __forceinline__ void prolong_cell(const Prm<T>& P, const LV& F, const
       int q0 = C.at(I, (j - 1) >> 1), q1 = C.at(I, (j + 1) >> 1);
       e = T(0.5) * ((C.v[q0] - C.sv[q0]) + (C.v[q1] - C.sv[q1]));
     }
-    F.v[k] += e;
+    v = F.v[k] + e;
+  }
+  const bool ghosts = has_ghosts(F, i, j);
+  put_cell(F, F.c, i, j, ghosts, c);
+  if constexpr (LV::has_rho)
+    if (F.rhoc) put_cell(F, F.rhoc, i, j, ghosts, rho_of(P, c));
+  put_cell(F, F.mu, i, j, ghosts, mu);
+  put_cell(F, F.p, i, j, ghosts, p);
+  if (hu) {
+    if (ghosts) store_u(F, i, j, u);
+    else F.u[k] = u;
+  }
+  if (hv) {
+    if (ghosts) store_v(F, i, j, v);
+    else F.v[k] = v;
   }
 }
 
@@ -1730,19 +1759,24 @@ __global__ void __launch_bounds__(NT, 2) k_prolong(Prm<T> P, Lv<T> F, Lv<T> C) {
 // launch instead of dozens.  Per-cell work is the same device code as the grid
 // kernels above, in the same colour order, so the results are the same.
 // --------------------------------------------------------------------------
-// coarse base X_H = R X_h (cells: 4-mean; edges: 2 coincident fine edges), one entry
+// coarse base X_H = R X_h (cells: 4-mean; edges: 2 coincident fine edges), one
+// entry, with the ghosts that the rows read: those of c and rho(c)
 template <typename T, class LV>
 __device__ __forceinline__ void restrict_base_cell(const Prm<T>& P, const LV& F, const LV& C, int I,
                                                    int J) {
-  int kc = C.at(I, J);
+  const int kc = C.at(I, J);
+  const bool ghosts = has_ghosts(C, I, J);
   if (I >= 1 && J >= 1) {
     int kf = F.at(2 * I - 1, 2 * J - 1), W = F.pitch;
     const T B = T(0.25) * (F.Bc[kf] + F.Bc[kf + 1] + F.Bc[kf + W] + F.Bc[kf + W + 1]);
-    C.Bc[kc] = B;
-    C.rB[kc] = rho_of(P, B);
-    C.Bmu[kc] = T(0.25) * (F.Bmu[kf] + F.Bmu[kf + 1] + F.Bmu[kf + W] + F.Bmu[kf + W + 1]);
-    C.Bdc[kc] = T(0.25) * (F.Bdc[kf] + F.Bdc[kf + 1] + F.Bdc[kf + W] + F.Bdc[kf + W + 1]);
+    const T m = T(0.25) * (F.Bmu[kf] + F.Bmu[kf + 1] + F.Bmu[kf + W] + F.Bmu[kf + W + 1]);
+    const T d = T(0.25) * (F.Bdc[kf] + F.Bdc[kf + 1] + F.Bdc[kf + W] + F.Bdc[kf + W + 1]);
+    put_cell(C, C.Bc, I, J, ghosts, B);
+    put_cell(C, C.rB, I, J, ghosts, rho_of(P, B));
+    C.Bmu[kc] = m;
+    C.Bdc[kc] = d;
   }
+  // velocities at the edges of the cells, column 0 (periodic x) included
   if (J >= 1) {
     int kf = F.at(2 * I, 2 * J - 1);
     C.Bu[kc] = T(0.5) * (F.Bu[kf] + F.Bu[kf + F.pitch]);
@@ -1751,18 +1785,6 @@ __device__ __forceinline__ void restrict_base_cell(const Prm<T>& P, const LV& F,
     int kf = F.at(2 * I - 1, 2 * J);
     C.Bv[kc] = T(0.5) * (F.Bv[kf] + F.Bv[kf + 1]);
   }
-}
-
-// ghosts of the base arrays
-template <class LV>
-__device__ __forceinline__ void bc_base_cell(const LV& L, int I, int J) {
-  typedef typename LV::real T;
-  fill_cell_ghost(L, L.Bc, I, J);
-  fill_cell_ghost(L, L.rB, I, J);
-  fill_cell_ghost(L, L.Bmu, I, J);
-  fill_cell_ghost(L, L.Bdc, I, J);
-  fill_u_ghost(L, L.Bu, I, J);
-  fill_v_ghost(L, L.Bv, I, J);
 }
 
 // The fused V-cycle runs in one thread block or in one thread-block cluster of
@@ -1794,24 +1816,6 @@ struct CoarseLevels {
   int n;
   int base;  // error equation: restrict the base state to L[1..n-1] first
 };
-
-template <class LV>
-__device__ __forceinline__ void bc_unknowns_block(const LV& L) {
-  typedef typename LV::real T;
-  int n = 4 * (L.m1 + 3) + 4 * (L.m2 + 3);
-  for (int t = grp_rank(); t < n; t += grp_size()) {
-    int I, J;
-    if (!frame_pos(t, L.m1, L.m2, I, J)) continue;
-    fill_cell_ghost(L, L.c, I, J);
-    if constexpr (LV::has_rho)
-      if (L.rhoc) fill_cell_ghost(L, L.rhoc, I, J);
-    fill_cell_ghost(L, L.mu, I, J);
-    fill_cell_ghost(L, L.p, I, J);
-    fill_u_ghost(L, L.u, I, J);
-    fill_v_ghost(L, L.v, I, J);
-  }
-  grp_sync();
-}
 
 // --------------------------------------------------------------------------
 // single-block smoothing of the coarse levels.  An FP64 warp instruction
@@ -2471,12 +2475,6 @@ __device__ __forceinline__ void coarse_vcycle_body(const Prm<T>& P, const Get& g
       for (int t = grp_rank(); t < (G.m1 + 1) * (G.m2 + 1); t += grp_size())
         restrict_base_cell(P, F, G, t % (G.m1 + 1), t / (G.m1 + 1));
       grp_sync();
-      const int nf = 4 * (G.m1 + 3) + 4 * (G.m2 + 3);
-      for (int t = grp_rank(); t < nf; t += grp_size()) {
-        int I, J;
-        if (frame_pos(t, G.m1, G.m2, I, J)) bc_base_cell(G, I, J);
-      }
-      grp_sync();
     }
   }
   for (int visit = 0; visit < 2 * n - 1; ++visit) {
@@ -2488,7 +2486,6 @@ __device__ __forceinline__ void coarse_vcycle_body(const Prm<T>& P, const Get& g
       for (int t = grp_rank(); t < F.m1 * F.m2; t += grp_size())
         prolong_cell(P, F, G, t % F.m1 + 1, t / F.m1 + 1);
       grp_sync();
-      bc_unknowns_block(F);
     }
     const int sweeps = down ? nu1 : up ? nu2 : nuc;
     for (int s = 0; s < sweeps; ++s) smooth_block<T, Form>(P, F, omega, coupled, team8);
@@ -2502,7 +2499,6 @@ __device__ __forceinline__ void coarse_vcycle_body(const Prm<T>& P, const Get& g
       for (int t = grp_rank(); t < G.m1 * G.m2; t += grp_size())
         restrict_res_cell(F, G, t % G.m1 + 1, t / G.m1 + 1);
       grp_sync();
-      bc_unknowns_block(G);
       for (int t = grp_rank(); t < G.m1 * G.m2; t += grp_size())
         residual_cell<T, 1, Form>(P, G, t % G.m1 + 1, t / G.m1 + 1, dummy);
       grp_sync();
@@ -3022,16 +3018,6 @@ __global__ void __launch_bounds__(NT, 2) k_restrict_base(Prm<T> P, Lv<T> F, Lv<T
   if (I > C.m1 || J > C.m2) return;
   restrict_base_cell(P, F, C, I, J);
 }
-
-template <typename T>
-__global__ void __launch_bounds__(NT, 2) k_bc_base(Lv<T> L) {
-  pdl_enter();
-  int t = blockIdx.x * blockDim.x + threadIdx.x;
-  int I, J;
-  if (!frame_pos(t, L.m1, L.m2, I, J)) return;
-  bc_base_cell(L, I, J);
-}
-
 
 // --------------------------------------------------------------------------
 // reductions
@@ -3715,9 +3701,6 @@ template <typename T>
 void launch_restrict_base(const Prm<T>& P, const Lv<T>& F, const Lv<T>& C, cudaStream_t s) {
   qlaunch(&k_restrict_base<T>, grid2(C.m1 + 1, C.m2 + 1), dim3(BX, BY), 0, s, P, F, C);
   ++g_launches;
-  int n = frame_threads(C.m1, C.m2);
-  qlaunch(&k_bc_base<T>, (n + 255) / 256, 256, 0, s, C);
-  ++g_launches;
 }
 template <typename T>
 void launch_bc_unknowns(const Lv<T>& L, cudaStream_t s) {
@@ -3742,13 +3725,8 @@ void launch_frozen(const Prm<T>& P, const Lv<T>& L, cudaStream_t s) {
   ++g_launches;
 }
 template <typename T>
-void launch_restrict_state(const Prm<T>& P, const Lv<T>& F, const Lv<T>& C, cudaStream_t s) {
-  qlaunch(&k_restrict_state<T>, grid2(C.m1 + 1, C.m2 + 1), dim3(BX, BY), 0, s, P, F, C);
-  ++g_launches;
-}
-template <typename T>
-void launch_restrict_res(const Lv<T>& F, const Lv<T>& C, cudaStream_t s) {
-  qlaunch(&k_restrict_res<T>, grid2(C.m1, C.m2), dim3(BX, BY), 0, s, F, C);
+void launch_restrict(const Prm<T>& P, const Lv<T>& F, const Lv<T>& C, cudaStream_t s) {
+  qlaunch(&k_restrict<T>, grid2(C.m1 + 1, C.m2 + 1), dim3(BX, BY), 0, s, P, F, C);
   ++g_launches;
 }
 template <typename T>
@@ -3964,8 +3942,7 @@ int partial_rows_needed(int m1, int m2) {
   template void launch_restrict_base<T>(const Prm<T>&, const Lv<T>&, const Lv<T>&, cudaStream_t); \
   template void launch_bc_unknowns<T>(const Lv<T>&, cudaStream_t);                               \
   template void launch_frozen<T>(const Prm<T>&, const Lv<T>&, cudaStream_t);                     \
-  template void launch_restrict_state<T>(const Prm<T>&, const Lv<T>&, const Lv<T>&, cudaStream_t); \
-  template void launch_restrict_res<T>(const Lv<T>&, const Lv<T>&, cudaStream_t);                \
+  template void launch_restrict<T>(const Prm<T>&, const Lv<T>&, const Lv<T>&, cudaStream_t);      \
   template void launch_restrict_frozen<T>(const Lv<T>&, const Lv<T>&, cudaStream_t);             \
   template void launch_prolong<T>(const Prm<T>&, const Lv<T>&, const Lv<T>&, cudaStream_t);        \
   template void launch_gauge<T>(const Lv<T>&, double*, double*, cudaStream_t);                   \

@@ -119,8 +119,8 @@ template <typename T>
 void launch_restrict_base(const Prm<T>& P, const Lv<T>& F, const Lv<T>& C, cudaStream_t s);
 template <typename T> void launch_bc_unknowns(const Lv<T>& L, cudaStream_t s);
 template <typename T> void launch_frozen(const Prm<T>& P, const Lv<T>& L, cudaStream_t s);
-template <typename T> void launch_restrict_state(const Prm<T>& P, const Lv<T>& F, const Lv<T>& C, cudaStream_t s);
-template <typename T> void launch_restrict_res(const Lv<T>& F, const Lv<T>& C, cudaStream_t s);
+// the coarse level's iterate with its ghosts, and its right-hand side R r_h
+template <typename T> void launch_restrict(const Prm<T>& P, const Lv<T>& F, const Lv<T>& C, cudaStream_t s);
 template <typename T> void launch_restrict_frozen(const Lv<T>& F, const Lv<T>& C, cudaStream_t s);
 template <typename T> void launch_prolong(const Prm<T>& P, const Lv<T>& F, const Lv<T>& C, cudaStream_t s);
 template <typename T> void launch_gauge(const Lv<T>& L, double* part, double* scal, cudaStream_t s);

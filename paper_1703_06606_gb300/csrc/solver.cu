@@ -723,13 +723,10 @@ void vcycle(qnsch_s* s, const std::vector<Lv<T>>& Ls, const Prm<T>& P, int l) {
   const Lv<T>& F = Ls[l];
   const Lv<T>& C = Ls[l + 1];
   qn::launch_residual<T, Form>(P, F, (double*)nullptr, s->stream);
-  qn::launch_restrict_state(P, F, C, s->stream);
-  qn::launch_bc_unknowns(C, s->stream);
-  qn::launch_restrict_res(F, C, s->stream);
+  qn::launch_restrict(P, F, C, s->stream);
   qn::launch_add_op<T, Form>(P, C, s->stream);
   vcycle<T, Form>(s, Ls, P, l + 1);
   qn::launch_prolong(P, F, C, s->stream);
-  qn::launch_bc_unknowns(F, s->stream);
   smooth_steps<T, Form>(s, Ls, P, l, nu_post(s, l));
 }
 
