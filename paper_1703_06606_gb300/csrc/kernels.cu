@@ -41,15 +41,21 @@ long long launches_issued() { return g_launches.load(); }
 // (griddepcontrol.wait) until the predecessor grid has completed and its
 // memory is visible.  The wait comes before any access to global memory, so
 // the order of effects is that of plain stream order; what is saved is part of
-// the gap between dependent launches (measured: ~1.3 % of a droplet step).  An
-// explicit early trigger (griddepcontrol.launch_dependents at kernel entry)
-// measured 13 % slower: the successor's blocks were placed while the
-// predecessor still held the SMs, and these latency-bound launches lost their
-// even spread over the sub-partitions.
+// the gap between dependent launches (measured: ~1.3 % of a droplet step).  A
+// grid of at most PDL_EARLY blocks also lets its successor's blocks come in
+// while it runs (launch_dependents), to fetch their code and parameters and
+// wait: 256x512 mixed step 17.9 -> 17.4 ms, 512x512 coupled mixed 7.6 -> 7.4 ms,
+// the rest within 1 %.  Not above that: the waiting blocks would take the SMs
+// that the running grid's neighbours in time are meant to spread over (every
+// grid early: 256x512 FP64 51.6 -> 57.5 ms; up to 76 blocks: a batch of
+// instances, whose streams compete for the SMs, 9.8 -> 10.0 ms).
+constexpr unsigned PDL_EARLY = 32;
 static std::atomic<int> g_pdl{1};
 void set_pdl(int on) { g_pdl = on ? 1 : 0; }
 __device__ __forceinline__ void pdl_enter() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (gridDim.x * gridDim.y * gridDim.z <= PDL_EARLY)
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 template <typename... KArgs, typename... Args>
 static void qlaunch(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
