@@ -110,7 +110,15 @@ __device__ __forceinline__ void warp_sum5(double& a, double& b, double& c, doubl
   e = __shfl_sync(FULL, wz, 4);
 }
 
-template <int NV>
+// the rows a thread evaluates: all, or a third of their work (ROLE 0: N_c and
+// N_p, which share the flux sum; 1: N_mu; 2: the momentum rows)
+constexpr int ROLE_ALL = -1;
+template <int ROLE>
+__host__ __device__ constexpr bool role_has(int q) {
+  return ROLE == ROLE_ALL || (ROLE == 0 ? q == 0 || q == 2 : ROLE == 1 ? q == 1 : q >= 3);
+}
+// ROLE: only the entries q and 5 + q of the residual families q of that role
+template <int NV, int ROLE = -1>
 __device__ __forceinline__ void block_sum_store(double (&val)[NV], double* part, int nmax_first) {
   // first `nmax_first` values are reduced with max, the rest with sum.  The
   // max values are non-negative (or NaN), whose bit patterns order as the
@@ -118,9 +126,11 @@ __device__ __forceinline__ void block_sum_store(double (&val)[NV], double* part,
   // 64-bit integers, off the FP64 pipe.
   __shared__ double sh[NT / 32][NV];
   int lane = (threadIdx.y * BX + threadIdx.x) & 31, warp = (threadIdx.y * BX + threadIdx.x) >> 5;
-  if constexpr (NV == 10) warp_sum5(val[5], val[6], val[7], val[8], val[9]);
+  constexpr bool FIVE = NV == 10 && ROLE == -1;
+  if constexpr (FIVE) warp_sum5(val[5], val[6], val[7], val[8], val[9]);
 #pragma unroll
   for (int q = 0; q < NV; ++q) {
+    if (!role_has<ROLE>(q % 5)) continue;
     double x = val[q];
     if (q < nmax_first) {
       long long b = __double_as_longlong(x);
@@ -129,7 +139,7 @@ __device__ __forceinline__ void block_sum_store(double (&val)[NV], double* part,
         b = c > b ? c : b;
       }
       x = __longlong_as_double(b);
-    } else if (NV != 10) {
+    } else if (!FIVE) {
       for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
     }
     if (lane == 0) sh[warp][q] = x;
@@ -138,6 +148,7 @@ __device__ __forceinline__ void block_sum_store(double (&val)[NV], double* part,
   if (warp == 0) {
 #pragma unroll
     for (int q = 0; q < NV; ++q) {
+      if (!role_has<ROLE>(q % 5)) continue;
       double x = sh[lane & (NT / 32 - 1)][q];  // lane 0 reduces the values of lanes 0 .. NT/32 - 1
       for (int o = NT / 64; o > 0; o >>= 1) {
         const double y = __shfl_down_sync(0xffffffffu, x, o);
@@ -257,48 +268,50 @@ template <typename T>
 struct Rows5 {
   T r[5];
 };
-// at thread (i,j): cell families at (i,j), u-edge (i,j) and v-edge (i,j)
-template <typename T, int MODE, class Form, class LV>
+// at thread (i,j): cell families at (i,j), u-edge (i,j) and v-edge (i,j); the
+// edge rows also on boundary edges (padded arrays), which are masked later
+template <typename T, int MODE, class Form, int ROLE, class LV>
 __device__ __forceinline__ Rows5<T> residual_rows5(const Prm<T>& P, const LV& L, int i, int j) {
-  int k = L.at(i, j);
-  const T f[5] = {L.fc[k], L.fmu[k], L.fp[k], L.fu[k], L.fv[k]};
-  T nc, nm, np, nu, nv;
-  if constexpr (std::is_same<Form, FullForm>::value) {
-    // rho(c) of the cell and its neighbours, shared by the five rows, and the
-    // flux sum shared by N_c and N_p
-    const int W = L.pitch;
-    auto rc = L.rhoc;
-    T rk = rc[k];
-    const T rq[4] = {rc[k + 1], rc[k - 1], rc[k + W], rc[k - W]};
-    T flux = flux_sum(P, L, k);
-    nc = rk * (L.c[k] - L.cn[k]) * P.idt + adv_sum(L, k) - L.k.dif * flux;
-    nm = chem_full(P, L, k, rk, rq);
-    np = (L.u[k] - L.u[k - 1] + L.v[k] - L.v[k - W]) * L.ih - L.k.adif * flux;
-    nu = mom_asm<true>(L, 0, k, rk + rq[0]);  // also on boundary edges (padded arrays); masked below
-    nv = mom_asm<true>(L, 1, k, rk + rq[2]);
-  } else if constexpr (std::is_same<Form, ProjForm>::value) {
-    const int W = L.pitch;
-    auto rc = L.rhoc;
-    T rk = rc[k];
-    const T rq[4] = {rc[k + 1], rc[k - 1], rc[k + W], rc[k - W]};
-    T w[4];
-    proj_faces(P, L, i, j, rk, rq, w);
-    T flux = flux_sum(P, L, k);
-    nc = opp_c_w(P, L, k, rq, w, flux);
-    nm = chem_full(P, L, k, rk, rq) + (L.rhon[k] - rk) * L.mu[k];  // rho^n in front of mu
-    np = opp_p_w(L, w, flux);
-    nu = mom_asm<false>(L, 0, k, rk + rq[0]);
-    nv = mom_asm<false>(L, 1, k, rk + rq[2]);
-  } else {
+  const int k = L.at(i, j), W = L.pitch;
+  constexpr bool CP = role_has<ROLE>(0), MU = role_has<ROLE>(1), UV = role_has<ROLE>(3);
+  const T f[5] = {CP ? L.fc[k] : T(0), MU ? L.fmu[k] : T(0), CP ? L.fp[k] : T(0),
+                  UV ? L.fu[k] : T(0), UV ? L.fv[k] : T(0)};
+  T n[5] = {T(0), T(0), T(0), T(0), T(0)};
+  if constexpr (std::is_same<Form, ErrForm>::value) {
     const ErrCell<T> X = err_cell(P, L, k);
     T flux = flux_sum(P, L, k);
-    nc = err_c(P, L, k, X.r[0]) - L.k.dif * flux;
-    nm = err_mu(P, L, k, X);
-    np = (L.u[k] - L.u[k - 1] + L.v[k] - L.v[k - L.pitch]) * L.ih - L.k.adif * flux;
-    nu = err_row(P, L, 0, k, X.r[0] + X.r[1], X.dr[0] + X.dr[1]);  // wall edges too, as above
-    nv = err_row(P, L, 1, k, X.r[0] + X.r[3], X.dr[0] + X.dr[3]);
+    n[0] = err_c(P, L, k, X.r[0]) - L.k.dif * flux;
+    n[1] = err_mu(P, L, k, X);
+    n[2] = (L.u[k] - L.u[k - 1] + L.v[k] - L.v[k - W]) * L.ih - L.k.adif * flux;
+    n[3] = err_row(P, L, 0, k, X.r[0] + X.r[1], X.dr[0] + X.dr[1]);
+    n[4] = err_row(P, L, 1, k, X.r[0] + X.r[3], X.dr[0] + X.dr[3]);
+  } else {
+    constexpr bool PROJ = std::is_same<Form, ProjForm>::value;
+    // rho(c) of the cell and its neighbours, shared by the rows
+    auto rc = L.rhoc;
+    const T rk = rc[k];
+    const T rq[4] = {rc[k + 1], rc[k - 1], rc[k + W], rc[k - W]};
+    if constexpr (CP) {
+      T flux = flux_sum(P, L, k);
+      if constexpr (PROJ) {
+        T w[4];
+        proj_faces(P, L, i, j, rk, rq, w);
+        n[0] = opp_c_w(P, L, k, rq, w, flux);
+        n[2] = opp_p_w(L, w, flux);
+      } else {
+        n[0] = rk * (L.c[k] - L.cn[k]) * P.idt + adv_sum(L, k) - L.k.dif * flux;
+        n[2] = (L.u[k] - L.u[k - 1] + L.v[k] - L.v[k - W]) * L.ih - L.k.adif * flux;
+      }
+    }
+    if constexpr (MU) {
+      n[1] = chem_full(P, L, k, rk, rq);
+      if constexpr (PROJ) n[1] += (L.rhon[k] - rk) * L.mu[k];  // rho^n in front of mu
+    }
+    if constexpr (UV) {
+      n[3] = mom_asm<!PROJ>(L, 0, k, rk + rq[0]);
+      n[4] = mom_asm<!PROJ>(L, 1, k, rk + rq[2]);
+    }
   }
-  const T n[5] = {nc, nm, np, nu, nv};
   Rows5<T> X;
 #pragma unroll
   for (int q = 0; q < 5; ++q) X.r[q] = MODE == 0 ? f[q] - n[q] : f[q] + n[q];
@@ -306,37 +319,34 @@ __device__ __forceinline__ Rows5<T> residual_rows5(const Prm<T>& P, const LV& L,
 }
 // stores them (MODE 0: into r, MODE 1: into f) and adds to val: the largest |r|
 // and the sum of r^2 per family (MODE 0)
-template <typename T, int MODE, class LV>
+template <typename T, int MODE, int ROLE, class LV>
 __device__ __forceinline__ void residual_store(const LV& L, int i, int j, const Rows5<T>& X,
                                                double (&val)[10]) {
   const int k = L.at(i, j);
   const bool own[5] = {true, true, true, i <= L.uhi(), j < L.m2};
+  const bool has[5] = {role_has<ROLE>(0), role_has<ROLE>(1), role_has<ROLE>(2),
+                       role_has<ROLE>(3) && own[3], role_has<ROLE>(4) && own[4]};
+  if (has[0]) (MODE == 0 ? L.rc[k] : L.fc[k]) = X.r[0];
+  if (has[1]) (MODE == 0 ? L.rmu[k] : L.fmu[k]) = X.r[1];
+  if (has[2]) (MODE == 0 ? L.rp[k] : L.fp[k]) = X.r[2];
+  if (has[3]) (MODE == 0 ? L.ru[k] : L.fu[k]) = X.r[3];
+  if (has[4]) (MODE == 0 ? L.rv[k] : L.fv[k]) = X.r[4];
   if (MODE == 0) {
-    L.rc[k] = X.r[0];
-    L.rmu[k] = X.r[1];
-    L.rp[k] = X.r[2];
-    if (own[3]) L.ru[k] = X.r[3];
-    if (own[4]) L.rv[k] = X.r[4];
 #pragma unroll
     for (int q = 0; q < 5; ++q) {
+      if (!role_has<ROLE>(q)) continue;
       const double a = own[q] ? (double)X.r[q] : 0.0;
       // |r| >= 0 or NaN: the bit patterns order as the values
       const long long b = __double_as_longlong(fabs(a)), m = __double_as_longlong(val[q]);
       val[q] = __longlong_as_double(b > m ? b : m);
       val[5 + q] += a * a;
     }
-  } else {
-    L.fc[k] = X.r[0];
-    L.fmu[k] = X.r[1];
-    L.fp[k] = X.r[2];
-    if (own[3]) L.fu[k] = X.r[3];
-    if (own[4]) L.fv[k] = X.r[4];
   }
 }
 template <typename T, int MODE, class Form, class LV>
 __device__ __forceinline__ void residual_cell(const Prm<T>& P, const LV& L, int i, int j,
                                               double (&val)[10]) {
-  residual_store<T, MODE>(L, i, j, residual_rows5<T, MODE, Form>(P, L, i, j), val);
+  residual_store<T, MODE, ROLE_ALL>(L, i, j, residual_rows5<T, MODE, Form, ROLE_ALL>(P, L, i, j), val);
 }
 
 // ROWS > 1 (large levels): each thread takes ROWS / 2 pairs of rows BY apart, so
@@ -356,13 +366,34 @@ __global__ void __launch_bounds__(NT, 2) k_residual(Prm<T> P, Lv<T> L, double* p
     for (int r = 0; r < ROWS; r += 2, j += 2 * BY) {
       if (i > L.m1 || j > L.m2) break;
       const bool two = j + BY <= L.m2;
-      const Rows5<T> A = residual_rows5<T, MODE, Form>(P, L, i, j);
-      const Rows5<T> B = residual_rows5<T, MODE, Form>(P, L, i, two ? j + BY : j);
-      residual_store<T, MODE>(L, i, j, A, val);
-      if (two) residual_store<T, MODE>(L, i, j + BY, B, val);
+      const Rows5<T> A = residual_rows5<T, MODE, Form, ROLE_ALL>(P, L, i, j);
+      const Rows5<T> B = residual_rows5<T, MODE, Form, ROLE_ALL>(P, L, i, two ? j + BY : j);
+      residual_store<T, MODE, ROLE_ALL>(L, i, j, A, val);
+      if (two) residual_store<T, MODE, ROLE_ALL>(L, i, j + BY, B, val);
     }
   }
   if (MODE == 0 && part) block_sum_store<10>(val, part, 5);
+}
+
+// The rows of a cell by three threads (ROLE: the block's z), for levels that
+// leave most of the FP64 pipes idle: a thread's chain of FP64 instructions, 64
+// cycles each, is what such a launch takes, and the longest third is 50 of the
+// 134.  A role's blocks write its families' entries of the partials.
+template <typename T, int MODE, class Form, int ROLE>
+__device__ __forceinline__ void residual_role(const Prm<T>& P, const Lv<T>& L, double* part) {
+  int i = blockIdx.x * BX + threadIdx.x + 1;
+  int j = blockIdx.y * BY + threadIdx.y + 1;
+  double val[10] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
+  if (i <= L.m1 && j <= L.m2)
+    residual_store<T, MODE, ROLE>(L, i, j, residual_rows5<T, MODE, Form, ROLE>(P, L, i, j), val);
+  if (MODE == 0 && part) block_sum_store<10, ROLE>(val, part, 5);
+}
+template <typename T, int MODE, class Form>
+__global__ void __launch_bounds__(NT, 2) k_residual_split(Prm<T> P, Lv<T> L, double* part) {
+  pdl_enter();
+  if (blockIdx.z == 0) residual_role<T, MODE, Form, 0>(P, L, part);
+  else if (blockIdx.z == 1) residual_role<T, MODE, Form, 1>(P, L, part);
+  else residual_role<T, MODE, Form, 2>(P, L, part);
 }
 
 // rows per residual thread on level L: two on levels of at least 65536 cells,
@@ -2222,7 +2253,6 @@ __global__ void __launch_bounds__(SNT, 4) k_vanka_team(Prm<T> P, Lv<T> L, int co
 template <typename T, class Form, class LV>
 __device__ __forceinline__ void vanka_pair(const Prm<T>& P, const LV& L, int i, int j, bool ok,
                                            T omega) {
-  const unsigned FULL = 0xffffffffu;
   const int W = L.pitch;
   const int d = threadIdx.x & 1;
   const T ih = L.ih, ih2 = L.ih2;
@@ -3323,6 +3353,21 @@ int nparts_cells(const Lv<T>& L) {
   return g.x * g.y;
 }
 
+// Three threads a cell on FP64 full-iterate levels of at most 32768 cells: three
+// threads' warps then still are at most five a sub-partition.  (FP32 levels: a
+// thread's chain is its loads, which the roles would repeat.)
+template <typename T, class Form>
+static bool residual_split(const Lv<compute_t<T, Form>>& L) {
+  return !std::is_same<Form, ErrForm>::value && (long long)L.m1 * L.m2 <= 32768;
+}
+template <typename R, int MODE, class Form>
+static void launch_residual_split(const Prm<R>& P, const Lv<R>& L, double* part, cudaStream_t s) {
+  if constexpr (!std::is_same<Form, ErrForm>::value) {
+    dim3 g = grid2(L.m1, L.m2);
+    g.z = 3;
+    qlaunch(&k_residual_split<R, MODE, Form>, g, dim3(BX, BY), 0, s, P, L, part);
+  }
+}
 template <typename T, class Form>
 void launch_residual(const Prm<T>& P0, const Lv<T>& L0, double* part, cudaStream_t s) {
   typedef compute_t<T, Form> R;
@@ -3333,6 +3378,8 @@ void launch_residual(const Prm<T>& P0, const Lv<T>& L0, double* part, cudaStream
     qlaunch(&k_residual<R, 0, Form, 8>, grid2(L.m1, (L.m2 + 7) / 8), dim3(BX, BY), 0, s, P, L, part);
   else if (rows == 2)
     qlaunch(&k_residual<R, 0, Form, 2>, grid2(L.m1, (L.m2 + 1) / 2), dim3(BX, BY), 0, s, P, L, part);
+  else if (residual_split<T, Form>(L))
+    launch_residual_split<R, 0, Form>(P, L, part, s);
   else
     qlaunch(&k_residual<R, 0, Form, 1>, grid2(L.m1, L.m2), dim3(BX, BY), 0, s, P, L, part);
   ++g_launches;
@@ -3347,6 +3394,8 @@ void launch_add_op(const Prm<T>& P0, const Lv<T>& L0, cudaStream_t s) {
     qlaunch(&k_residual<R, 1, Form, 8>, grid2(L.m1, (L.m2 + 7) / 8), dim3(BX, BY), 0, s, P, L, nullptr);
   else if (rows == 2)
     qlaunch(&k_residual<R, 1, Form, 2>, grid2(L.m1, (L.m2 + 1) / 2), dim3(BX, BY), 0, s, P, L, nullptr);
+  else if (residual_split<T, Form>(L))
+    launch_residual_split<R, 1, Form>(P, L, nullptr, s);
   else
     qlaunch(&k_residual<R, 1, Form, 1>, grid2(L.m1, L.m2), dim3(BX, BY), 0, s, P, L, nullptr);
   ++g_launches;
