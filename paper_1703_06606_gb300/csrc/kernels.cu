@@ -17,10 +17,9 @@ namespace qn {
 
 constexpr int BX = 32, BY = 8, NT = BX * BY;
 
-// the type a kernel computes in for data of type T: the error equation's
-// kernels with their contraction fixed (Fused)
+// the type a kernel computes in for data of type T: with its contraction fixed
 template <typename T, class Form>
-using compute_t = typename std::conditional<std::is_same<Form, ErrForm>::value, Fused<T>, T>::type;
+using compute_t = Fused<T>;
 // the same bits as data of the kernel's type
 template <typename R, template <typename> class S, typename T>
 static inline const S<R>& as_compute(const S<T>& x) {
@@ -619,7 +618,10 @@ __device__ __forceinline__ T proj_face_team(const Prm<T>& P, const LV& L, int k,
   const int d = q >> 1, off = d ? L.pitch : 1;
   const bool hi = q & 1;  // E or N: the face's velocity sits at k
   const int a = hi ? k : k - off;
-  auto vel = d ? L.v : L.u; auto c = L.c; auto mu = L.mu; auto p = L.p;
+  auto vel = L.pair(d, L.u, L.v);
+  auto c = L.c;
+  auto mu = L.mu;
+  auto p = L.p;
   T ra = hi ? rk : rn, rb = hi ? rn : rk;
   return open ? vel[a] + proj_kick(L, ra, rb, mu[a], mu[a + off], c[a + off] - c[a], p[a + off] - p[a]) -
                     (d ? L.k.gdt : T(0))
@@ -654,24 +656,24 @@ constexpr bool lane_teams = sizeof(T) == 8;
 // lane receiving all eight: the first exchange halves what a lane adds up
 // (4 + 2 additions a lane where eight butterflies take 16; each addition is
 // that of team_sum, so the sums are the same)
-__device__ __forceinline__ void team_sum8(double (&v)[8]) {
-  const unsigned FULL = 0xffffffffu;
+template <typename T>
+__device__ __forceinline__ void team_sum8(T (&v)[8]) {
   const int lane = threadIdx.x & 31;
   const bool b0 = lane & 1, b1 = lane & 2;
-  double r[4], t[2];
+  T r[4], t[2];
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
-    double send = b0 ? v[i] : v[i + 4], keep = b0 ? v[i + 4] : v[i];
+    T send = b0 ? v[i] : v[i + 4], keep = b0 ? v[i + 4] : v[i];
     r[i] = keep + shfl_xor(send, 1);
   }
 #pragma unroll
   for (int i = 0; i < 2; ++i) {
-    double send = b1 ? r[i] : r[i + 2], keep = b1 ? r[i + 2] : r[i];
+    T send = b1 ? r[i] : r[i + 2], keep = b1 ? r[i + 2] : r[i];
     t[i] = keep + shfl_xor(send, 2);
   }
 #pragma unroll
   for (int m = 0; m < 8; ++m)
-    v[m] = __shfl_sync(FULL, t[m & 1], (lane & 28) | (m >> 2) | (m & 2));
+    v[m] = shfl_from(t[m & 1], (lane & 28) | (m >> 2) | (m & 2));
 }
 
 // The CH rows of cell (i,j) for a team of four lanes (lane & 3 = q: face W,
@@ -688,11 +690,9 @@ struct ChRows {
 };
 
 // ch_team_rows for the full iterate: ch_system_full's sums, a face a lane
-template <bool PROJ>
-__device__ __forceinline__ ChRows<double> ch_team_rows_full(const Prm<double>& P,
-                                                            const Lv<double>& L, int i, int j,
-                                                            int q, bool open, double rk, double rq) {
-  typedef double T;
+template <bool PROJ, typename T, class LV>
+__device__ __forceinline__ ChRows<T> ch_team_rows_full(const Prm<T>& P, const LV& L, int i, int j,
+                                                       int q, bool open, T rk, T rq) {
   const int W = L.pitch;
   const int d = q >> 1;
   const int k = L.at(i, j);
@@ -913,7 +913,7 @@ __device__ __forceinline__ void vanka_system(const Prm<T>& P, const LV& L, int i
     constexpr bool PST = std::is_same<Form, FullForm>::value;
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-      A[q][q] = (q < 2 ? L.Dgu : L.Dgv)[ke[q]] + L.k.qidt * rs[q];  // per-step coefficients
+      A[q][q] = L.pair(q >> 1, L.Dgu, L.Dgv)[ke[q]] + L.k.qidt * rs[q];  // per-step coefficients
       rows[q] = mom_asm<PST>(L, q >> 1, ke[q], rs[q]);
     }
     const T v1 = vis[k] * L.k.v1, sx = L.k.hih * L.Sx[k], sy = L.k.hih * L.Sy[k];
@@ -2214,8 +2214,9 @@ __global__ void __launch_bounds__(SNT, 4) k_coupled_team(Prm<T> P, Lv<T> L, int 
 
 // per-level launch with eight lanes per Vanka block (vanka_team8; FP64 full
 // iterate)
-__global__ void __launch_bounds__(SNT, 4) k_vanka_team8(Prm<double> P, Lv<double> L, int colour,
-                                                     double omega) {
+template <typename T>
+__global__ void __launch_bounds__(SNT, 4) k_vanka_team8(Prm<T> P, Lv<T> L, int colour,
+                                                     T omega) {
   pdl_enter();
   ColourSlots cs = vanka_slots(L, colour);
   int t = blockIdx.x * SNT + threadIdx.x;
@@ -2223,7 +2224,7 @@ __global__ void __launch_bounds__(SNT, 4) k_vanka_team8(Prm<double> P, Lv<double
   int i = 1, j = 1;
   bool ok = (t >> 3) < cs.n && vanka_slot_cell(L, colour, cs, t >> 3, i, j);
   if (!ok) i = j = 1;
-  vanka_team8<double>(P, L, i, j, ok, omega);
+  vanka_team8<T>(P, L, i, j, ok, omega);
 }
 
 template <typename T, class Form>
@@ -2474,7 +2475,7 @@ __device__ __forceinline__ void smooth_block(const Prm<T>& P, const LV& L, T ome
         int i = 1, j = 1;
         bool ok = (t >> 3) < cs.n && vanka_slot_cell(L, col, cs, t >> 3, i, j);
         if (!ok) i = j = 1;
-        if constexpr (team_ok) vanka_team8<double>(P, L, i, j, ok, omega);
+        if constexpr (team_ok && LV::all_arrays) vanka_team8<T>(P, L, i, j, ok, omega);
       }
     } else if (vteam_ok && cs.n <= team_slots) {
       int t = grp_rank();
@@ -2504,8 +2505,8 @@ __device__ __forceinline__ void coarse_vcycle_body(const Prm<T>& P, const Get& g
                                                    int nu1, int nu2, int nuc, T omega, int coupled,
                                                    int team8) {
   double dummy[10];
-  if (base) {
-    for (int l = 1; l < n; ++l) {
+  if constexpr (std::is_same<Form, ErrForm>::value) {
+    for (int l = 1; base && l < n; ++l) {
       const auto& F = get(l - 1);
       const auto& G = get(l);
       for (int t = grp_rank(); t < (G.m1 + 1) * (G.m2 + 1); t += grp_size())
@@ -2566,9 +2567,9 @@ __global__ void __launch_bounds__(NT, 1) k_coarse_vcycle(Prm<T> P, CoarseLevels<
 // writes) into shared memory at the compact pitch m1 + 3, runs the V-cycle
 // body unchanged on level descriptors that point into the copy, and writes
 // back the arrays the V-cycle writes: the unknowns, sources, residuals and the
-// kept restricted iterate (the first 20 arrays) and rho(c).  copy = 0 leaves
-// the descriptors on the level's own arrays: one instance of the code serves
-// both, so the two give the same bits.
+// kept restricted iterate (the first 20 arrays) and rho(c).  For eight-lane
+// Vanka blocks (vanka_team8), which read arrays that the records of
+// k_coarse_records leave out.
 // --------------------------------------------------------------------------
 constexpr int QN_LV_NARR = 59;     // arrays of QN_LV_ARRAYS
 constexpr int QN_LV_WRITTEN = 20;  // arrays 0..19 are written; and rho(c):
@@ -2610,167 +2611,199 @@ __device__ __forceinline__ void coarse_copy(double* __restrict__ g, int pg, long
 }
 
 template <int NT>
-__global__ void __launch_bounds__(NT, 1) k_coarse_vcycle_smem(Prm<double> P, CoarseLevels<double> C,
-                                                           CoarseSmem M, int copy, int nu1, int nu2,
-                                                           int nuc, double omega, int coupled,
+__global__ void __launch_bounds__(NT, 1) k_coarse_vcycle_smem(Prm<rf64> P, CoarseLevels<rf64> C,
+                                                           CoarseSmem M, int nu1, int nu2,
+                                                           int nuc, rf64 omega, int coupled,
                                                            int team8) {
   extern __shared__ __align__(16) double qn_coarse_smem[];
   pdl_enter();
-  CoarseLevels<double>* S = reinterpret_cast<CoarseLevels<double>*>(qn_coarse_smem);
+  CoarseLevels<rf64>* S = reinterpret_cast<CoarseLevels<rf64>*>(qn_coarse_smem);
   double* arr = qn_coarse_smem + M.head;
   const int n = C.n;
-  for (int l = 0; copy && l < n; ++l) {
-    const Lv<double>& G = C.L[l];
+  for (int l = 0; l < n; ++l) {
+    const Lv<rf64>& G = C.L[l];
     const int cc = G.m1 + 3, rr = G.m2 + 3;
-    coarse_copy<NT, true>(G.c - (G.pitch + 1), G.pitch, M.ng[l], arr + M.off[l], cc, rr, 0,
+    coarse_copy<NT, true>(&G.c->v - (G.pitch + 1), G.pitch, M.ng[l], arr + M.off[l], cc, rr, 0,
                           QN_LV_NARR);
   }
   if (threadIdx.x < n) {  // the descriptor of level l, its arrays in the copy
     const int l = threadIdx.x;
-    Lv<double> X = C.L[l];
-    if (copy) {
-      const int cc = X.m1 + 3, ns = cc * (X.m2 + 3);
-      double* o = arr + M.off[l] + cc + 1;  // origin (0,0) of array 0
-      int q = 0;
+    Lv<rf64> X = C.L[l];
+    const int cc = X.m1 + 3, ns = cc * (X.m2 + 3);
+    rf64* o = reinterpret_cast<rf64*>(arr + M.off[l] + cc + 1);  // origin (0,0) of array 0
+    int q = 0;
 #define QN_REBASE(m) X.m = o + (q++) * ns;
-      QN_LV_ARRAYS(QN_REBASE)
+    QN_LV_ARRAYS(QN_REBASE)
 #undef QN_REBASE
-      X.pitch = cc;
-      X.nst = ns;
-    }
+    X.pitch = cc;
+    X.nst = ns;
     S->L[l] = X;
   }
   asm volatile("cp.async.wait_all;" ::: "memory");
   __syncthreads();
-  coarse_vcycle_body<double, FullForm>(P, LevelsOf<double>{*S}, n, 0, nu1, nu2, nuc, omega, coupled,
+  coarse_vcycle_body<rf64, FullForm>(P, LevelsOf<rf64>{*S}, n, 0, nu1, nu2, nuc, omega, coupled,
                                        team8);
   __syncthreads();
-  for (int l = 0; copy && l < n; ++l) {
-    const Lv<double>& G = C.L[l];
+  for (int l = 0; l < n; ++l) {
+    const Lv<rf64>& G = C.L[l];
     const int cc = G.m1 + 3, rr = G.m2 + 3;
-    double* g = G.c - (G.pitch + 1);
+    double* g = &G.c->v - (G.pitch + 1);
     coarse_copy<NT, false>(g, G.pitch, M.ng[l], arr + M.off[l], cc, rr, 0, QN_LV_WRITTEN);
     coarse_copy<NT, false>(g, G.pitch, M.ng[l], arr + M.off[l], cc, rr, QN_LV_RHOC, QN_LV_RHOC + 1);
   }
 }
 
 // --------------------------------------------------------------------------
-// The fused V-cycle of FP32 error-equation levels on a shared-memory copy.  Its
-// visits have no slow arithmetic: what a colour step cost was the chain of
-// address arithmetic (a 64-bit address for each of the ~60 array elements a
-// visit reads) and L2 round trips.  The copy interleaves the level's arrays:
-// cell k's 43 values sit together (LvS), so that a visit forms three
-// addresses (its row and the rows beside it) and reads everything else at
-// constant offsets from them.  43 words a cell is odd, so lanes on cells any
-// power of two (or 5) apart fall into different banks.
-// Measured (GB300, ncu, caches warm): the 16x32 .. 2x4 levels of the 256x512
-// drop 245 -> 139 us, the 28x28 and 14x14 levels of a served 448x448 request
-// (64 coupled sweeps on the coarsest) 1504 -> 1121 us.  Launched wherever the
-// records fit the opt-in shared memory (option coarse_smem; about 1350 padded
-// cells); a larger group reads global memory.
+// The fused V-cycle on interleaved shared-memory records.  What a colour step
+// cost beside its arithmetic was the chain of address arithmetic (a 64-bit
+// address for each of the ~60 array elements a visit reads) and L2 round
+// trips.  The copy interleaves the arrays that the V-cycle touches: a cell's
+// values sit together, so that a visit forms three addresses (its row and the
+// rows beside it) and reads everything else at constant offsets from them.  An
+// odd number of values a cell keeps lanes on cells any power of two (or 5)
+// apart in different banks.  The operators are the grid kernels' own
+// (templates over the level), in the type whose rounding the source fixes, so
+// the results are those of the launch that reads global memory.
+// Measured (GB300, ncu, caches warm), FP32 error levels: 16x32 .. 2x4 of the
+// 256x512 drop 245 -> 139 us, 28x28 and 14x14 of a served 448x448 request (64
+// coupled sweeps on the coarsest) 1504 -> 1121 us (89 and 990 us with the
+// launch bounds and one lane a visit that came after).
 // --------------------------------------------------------------------------
-// the arrays of an error-equation level that its V-cycle touches, in the order
-// of a cell's record
-#define QN_ERR_ARRAYS(X)                                                                       \
-  X(c) X(mu) X(p) X(u) X(v) X(fc) X(fmu) X(fp) X(fu) X(fv) X(rc) X(rmu) X(rp) X(ru) X(rv)     \
-  X(sc) X(smu) X(sp) X(su) X(sv) X(cn) X(rhon) X(mobn) X(visn) X(Gn) X(T1u) X(T1v) X(aPu)    \
-  X(aPv) X(aMu) X(aMv) X(tPu) X(tPv) X(tMu) X(tMv) X(Tx) X(Ty) X(Bc) X(Bmu) X(Bu) X(Bv)       \
-  X(Bdc) X(rB)
-enum {
-#define QN_ERR_INDEX(m) ERR_##m,
-  QN_ERR_ARRAYS(QN_ERR_INDEX)
-#undef QN_ERR_INDEX
-      ERR_N
-};
-static_assert(ERR_N % 2 == 1, "an odd record keeps strided lanes in different banks");
-
-// array OFF of the records at b: element k as if it were a plain array
-template <typename T, int OFF>
+// array OFF of records of N values at b: element k as if it were a plain array
+template <typename T, int OFF, int N>
 struct Fld {
   T* b;
-  __device__ __forceinline__ T& operator[](int k) const { return b[k * ERR_N + OFF]; }
+  __device__ __forceinline__ T& operator[](int k) const { return b[k * N + OFF]; }
+  __device__ __forceinline__ explicit operator bool() const { return true; }  // it is there
 };
-// an error-equation level in records (the members and constants of Lv)
-template <typename T>
-struct LvS {
-  typedef T real;
-  static constexpr bool has_rho = false;
-  LvK<T> k;
-  FastDiv vrow, crow, kdiv;
-  int m1, m2, px, pitch, kcol, c8;
-  T h, ih, ih2;
-#define QN_ERR_MEMBER(m) Fld<T, ERR_##m> m;
-  QN_ERR_ARRAYS(QN_ERR_MEMBER)
-#undef QN_ERR_MEMBER
-  // level L with its record of cell (0,0) at b
-  __device__ __forceinline__ LvS(const Lv<T>& L, T* b)
-      : k(L.k), vrow(L.vrow), crow(L.crow), kdiv(L.kdiv), m1(L.m1), m2(L.m2), px(L.px), pitch(L.m1 + 3), kcol(L.kcol), c8(L.c8), h(L.h),
-        ih(L.ih), ih2(L.ih2) {
-#define QN_ERR_SET(m) m.b = b;
-    QN_ERR_ARRAYS(QN_ERR_SET)
-#undef QN_ERR_SET
+// A level in records (the members and constants of Lv); pairs of directions are
+// neighbours in the record.  From level L and its record of cell (0,0) at b.
+#define QN_RECORD_INDEX(m) I_##m,
+#define QN_RECORD_MEMBER(m) Fld<T, I_##m, N> m;
+#define QN_RECORD_SET(m) m.b = b;
+#define QN_RECORD_LEVEL(NAME, ARRAYS, RHO)                                                     \
+  template <typename T>                                                                        \
+  struct NAME {                                                                                \
+    typedef T real;                                                                            \
+    enum { ARRAYS(QN_RECORD_INDEX) COUNT, N = COUNT | 1 };                                     \
+    static constexpr bool has_rho = RHO, all_arrays = false;                                   \
+    LvK<T> k;                                                                                  \
+    FastDiv vrow, crow, kdiv;                                                                  \
+    int m1, m2, px, pitch, kcol, c8;                                                           \
+    T h, ih, ih2;                                                                              \
+    ARRAYS(QN_RECORD_MEMBER)                                                                   \
+    __device__ __forceinline__ NAME(const Lv<T>& L, T* b)                                      \
+        : k(L.k), vrow(L.vrow), crow(L.crow), kdiv(L.kdiv), m1(L.m1), m2(L.m2), px(L.px),      \
+          pitch(L.m1 + 3), kcol(L.kcol), c8(L.c8), h(L.h), ih(L.ih), ih2(L.ih2) {              \
+      ARRAYS(QN_RECORD_SET)                                                                    \
+    }                                                                                          \
+    __device__ __forceinline__ int at(int i, int j) const { return j * pitch + i; }            \
+    __device__ __forceinline__ int uhi() const { return px ? m1 : m1 - 1; }                    \
+    template <int OFF>                                                                         \
+    __device__ __forceinline__ Fld<T, OFF, N> pair(int d, Fld<T, OFF, N> x,                    \
+                                                   Fld<T, OFF + 1, N>) const {                 \
+      return {x.b + d};                                                                        \
+    }                                                                                          \
+    template <int OFF>                                                                         \
+    __device__ __forceinline__ Fld<T, OFF, N> row_pair(int d, Fld<T, OFF, N> x,                \
+                                                       Fld<T, OFF + 1, N>) const {             \
+      return {x.b + d};                                                                        \
+    }                                                                                          \
   }
-  __device__ __forceinline__ int at(int i, int j) const { return j * pitch + i; }
-  __device__ __forceinline__ int uhi() const { return px ? m1 : m1 - 1; }
-  // neighbours in the record: the pair's second array is the first one element on
-  template <int OFF>
-  __device__ __forceinline__ Fld<T, OFF> pair(int d, Fld<T, OFF> x, Fld<T, OFF + 1>) const {
-    return {x.b + d};
-  }
+// the unknowns, right-hand sides, residuals, the kept iterate; c^n and its fields
+#define QN_COMMON_ARRAYS(X)                                                                    \
+  X(c) X(mu) X(p) X(u) X(v) X(fc) X(fmu) X(fp) X(fu) X(fv) X(rc) X(rmu) X(rp) X(ru) X(rv)      \
+  X(sc) X(smu) X(sp) X(su) X(sv) X(cn) X(rhon) X(mobn) X(visn) X(Gn) X(Tx) X(Ty)
+// error equation: the rows' coefficients and the base
+#define QN_ERR_ARRAYS(X)                                                                       \
+  QN_COMMON_ARRAYS(X) X(T1u) X(T1v) X(aPu) X(aPv) X(aMu) X(aMv) X(tPu) X(tPv) X(tMu) X(tMv)    \
+  X(Bc) X(Bmu) X(Bu) X(Bv) X(Bdc) X(rB)
+// full iterate: rho(c), the rows' stencils, their diagonals and couplings
+#define QN_FULL_ARRAYS(X)                                                                      \
+  QN_COMMON_ARRAYS(X) X(T0u) X(T0v) X(Cu) X(Cv) X(aPu) X(aPv) X(aMu) X(aMv) X(tPu) X(tPv)      \
+  X(tMu) X(tMv) X(M0u) X(M0v) X(M1u) X(M1v) X(Dgu) X(Dgv) X(Sx) X(Sy) X(rhoc)
+QN_RECORD_LEVEL(LvErr, QN_ERR_ARRAYS, false);
+QN_RECORD_LEVEL(LvFull, QN_FULL_ARRAYS, true);
+
+template <class Form>
+struct RecordOf {  // FullForm, ProjForm
+  template <typename T> using level = LvFull<T>;
+  static constexpr int values = LvFull<rf64>::N;
+};
+template <>
+struct RecordOf<ErrForm> {
+  template <typename T> using level = LvErr<T>;
+  static constexpr int values = LvErr<rf32>::N;
 };
 
-struct ErrSmem {
-  int off[QN_MAX_FUSED_LEVELS];  // first word of level l's records
+struct RecordPlan {
+  int off[QN_MAX_FUSED_LEVELS];  // first value of level l's records
 };
 
-template <typename T>
-struct ErrLevels {
+template <typename T, class Form>
+struct RecordLevels {
   const CoarseLevels<T>& C;
-  const ErrSmem& M;
+  const RecordPlan& M;
   T* base;
-  __device__ __forceinline__ LvS<T> operator()(int l) const {
+  __device__ __forceinline__ typename RecordOf<Form>::template level<T> operator()(int l) const {
+    typedef typename RecordOf<Form>::template level<T> R;
     const Lv<T>& L = C.L[l];
-    return LvS<T>(L, base + M.off[l] + (L.m1 + 4) * ERR_N);  // cell (0,0) of the frame from (-1,-1)
+    return R(L, base + M.off[l] + (L.m1 + 4) * R::N);  // cell (0,0) of the frame from (-1,-1)
   }
 };
 
-template <int NT>
-__global__ void __launch_bounds__(NT, 1) k_coarse_err(Prm<rf32> P, const __grid_constant__ CoarseLevels<rf32> C,
-                                                   const __grid_constant__ ErrSmem M, int nu1, int nu2,
-                                                   int nuc, rf32 omega, int coupled) {
-  extern __shared__ __align__(16) float qn_err_words[];
-  rf32* qn_err_smem = reinterpret_cast<rf32*>(qn_err_words);
+// copies array m of a level's records in (asynchronously)
+template <typename T>
+__device__ __forceinline__ void record_in(T* to, const T* from) {
+  const unsigned sa = (unsigned)__cvta_generic_to_shared(to);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(sa), "l"(from),
+               "n"((int)sizeof(T))
+               : "memory");
+}
+
+template <typename T, class Form, int NT>
+__global__ void __launch_bounds__(NT, 1) k_coarse_records(Prm<T> P,
+                                                          const __grid_constant__ CoarseLevels<T> C,
+                                                          const __grid_constant__ RecordPlan M,
+                                                          int nu1, int nu2, int nuc, T omega,
+                                                          int coupled) {
+  typedef typename RecordOf<Form>::template level<T> R;
+  extern __shared__ __align__(16) char qn_records[];
+  T* const base = reinterpret_cast<T*>(qn_records);
   pdl_enter();
   const int n = C.n;
   for (int l = 0; l < n; ++l) {  // the padded frame of every array, all copies in flight at once
-    const Lv<rf32>& L = C.L[l];
+    const Lv<T>& L = C.L[l];
     const int cc = L.m1 + 3, cells = cc * (L.m2 + 3);
     for (int t = threadIdx.x; t < cells; t += NT) {
       const int g = (t / cc - 1) * L.pitch + t % cc - 1;
-      const unsigned sa = (unsigned)__cvta_generic_to_shared(qn_err_smem + M.off[l] + t * ERR_N);
-#define QN_ERR_IN(m)                                                                        \
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(sa + 4 * ERR_##m), "l"(L.m + g) \
-               : "memory");
-      QN_ERR_ARRAYS(QN_ERR_IN)
-#undef QN_ERR_IN
+      T* const r = base + M.off[l] + t * R::N;
+#define QN_RECORD_IN(m) record_in(r + R::I_##m, L.m + g);
+      if constexpr (std::is_same<Form, ErrForm>::value) {
+        QN_ERR_ARRAYS(QN_RECORD_IN)
+      } else {
+        QN_FULL_ARRAYS(QN_RECORD_IN)
+      }
+#undef QN_RECORD_IN
     }
   }
   asm volatile("cp.async.wait_all;" ::: "memory");
   __syncthreads();
-  const ErrLevels<rf32> get{C, M, qn_err_smem};
-  coarse_vcycle_body<rf32, ErrForm>(P, get, n, 1, nu1, nu2, nuc, omega, coupled, 0);
+  coarse_vcycle_body<T, Form>(P, RecordLevels<T, Form>{C, M, base}, n, C.base, nu1, nu2, nuc, omega,
+                              coupled, 0);
   __syncthreads();
   // what the levels above read of the group: the iterate of its finest level
-  const Lv<rf32>& L = C.L[0];
+  const Lv<T>& L = C.L[0];
   const int cc = L.m1 + 3, cells = cc * (L.m2 + 3);
   for (int t = threadIdx.x; t < cells; t += NT) {
     const int g = (t / cc - 1) * L.pitch + t % cc - 1;
-    const rf32* r = qn_err_smem + M.off[0] + t * ERR_N;
-    L.c[g] = r[ERR_c];
-    L.mu[g] = r[ERR_mu];
-    L.p[g] = r[ERR_p];
-    L.u[g] = r[ERR_u];
-    L.v[g] = r[ERR_v];
+    const T* r = base + M.off[0] + t * R::N;
+    L.c[g] = r[R::I_c];
+    L.mu[g] = r[R::I_mu];
+    L.p[g] = r[R::I_p];
+    L.u[g] = r[R::I_u];
+    L.v[g] = r[R::I_v];
+    if constexpr (R::has_rho) L.rhoc[g] = r[R::I_rhoc];
   }
 }
 
@@ -3468,7 +3501,7 @@ void launch_vanka(const Prm<T>& P0, const Lv<T>& L0, int colour, T omega, cudaSt
   if (n <= 0) return;
   if constexpr (std::is_same<Form, FullForm>::value && sizeof(T) == 8) {
     if (n <= team8_max) {  // eight lanes per block: half a momentum row per lane
-      qlaunch(&k_vanka_team8, (8 * n + SNT - 1) / SNT, SNT, 0, s, P, L, colour, omega);
+      qlaunch(&k_vanka_team8<R>, (8 * n + SNT - 1) / SNT, SNT, 0, s, P, L, colour, omega);
       ++g_launches;
       return;
     }
@@ -3538,16 +3571,17 @@ static size_t coarse_smem_plan(const Lv<double>* levels, int n, CoarseSmem& M) {
   return bytes <= (size_t)smem_optin() ? bytes : 0;
 }
 
-// Plan of k_coarse_err's copy; returns its bytes, 0 if it does not fit
-static size_t coarse_err_plan(const Lv<float>* levels, int n, ErrSmem& M) {
-  const long long limit = smem_optin();
-  long long words = 0;
+// Plan of k_coarse_records' copy; returns its bytes, 0 if it does not fit
+template <typename T, class Form>
+static size_t record_plan(const Lv<T>* levels, int n, RecordPlan& M) {
+  const long long limit = smem_optin() / (long long)sizeof(T);
+  long long values = 0;
   for (int l = 0; l < n; ++l) {
-    M.off[l] = (int)words;
-    words += (long long)(levels[l].m1 + 3) * (levels[l].m2 + 3) * ERR_N;
-    if (4 * words > limit) return 0;
+    M.off[l] = (int)values;
+    values += (long long)(levels[l].m1 + 3) * (levels[l].m2 + 3) * RecordOf<Form>::values;
+    if (values > limit) return 0;
   }
-  return (size_t)words * sizeof(float);
+  return (size_t)values * sizeof(T);
 }
 
 void coarse_smem_prepare() {
@@ -3556,7 +3590,14 @@ void coarse_smem_prepare() {
   if (cudaDeviceGetAttribute(&v, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) == cudaSuccess &&
       v > 0) {
     cudaFuncSetAttribute(&k_coarse_vcycle_smem<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, v);
-    cudaFuncSetAttribute(&k_coarse_err<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, v);
+    cudaFuncSetAttribute(&k_coarse_records<rf32, ErrForm, 256>,
+                         cudaFuncAttributeMaxDynamicSharedMemorySize, v);
+    cudaFuncSetAttribute(&k_coarse_records<rf64, ErrForm, 256>,
+                         cudaFuncAttributeMaxDynamicSharedMemorySize, v);
+    cudaFuncSetAttribute(&k_coarse_records<rf64, FullForm, 256>,
+                         cudaFuncAttributeMaxDynamicSharedMemorySize, v);
+    cudaFuncSetAttribute(&k_coarse_records<rf64, ProjForm, 256>,
+                         cudaFuncAttributeMaxDynamicSharedMemorySize, v);
   }
   cudaGetLastError();
 }
@@ -3572,23 +3613,27 @@ int launch_coarse_vcycle(const Prm<T>& P0, const Lv<T>* levels, int n, int nu1, 
   C.base = std::is_same<Form, ErrForm>::value;
   for (int l = 0; l < n; ++l) C.L[l] = as_compute<R>(level_consts(P0, levels[l]));
   constexpr int NT = sizeof(T) == 8 ? 256 : 512;
-  if constexpr (std::is_same<Form, FullForm>::value && sizeof(T) == 8) {
-    if (ctas <= 1) {
-      CoarseSmem M = {};
-      const size_t bytes = smem ? coarse_smem_plan(levels, n, M) : 0;
-      qlaunch(&k_coarse_vcycle_smem<NT>, 1, NT, bytes ? bytes : sizeof(CoarseLevels<double>), s, P,
-              C, M, bytes ? 1 : 0, nu1, nu2, nuc, omega, coupled, team8);
+  if (smem && ctas <= 1 && !team8) {  // on shared-memory records, where they fit
+    RecordPlan M = {};
+    const size_t bytes = record_plan<T, Form>(levels, n, M);
+    if (bytes) {
+      qlaunch(&k_coarse_records<R, Form, 256>, 1, 256, bytes, s, P, C, M, nu1, nu2, nuc, R(omega),
+              coupled);
       ++g_launches;
-      return bytes ? 1 : 0;
+      return std::is_same<Form, ErrForm>::value ? 0 : 1;
     }
   }
-  if constexpr (std::is_same<Form, ErrForm>::value && sizeof(T) == 4) {
-    ErrSmem M = {};
-    const size_t bytes = smem && ctas <= 1 ? coarse_err_plan(levels, n, M) : 0;
-    if (bytes) {
-      qlaunch(&k_coarse_err<256>, 1, 256, bytes, s, P, C, M, nu1, nu2, nuc, omega, coupled);
-      ++g_launches;
-      return 0;
+  if constexpr (std::is_same<Form, FullForm>::value && sizeof(T) == 8) {
+    // eight-lane blocks read arrays that the records leave out: on a copy of all
+    if (smem && ctas <= 1 && team8) {
+      CoarseSmem M = {};
+      const size_t bytes = coarse_smem_plan(levels, n, M);
+      if (bytes) {
+        qlaunch(&k_coarse_vcycle_smem<NT>, 1, NT, bytes, s, P, C, M, nu1, nu2, nuc, R(omega),
+                coupled, team8);
+        ++g_launches;
+        return 1;
+      }
     }
   }
   if (ctas <= 1) {

@@ -84,6 +84,11 @@ template <typename F>
 QN_F Fused<F> shfl_xor(Fused<F> x, int o) {
   return __shfl_xor_sync(0xffffffffu, x.v, o);
 }
+// lane src's value
+template <typename F>
+QN_F Fused<F> shfl_from(Fused<F> x, int src) {
+  return __shfl_sync(0xffffffffu, x.v, src);
+}
 #undef QN_F
 #endif
 
@@ -143,7 +148,8 @@ struct LvK {
 template <typename T>
 struct Lv {
   typedef T real;
-  static constexpr bool has_rho = true;
+  static constexpr bool has_rho = true;  // rhoc may be set
+  static constexpr bool all_arrays = true;  // also those that only some kernels read
   LvK<T> k;
   // slot-to-cell mapping: cells of a Vanka colour in one of its rows, of a CH
   // colour in a row, and the number of Vanka colours

@@ -1,5 +1,5 @@
 """The fused coarse V-cycle of FP32 error-equation levels on its shared-memory
-records (k_coarse_err; option coarse_smem, on by default) against the launch
+records (k_coarse_records; option coarse_smem, on by default) against the launch
 that reads global memory.  Both run the same operators on the same values, so
 one defect-correction cycle gives the same correction up to FP32 rounding: each
 of the few hundred dependent visits of a cycle rounds at 6e-8 of the
@@ -8,7 +8,10 @@ a wrong neighbour or array shows at its own size.  Grids: walls and periodic x
 (5, 8 and 6-multiple colourings), sides that coarsen to odd sizes, a group that
 starts on the finest level, the 2 x 2 and 4 x 2 grids, the coupled block, the
 server's larger groups, and a group too large for the records, which falls
-back.  Steps meet the mixed-precision bars against the FP64 oracle."""
+back.  Steps meet the mixed-precision bars against the FP64 oracle.  The FP64
+records of the full iterate and of the projection method round as the launch on
+global memory does: the same bits.  (Too large for the records, the group
+reports that it read global memory.)"""
 import numpy as np
 import pytest
 
@@ -73,3 +76,28 @@ def test_mixed_steps_meet_the_bars(qn, m1, m2, px, opts):
     for _ in range(2):
         assert g.step(P.dt)[1] <= P.tol and r.step(P.dt)[1] <= P.tol
     check_mixed(g.get_fields(), r.get_fields())
+
+
+@pytest.mark.parametrize("name,m1,m2,px,opts,used", [
+    ("full_one_odd_level", 15, 9, False, {"fuse_cells": 256}, 1),
+    ("full_smallest_coupled", 4, 2, True, {"coupled": 1}, 1),
+    ("full_too_large", 40, 40, False, {"fuse_cells": 4096}, 0),
+    ("projection_walls", 64, 96, False, {"scheme": 1}, 1),
+    ("projection_periodic", 48, 72, True, {"scheme": 1}, 1),
+    ("projection_one_odd_level", 15, 9, False, {"scheme": 1, "fuse_cells": 256}, 1),
+    ("projection_smallest", 2, 2, False, {"scheme": 1}, 1),
+    ("projection_too_large", 40, 40, False, {"scheme": 1, "fuse_cells": 4096}, 0)],
+    ids=lambda x: x if isinstance(x, str) else "")
+def test_fp64_records_match_global_bitwise(qn, name, m1, m2, px, opts, used):
+    P = W.small_case(m1, m2, px)
+    out = []
+    for smem in (1, 0):
+        s = qn.Solver(**P.create_kwargs(), coarse_smem=smem, **opts)
+        s.set_fields(P.fields())
+        s.begin_step(P.dt)
+        norms = [s.vcycle() for _ in range(2)]
+        assert s.get_option("coarse_smem_used") == (used if smem else 0)
+        out.append((norms, s.get_iterate()))
+    assert np.array_equal(out[0][0], out[1][0])
+    for k in out[0][1]:
+        assert np.array_equal(out[0][1][k], out[1][1][k]), k
