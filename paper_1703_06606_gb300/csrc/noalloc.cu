@@ -58,13 +58,16 @@ int partials_address(void** out) {
 }
 
 // The FP64 pipe bounds the kernel (a warp's FP64 instruction takes 19 cycles of
-// an SM, and 2048 x 4096 cells are 1724 warps an SM: 15.8 us an instruction),
-// not HBM (67 MB, 10 us): a division's ten FP64 instructions were two thirds
-// of it.  With rcp_any 152 -> 100 us at that size.
+// an SM, and 2048 x 4096 cells are 1724 warps an SM: 15.8 us an instruction a
+// cell), not HBM (67 MB, 10 us).  A cell takes 6: rho's argument, three of
+// rcp_any (a division has ten), two sums.  Eight warps that each reduce two
+// sums by shuffles add 1.4 to that, two warps that add up the block's sums from
+// shared memory 0.4.  Measured at that size, both kernels: 152 us with the
+// division, 123 with rcp_any, 105 with the sums in shared memory.
 // rho(c) = 1 / (ia c + ib) with ia = (rho2 - rho1)/(rho1 rho2), ib = 1/rho2 (Sec. 2.1)
 __global__ void k_mass_partials(const double* __restrict__ c, long long n, double ia, double ib,
                                 double* __restrict__ part) {
-  __shared__ double sr[NA_THREADS / 32], src[NA_THREADS / 32];
+  __shared__ double sums[2][NA_THREADS];
   long long base = (long long)blockIdx.x * NA_CELLS_PER_BLOCK;
   double a = 0.0, b = 0.0;
 #pragma unroll
@@ -77,27 +80,16 @@ __global__ void k_mass_partials(const double* __restrict__ c, long long n, doubl
       b += r * cc;
     }
   }
-  for (int o = 16; o > 0; o >>= 1) {
-    a += __shfl_down_sync(0xffffffffu, a, o);
-    b += __shfl_down_sync(0xffffffffu, b, o);
-  }
-  int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (lane == 0) {
-    sr[warp] = a;
-    src[warp] = b;
-  }
+  sums[0][threadIdx.x] = a;
+  sums[1][threadIdx.x] = b;
   __syncthreads();
-  if (warp == 0) {
-    a = lane < NA_THREADS / 32 ? sr[lane] : 0.0;
-    b = lane < NA_THREADS / 32 ? src[lane] : 0.0;
-    for (int o = 16; o > 0; o >>= 1) {
-      a += __shfl_down_sync(0xffffffffu, a, o);
-      b += __shfl_down_sync(0xffffffffu, b, o);
-    }
-    if (lane == 0) {
-      part[2 * blockIdx.x] = a;
-      part[2 * blockIdx.x + 1] = b;
-    }
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (warp < 2) {  // warp 0 adds up the first sums, warp 1 the second
+    a = sums[warp][lane];
+#pragma unroll
+    for (int q = 32; q < NA_THREADS; q += 32) a += sums[warp][lane + q];
+    for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
+    if (lane == 0) part[2 * blockIdx.x + warp] = a;
   }
 }
 
