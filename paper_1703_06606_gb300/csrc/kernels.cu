@@ -317,10 +317,12 @@ __device__ __forceinline__ Rows5<T> residual_rows5(const Prm<T>& P, const LV& L,
   return X;
 }
 // stores them (MODE 0: into r, MODE 1: into f) and adds to val: the largest |r|
-// and the sum of r^2 per family (MODE 0)
+// and the sum of r^2 per family (MODE 0 with norms: a cycle's own residuals need
+// none, and in FP32 their conversions and sums, ten FP64 instructions a cell,
+// were a quarter of the launch: 219 -> 164 us on 1024x4096)
 template <typename T, int MODE, int ROLE, class LV>
 __device__ __forceinline__ void residual_store(const LV& L, int i, int j, const Rows5<T>& X,
-                                               double (&val)[10]) {
+                                               double (&val)[10], bool norms) {
   const int k = L.at(i, j);
   const bool own[5] = {true, true, true, i <= L.uhi(), j < L.m2};
   const bool has[5] = {role_has<ROLE>(0), role_has<ROLE>(1), role_has<ROLE>(2),
@@ -330,7 +332,7 @@ __device__ __forceinline__ void residual_store(const LV& L, int i, int j, const 
   if (has[2]) (MODE == 0 ? L.rp[k] : L.fp[k]) = X.r[2];
   if (has[3]) (MODE == 0 ? L.ru[k] : L.fu[k]) = X.r[3];
   if (has[4]) (MODE == 0 ? L.rv[k] : L.fv[k]) = X.r[4];
-  if (MODE == 0) {
+  if (MODE == 0 && norms) {
 #pragma unroll
     for (int q = 0; q < 5; ++q) {
       if (!role_has<ROLE>(q)) continue;
@@ -344,8 +346,9 @@ __device__ __forceinline__ void residual_store(const LV& L, int i, int j, const 
 }
 template <typename T, int MODE, class Form, class LV>
 __device__ __forceinline__ void residual_cell(const Prm<T>& P, const LV& L, int i, int j,
-                                              double (&val)[10]) {
-  residual_store<T, MODE, ROLE_ALL>(L, i, j, residual_rows5<T, MODE, Form, ROLE_ALL>(P, L, i, j), val);
+                                              double (&val)[10], bool norms) {
+  residual_store<T, MODE, ROLE_ALL>(L, i, j, residual_rows5<T, MODE, Form, ROLE_ALL>(P, L, i, j), val,
+                                    norms);
 }
 
 // ROWS > 1 (large levels): each thread takes ROWS / 2 pairs of rows BY apart, so
@@ -357,9 +360,10 @@ __global__ void __launch_bounds__(NT, 2) k_residual(Prm<T> P, Lv<T> L, double* p
   pdl_enter();
   int i = blockIdx.x * BX + threadIdx.x + 1;
   int j = blockIdx.y * (ROWS * BY) + threadIdx.y + 1;
+  const bool norms = MODE == 0 && part;
   double val[10] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};  // max x5 then sum of squares x5
   if (ROWS == 1) {
-    if (i <= L.m1 && j <= L.m2) residual_cell<T, MODE, Form>(P, L, i, j, val);
+    if (i <= L.m1 && j <= L.m2) residual_cell<T, MODE, Form>(P, L, i, j, val, norms);
   } else {
 #pragma unroll 1
     for (int r = 0; r < ROWS; r += 2, j += 2 * BY) {
@@ -367,11 +371,11 @@ __global__ void __launch_bounds__(NT, 2) k_residual(Prm<T> P, Lv<T> L, double* p
       const bool two = j + BY <= L.m2;
       const Rows5<T> A = residual_rows5<T, MODE, Form, ROLE_ALL>(P, L, i, j);
       const Rows5<T> B = residual_rows5<T, MODE, Form, ROLE_ALL>(P, L, i, two ? j + BY : j);
-      residual_store<T, MODE, ROLE_ALL>(L, i, j, A, val);
-      if (two) residual_store<T, MODE, ROLE_ALL>(L, i, j + BY, B, val);
+      residual_store<T, MODE, ROLE_ALL>(L, i, j, A, val, norms);
+      if (two) residual_store<T, MODE, ROLE_ALL>(L, i, j + BY, B, val, norms);
     }
   }
-  if (MODE == 0 && part) block_sum_store<10>(val, part, 5);
+  if (norms) block_sum_store<10>(val, part, 5);
 }
 
 // The rows of a cell by three threads (ROLE: the block's z), for levels that
@@ -382,10 +386,11 @@ template <typename T, int MODE, class Form, int ROLE>
 __device__ __forceinline__ void residual_role(const Prm<T>& P, const Lv<T>& L, double* part) {
   int i = blockIdx.x * BX + threadIdx.x + 1;
   int j = blockIdx.y * BY + threadIdx.y + 1;
+  const bool norms = MODE == 0 && part;
   double val[10] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
   if (i <= L.m1 && j <= L.m2)
-    residual_store<T, MODE, ROLE>(L, i, j, residual_rows5<T, MODE, Form, ROLE>(P, L, i, j), val);
-  if (MODE == 0 && part) block_sum_store<10, ROLE>(val, part, 5);
+    residual_store<T, MODE, ROLE>(L, i, j, residual_rows5<T, MODE, Form, ROLE>(P, L, i, j), val, norms);
+  if (norms) block_sum_store<10, ROLE>(val, part, 5);
 }
 template <typename T, int MODE, class Form>
 __global__ void __launch_bounds__(NT, 2) k_residual_split(Prm<T> P, Lv<T> L, double* part) {
@@ -2529,7 +2534,7 @@ __device__ __forceinline__ void coarse_vcycle_body(const Prm<T>& P, const Get& g
     if (down) {
       const auto& G = get(l + 1);
       for (int t = grp_rank(); t < F.m1 * F.m2; t += grp_size())
-        residual_cell<T, 0, Form>(P, F, t % F.m1 + 1, t / F.m1 + 1, dummy);
+        residual_cell<T, 0, Form>(P, F, t % F.m1 + 1, t / F.m1 + 1, dummy, false);
       grp_sync();
       for (int t = grp_rank(); t < (G.m1 + 1) * (G.m2 + 1); t += grp_size())
         restrict_state_cell(P, F, G, t % (G.m1 + 1), t / (G.m1 + 1));
@@ -2537,7 +2542,7 @@ __device__ __forceinline__ void coarse_vcycle_body(const Prm<T>& P, const Get& g
         restrict_res_cell(F, G, t % G.m1 + 1, t / G.m1 + 1);
       grp_sync();
       for (int t = grp_rank(); t < G.m1 * G.m2; t += grp_size())
-        residual_cell<T, 1, Form>(P, G, t % G.m1 + 1, t / G.m1 + 1, dummy);
+        residual_cell<T, 1, Form>(P, G, t % G.m1 + 1, t / G.m1 + 1, dummy, false);
       grp_sync();
     }
   }
@@ -3001,6 +3006,10 @@ __global__ void __launch_bounds__(NT, 2) k_predict(FiveArrays X, FiveArrays A, F
 // --------------------------------------------------------------------------
 // defect correction (mixed precision): FP64 level <-> error-equation level
 // --------------------------------------------------------------------------
+// These kernels move every array of a level once and are bound by its bytes.
+// They read all of a cell's values before the first store: a load behind a
+// store that may alias it waits for its turn, and a cell's ten loads in a row
+// are ten round trips (k_start_correction on 1024x4096: 113 -> 91 us).
 // error-equation frozen data = rounded FP64 frozen data (whole padded arrays)
 template <typename T>
 __global__ void __launch_bounds__(NT, 2) k_cast_frozen(Lv<double> D, Lv<T> E, long long n, int off) {
@@ -3008,23 +3017,13 @@ __global__ void __launch_bounds__(NT, 2) k_cast_frozen(Lv<double> D, Lv<T> E, lo
   long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= n) return;
   long long q = t - off;  // origin-relative index
-  E.cn[q] = (T)D.cn[q];
-  E.rhon[q] = (T)D.rhon[q];
-  E.mobn[q] = (T)D.mobn[q];
-  E.visn[q] = (T)D.visn[q];
-  E.Gn[q] = (T)D.Gn[q];
-  E.T1u[q] = (T)D.T1u[q];
-  E.T1v[q] = (T)D.T1v[q];
-  E.aPu[q] = (T)D.aPu[q];
-  E.aPv[q] = (T)D.aPv[q];
-  E.aMu[q] = (T)D.aMu[q];
-  E.aMv[q] = (T)D.aMv[q];
-  E.tPu[q] = (T)D.tPu[q];
-  E.tPv[q] = (T)D.tPv[q];
-  E.tMu[q] = (T)D.tMu[q];
-  E.tMv[q] = (T)D.tMv[q];
-  E.Tx[q] = (T)D.Tx[q];
-  E.Ty[q] = (T)D.Ty[q];
+  const double x[17] = {D.cn[q], D.rhon[q], D.mobn[q], D.visn[q], D.Gn[q], D.T1u[q], D.T1v[q],
+                        D.aPu[q], D.aPv[q], D.aMu[q], D.aMv[q], D.tPu[q], D.tPv[q],
+                        D.tMu[q], D.tMv[q], D.Tx[q], D.Ty[q]};
+  T* const to[17] = {E.cn, E.rhon, E.mobn, E.visn, E.Gn, E.T1u, E.T1v, E.aPu, E.aPv, E.aMu,
+                     E.aMv, E.tPu, E.tPv, E.tMu, E.tMv, E.Tx, E.Ty};
+#pragma unroll
+  for (int m = 0; m < 17; ++m) to[m][q] = (T)x[m];
 }
 
 // base X = x (rounded), X.c - c^n formed in FP64, right-hand side = FP64 residual
@@ -3035,17 +3034,20 @@ __global__ void __launch_bounds__(NT, 2) k_start_correction(Prm<T> P, Lv<double>
   long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= n) return;
   long long q = t - off;
-  E.Bc[q] = (T)D.c[q];
-  E.rB[q] = rho_of(P, E.Bc[q]);
-  E.Bmu[q] = (T)D.mu[q];
-  E.Bu[q] = (T)D.u[q];
-  E.Bv[q] = (T)D.v[q];
-  E.Bdc[q] = (T)(D.c[q] - D.cn[q]);
-  E.fc[q] = (T)D.rc[q];
-  E.fmu[q] = (T)D.rmu[q];
-  E.fp[q] = (T)D.rp[q];
-  E.fu[q] = (T)D.ru[q];
-  E.fv[q] = (T)D.rv[q];
+  const double c = D.c[q], dc = c - D.cn[q], mu = D.mu[q], u = D.u[q], v = D.v[q];
+  const double rc = D.rc[q], rmu = D.rmu[q], rp = D.rp[q], ru = D.ru[q], rv = D.rv[q];
+  const T Bc = (T)c;
+  E.Bc[q] = Bc;
+  E.rB[q] = rho_of(P, Bc);
+  E.Bmu[q] = (T)mu;
+  E.Bu[q] = (T)u;
+  E.Bv[q] = (T)v;
+  E.Bdc[q] = (T)dc;
+  E.fc[q] = (T)rc;
+  E.fmu[q] = (T)rmu;
+  E.fp[q] = (T)rp;
+  E.fu[q] = (T)ru;
+  E.fv[q] = (T)rv;
   E.c[q] = T(0);
   E.mu[q] = T(0);
   E.p[q] = T(0);
@@ -3060,12 +3062,15 @@ __global__ void __launch_bounds__(NT, 2) k_apply_correction(Prm<double> P, Lv<do
   long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= n) return;
   long long q = t - off;
-  D.c[q] += (double)E.c[q];
-  D.rhoc[q] = rho_of(P, D.c[q]);
-  D.mu[q] += (double)E.mu[q];
-  D.p[q] += (double)E.p[q];
-  D.u[q] += (double)E.u[q];
-  D.v[q] += (double)E.v[q];
+  const double c = D.c[q] + (double)E.c[q], mu = D.mu[q] + (double)E.mu[q],
+               p = D.p[q] + (double)E.p[q], u = D.u[q] + (double)E.u[q],
+               v = D.v[q] + (double)E.v[q];
+  D.c[q] = c;
+  D.rhoc[q] = rho_of(P, c);
+  D.mu[q] = mu;
+  D.p[q] = p;
+  D.u[q] = u;
+  D.v[q] = v;
 }
 
 // rho(c) of the iterate over the whole padded array, after c was written in
