@@ -754,31 +754,26 @@ def run_ours(args, rank, world, local_rank):
         dist.destroy_process_group()
 
 
-# algorithmic FP64 operations per Vanka cell visit (add/sub/mul/div = 1, fused
-# multiply-add = 2), counted from the formulas of one 5x5 Vanka block (Sec. 7.1)
-# as the kernel evaluates it: 4 edge averages of the densities rho(c) (read from
-# the array the smoothers keep), 4 diagonals from the per-step row
-# coefficients, off-diagonals and the mass row, 4 momentum residuals from the
-# per-step assembled stencils and 1 mass residual, the structured block solve,
-# 5 updates
-VANKA_FP64_FLOPS_PER_VISIT = 287.0
-# FP64 operations per CH cell visit (N_c, N_mu, the 2x2 Jacobian, its solve and
-# rho of the new c) and per residual cell (all five families), as ncu counts
-# them executed (add, mul = 1, fma = 2) on the FP64 kernels
-CH_FP64_FLOPS_PER_VISIT = 241.0
-RESIDUAL_FP64_FLOPS_PER_CELL = 223.0
+# FP64 operations per Vanka cell visit (one 5x5 block: its densities' sums, the
+# diagonals, off-diagonals and the mass row, 5 residuals, the structured solve,
+# 5 updates), per CH cell visit (N_c, N_mu, the 2x2 Jacobian, its solve and rho
+# of the new c) and per residual cell (all five families; the mean of a launch
+# with norms and one without), as ncu counts them executed (add, mul = 1,
+# fma = 2) on the FP64 kernels with one lane per visit
+VANKA_FP64_FLOPS_PER_VISIT = 272.0
+CH_FP64_FLOPS_PER_VISIT = 180.0
+RESIDUAL_FP64_FLOPS_PER_CELL = 181.0
 # dram__bytes_read.sum + dram__bytes_write.sum per launch of a timed kind (average
 # over its launches), from one ncu capture of the same kernel build (the
 # profiles/ file named beside it; cold-cache, serialised); a kind without a
 # capture of the current build reports traffic null.  Drop these entries when
 # the kernels change.
+_DRAM_PROFILE = "profiles/launches_and_fp64_instructions_after_the_record_kernels.md"
 TRAFFIC_BYTES = {
-    "vanka_levels": (3.08e6, "profiles/dram_per_kernel_fp64_step_rising_drop_256x512.md"),
-    "vanka_finest": (33.99e6, "profiles/dram_per_kernel_fp64_step_rising_drop_256x512.md"),
-    "coarse_vcycle": (0.39e6, "profiles/dram_per_kernel_fp64_step_rising_drop_256x512.md"),
-    "ch": (15.66e6, "profiles/dram_per_kernel_fp64_step_rising_drop_256x512.md"),
-    "vanka_finest_fp32": (431.99e6, "profiles/dram_per_kernel_rayleigh_taylor_1024x4096.md"),
-    "ch_fp32": (299.10e6, "profiles/dram_per_kernel_rayleigh_taylor_1024x4096.md"),
+    "vanka_levels": (2.95e6, _DRAM_PROFILE),
+    "vanka_finest": (32.86e6, _DRAM_PROFILE),
+    "coarse_vcycle": (0.34e6, _DRAM_PROFILE),
+    "ch": (15.65e6, _DRAM_PROFILE),
 }
 # words per cell a sweep moves at one pass over the arrays it needs (Sec. 7.1
 # smoothers; read c^n, u^n, v^n, c, mu, u, v, p and the three right-hand sides,
@@ -874,7 +869,7 @@ def roofline_of(kinds, fp64_peak, coarse_smem=False):
     achieved = flops / (k["avg_launch_us"] * 1e-6) / 1e12
     kernel = {"vanka_finest": "k_vanka<double> (finest level)",
               "vanka_levels": "k_vanka_team<double> (levels below the finest)",
-              "coarse_vcycle": ("k_coarse_vcycle_smem (fused coarse levels, shared-memory copy)"
+              "coarse_vcycle": ("k_coarse_records (fused coarse levels, shared-memory records)"
                                 if coarse_smem else "k_coarse_vcycle<double> (fused coarse levels)"),
               "ch": "k_ch<double> (finest level)"}[name]
     tr = TRAFFIC_BYTES.get(name)

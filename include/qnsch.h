@@ -191,7 +191,8 @@ int qnsch_footprint(const qnsch_grid* grid, int precision, size_t* bytes);
    are independent and stream order orders the rest.  The results are those
    of the per-colour launches with one lane per visit, bit for bit (the same
    device code on the same values).  Measured on the 1024 x 4096 mixed
-   workload: 1.7x less DRAM traffic per smoothing block and 1.25x more time.
+   workload: 1.7x less DRAM traffic per smoothing block, and 5.51 ms a V-cycle
+   at the best chunk height against 5.21 ms.
    device_loop: 1 (with graphs = 1 and profiling off) runs qnsch_step and
    qnsch_step_launch as one graph per step: the initial residual, a
    conditional WHILE node around the outer cycle whose last kernel applies the
@@ -216,8 +217,9 @@ int qnsch_footprint(const qnsch_grid* grid, int precision, size_t* bytes);
    idle); ch_team_max does the same for the CH 2x2 Newton launches (four lanes
    per cell, one face each); vanka_team_max32 for the Vanka launches on the
    error-equation levels of the defect correction (precision 1 and 2), which
-   are latency-bound up to a few hundred thousand cells per colour, and
-   ch_team_max32 for their CH launches.
+   in FP64 (precision 2), and ch_team_max32 for their CH launches; FP32 error
+   levels (precision 1) run one lane per visit whatever these two say, which
+   measured as fast or faster at every size.
    vanka_team_max and vanka_team_max32 also choose the four-lane launches of
    the coupled 7x7 block (coupled = 1).
    vanka_team8_max: FP64 full-iterate levels with at most this many cells per
@@ -245,10 +247,12 @@ int qnsch_footprint(const qnsch_grid* grid, int precision, size_t* bytes);
    full-iterate levels (fuse_cells, in one thread block: fuse_ctas = 1) on a
    copy of those levels in shared memory, made at the start of the launch and
    written back at its end, wherever the copy fits the device's shared memory
-   per block (about 151 KB for the 8x16, 4x8 and 2x4 levels); 0 runs it from
-   global memory.  The same device code runs on the same values, so the
-   results are the same.  Reading the key "coarse_smem_used" (get only) gives
-   1 if the last fused launch ran on the shared-memory copy.
+   per block (392 bytes a padded cell: about 126 KB for the 8x16, 4x8 and 2x4
+   levels); 0 runs it from global memory.  The projection method's levels and
+   the error-equation levels (fuse_cells32; 172 bytes a padded cell in FP32)
+   do the same.  The same operators run on the same values, so the results are
+   the same.  Reading the key "coarse_smem_used" (get only) gives 1 if the
+   last fused launch of FP64 full-iterate levels ran on the copy.
    pdl: 1 launches every kernel with programmatic dependent launch, so that
    a kernel is scheduled as its predecessor's blocks exit and waits on the GPU
    for the predecessor's results before touching memory (same results); 0

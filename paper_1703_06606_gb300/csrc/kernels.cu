@@ -160,7 +160,9 @@ __device__ __forceinline__ void block_sum_store(double (&val)[NV], double* part,
 
 // Sum (or max) nparts rows of nv <= 32 partials in a fixed order, in one block:
 // consecutive threads read consecutive partials (a thread's all of one
-// column), and a warp then adds each column's share.
+// column), and a warp then adds each column's share.  One block's dependent
+// loads bound it: with 1024 threads reading in rows 11.6 -> 6 us on 256x512 and
+// 41.7 -> 12 us on 1024x4096 (256 threads, a column each, before).
 constexpr int FIN_NT = 1024;
 __global__ void __launch_bounds__(FIN_NT) k_finalize(const double* part, int nparts, int nv,
                                                      int nmax_first, double scale_sum, double* out) {
@@ -402,7 +404,8 @@ __global__ void __launch_bounds__(NT, 2) k_residual_split(Prm<T> P, Lv<T> L, dou
 
 // rows per residual thread on level L: two on levels of at least 65536 cells,
 // eight where that still leaves the GPU several blocks an SM (2^21 cells: 1024
-// blocks), so that one block sums a quarter of the partials
+// blocks), so that one block sums a quarter of the partials (with the wider
+// k_finalize 30 us of a 1024x4096 residual and its norms)
 template <typename T>
 static int residual_rows(const Lv<T>& L) {
   const long long n = (long long)L.m1 * L.m2;
@@ -1200,7 +1203,12 @@ __device__ __forceinline__ int vanka_colour(const LV& L, int i, int j) {
 
 // per-level smoother launches: one thread per cell of the colour, packed into
 // 64-thread blocks so that a level's warps spread over many SMs (on the FP64
-// pipe a warp costs the same with 1 or 32 lanes busy)
+// pipe a warp costs the same with 1 or 32 lanes busy).  The launch bounds ask for
+// four blocks an SM: without them the compiler keeps these kernels at 48 to 80
+// registers and issues a visit's 60 to 110 loads in batches, each an exposed L2
+// round trip; with them all are in flight (FP32 coupled visits 8.2 -> 4.4 us a
+// colour on small levels, 9.9 -> 6.1 us on 448x448).  Eight blocks an SM measured
+// slower (1024x4096 mixed 83.6 against 78.5 ms a step), two the same.
 constexpr int SNT = 64;
 
 template <typename T, class Form>
@@ -1701,7 +1709,10 @@ __device__ __forceinline__ void restrict_res_cell(const LV& F, const LV& C, int 
   if (J < C.m2) C.fv[kc] = T(0.5) * v;
 }
 
-// the coarse level's iterate (restrict_state_cell) and right-hand side R r_h in one launch
+// The coarse level's iterate (restrict_state_cell) and right-hand side R r_h in
+// one launch, ghosts stored with their cells: three launches before, one of
+// them a frame fill of 2 to 6 us (with k_prolong's, 256x512 mixed 20.2 -> 18.1 ms
+// for three steps).  Bound by the launch on small levels, by bytes on large.
 template <typename T>
 __global__ void __launch_bounds__(NT, 2) k_restrict(Prm<T> P, Lv<T> F, Lv<T> C) {
   pdl_enter();
@@ -2670,9 +2681,14 @@ __global__ void __launch_bounds__(NT, 1) k_coarse_vcycle_smem(Prm<rf64> P, Coars
 // (templates over the level), in the type whose rounding the source fixes, so
 // the results are those of the launch that reads global memory.
 // Measured (GB300, ncu, caches warm), FP32 error levels: 16x32 .. 2x4 of the
-// 256x512 drop 245 -> 139 us, 28x28 and 14x14 of a served 448x448 request (64
-// coupled sweeps on the coarsest) 1504 -> 1121 us (89 and 990 us with the
-// launch bounds and one lane a visit that came after).
+// 256x512 drop 245 -> 84 us, 28x28 and 14x14 of a served 448x448 request (64
+// coupled sweeps on the coarsest) 1504 -> 630 us.  FP64: 8x16 .. 2x4 of the drop
+// 290 -> 246 us, a 128x256 projection step's group 719 -> 661 us, the 6x9
+// coupled group of 96x144 1640 -> 1438 us (the FP64 figures against a copy array
+// by array, the projection's against global memory).  What is left is one
+// warp's visit, about 1000 instructions, colour after colour; two warps that
+// shared a coupled visit (CH block, NS block) were slower, 23.8 -> 24.6 ms for
+// two served steps.
 // --------------------------------------------------------------------------
 // array OFF of records of N values at b: element k as if it were a plain array
 template <typename T, int OFF, int N>
@@ -2823,9 +2839,8 @@ __global__ void __launch_bounds__(NT, 1) k_coarse_records(Prm<T> P,
 // k - 1 (per-band counters of finished passes), runs the pass's visits on its
 // band and publishes the band's new count.  Each visit sees exactly the
 // values it sees when every pass is a launch over the whole level and runs the
-// same device code, so the results are those of the per-colour launches up to
-// the compiler's contraction of multiply-adds, which may differ between the
-// two kernels; what changes is that a band's arrays stay in L2 across its
+// same device code in the same type (Fused), so the results are those of the
+// per-colour launches with as many lanes a visit; what changes is that a band's arrays stay in L2 across its
 // passes instead of every colour launch streaming the whole level.
 // A ticket's dependencies hold earlier tickets, taken by blocks that are
 // running or done, so the wavefront progresses whatever the number of
@@ -3392,7 +3407,10 @@ int nparts_cells(const Lv<T>& L) {
 }
 
 // Three threads a cell on FP64 full-iterate levels of at most 32768 cells: three
-// threads' warps then still are at most five a sub-partition.  (FP32 levels: a
+// threads' warps then still are at most five a sub-partition, and a launch is
+// one thread's chain (a V-cycle of 256x256 2.16 -> 2.04 ms, a 64x64 step 7.72 ->
+// 7.37 ms); on a level that fills the pipes the roles' shared loads and sums
+// would be done three times.  (FP32 levels: a
 // thread's chain is its loads, which the roles would repeat.)
 template <typename T, class Form>
 static bool residual_split(const Lv<compute_t<T, Form>>& L) {
