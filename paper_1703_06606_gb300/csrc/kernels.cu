@@ -2685,10 +2685,11 @@ __global__ void __launch_bounds__(NT, 1) k_coarse_vcycle_smem(Prm<rf64> P, Coars
 // coupled sweeps on the coarsest) 1504 -> 630 us.  FP64: 8x16 .. 2x4 of the drop
 // 290 -> 246 us, a 128x256 projection step's group 719 -> 661 us, the 6x9
 // coupled group of 96x144 1640 -> 1438 us (the FP64 figures against a copy array
-// by array, the projection's against global memory).  What is left is one
-// warp's visit, about 1000 instructions, colour after colour; two warps that
-// shared a coupled visit (CH block, NS block) were slower, 23.8 -> 24.6 ms for
-// two served steps.
+// by array, the projection's against global memory).  What is left is the
+// chain of one warp's visit, colour after colour: per instruction issued it
+// waits 1.2 cycles for a result in FP32 and 7.8 in FP64 (0.2 for code).  Two
+// warps that shared a coupled visit (CH block; NS block and solve, the longer
+// chain) were slower, 23.8 -> 24.6 ms for two served steps.
 // --------------------------------------------------------------------------
 // array OFF of records of N values at b: element k as if it were a plain array
 template <typename T, int OFF, int N>
