@@ -1976,6 +1976,22 @@ struct TeamSolve {
     pr = (r4 + ih * tg) * iden;
     return y - z * (v3 * tg + ga * pr);
   }
+  // the same for the transposed system: B transposed, the pressure column
+  // -w/h, the pressure row a w (a = 1/(M h)); ap0, ap1 as in the constructor.
+  // Sherman-Morrison's g and the pivot of p are the system's own.
+  __device__ __forceinline__ T apply_t(T rq, T r4, bool ap0, bool ap1, T a, T& pr) const {
+    T rqo = shfl_xor(rq, 1);
+    T r0 = odd ? rqo : rq, r1 = odd ? rq : rqo;
+    T y = ((odd ? B00 : B11) * (odd ? r1 : r0) - (odd ? B01 : B10) * (odd ? r0 : r1)) * idet;
+    T zn = odd ? ((ap1 ? B00 : T(0)) + (ap0 ? B01 : T(0))) : ((ap0 ? B11 : T(0)) + (ap1 ? B10 : T(0)));
+    T zt = (odd ? -zn : zn) * idet;
+    T tdot = odd ? -y : y;
+    tdot += shfl_xor(tdot, 1);
+    tdot += shfl_xor(tdot, 2);
+    const T tg = tdot * g;
+    pr = (r4 - a * tg) * iden;
+    return y - zt * (v3 * tg - ih * g * pr);
+  }
 };
 
 // Vanka block of cell (i,j) by a team of four lanes (lane & 3 = q): lane q
@@ -2137,9 +2153,9 @@ __device__ __forceinline__ void vanka4_team(const Prm<T>& P, const LV& L, int i,
 // edge and face W, E, S, N).  Lane q builds momentum row q, face q's terms of
 // the mass row, of N_c, N_mu and of the CH Jacobian's face sums, and the
 // couplings of edge q; butterflies add the face terms and every lane forms
-// the cell terms.  The solve follows solve_coupled7: the NS block's
-// structured solve (TeamSolve) applied to three right-hand sides, then the
-// 2x2 Schur system for (dc, dmu).  Lane q writes edge q, lane 0 c, mu, p.
+// the cell terms.  The solve is solve_coupled7's by the NS block's structured
+// solve (TeamSolve): the 2x2 Schur system for (dc, dmu), then the NS unknowns.
+// Lane q writes edge q, lane 0 c, mu, p.
 template <typename T, class Form, class LV>
 __device__ __forceinline__ void coupled_team(const Prm<T>& P, const LV& L, int i, int j, bool ok,
                                              T omega) {
@@ -2174,18 +2190,21 @@ __device__ __forceinline__ void coupled_team(const Prm<T>& P, const LV& L, int i
   T b01, b10;
   pair_couplings<T, Form>(L, d, k, vc, b01, b10);
   TeamSolve<T> ts(L, q, dq, d ? a2 : a0, d ? a3 : a1, b01, b10, vc, A44);
-  T p0, p1, p2;
-  T x0 = ts.apply(bq, b4, p0);
-  T x1 = ts.apply(cq0, T(0), p1);
-  T x2 = ts.apply(cq1, diffc, p2);
-  T S00 = J11 - (team_sum<T>(gm * x1) + diffc * p1);
-  T S01 = J12 - (team_sum<T>(gm * x2) + diffc * p2);
-  T rhs0 = Rc - (team_sum<T>(gm * x0) + diffc * p0);
+  // The Schur system of (dc, dmu) needs the CH row's products with the solved
+  // columns, g^T A_NS^-1 r for three r: one transposed solve gives g^T A_NS^-1,
+  // and one solve with the whole right-hand side then the NS unknowns (FP64
+  // instructions, which bound the visit: 53 where three solves took 63; 96x144
+  // coupled, three steps 19.6 -> 19.3 ms)
+  T gp;
+  const T gx = ts.apply_t(gm, diffc, d ? a2 : a0, d ? a3 : a1, L.k.ihM, gp);
+  T S00 = J11 - team_sum<T>(gx * cq0);
+  T S01 = J12 - (team_sum<T>(gx * cq1) + diffc * gp);
+  T rhs0 = Rc - (team_sum<T>(gx * bq) + b4 * gp);
   T id2 = qrcp(S00 * J22 - S01 * J21);
   T dc = (J22 * rhs0 - S01 * Rm) * id2;
   T dm = (S00 * Rm - J21 * rhs0) * id2;
-  T x = x0 - x1 * dc - x2 * dm;
-  T pr = p0 - p1 * dc - p2 * dm;
+  T pr;
+  T x = ts.apply(bq - cq0 * dc - cq1 * dm, b4 - diffc * dm, pr);
   if (!ok) return;
   const bool ghosts = has_ghosts(L, i, j);
   const T xn = L.pair(d, L.u, L.v)[ke] - omega * x, pn = L.p[k] - omega * pr;
