@@ -205,27 +205,27 @@ __global__ void __launch_bounds__(FIN_NT) k_finalize(const double* part, int npa
 // bounds the kernels that evaluate it): sums over the four faces of unscaled
 // differences, scaled once by the level's constants.
 // sum over the faces of (m(c^n) of both cells) (d mu + alpha d p): 2 h^2 Pe
-// times the diffusion of N_c
+// times the diffusion of N_c.  Differences of mu and of p first: those of
+// mu + alpha p would round at alpha p's own size, 20 to 300 times the error on
+// 64 to 1024 cells across, and grow as 1/h^2 in the row.
 template <typename T, class LV>
 __device__ __forceinline__ T flux_sum(const Prm<T>& P, const LV& L, int k) {
   const int W = L.pitch;
   auto mob = L.mobn; auto mu = L.mu; auto p = L.p;
   const int off[4] = {1, -1, W, -W};
-  T mk = mob[k], s = T(0);
-  if constexpr (sizeof(T) == 8) {
-    T fk = mu[k] + P.alpha * p[k];
+  T mk = mob[k], s = T(0), sp = T(0);
 #pragma unroll
-    for (int f = 0; f < 4; ++f) {
-      int q = k + off[f];
-      s += (mk + mob[q]) * (mu[q] + P.alpha * p[q] - fk);
-    }
-  } else {  // differences first: the sums would round at the fields' own size
-#pragma unroll
-    for (int f = 0; f < 4; ++f) {
-      int q = k + off[f];
-      s += (mk + mob[q]) * ((mu[q] - mu[k]) + P.alpha * (p[q] - p[k]));
+  for (int f = 0; f < 4; ++f) {
+    int q = k + off[f];
+    T m = mk + mob[q], dmu = mu[q] - mu[k], dp = p[q] - p[k];
+    if constexpr (sizeof(T) == 8) {  // the two fields' sums apart: alpha once, one rounding a face less
+      s += m * dmu;
+      sp += m * dp;
+    } else {
+      s += m * (dmu + P.alpha * dp);
     }
   }
+  if constexpr (sizeof(T) == 8) s += P.alpha * sp;
   return s;
 }
 // the advection (e1e2) of N_c
@@ -420,7 +420,7 @@ static int residual_rows(const Lv<T>& L) {
 // ch_system for the full iterate (PROJ: the projection method's form), with the
 // constants and the terms
 // common to the residuals and the Jacobian folded (chem_full's notation; E =
-// K ((F + F^n)/2) + (Lam/4) Gbar): about 115 FP64 instructions where the
+// K ((F + F^n)/2) + (Lam/4) Gbar): about 119 FP64 instructions where the
 // unfolded sums take about 190.  On a wall face the ghost's c and c^n are the
 // cell's own, so its differences vanish and only the coefficients of c (2 rho
 // sums) and the mobilities need the face left out.
@@ -433,14 +433,15 @@ __device__ __forceinline__ void ch_system_full(const Prm<T>& P, const LV& L, int
   const bool wall[4] = {!L.px && i == L.m1, !L.px && i == 1, j == L.m2, j == 1};
   auto c = L.c; auto cn = L.cn; auto rn = L.rhon; auto rc = L.rhoc; auto mob = L.mobn; auto mu = L.mu; auto p = L.p;
   T ck = c[k], cnk = cn[k], rk = rc[k], rnk = rn[k], muk = mu[k];
-  T mk = mob[k], fk = muk + P.alpha * p[k];
+  T mk = mob[k], pk = p[k];
   T S = rk + rnk, ch = ck + cnk;
-  T flux = T(0), sm = T(0), G2 = T(0), sd = T(0), div = T(0), SD = T(0), SW = T(0);
+  T flux = T(0), fluxp = T(0), sm = T(0), G2 = T(0), sd = T(0), div = T(0), SD = T(0), SW = T(0);
 #pragma unroll
   for (int f = 0; f < 4; ++f) {
     const int q = k + off[f];
     T m = mk + mob[q], cq = c[q];
-    flux += m * (mu[q] + P.alpha * p[q] - fk);
+    flux += m * (mu[q] - muk);  // flux_sum's two sums
+    fluxp += m * (p[q] - pk);
     T d = cq - ck, D = (cq + cn[q]) - ch, H = rc[q] + rn[q];
     G2 += d * d;
     sd += d;
@@ -452,6 +453,7 @@ __device__ __forceinline__ void ch_system_full(const Prm<T>& P, const LV& L, int
   const int open = 4 - (wall[0] + wall[1] + wall[2] + wall[3]);
   SW += (open == 4 ? T(4) : open == 3 ? T(3) : open == 2 ? T(2) : open == 1 ? T(1) : T(0)) * S;
   div += S * SD;
+  flux += P.alpha * fluxp;
   T dck = ck - cnk, ar = -P.alpha * rk, drho = ar * rk, r = ar * rnk;
   T dr = -P.alpha * rnk * drho;
   T A = ck * ck - ck, An = cnk * cnk - cnk, sA = A + An, t = ch - T(1), g4 = sA * t;
@@ -718,7 +720,7 @@ __device__ __forceinline__ ChRows<T> ch_team_rows_full(const Prm<T>& P, const LV
     wq = proj_face_team(P, L, k, q, open, rk, rq);
     rw = rq * wq;
   }
-  T v[8] = {m * (L.mu[nq] + P.alpha * L.p[nq] - (muk + P.alpha * L.p[k])),
+  T v[8] = {m * ((L.mu[nq] - muk) + P.alpha * (L.p[nq] - L.p[k])),  // differences first (flux_sum)
             open ? m : T(0),
             PROJ ? rw * ((q & 1) ? dq : -dq) : gq * L.pair(d, L.u, L.v)[kf],
             dq * dq,
