@@ -309,8 +309,8 @@ __device__ __forceinline__ Rows5<T> residual_rows5(const Prm<T>& P, const LV& L,
       if constexpr (PROJ) n[1] += (L.rhon[k] - rk) * L.mu[k];  // rho^n in front of mu
     }
     if constexpr (UV) {
-      n[3] = mom_asm<!PROJ>(L, 0, k, rk + rq[0]);
-      n[4] = mom_asm<!PROJ>(L, 1, k, rk + rq[2]);
+      n[3] = full_mom_row<PROJ>(L, 0, k, rk + rq[0]);
+      n[4] = full_mom_row<PROJ>(L, 1, k, rk + rq[2]);
     }
   }
   Rows5<T> X;
@@ -920,11 +920,11 @@ __device__ __forceinline__ void vanka_system(const Prm<T>& P, const LV& L, int i
     const T rk = Form::rho(P, L, k);
     const T rs[4] = {Form::rho(P, L, k - 1) + rk, rk + Form::rho(P, L, k + 1),
                      Form::rho(P, L, k - W) + rk, rk + Form::rho(P, L, k + W)};
-    constexpr bool PST = std::is_same<Form, FullForm>::value;
+    constexpr bool PROJ = std::is_same<Form, ProjForm>::value;
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       A[q][q] = L.pair(q >> 1, L.Dgu, L.Dgv)[ke[q]] + L.k.qidt * rs[q];  // per-step coefficients
-      rows[q] = mom_asm<PST>(L, q >> 1, ke[q], rs[q]);
+      rows[q] = full_mom_row<PROJ>(L, q >> 1, ke[q], rs[q]);
     }
     const T v1 = vis[k] * L.k.v1, sx = L.k.hih * L.Sx[k], sy = L.k.hih * L.Sy[k];
     A[0][1] = sx - v1 - v3;
@@ -1881,7 +1881,7 @@ struct CoarseLevels {
 // Vanka block (one edge row each).
 // --------------------------------------------------------------------------
 // N - f of the momentum row in direction d (0: the x row, unknown u; 1:
-// the y row, unknown v) at edge index k: mom_asm, or err_row for ErrForm, from
+// the y row, unknown v) at edge index k: full_mom_row, or err_row for ErrForm, from
 // rho(c) of the edge's two cells; kf is the index of its right-hand side.  Both
 // directions run the same instructions on different arrays and strides (s
 // along the edge normal, t across it).
@@ -1892,7 +1892,7 @@ __device__ __forceinline__ T mom_residual(const Prm<T>& P, const LV& L, int d, i
   if constexpr (std::is_same<Form, ErrForm>::value)
     return err_row(P, L, d, k, l.r + r.r, l.d + r.d) - f;
   else
-    return mom_asm<std::is_same<Form, FullForm>::value>(L, d, k, l.r + r.r) - f;
+    return full_mom_row<std::is_same<Form, ProjForm>::value>(L, d, k, l.r + r.r) - f;
 }
 
 // Diagonal entry dq and residual bq = N - f (0 on a wall edge) of momentum row
@@ -2761,17 +2761,27 @@ struct Fld {
 #define QN_ERR_ARRAYS(X)                                                                       \
   QN_COMMON_ARRAYS(X) X(T1u) X(T1v) X(aPu) X(aPv) X(aMu) X(aMv) X(tPu) X(tPv) X(tMu) X(tMv)    \
   X(Bc) X(Bmu) X(Bu) X(Bv) X(Bdc) X(rB)
-// full iterate: rho(c), the rows' stencils, their diagonals and couplings
+// full iterate: rho(c), the rows' stencils, their diagonals and couplings; the
+// projection method's rows hold their flux coefficients instead
 #define QN_FULL_ARRAYS(X)                                                                      \
   QN_COMMON_ARRAYS(X) X(T0u) X(T0v) X(Cu) X(Cv) X(aPu) X(aPv) X(aMu) X(aMv) X(tPu) X(tPv)      \
   X(tMu) X(tMv) X(M0u) X(M0v) X(M1u) X(M1v) X(Dgu) X(Dgv) X(Sx) X(Sy) X(rhoc)
+#define QN_PROJ_ARRAYS(X)                                                                      \
+  QN_COMMON_ARRAYS(X) X(T0u) X(T0v) X(T1u) X(T1v) X(Dgu) X(Dgv) X(Sx) X(Sy) X(Qx) X(Qy) X(Av)  \
+  X(rhoc)
 QN_RECORD_LEVEL(LvErr, QN_ERR_ARRAYS, false);
 QN_RECORD_LEVEL(LvFull, QN_FULL_ARRAYS, true);
+QN_RECORD_LEVEL(LvProj, QN_PROJ_ARRAYS, true);
 
 template <class Form>
-struct RecordOf {  // FullForm, ProjForm
+struct RecordOf {  // FullForm
   template <typename T> using level = LvFull<T>;
   static constexpr int values = LvFull<rf64>::N;
+};
+template <>
+struct RecordOf<ProjForm> {
+  template <typename T> using level = LvProj<T>;
+  static constexpr int values = LvProj<rf64>::N;
 };
 template <>
 struct RecordOf<ErrForm> {
@@ -2824,6 +2834,8 @@ __global__ void __launch_bounds__(NT, 1) k_coarse_records(Prm<T> P,
 #define QN_RECORD_IN(m) record_in(r + R::I_##m, L.m + g);
       if constexpr (std::is_same<Form, ErrForm>::value) {
         QN_ERR_ARRAYS(QN_RECORD_IN)
+      } else if constexpr (std::is_same<Form, ProjForm>::value) {
+        QN_PROJ_ARRAYS(QN_RECORD_IN)
       } else {
         QN_FULL_ARRAYS(QN_RECORD_IN)
       }

@@ -118,3 +118,44 @@ def test_flux_of_the_ch_visit(qn, px, team):
     own = (i + j) % 2 == 0
     assert np.all(abs(g["c"].astype(LD) - (1 - dc))[own] <= bc[own])
     assert np.all(abs(g["mu"].astype(LD) - (mu - dm))[own] <= bm[own])
+
+
+@pytest.mark.parametrize("m2", [32, 64])
+def test_rows_of_the_intermediate_velocity(qn, m2):
+    """The projection method's momentum rows from rest (no convection) with
+    density and viscosity uniform: rho x / dt and the viscous fluxes, away from
+    the walls.  The time term takes at most 6 roundings, a viscous flux 8 from its
+    difference to the row."""
+    m1, a = 1024, (1.0 - 0.01) / 0.01
+    s = qn.Solver(m1, m2, periodic_x=True, scheme=1, levels=1, **KW)
+    f = resting(m1, m2)
+    s.set_fields(f)
+    s.begin_step(1.0)
+    x, y = np.arange(m1 + 1) / m1, (np.arange(m2) + 0.5) / m1
+    f["u"] = np.sin(2 * np.pi * x + 0.3)[None, :] * np.cos(3.0 * y)[:, None]
+    f["u"][:, 0] = f["u"][:, m1]
+    f["v"][1:-1] = (np.cos(2 * np.pi * (x[1:] - 0.5 / m1) + 0.4)[None, :]
+                    * np.sin(3.0 * np.arange(1, m2) / m1 + 0.2)[:, None])
+    s.set_iterate(f)
+    r, _ = s.residual()
+    s.close()
+    rho, hv = LD(1.0 / (a + 1.0)), LD(0.1) * LD(m1) ** 2
+    u, v = f["u"][:, 1:].astype(LD), f["v"].astype(LD)  # u of edges 1 .. m1
+
+    def row(c, dr, dl, dp, dm, br, bl):
+        n = rho * c - hv * ((dr - dl) + (dp - dm) + ((dr + br) - (dl + bl)) / 3)
+        size = abs(dr) + abs(dl) + abs(dp) + abs(dm) + (abs(dr) + abs(br) + abs(dl) + abs(bl)) / 3
+        return n, U * (6 * rho * abs(c) + 8 * hv * size)
+
+    east, west = np.roll(u, -1, 1), np.roll(u, 1, 1)
+    b = v[1:] - v[:-1]  # v across the cells of each row
+    i = slice(1, -1)    # rows away from the walls
+    n, tol = row(u[i], (east - u)[i], (u - west)[i], u[2:] - u[i], u[i] - u[:-2],
+                 np.roll(b, -1, 1)[i], b[i])
+    assert np.all(abs(r["u"][i, 1:].astype(LD) + n) <= tol)
+    i = slice(2, -2)
+    c = v[i]
+    b = u - west        # u across the cells of each row
+    n, tol = row(c, v[3:-1] - c, c - v[1:-3], (np.roll(v, -1, 1) - v)[i], (v - np.roll(v, 1, 1))[i],
+                 b[2:-1], b[1:-2])
+    assert np.all(abs(r["v"][i].astype(LD) + n) <= tol)
