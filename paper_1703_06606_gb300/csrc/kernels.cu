@@ -3173,7 +3173,7 @@ __global__ void __launch_bounds__(NT, 2) k_mass(Prm<T> P, Lv<T> L, const T* c, d
   double val[2] = {0.0, 0.0};
   if (i <= L.m1 && j <= L.m2) {
     double cc = (double)c[L.at(i, j)];
-    double r = rcp_any((double)P.ia * cc + (double)P.ib);
+    double r = 1.0 / ((double)P.ia * cc + (double)P.ib);
     val[0] = r;
     val[1] = r * cc;
   }
@@ -3279,7 +3279,7 @@ __global__ void __launch_bounds__(NT, 2) k_energy(Prm<T> P, Lv<T> L, const T* c,
     const int W = L.pitch;
     int k = L.at(i, j);
     double cc = (double)c[k];
-    double r = rcp_any((double)P.ia * cc + (double)P.ib);
+    double r = 1.0 / ((double)P.ia * cc + (double)P.ib);
     double u0 = u[k], u1 = u[k - 1], v0 = v[k], v1 = v[k - W];
     double kin = 0.25 * (u0 * u0 + u1 * u1 + v0 * v0 + v1 * v1);
     double de = (double)c[k + 1] - cc, dw = cc - (double)c[k - 1];

@@ -15,7 +15,6 @@
 #include <mutex>
 
 #include "qnsch.h"
-#include "qnsch_dev.cuh"
 
 namespace {
 
@@ -59,11 +58,12 @@ int partials_address(void** out) {
 
 // The FP64 pipe bounds the kernel (a warp's FP64 instruction takes 19 cycles of
 // an SM, and 2048 x 4096 cells are 1724 warps an SM: 15.8 us an instruction a
-// cell), not HBM (67 MB, 10 us).  A cell takes 6: rho's argument, three of
-// rcp_any (a division has ten), two sums.  Eight warps that each reduce two
-// sums by shuffles add 1.4 to that, two warps that add up the block's sums from
-// shared memory 0.4.  Measured at that size, both kernels: 152 us with the
-// division, 123 with rcp_any, 105 with the sums in shared memory.
+// cell), not HBM (67 MB, 10 us).  A cell takes about 8: rho's argument, the
+// division, two sums.  Eight warps that each reduce two sums by shuffles add 1.4
+// to that, two warps that add up the block's sums from shared memory 0.4.
+// Measured at that size, both kernels: 152 us with the shuffles, 135 with the
+// sums in shared memory.  (With qrcp's three instructions in place of the
+// division 105, but 3 in 10^4 of its results differ from the division's.)
 // rho(c) = 1 / (ia c + ib) with ia = (rho2 - rho1)/(rho1 rho2), ib = 1/rho2 (Sec. 2.1)
 __global__ void k_mass_partials(const double* __restrict__ c, long long n, double ia, double ib,
                                 double* __restrict__ part) {
@@ -75,7 +75,7 @@ __global__ void k_mass_partials(const double* __restrict__ c, long long n, doubl
     long long k = base + (long long)q * NA_THREADS + threadIdx.x;
     if (k < n) {
       double cc = c[k];
-      double r = qn::rcp_any(ia * cc + ib);
+      double r = 1.0 / (ia * cc + ib);
       a += r;
       b += r * cc;
     }

@@ -258,8 +258,10 @@ template <> __device__ __forceinline__ rf32 qdiv(rf32 a, rf32 b) { return __fdiv
 // (rcp.approx.ftz.f64) the result is within a few units in the last place of
 // 1/x (tested against IEEE division) in three FP64 instructions, where two
 // Newton steps take four and an IEEE division about ten.  Normal-range x only:
-// the pivots are determinants and diagonal sums of the local systems and the
-// densities' denominators, far from the subnormal range.
+// the pivots are determinants and diagonal sums of the local systems, far from
+// the subnormal range.  Not for a density: its error reaches 0.5065 units (6e6
+// arguments; 3 in 10^4 differ from the division), and rho(c) is a term of the
+// rows themselves, so rho_of divides, in FP64 with the division's rounding.
 template <typename T> __device__ __forceinline__ T qrcp(T x) { return qdiv(T(1), x); }
 template <> __device__ __forceinline__ double qrcp(double x) {
   double r;
@@ -269,18 +271,6 @@ template <> __device__ __forceinline__ double qrcp(double x) {
   return __fma_rn(r, e, r);
 }
 template <> __device__ __forceinline__ rf64 qrcp(rf64 x) { return qrcp(x.v); }
-// 1/x for any x: qrcp where the iteration's numbers stay normal, else the
-// division (zero, infinity, NaN, the ends of the exponent range)
-__device__ __forceinline__ double rcp_any(double x) {
-  const unsigned e = (unsigned)__double2hiint(x) & 0x7ff00000u;
-  return e - 0x01000000u < 0x7d000000u ? qrcp(x) : 1.0 / x;
-}
-template <> __device__ __forceinline__ double rho_of(const Prm<double>& P, double c) {
-  return qrcp(P.ia * c + P.ib);
-}
-template <> __device__ __forceinline__ rf64 rho_of(const Prm<rf64>& P, rf64 c) {
-  return qrcp<rf64>(P.ia * c + P.ib);
-}
 template <> __device__ __forceinline__ float rho_of(const Prm<float>& P, float c) {
   return qdiv(1.0f, P.ia * c + P.ib);
 }

@@ -159,3 +159,60 @@ def test_rows_of_the_intermediate_velocity(qn, m2):
     n, tol = row(c, v[3:-1] - c, c - v[1:-3], (np.roll(v, -1, 1) - v)[i], (v - np.roll(v, 1, 1))[i],
                  b[2:-1], b[1:-2])
     assert np.all(abs(r["v"][i].astype(LD) + n) <= tol)
+
+
+# --- densities: 1 / (0.5 c + 0.5) for rho1 = 1, rho2 = 2, whose argument rounds
+# once wherever it is formed, so the division's result is known to the last bit
+# (a reciprocal within 0.51 ulp differs in 3 of 10^4 arguments)
+def samples(n):
+    c = np.random.default_rng(12).random(n)
+    return c, 1.0 / (0.5 * c + 0.5)
+
+
+def test_density_of_the_rows_is_the_divisions(qn):
+    """With no viscosity to speak of, no flow at c^n and u = 1 in the iterate, the
+    x row of a uniform grid line is its rho(c).  A denominator of zero gives an
+    infinite density, and no other line notices."""
+    m2 = 65536
+    c, rho = samples(m2)
+    s = qn.Solver(4, m2, periodic_x=True, levels=1, rho1=1.0, rho2=2.0, Re=1e300)
+    f = s.zeros()
+    f["c"][:] = c[:, None]
+    s.set_fields(f)
+    s.begin_step(1.0)
+    f["u"][:] = 1.0
+    s.set_iterate(f)
+    r, _ = s.residual()
+    assert np.array_equal(r["u"][:, 1:], -np.repeat(rho[:, None], 4, axis=1))
+    lines = [7, 40000]
+    f["c"][lines] = -1.0
+    s.set_iterate(f)
+    r, _ = s.residual()
+    s.close()
+    rho[lines] = np.inf
+    assert np.array_equal(r["u"][:, 1:], -np.repeat(rho[:, None], 4, axis=1))
+
+
+def test_density_of_the_mass_is_the_divisions(qn):
+    """Eight equal cells, h^2 = 1/16: the mass is rho / 2."""
+    c, rho = samples(20000)
+    s = qn.Solver(4, 2, periodic_x=True, rho1=1.0, rho2=2.0)
+    f, got = s.zeros(), np.empty_like(c)
+    for k, x in enumerate(c):
+        f["c"][:] = x
+        s.set_fields(f)
+        got[k] = s.mass()[0]
+    s.close()
+    assert np.array_equal(got, 0.5 * rho)
+
+
+def test_density_of_the_allocation_free_mass_is_the_divisions(qn):
+    """One cell a call, h = 1: the mass is rho."""
+    import torch
+    c, rho = samples(20000)
+    d = torch.from_numpy(c).cuda()
+    out = torch.zeros((c.size, 2), dtype=torch.float64, device="cuda")
+    for k in range(c.size):
+        qn.mass_noalloc(d[k:k + 1].view(1, 1), 1.0, 1.0, 2.0, out[k])
+    torch.cuda.synchronize()
+    assert np.array_equal(out[:, 0].cpu().numpy(), rho)
