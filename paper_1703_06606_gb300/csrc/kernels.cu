@@ -3194,11 +3194,12 @@ __device__ __forceinline__ double diag_v(const Lv<double>& L, const double* v, i
   if (j == 0 || j == L.m2) return 0.0;
   return v[L.at(i, j)];
 }
-// d_x u + d_y v of cell (i,j)
+// d_x u + d_y v of cell (i,j), by division: 1/h is itself rounded, which on a
+// third of the sizes up to 1024 is up to 1.4 times the error
 __device__ __forceinline__ double diag_div(const Lv<double>& L, const double* u, const double* v,
                                            int i, int j) {
-  return (diag_u(L, u, i, j) - diag_u(L, u, i - 1, j)) * L.ih +
-         (diag_v(L, v, i, j) - diag_v(L, v, i, j - 1)) * L.ih;
+  return (diag_u(L, u, i, j) - diag_u(L, u, i - 1, j)) / L.h +
+         (diag_v(L, v, i, j) - diag_v(L, v, i, j - 1)) / L.h;
 }
 
 // per cell: [0] |div|, [1] max(div, 0), [2] max(-div, 0) (block maxima), then

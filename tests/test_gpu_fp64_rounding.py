@@ -216,3 +216,21 @@ def test_density_of_the_allocation_free_mass_is_the_divisions(qn):
         qn.mass_noalloc(d[k:k + 1].view(1, 1), 1.0, 1.0, 2.0, out[k])
     torch.cuda.synchronize()
     assert np.array_equal(out[:, 0].cpu().numpy(), rho)
+
+
+@pytest.mark.parametrize("m1,m2,px", [(737, 5, False), (96, 144, True), (49, 1000, False)])
+def test_divergence_is_the_differences_divided_by_h(qn, m1, m2, px):
+    s = qn.Solver(m1, m2, periodic_x=px, levels=1)
+    rng = np.random.default_rng(3)
+    f = {k: rng.standard_normal(v.shape) for k, v in s.zeros().items()}
+    f["v"][[0, -1]] = 0.0
+    f["u"][:, 0] = f["u"][:, -1] if px else 0.0
+    if not px:
+        f["u"][:, -1] = 0.0
+    s.set_fields(f)
+    d = (f["u"][:, 1:] - f["u"][:, :-1]) / s.h + (f["v"][1:] - f["v"][:-1]) / s.h
+    assert np.array_equal(s.divergence(), d)
+    g = s.diagnostics()
+    s.close()
+    assert (g["div_max"], g["div_expansion"], g["div_compression"]) == (
+        np.max(abs(d)), max(d.max(), 0.0), max((-d).max(), 0.0))
