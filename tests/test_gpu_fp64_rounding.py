@@ -234,3 +234,25 @@ def test_divergence_is_the_differences_divided_by_h(qn, m1, m2, px):
     s.close()
     assert (g["div_max"], g["div_expansion"], g["div_compression"]) == (
         np.max(abs(d)), max(d.max(), 0.0), max((-d).max(), 0.0))
+
+
+def test_projection_constant_rounds_once(qn):
+    """From rest with density 1 and pressures of 0 and 1 in turn, the projected
+    velocity is dt / (M h) and nothing else: 1/h, 1/M and 1/dt as they are held,
+    their product rounded once."""
+    from fractions import Fraction
+    rng = np.random.default_rng(8)
+    for m1 in range(4, 124, 2):
+        dt, M = rng.uniform(1e-4, 1e-3), rng.uniform(0.01, 0.05)
+        s = qn.Solver(m1, 2, periodic_x=True, scheme=1, levels=1, M=M)
+        f = s.zeros()
+        f["c"][:] = 1.0
+        s.set_fields(f)
+        s.begin_step(dt)
+        f["p"][:, 1::2] = 1.0
+        s.set_iterate(f)
+        s.commit_step()
+        u = s.get_fields()["u"][:, 1:]
+        k = float(Fraction(1.0 / s.h) * Fraction(1.0 / M) / Fraction(1.0 / dt))
+        s.close()
+        assert np.array_equal(u, np.where(np.arange(m1) % 2, k, -k) + np.zeros((2, 1))), m1
