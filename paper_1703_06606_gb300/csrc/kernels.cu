@@ -20,12 +20,6 @@ constexpr int BX = 32, BY = 8, NT = BX * BY;
 // the type a kernel computes in for data of type T: with its contraction fixed
 template <typename T, class Form>
 using compute_t = Fused<T>;
-// the same bits as data of the kernel's type
-template <typename R, template <typename> class S, typename T>
-static inline const S<R>& as_compute(const S<T>& x) {
-  static_assert(sizeof(S<T>) == sizeof(S<R>), "one layout");
-  return reinterpret_cast<const S<R>&>(x);
-}
 
 static inline dim3 grid2(int nx, int ny) { return dim3((nx + BX - 1) / BX, (ny + BY - 1) / BY); }
 

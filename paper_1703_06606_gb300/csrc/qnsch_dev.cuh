@@ -14,6 +14,7 @@
 #include <cuda_runtime.h>
 
 #include <cmath>
+#include <cstring>
 #include <type_traits>
 
 namespace qn {
@@ -39,6 +40,17 @@ typedef Fused<double> rf64;
 static_assert(sizeof(rf32) == 4 && sizeof(rf64) == 8 && std::is_trivially_copyable<rf32>::value &&
                   std::is_trivially_copyable<rf64>::value,
               "the bits of a float and a double");
+// the same bits as an object of the kernel's type: a copy, since an object may
+// not be read as one of another class
+template <typename R, template <typename> class S, typename T>
+inline S<R> as_compute(const S<T>& x) {
+  static_assert(sizeof(S<T>) == sizeof(S<R>) && std::is_trivially_copyable<S<T>>::value &&
+                    std::is_trivially_copyable<S<R>>::value,
+                "one layout");
+  S<R> y;
+  std::memcpy(static_cast<void*>(&y), &x, sizeof(y));
+  return y;
+}
 #ifdef __CUDACC__
 #define QN_F __device__ __forceinline__
 QN_F float rn_add(float x, float y) { return __fadd_rn(x, y); }
