@@ -248,11 +248,13 @@ int qnsch_footprint(const qnsch_grid* grid, int precision, size_t* bytes);
    copy of those levels in shared memory, made at the start of the launch and
    written back at its end, wherever the copy fits the device's shared memory
    per block (392 bytes a padded cell: about 126 KB for the 8x16, 4x8 and 2x4
-   levels); 0 runs it from global memory.  The projection method's levels and
-   the error-equation levels (fuse_cells32; 172 bytes a padded cell in FP32)
-   do the same.  The same operators run on the same values, so the results are
-   the same.  Reading the key "coarse_smem_used" (get only) gives 1 if the
-   last fused launch of FP64 full-iterate levels ran on the copy.
+   levels); 0 runs it from global memory.  The projection method's levels (312
+   bytes) and the error-equation levels (fuse_cells32; 172 bytes in FP32, 344 in
+   FP64) do the same.  The same operators run on the same values, so the results
+   are the same bits.  Reading the key "coarse_smem_used" (get only) gives 1 if
+   the last fused launch ran on the copy, whatever its levels: a group whose
+   copy does not fit (FP32 groups that start at 32x32, say: 302 KB) runs from
+   global memory.
    pdl: 1 launches every kernel with programmatic dependent launch, so that
    a kernel is scheduled as its predecessor's blocks exit and waits on the GPU
    for the predecessor's results before touching memory (same results); 0

@@ -3672,7 +3672,7 @@ int launch_coarse_vcycle(const Prm<T>& P0, const Lv<T>* levels, int n, int nu1, 
       qlaunch(&k_coarse_records<R, Form, 256>, 1, 256, bytes, s, P, C, M, nu1, nu2, nuc, R(omega),
               coupled);
       ++g_launches;
-      return std::is_same<Form, ErrForm>::value ? 0 : 1;
+      return 1;
     }
   }
   if constexpr (std::is_same<Form, FullForm>::value && sizeof(T) == 8) {

@@ -73,10 +73,10 @@ void launch_predict(double* const x[5], double* const a[5], double* const b[5],
 // the V-cycle on levels[0..n-1] (levels[0] is its finest) in one launch: one
 // thread block (ctas = 1) or one thread-block cluster of ctas blocks, a size
 // coarse_cluster_blocks returned (team8: the FP64 full-iterate Vanka blocks use
-// eight lanes where a colour fits the group in one pass).  smem: an FP64
-// full-iterate group in one block runs on a shared-memory copy of its levels
-// where the copy fits (k_coarse_vcycle_smem, same results).  Returns 1 if it
-// ran on the shared-memory copy, else 0.
+// eight lanes where a colour fits the group in one pass).  smem: a group in one
+// block runs on a shared-memory copy of its levels where the copy fits
+// (k_coarse_records; k_coarse_vcycle_smem for eight lanes; same results).
+// Returns 1 if it ran on the shared-memory copy, else 0.
 template <typename T, class Form>
 int launch_coarse_vcycle(const Prm<T>& P, const Lv<T>* levels, int n, int nu1, int nu2, int nuc,
                          int kcol, T omega, int coupled, cudaStream_t s, int team8 = 0,
