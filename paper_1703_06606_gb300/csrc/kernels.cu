@@ -3665,7 +3665,9 @@ int launch_coarse_vcycle(const Prm<T>& P0, const Lv<T>* levels, int n, int nu1, 
   C.base = std::is_same<Form, ErrForm>::value;
   for (int l = 0; l < n; ++l) C.L[l] = as_compute<R>(level_consts(P0, levels[l]));
   constexpr int NT = sizeof(T) == 8 ? 256 : 512;
-  if (smem && ctas <= 1 && !team8) {  // on shared-memory records, where they fit
+  // eight lanes a block: the uncoupled FP64 primitive visits only (smooth_block)
+  const bool eight = team8 && !coupled && std::is_same<Form, FullForm>::value && sizeof(T) == 8;
+  if (smem && ctas <= 1 && !eight) {  // on shared-memory records, where they fit
     RecordPlan M = {};
     const size_t bytes = record_plan<T, Form>(levels, n, M);
     if (bytes) {
@@ -3677,7 +3679,7 @@ int launch_coarse_vcycle(const Prm<T>& P0, const Lv<T>* levels, int n, int nu1, 
   }
   if constexpr (std::is_same<Form, FullForm>::value && sizeof(T) == 8) {
     // eight-lane blocks read arrays that the records leave out: on a copy of all
-    if (smem && ctas <= 1 && team8) {
+    if (smem && ctas <= 1 && eight) {
       CoarseSmem M = {};
       const size_t bytes = coarse_smem_plan(levels, n, M);
       if (bytes) {

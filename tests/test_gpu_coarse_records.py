@@ -52,3 +52,26 @@ def test_records_match_global_memory_bitwise(qn, name, m1, m2, px, opts, used, p
     assert np.array_equal(out[0][0], out[1][0])
     for k in out[0][1]:
         assert np.array_equal(out[0][1][k], out[1][1][k]), k
+
+
+@pytest.mark.parametrize("m1,m2,px,opts", [
+    (64, 96, False, {"scheme": 1}), (48, 72, True, {"scheme": 1}),
+    (64, 96, False, {"precision": 1}), (64, 64, True, {"precision": 1, "coupled": 1}),
+    (64, 64, False, {"precision": 2}), (48, 72, False, {"coupled": 1})],
+    ids=["projection", "projection_periodic", "mixed", "mixed_coupled", "fp64_error", "coupled"])
+def test_eight_lanes_leave_other_visits_on_records(qn, m1, m2, px, opts):
+    """vanka_team8_max > 0 shapes the uncoupled FP64 primitive visits only: the
+    other groups' launch and results do not change with it."""
+    P = W.small_case(m1, m2, px)
+    out = []
+    for team8 in (0, 1 << 20):
+        s = qn.Solver(**P.create_kwargs(), vanka_team8_max=team8, **opts)
+        s.set_fields(P.fields())
+        s.begin_step(P.dt)
+        norms = s.vcycle()
+        assert s.get_option("coarse_smem_used") == 1
+        out.append((norms, s.get_iterate()))
+        s.close()
+    assert np.array_equal(out[0][0], out[1][0])
+    for k in out[0][1]:
+        assert np.array_equal(out[0][1][k], out[1][1][k]), k
