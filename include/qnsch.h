@@ -215,11 +215,11 @@ int qnsch_footprint(const qnsch_grid* grid, int precision, size_t* bytes);
    run the per-level Vanka launches with four lanes per 5x5 block (same
    arithmetic, shorter critical path when the colour leaves most of the GPU
    idle); ch_team_max does the same for the CH 2x2 Newton launches (four lanes
-   per cell, one face each); vanka_team_max32 for the Vanka launches on the
-   error-equation levels of the defect correction (precision 1 and 2), which
-   in FP64 (precision 2), and ch_team_max32 for their CH launches; FP32 error
-   levels (precision 1) run one lane per visit whatever these two say, which
-   measured as fast or faster at every size.
+   per cell, one face each).  vanka_team_max32 and ch_team_max32 are the two
+   thresholds of the error-equation levels of precision 2, which are FP64 too.
+   The FP32 error levels of precision 1 run one lane per visit whatever these
+   two say (measured as fast or faster at every size); they are still checked,
+   kept and reported.
    vanka_team_max and vanka_team_max32 also choose the four-lane launches of
    the coupled 7x7 block (coupled = 1).
    vanka_team8_max: FP64 full-iterate levels with at most this many cells per

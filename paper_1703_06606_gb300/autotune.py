@@ -41,8 +41,8 @@ CANDIDATES = {
     # single-lane FP64 Vanka launches split between one lane per block and
     # lane pairs (0: never, 1: by the cost model)
     "vanka_split": [0, 1],
-    # the fused coarse V-cycle of the FP64 levels on a shared-memory copy (1) or
-    # from global memory (0)
+    # the fused coarse V-cycle on a shared-memory copy of its levels (1) or from
+    # global memory (0)
     "coarse_smem": [1, 0],
     "ch_team_max": [4096, 0, 16384],
     "fuse_cells": [128, 32, 512, 4096],
@@ -74,14 +74,15 @@ CUTOFF = 20.0
 # (relative), so that timing noise does not move a knob
 MIN_GAIN = 0.005
 # the options that shape the launches of each precision (0 FP64, 1 mixed,
-# 2 FP64 error form: its error levels use the FP64 thresholds)
+# 2 FP64 error form: its error levels use the FP64 thresholds), less those the
+# solver class names as idle
 KNOBS = {
     0: ["vanka_team_max", "vanka_team8_max", "vanka_pair_max", "vanka_split", "ch_team_max",
         "fuse_cells", "fuse_ctas", "coarse_smem", "nu1", "nu2", "nu_coarse", "nu1_fine",
         "nu2_fine"],
-    1: ["vanka_team_max32", "ch_team_max32", "fuse_cells32", "fuse_ctas", "wave_cells32",
+    1: ["vanka_team_max32", "ch_team_max32", "fuse_cells32", "fuse_ctas", "coarse_smem", "wave_cells32",
         "wave_rows", "skew_cells32", "skew_rows", "nu1", "nu2", "nu_coarse", "nu1_fine", "nu2_fine"],
-    2: ["vanka_team_max32", "ch_team_max32", "fuse_cells", "fuse_ctas", "wave_cells32",
+    2: ["vanka_team_max32", "ch_team_max32", "fuse_cells", "fuse_ctas", "coarse_smem", "wave_cells32",
         "wave_rows", "skew_cells32", "skew_rows", "nu1", "nu2", "nu_coarse", "nu1_fine", "nu2_fine"],
 }
 
@@ -122,7 +123,9 @@ def tune(P, precision=0, coupled=0, scheme=0, steps=4, warmup=2, solver_cls=None
          candidates=None, rounds=2):
     """Coordinate descent over the launch-shape options of `precision`: each
     option in turn takes the candidate value with the shortest time per step,
-    the others held, for `rounds` passes or until nothing changes.  Returns
+    the others held, for `rounds` passes or until nothing changes.  Options that
+    solver_cls names as idle at the precision (IDLE_OPTIONS) keep their defaults:
+    their candidates are one program, which noise would tell apart.  Returns
     (best options, best seconds per step, every (options, seconds) measured)."""
     if solver_cls is None:
         from . import qnsch
@@ -131,6 +134,7 @@ def tune(P, precision=0, coupled=0, scheme=0, steps=4, warmup=2, solver_cls=None
     cand = dict(CANDIDATES, **(candidates or {}))
     base = {"precision": precision, "coupled": coupled, "scheme": scheme}
     best = {k: cand[k][0] for k in KNOBS[precision]}
+    idle = getattr(solver_cls, "IDLE_OPTIONS", {}).get(precision, ())
     seen = {}
 
     def measure(opts):
@@ -149,7 +153,7 @@ def tune(P, precision=0, coupled=0, scheme=0, steps=4, warmup=2, solver_cls=None
     for _ in range(rounds):
         changed = False
         for k in KNOBS[precision]:
-            for v in cand[k]:
+            for v in () if k in idle else cand[k]:
                 if v == best[k]:
                     continue
                 trial = dict(best, **{k: v})

@@ -150,6 +150,9 @@ class Solver:
     """One q-NSCH instance on the GPU (the handle of qnsch_create)."""
 
     FIELDS = ("c", "mu", "u", "v", "p")  # argument order of the C calls
+    # options that shape no launch at a precision (kept and reported, see
+    # include/qnsch.h): FP32 error levels run one lane per visit
+    IDLE_OPTIONS = {1: ("vanka_team_max32", "ch_team_max32")}
 
     def __init__(self, m1, m2, Lx=1.0, periodic_x=False, levels=0, rho1=1.0, rho2=1.0,
                  eta1=1.0, eta2=1.0, Re=100.0, We=10.0, Pe=100.0, Cn=0.01, Fr=math.inf,

@@ -35,7 +35,8 @@ from . import autotune, qnsch, workloads
 
 # Options for many simulations in flight at once (mixed precision, coupled
 # block), where the GPU is full and work, not one simulation's latency,
-# decides.  One lane per coupled block in the per-level launches: the
+# decides.  One lane per coupled block in the per-level launches, which FP32
+# error levels run anyway (the option shapes those of precision 2): the
 # four-lane teams repeat part of each visit on every lane.  Levels up to 2048
 # cells go into each simulation's single-block V-cycle, which holds one SM.
 # One smoothing step before the coarse-grid correction and two after it: more
