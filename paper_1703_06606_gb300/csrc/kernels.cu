@@ -541,7 +541,9 @@ __device__ __forceinline__ void ch_cell(const Prm<T>& P, const LV& L, int i, int
   put_cell(L, L.mu, i, j, ghosts, mnew);
 }
 
-// first cell i0 >= 1 of colour `colour` in row j and the stride between cells
+// Vanka colour of cell (i,j): (2i + j) mod 8 (c8: periodic x, m1 = 0 mod 4) or
+// (i + 2j) mod kcol (kcol = 5 with walls, the smallest divisor >= 5 of m1 otherwise).
+// First cell i0 >= 1 of colour `colour` in row j and the stride between cells
 // of that colour in the row; false if the row has none
 template <class LV>
 __device__ __forceinline__ bool colour_row(const LV& L, int colour, int j, int& i0, int& stride) {
@@ -1187,14 +1189,6 @@ __device__ __forceinline__ void coupled_cell(const Prm<T>& P, const LV& L, int i
   put_cell(L, L.mu, i, j, ghosts, mnew);
   put_edges(L, i, j, ghosts, act, w, e, so, n);
   put_cell(L, L.p, i, j, ghosts, pn);
-}
-
-// Vanka colour of cell (i,j): (2i + j) mod 8 (periodic x, m1 = 0 mod 4) or
-// (i + 2j) mod kcol (kcol = 5 with walls, the smallest divisor >= 5 of m1 otherwise)
-template <class LV>
-__device__ __forceinline__ int vanka_colour(const LV& L, int i, int j) {
-  typedef typename LV::real T;
-  return L.c8 ? (2 * i + j) & 7 : (i + 2 * j) % L.kcol;
 }
 
 // per-level smoother launches: one thread per cell of the colour, packed into
@@ -1940,7 +1934,6 @@ struct TeamSolve {
   template <class LV>
   __device__ __forceinline__ TeamSolve(const LV& L, int q, T dq, bool ap0, bool ap1, T b01, T b10,
                                        T vc, T A44, bool with_p = true) {
-    const unsigned FULL = 0xffffffffu;
     ih = L.ih;
     v3 = vc * L.k.v3;
     odd = q & 1;
@@ -1961,7 +1954,6 @@ struct TeamSolve {
     ga = with_p ? g * L.k.ihM : T(0);
   }
   __device__ __forceinline__ T apply(T rq, T r4, T& pr) const {
-    const unsigned FULL = 0xffffffffu;
     T rqo = shfl_xor(rq, 1);
     T r0 = odd ? rqo : rq, r1 = odd ? rq : rqo;
     T y = ((odd ? B00 : B11) * (odd ? r1 : r0) - (odd ? B10 : B01) * (odd ? r0 : r1)) * idet;
@@ -2001,7 +1993,7 @@ __device__ __forceinline__ void vanka_team(const Prm<T>& P, const LV& L, int i, 
                                            T omega) {
   const int W = L.pitch;
   const int q = threadIdx.x & 3, d = q >> 1;
-  const T ih = L.ih, ih2 = L.ih2;
+  const T ih = L.ih;
   int k = L.at(i, j);
   int eW = (L.px && i == 1) ? L.m1 : i - 1;
   int kW = L.at(eW, j);
@@ -2081,7 +2073,7 @@ __device__ __forceinline__ void vanka_team8(const Prm<T>& P, const LV& L, int i,
                                             T omega) {
   const int W = L.pitch;
   const int q = threadIdx.x & 3, d = q >> 1, half = (threadIdx.x >> 2) & 1;
-  const T ih = L.ih, ih2 = L.ih2;
+  const T ih = L.ih;
   int k = L.at(i, j);
   int eW = (L.px && i == 1) ? L.m1 : i - 1;
   int kW = L.at(eW, j);
@@ -2157,7 +2149,7 @@ __device__ __forceinline__ void coupled_team(const Prm<T>& P, const LV& L, int i
                                              T omega) {
   const int W = L.pitch;
   const int q = threadIdx.x & 3, d = q >> 1;
-  const T ih = L.ih, ih2 = L.ih2;
+  const T ih = L.ih;
   int k = L.at(i, j);
   int eW = (L.px && i == 1) ? L.m1 : i - 1;
   int kW = L.at(eW, j);
@@ -2287,7 +2279,7 @@ __device__ __forceinline__ void vanka_pair(const Prm<T>& P, const LV& L, int i, 
                                            T omega) {
   const int W = L.pitch;
   const int d = threadIdx.x & 1;
-  const T ih = L.ih, ih2 = L.ih2;
+  const T ih = L.ih;
   int k = L.at(i, j);
   int eW = (L.px && i == 1) ? L.m1 : i - 1;
   int kW = L.at(eW, j);
@@ -2583,7 +2575,7 @@ struct LevelsOf {
 
 template <typename T, class Form, int NT>
 __global__ void __launch_bounds__(NT, 1) k_coarse_vcycle(Prm<T> P, CoarseLevels<T> C, int nu1, int nu2,
-                                                      int nuc, int kcol, T omega, int coupled,
+                                                      int nuc, T omega, int coupled,
                                                       int team8) {
   pdl_enter();
   coarse_vcycle_body<T, Form>(P, LevelsOf<T>{C}, C.n, C.base, nu1, nu2, nuc, omega, coupled, team8);
@@ -3656,7 +3648,7 @@ void coarse_smem_prepare() {
 
 template <typename T, class Form>
 int launch_coarse_vcycle(const Prm<T>& P0, const Lv<T>* levels, int n, int nu1, int nu2, int nuc,
-                         int kcol, T omega, int coupled, cudaStream_t s, int team8, int ctas,
+                         T omega, int coupled, cudaStream_t s, int team8, int ctas,
                          int smem) {
   typedef compute_t<T, Form> R;
   const Prm<R>& P = as_compute<R>(P0);
@@ -3691,7 +3683,7 @@ int launch_coarse_vcycle(const Prm<T>& P0, const Lv<T>* levels, int n, int nu1, 
     }
   }
   if (ctas <= 1) {
-    qlaunch(&k_coarse_vcycle<R, Form, NT>, 1, NT, 0, s, P, C, nu1, nu2, nuc, kcol, omega, coupled,
+    qlaunch(&k_coarse_vcycle<R, Form, NT>, 1, NT, 0, s, P, C, nu1, nu2, nuc, omega, coupled,
             team8);
   } else {  // one cluster of ctas blocks (a size coarse_cluster_blocks accepted)
     cudaLaunchConfig_t cfg = {};
@@ -3707,7 +3699,7 @@ int launch_coarse_vcycle(const Prm<T>& P0, const Lv<T>* levels, int n, int nu1, 
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = g_pdl ? 2 : 1;
-    cudaLaunchKernelEx(&cfg, &k_coarse_vcycle<R, Form, NT>, P, C, nu1, nu2, nuc, kcol, omega,
+    cudaLaunchKernelEx(&cfg, &k_coarse_vcycle<R, Form, NT>, P, C, nu1, nu2, nuc, omega,
                        coupled, team8);
   }
   ++g_launches;
@@ -4079,7 +4071,7 @@ int partial_rows_needed(int m1, int m2) {
 }
 
 #define QN_INSTANTIATE_FORM(T, F)                                                                \
-  template int launch_coarse_vcycle<T, F>(const Prm<T>&, const Lv<T>*, int, int, int, int, int,   \
+  template int launch_coarse_vcycle<T, F>(const Prm<T>&, const Lv<T>*, int, int, int, int,        \
                                           T, int, cudaStream_t, int, int, int);                  \
   template void launch_coupled<T, F>(const Prm<T>&, const Lv<T>&, int, T, cudaStream_t, int);     \
   template void launch_residual<T, F>(const Prm<T>&, const Lv<T>&, double*, cudaStream_t);       \
@@ -4127,7 +4119,7 @@ template int launch_skew<double, ErrForm>(const Prm<double>&, const Lv<double>&,
 template void launch_residual<double, ProjForm>(const Prm<double>&, const Lv<double>&, double*,
                                                 cudaStream_t);
 template int launch_coarse_vcycle<double, ProjForm>(const Prm<double>&, const Lv<double>*, int, int,
-                                                    int, int, int, double, int, cudaStream_t, int,
+                                                    int, int, double, int, cudaStream_t, int,
                                                     int, int);
 template void launch_add_op<double, ProjForm>(const Prm<double>&, const Lv<double>&, cudaStream_t);
 template void launch_ch<double, ProjForm>(const Prm<double>&, const Lv<double>&, int, cudaStream_t,

@@ -79,7 +79,7 @@ void launch_predict(double* const x[5], double* const a[5], double* const b[5],
 // Returns 1 if it ran on the shared-memory copy, else 0.
 template <typename T, class Form>
 int launch_coarse_vcycle(const Prm<T>& P, const Lv<T>* levels, int n, int nu1, int nu2, int nuc,
-                         int kcol, T omega, int coupled, cudaStream_t s, int team8 = 0,
+                         T omega, int coupled, cudaStream_t s, int team8 = 0,
                          int ctas = 1, int smem = 0);
 // lets the shared-memory fused V-cycle use the device's opt-in shared memory
 // per block (call with the device current, outside stream capture)

@@ -710,7 +710,7 @@ void vcycle(qnsch_s* s, const std::vector<Lv<T>>& Ls, const Prm<T>& P, int l) {
                 (m == s->nlev - 1 ? coarse_sweeps(s) : s->nu1 + s->nu2);
     int q = prof_open(s, PK_COARSE, visits);
     s->coarse_smem_used = qn::launch_coarse_vcycle<T, Form>(
-        P, &Ls[l], s->nlev - l, s->nu1, s->nu2, coarse_sweeps(s), s->kcol, (T)s->omega, s->coupled,
+        P, &Ls[l], s->nlev - l, s->nu1, s->nu2, coarse_sweeps(s), (T)s->omega, s->coupled,
         s->stream, s->team8_max > 0 ? 1 : 0, s->fuse_ctas, s->coarse_smem);
     prof_close(s, q);
     return;
