@@ -760,9 +760,9 @@ def run_ours(args, rank, world, local_rank):
 # of the new c) and per residual cell (all five families; the mean of a launch
 # with norms and one without), as ncu counts them executed (add, mul = 1,
 # fma = 2) on the FP64 kernels with one lane per visit
-VANKA_FP64_FLOPS_PER_VISIT = 272.0
-CH_FP64_FLOPS_PER_VISIT = 180.0
-RESIDUAL_FP64_FLOPS_PER_CELL = 181.0
+VANKA_FP64_FLOPS_PER_VISIT = 276.0
+CH_FP64_FLOPS_PER_VISIT = 188.0
+RESIDUAL_FP64_FLOPS_PER_CELL = 184.0
 # dram__bytes_read.sum + dram__bytes_write.sum per launch of a timed kind (average
 # over its launches), from one ncu capture of the same kernel build (the
 # profiles/ file named beside it; cold-cache, serialised); a kind without a

@@ -377,7 +377,7 @@ __global__ void __launch_bounds__(NT, 2) k_residual(Prm<T> P, Lv<T> L, double* p
 // The rows of a cell by three threads (ROLE: the block's z), for levels that
 // leave most of the FP64 pipes idle: a thread's chain of FP64 instructions, 64
 // cycles each, is what such a launch takes, and the longest third is 50 of the
-// 134.  A role's blocks write its families' entries of the partials.
+// 137.  A role's blocks write its families' entries of the partials.
 template <typename T, int MODE, class Form, int ROLE>
 __device__ __forceinline__ void residual_role(const Prm<T>& P, const Lv<T>& L, double* part) {
   int i = blockIdx.x * BX + threadIdx.x + 1;
@@ -2690,11 +2690,11 @@ __global__ void __launch_bounds__(NT, 1) k_coarse_vcycle_smem(Prm<rf64> P, Coars
 // Measured (GB300, ncu, caches warm), FP32 error levels: 16x32 .. 2x4 of the
 // 256x512 drop 245 -> 84 us, 28x28 and 14x14 of a served 448x448 request (64
 // coupled sweeps on the coarsest) 1504 -> 630 us.  FP64: 8x16 .. 2x4 of the drop
-// 290 -> 246 us, a 128x256 projection step's group 719 -> 661 us, the 6x9
-// coupled group of 96x144 1640 -> 1438 us (the FP64 figures against a copy array
-// by array, the projection's against global memory).  What is left is the
+// 290 -> 250 us, a 128x256 projection step's group 796 -> 721 us, the 6x9
+// coupled group of 96x144 1618 -> 1435 us (the FP64 figures event-timed against
+// global memory).  What is left is the
 // chain of one warp's visit, colour after colour: per instruction issued it
-// waits 1.2 cycles for a result in FP32 and 7.8 in FP64 (0.2 for code).  Two
+// waits 1.2 cycles for a result in FP32 and 7.7 in FP64 (0.2 for code).  Two
 // warps that shared a coupled visit (CH block; NS block and solve, the longer
 // chain) were slower, 23.8 -> 24.6 ms for two served steps.
 // --------------------------------------------------------------------------

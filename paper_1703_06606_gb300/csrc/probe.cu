@@ -45,7 +45,7 @@
 //
 //   int qnsch_rcp_check(int n, const double* x, double* y_fast, double* y_ieee);
 //     host arrays of n doubles: y_fast = the FP64 reciprocal the block solves
-//     use (qrcp of qnsch_dev.cuh: Newton-Raphson from rcp.approx.ftz.f64),
+//     use (qrcp of qnsch_dev.cuh: one third-order step from rcp.approx.ftz.f64),
 //     y_ieee = 1.0 / x (IEEE division), both computed on the device.
 //     n in [1, 2^24]; allocates and frees 3 n doubles; synchronises.
 #include <cuda_runtime.h>

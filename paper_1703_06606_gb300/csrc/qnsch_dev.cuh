@@ -279,7 +279,7 @@ template <> __device__ __forceinline__ rf32 qdiv(rf32 a, rf32 b) { return __fdiv
 // e^3; started from the hardware's approximate reciprocal
 // (rcp.approx.ftz.f64) the result is within a few units in the last place of
 // 1/x (tested against IEEE division) in three FP64 instructions, where two
-// Newton steps take four and an IEEE division about ten.  Normal-range x only:
+// Newton steps take four and the division 1/x five.  Normal-range x only:
 // the pivots are determinants and diagonal sums of the local systems, far from
 // the subnormal range.  Not for a density: its error reaches 0.5065 units (6e6
 // arguments; 3 in 10^4 differ from the division), and rho(c) is a term of the

@@ -39,14 +39,17 @@ from . import autotune, qnsch, workloads
 # error levels run anyway (the option shapes those of precision 2): the
 # four-lane teams repeat part of each visit on every lane.  Levels up to 2048
 # cells go into each simulation's single-block V-cycle, which holds one SM.
+# (A group that starts at 32x32 is too large for its shared-memory records and
+# runs from global memory: the 64-drop batch takes 76.0 ms a batch step, with
+# groups from 512 cells, all on records, 71.5.)
 # One smoothing step before the coarse-grid correction and two after it: more
 # V-cycles per time step, fewer smoothing visits in all.  Measured on the
-# 64-drop batch, in ms per batch step: 114.2 with (nu1, nu2) = (2, 2); 101.6
-# with (1, 2); 111.6 with (1, 1); 111.7 with (2, 1); 107.9 with (1, 3).  Each
-# step starting from the quadratic extrapolation in time of the last three
-# states (predictor 2): 83.2 against 98.7 without and 89.3 with the linear
-# one (after 5 warm-up steps).  The FP64 defect correction still decides the
-# answer at the same tolerance.
+# 64-drop batch with earlier kernels, in ms per batch step: 114.2 with
+# (nu1, nu2) = (2, 2); 101.6 with (1, 2); 111.6 with (1, 1); 111.7 with (2, 1);
+# 107.9 with (1, 3).  Each step starting from the quadratic extrapolation in
+# time of the last three states (predictor 2): 83.2 against 98.7 without and
+# 89.3 with the linear one (after 5 warm-up steps).  The FP64 defect correction
+# still decides the answer at the same tolerance.
 THROUGHPUT_OPTIONS = {"fuse_cells32": 2048, "vanka_team_max32": 0, "nu1": 1, "nu2": 2,
                       "predictor": 2}
 
